@@ -124,9 +124,9 @@ GLEAM_API int gleam_dc_workspace_size(const gleam_dims* dims, uint64_t* bytes);
 GLEAM_API int gleam_dc_check_status(const gleam_dims* dims);
 
 /*
- * Which kernels the separable 3-D path uses for phase-encode extents (n1, n2): the number of rows RY a block
- * of the row-tile kernels holds (n1 = RY * BY; every pass over the workspace contiguous), or 0 when the pair
- * has no row-tile kernels and the general strided middle pass is used.  Informational.
+ * How the row-tile passes split phase-encode extents (n1, n2): the number of rows RY a block of the outer passes
+ * holds (n1 = RY * BY) where both axes have two register stages with a middle radix BY of at most 24, or 0
+ * otherwise (the same passes, with one row per block, single-stage rows or a middle radix of 32).  Informational.
  */
 GLEAM_API int32_t gleam_dc_rowtile_split(int32_t n1, int32_t n2);
 

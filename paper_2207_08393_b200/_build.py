@@ -26,6 +26,11 @@ def _groups():
     return sorted({int(g) for g in re.findall(r"GLEAM_GROUP == (\d+)", text)})
 
 
+def _tile_rows():
+    text = open(os.path.join(CSRC, "gleam_dc.cu")).read()
+    return sorted({int(r) for r in re.findall(r"GLEAM_TILE_R\((\d+)\)", text)})
+
+
 def _sources_digest():
     h = hashlib.sha256()
     for name in sorted(os.listdir(CSRC)):
@@ -54,11 +59,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
         obj = os.path.join(BUILD, "kernels_group%d.o" % g)
         jobs.append((["nvcc"] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +
                      ["-DGLEAM_GROUP=%d" % g, "-c", os.path.join(CSRC, "kernels_group.cu"), "-o", obj], obj))
-    npair = len(set(re.findall(r"GLEAM_PAIR_GROUP == (\d+)", open(os.path.join(CSRC, "pairs.def")).read())))
-    for g in range(npair):
-        obj = os.path.join(BUILD, "kernels_pairs%d.o" % g)
+        for name in ("mid", "axis"):
+            obj = os.path.join(BUILD, "kernels_%s%d.o" % (name, g))
+            jobs.append((["nvcc"] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +
+                         ["-DGLEAM_GROUP=%d" % g, "-c", os.path.join(CSRC, "kernels_%s.cu" % name), "-o", obj], obj))
+    for ry in _tile_rows():
+        obj = os.path.join(BUILD, "kernels_tile%d.o" % ry)
         jobs.append((["nvcc"] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +
-                     ["-DGLEAM_PAIR_GROUP=%d" % g, "-c", os.path.join(CSRC, "kernels_pairs.cu"), "-o", obj], obj))
+                     ["-DGLEAM_TILE_RY=%d" % ry, "-c", os.path.join(CSRC, "kernels_tile.cu"), "-o", obj], obj))
     for name in ("gleam_dc", "kernels_fused", "modl_cg"):
         obj = os.path.join(BUILD, name + ".o")
         jobs.append((["nvcc"] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +

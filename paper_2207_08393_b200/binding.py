@@ -306,7 +306,7 @@ def gleam_measure_fp32_peak(scratch, stream=None) -> float:
 
 
 def gleam_dc_rowtile_split(n1: int, n2: int) -> int:
-    """Rows per block of the row-tile kernels for phase-encode extents (n1, n2), 0 if the pair has none."""
+    """Rows per block of the row-tile passes for phase-encode extents (n1, n2) that split into two register stages."""
     return int(load_library().gleam_dc_rowtile_split(int(n1), int(n2)))
 
 

@@ -6,8 +6,9 @@
 namespace gleam {
 
 // RUN_PREPARE: only what depends on y and the mask alone (rank map, z table) is computed and left in
-// the workspace; RUN_APPLY: the step with those tables taken from the workspace as they are.
-enum { RUN_ALL = 0, RUN_PREPARE = 1, RUN_APPLY = 2 };
+// the workspace; RUN_APPLY: the step with those tables taken from the workspace as they are; RUN_ADJOINT: A^H y
+// (x and eta are ignored; the transforms of a zero image are left out).
+enum { RUN_ALL = 0, RUN_PREPARE = 1, RUN_APPLY = 2, RUN_ADJOINT = 3 };
 
 // out = x - eta A^H (A x - y)   (y == nullptr: out = x - eta A^H A x).  Validates its arguments,
 // enqueues on d->stream, returns GLEAM_OK or a GLEAM_ERR_* code.  check_only: the argument checks

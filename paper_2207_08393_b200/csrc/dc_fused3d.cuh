@@ -1,4 +1,4 @@
-// One persistent kernel for the separable 3-D path: the three passes of dc_rowtile.cuh run as a
+// One persistent kernel for the separable 3-D path: the three passes of the row-tile scheme (dc_tile.cuh) run as a
 // dataflow over readout slabs, so that the coil workspace of a slab lives in L2 between its passes
 // instead of streaming through HBM three times.
 //

@@ -1,0 +1,306 @@
+// Pass 2 of the row-tile scheme (dc_tile.cuh): radix-BY transform over the rows j of one k0 group, the k-space work
+// of the call, and the mirror image back, in place on the workspace.  One thread per kz column, the BY values in
+// registers, no exchange through shared memory.  Bound by HBM: 16 bytes per element, 10 log2 BY + 12 flop.
+#pragma once
+#include "dc_tile.cuh"
+
+namespace gleam {
+
+enum MidMode {
+    MID_SEP = 0,     // readout-invariant mask, no measurements (VJP, normal-equations form)
+    MID_SEP_Z = 1,   // readout-invariant mask and the table z of the measurements
+    MID_ADJ_Z = 2,   // A^H y: minus the table z alone, nothing is read from the workspace
+    MID_FULL = 3,    // 2-D problem with an arbitrary mask; measurements may be null
+    MID_ADJ_FULL = 4,
+    MID_FWD = 5,     // forward half alone (arbitrary 3-D masks: the readout axis follows)
+    MID_INV = 6,     // inverse half alone
+    MID_GRADY = 7    // forward half and the mask, written to k-space: last step of the forward operator A, 2-D
+};
+
+struct MidArgs {
+    cf* V; long long v_unit, v_slab, v_k0, v_j;
+    const float* mask;                        // MID_SEP*: (B,T,N1,NZ); MID_FULL*, MID_GRADY: (B,T,N1,NZ) or (B,T,NZ)
+    int mask_row;                             // MID_GRADY: the mask has one row per (b,t)
+    const cf* zin; const int* zidx;           // compact z table and rank map
+    const float* m2c; const int* zstart;      // squared mask weights by rank; (B,T,33) first rank of each k0 group
+    const cf* y; cf* ky_out;
+    float scale, scale2;                      // g / sqrt(N1 NZ) (times eta: MID_GRADY), 1 / (N1 NZ)
+    int C, T, n0, G, i0_start, NZ, zcap;
+    long long nunits;                         // B*C*T
+};
+
+// The kernel streams: what matters is how many columns are in flight, so the register bound leaves little beyond the
+// column itself (a prime radix also holds its sums and differences) and everything else the k-space work needs is
+// fetched late or staged in shared memory.  Without the bound the compiler keeps mask weights and addresses of the
+// whole column: 100 registers, 2 blocks per SM, 907 us for the middle pass of a 320 x 320 x 256 volume with 8 coils
+// instead of 510 us.
+template <int BY> constexpr int mid_blocks() {
+    constexpr bool prime = BY > 4 && smallest_odd_factor(BY) == BY && BY % 2 == 1;
+    constexpr int regs = ((prime ? 4 : 2) * BY + 24 + 7) / 8 * 8;
+    return cmin(8, cmax(1, 65536 / (256 * regs)));
+}
+
+template <int RY, int BY, int MODE>
+__global__ void __launch_bounds__(256, mid_blocks<BY>())
+mid_kernel(const MidArgs a) {
+    constexpr int N1 = RY * BY;
+    constexpr bool FORWARD = MODE != MID_INV && MODE != MID_ADJ_Z && MODE != MID_ADJ_FULL;
+    constexpr bool INVERSE = MODE != MID_FWD && MODE != MID_GRADY;
+    constexpr bool Z = MODE == MID_SEP_Z || MODE == MID_ADJ_Z;
+    constexpr bool FULL = MODE == MID_FULL || MODE == MID_ADJ_FULL;
+    const int NZ = a.NZ;
+    const int kz = blockIdx.y * blockDim.x + threadIdx.x;          // gridDim.y covers NZ
+    const bool col_ok = kz < NZ;
+    const unsigned blk = blockIdx.x;                               // (unit, gi, k0)
+    const int k0 = (int)(blk % RY);
+    const unsigned gi = (blk / RY) % (unsigned)a.G;
+    const unsigned unit = blk / (RY * (unsigned)a.G);
+    const unsigned bc = unit / (unsigned)a.T;
+    const int t = (int)(unit - bc * (unsigned)a.T);
+    const int b = (int)(bc / (unsigned)a.C);
+    const long long bt = (long long)b * a.T + t;
+    const long long pe = (long long)N1 * NZ;
+    cf* Vp = a.V + unit * a.v_unit + gi * a.v_slab + k0 * a.v_k0 + kz;
+    __shared__ cf s_tw[BY];                                        // w_N1^(j k0)
+    if ((int)threadIdx.x < BY) s_tw[threadIdx.x] = unit_root_fwd<N1>(((int)threadIdx.x * k0) % N1);
+    // Each half of the kernel reads the twiddles for itself (volatile: a value kept from the first half to the second
+    // would cost 2 BY registers).
+    const unsigned tw_addr = (unsigned)__cvta_generic_to_shared(s_tw);
+    auto twiddle = [&](int j) -> cf {
+        cf w;
+        asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];" : "=f"(w.x), "=f"(w.y) : "r"(tw_addr + 8u * j));
+        return w;
+    };
+
+    // The z values of this block's ky group are contiguous in the compact table (ranks zstart[k0] .. zstart[k0+1]);
+    // they are staged in shared memory while the transform runs, with their scaled squared mask weights.  Slot zcap
+    // holds zero for the unsampled entries, which keeps the update free of branches.
+    extern __shared__ __align__(16) float2 mid_smem[];
+    cf* s_z = reinterpret_cast<cf*>(reinterpret_cast<float*>(mid_smem) + BY * blockDim.x);    // behind the slots of the threads
+    float* s_w = reinterpret_cast<float*>(s_z + a.zcap + 1);
+    int z_first = 0;
+    bool z_staged = false;
+    if (Z) {
+        z_first = a.zstart[bt * 33 + k0];
+        const int nz = a.zstart[bt * 33 + k0 + 1] - z_first;
+        z_staged = nz <= a.zcap;
+        if (z_staged) {
+            const cf* zsrc = a.zin + ((long long)unit * a.n0 + a.i0_start + (int)gi) * pe + z_first;
+            const float* wsrc = a.m2c + bt * pe + z_first;
+            for (int e = threadIdx.x; e < nz; e += blockDim.x) cp_async8(&s_z[e], zsrc + e);
+            cp_async_commit();
+            if (MODE == MID_SEP_Z) for (int e = threadIdx.x; e < nz; e += blockDim.x) s_w[e] = wsrc[e] * a.scale2;
+            if (threadIdx.x == 0) { s_z[a.zcap] = make_float2(0.f, 0.f); s_w[a.zcap] = 0.f; }
+        }
+    }
+    // What the k-space work of this column needs is copied to shared memory while the transform runs, into slots of the
+    // thread's own: mask weights (MID_SEP), ranks among the sampled positions (with z), weights and measurements
+    // (arbitrary mask; measurements at unsampled positions are not read, they may hold anything).
+    const int s2 = shift_half(kz, NZ);
+    const int TH = blockDim.x;
+    float* s_m = reinterpret_cast<float*>(mid_smem) + threadIdx.x;
+    cf* s_y = reinterpret_cast<cf*>(reinterpret_cast<float*>(mid_smem) + BY * TH) + threadIdx.x;
+    // centred ky of the raw index k0 + RY k1; an even BY turns the half shift into a rotation of k1
+    auto centred = [&](int k1) { return BY % 2 == 0 ? k0 + RY * ((k1 + BY / 2) % BY) : shift_half(k0 + RY * k1, N1); };
+    if (MODE == MID_SEP && col_ok) {
+        const float* mk = a.mask + bt * pe + s2;
+#pragma unroll
+        for (int k1 = 0; k1 < BY; ++k1) cp_async4(s_m + k1 * TH, mk + centred(k1) * NZ);
+        cp_async_commit();
+    }
+    if (Z && col_ok) {
+        const int* zi = a.zidx + bt * pe + (long long)k0 * NZ + kz;
+#pragma unroll
+        for (int k1 = 0; k1 < BY; ++k1) cp_async4(s_m + k1 * TH, zi + RY * k1 * NZ);
+        cp_async_commit();
+    }
+    cf c[BY];
+    if (col_ok && (FORWARD || MODE == MID_INV)) {
+        const cf* p = Vp;
+#pragma unroll
+        for (int j = 0; j < BY; ++j) { c[j] = *p; p += a.v_j; }
+    }
+    if (FULL && col_ok) {
+        const float* mk = a.mask + bt * pe + s2;
+        const cf* yy = a.y + (long long)unit * pe + s2;
+#pragma unroll
+        for (int k1 = 0; k1 < BY; ++k1) {
+            const int off = centred(k1) * NZ;
+            const float m = mk[off];
+            s_m[k1 * TH] = m;
+            if (a.y && m != 0.f) cp_async8(s_y + k1 * TH, yy + off);
+        }
+        cp_async_commit();
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    if (!col_ok) return;
+    if (FORWARD) {
+        if (RY > 1) {
+#pragma unroll
+            for (int j = 1; j < BY; ++j) c[j] = cmul(c[j], twiddle(j));
+        }
+        Dft<BY, -1>::run(c);
+    }
+    if (MODE == MID_SEP) {
+#pragma unroll
+        for (int k1 = 0; k1 < BY; ++k1) { const float m = s_m[k1 * TH]; c[k1] = cscale(c[k1], m * m * a.scale2); }
+    } else if (Z) {
+        const int* zi = reinterpret_cast<const int*>(s_m);
+        const cf* zz = a.zin + ((long long)unit * a.n0 + a.i0_start + (int)gi) * pe;
+        const float* m2 = a.m2c + bt * pe;
+#pragma unroll
+        for (int k1 = 0; k1 < BY; ++k1) {
+            const int r = zi[k1 * TH];
+            cf zv; float w = 0.f;
+            if (z_staged) {
+                const int e = (r >= 0) ? r - z_first : a.zcap;
+                zv = s_z[e];
+                if (MODE == MID_SEP_Z) w = s_w[e];
+            } else {                                                // more sampled entries than the staging area holds
+                zv = (r >= 0) ? zz[r] : make_float2(0.f, 0.f);
+                if (MODE == MID_SEP_Z) w = (r >= 0) ? m2[r] * a.scale2 : 0.f;
+            }
+            if (MODE == MID_SEP_Z) c[k1] = make_float2(fmaf(w, c[k1].x, -zv.x), fmaf(w, c[k1].y, -zv.y));
+            else c[k1] = make_float2(-zv.x, -zv.y);
+        }
+    } else if (FULL) {
+#pragma unroll
+        for (int k1 = 0; k1 < BY; ++k1) {
+            const float m = s_m[k1 * TH], w = m * m * a.scale2;
+            if (a.y) {
+                const cf yv = (m != 0.f) ? s_y[k1 * TH] : make_float2(0.f, 0.f);
+                const float f = (((centred(k1) + s2) & 1) ? -a.scale : a.scale) * m;
+                if (MODE == MID_FULL) c[k1] = make_float2(fmaf(w, c[k1].x, -f * yv.x), fmaf(w, c[k1].y, -f * yv.y));
+                else c[k1] = make_float2(-f * yv.x, -f * yv.y);
+            } else {
+                c[k1] = cscale(c[k1], w);
+            }
+        }
+    } else if (MODE == MID_GRADY) {
+        const float* mk = a.mask + bt * (a.mask_row ? NZ : pe) + s2;
+        cf* dst = a.ky_out + (long long)unit * pe + s2;
+#pragma unroll
+        for (int k1 = 0; k1 < BY; ++k1) {
+            const int s1 = centred(k1);
+            dst[s1 * NZ] = cscale(c[k1], (((s1 + s2) & 1) ? -a.scale : a.scale) * mk[a.mask_row ? 0 : s1 * NZ]);
+        }
+        return;
+    }
+    if (INVERSE) {
+        Dft<BY, +1>::run(c);
+        if (RY > 1) {
+#pragma unroll
+            for (int j = 1; j < BY; ++j) c[j] = cmulc(c[j], twiddle(j));
+        }
+    }
+    cf* p = Vp;
+#pragma unroll
+    for (int j = 0; j < BY; ++j) { *p = c[j]; p += a.v_j; }
+}
+
+// ---------------------------------------------------------------------------------------------
+// launch tables: passes 1 and 3 per (RY, kz plan), pass 2 per ky length
+// ---------------------------------------------------------------------------------------------
+struct TileOps {
+    int ry, n2;
+    // images: B*T; tiles: tiles of the whole problem (they decide how the coils are split, so that a volume gives the
+    // same bits whatever part of it one launch covers)
+    cudaError_t (*fwd)(const TileArgs&, long long images, long long tiles, cudaStream_t);
+    cudaError_t (*inv)(const TileArgs&, long long images, long long tiles, cudaStream_t);
+};
+struct MidOps {
+    int n1, ry, by;
+    cudaError_t (*launch)(int mode, const MidArgs&, cudaStream_t);
+};
+
+// Blocks that share the coils of a tile: doubled while that leaves no more than three blocks per SM.  Splitting only
+// fills SMs that would be idle (a single 320 x 256 slice with 8 coils, 20 tiles: 44 -> 29 us per call for 4 blocks a
+// tile); with more tiles the start-up of the additional blocks and the sum over the cluster cost more than the finer
+// grain gains (12 coils of 96 x 240 x 184, 1440 tiles: 512 us unsplit, 549 us for 2, 615 us for 4 blocks a tile).
+inline int coil_split(long long tiles, int sms, int C) {
+    int cs = 1;
+    while (cs < 4 && 2 * cs <= C && 2 * cs * tiles <= 3LL * sms) cs *= 2;
+    return cs;
+}
+
+template <class PZ, int RY>
+struct TileImpl {
+    using TL = Tile<PZ, RY>;
+    static cudaError_t fwd(const TileArgs& a0, long long images, long long tiles, cudaStream_t s) {
+        static PerDevice done;
+        cudaError_t e = ensure_smem(tile_fwd_kernel<PZ, RY>, TL::FWD_BYTES, done);
+        if (e != cudaSuccess) return e;
+        int sms = 0;
+        if ((e = device_sms(&sms)) != cudaSuccess) return e;
+        TileArgs a = a0;
+        a.csplit = coil_split(tiles, sms, a.C);
+        const long long blocks = images * a.G * a.BY * a.csplit;
+        if (blocks <= 0) return cudaSuccess;
+        if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
+        tile_fwd_kernel<PZ, RY><<<(unsigned)blocks, TL::TH, TL::FWD_BYTES, s>>>(a);
+        return cudaGetLastError();
+    }
+    static cudaError_t inv(const TileArgs& a0, long long images, long long tiles, cudaStream_t s) {
+        static PerDevice done;
+        cudaError_t e = ensure_smem(tile_inv_kernel<PZ, RY>, TL::INV_BYTES, done);
+        if (e != cudaSuccess) return e;
+        int sms = 0;
+        if ((e = device_sms(&sms)) != cudaSuccess) return e;
+        TileArgs a = a0;
+        a.csplit = coil_split(tiles, sms, a.C);
+        const long long blocks = images * a.G * a.BY * a.csplit;
+        if (blocks <= 0) return cudaSuccess;
+        if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3(TL::TH); cfg.dynamicSmemBytes = TL::INV_BYTES; cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)a.csplit; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        cfg.attrs = at; cfg.numAttrs = a.csplit > 1 ? 1 : 0;
+        return cudaLaunchKernelEx(&cfg, tile_inv_kernel<PZ, RY>, a);
+    }
+};
+
+template <int RY, int BY>
+struct MidImpl {
+    template <int MODE> static cudaError_t go(const MidArgs& a0, cudaStream_t s) {
+        MidArgs a = a0;
+        const int threads = a.NZ < 256 ? ((a.NZ + 31) / 32) * 32 : 256;
+        const long long blocks = a.nunits * a.G * RY;
+        if (blocks <= 0) return cudaSuccess;
+        if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
+        // shared memory: a weight or rank per element, and the measurements (arbitrary mask) or the z values and
+        // weights of one k0 group
+        constexpr bool Z = MODE == MID_SEP_Z || MODE == MID_ADJ_Z, FULL = MODE == MID_FULL || MODE == MID_ADJ_FULL;
+        size_t bytes = (Z || FULL || MODE == MID_SEP) ? (size_t)BY * threads * sizeof(float) : 0;
+        if (FULL) {
+            static PerDevice done;
+            cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * (sizeof(cf) + sizeof(float)), done);
+            if (e != cudaSuccess) return e;
+            if (a.y) bytes += (size_t)BY * threads * sizeof(cf);
+        }
+        if (Z) {
+            a.zcap = BY * a.NZ < 1024 ? BY * a.NZ : 1024;
+            bytes += (size_t)(a.zcap + 1) * (sizeof(cf) + sizeof(float)) + 8;
+        }
+        static_assert(!Z || BY * 256 * sizeof(float) + 1025 * 12 + 8 + (BY + 1) * 8 <= 48 * 1024, "over the default shared memory limit");
+        mid_kernel<RY, BY, MODE><<<dim3((unsigned)blocks, (unsigned)((a.NZ + threads - 1) / threads)), threads, bytes, s>>>(a);
+        return cudaGetLastError();
+    }
+    static cudaError_t launch(int mode, const MidArgs& a, cudaStream_t s) {
+        switch (mode) {
+            case MID_SEP: return go<MID_SEP>(a, s);
+            case MID_SEP_Z: return go<MID_SEP_Z>(a, s);
+            case MID_ADJ_Z: return go<MID_ADJ_Z>(a, s);
+            case MID_FULL: return go<MID_FULL>(a, s);
+            case MID_ADJ_FULL: return go<MID_ADJ_FULL>(a, s);
+            case MID_FWD: return go<MID_FWD>(a, s);
+            case MID_INV: return go<MID_INV>(a, s);
+            case MID_GRADY: return go<MID_GRADY>(a, s);
+        }
+        return cudaErrorInvalidValue;
+    }
+};
+
+}  // namespace gleam

@@ -1,0 +1,295 @@
+// Row-tile kernels: the phase-encode plane (ky, kz) of the 3-D path, or the whole slice (n1, n2) of a 2-D problem
+// with an arbitrary mask, is transformed so that every pass over the coil workspace is contiguous in memory.
+//
+// ky has the split N1 = RY * BY, kz the one- or two-stage plan PZ.  With ky = j + BY m (m < RY) on the image side
+// and ky = k0 + RY k1 (k1 < BY) on the k-space side:
+//   pass 1  tile_fwd : block (b,t,i0,j) takes the RY rows ky = j + BY m, multiplies by S_c, transforms the rows
+//                      against each other (radix RY, one thread per kz), then each row along kz, and stores
+//                      V[unit][i0][k0][j][kz].
+//   pass 2  mid      : block (unit,i0,k0) reads the BY rows V[..][k0][0..BY)[kz], applies the ky twiddles
+//                      w_N1^(j k0), radix-BY transform over j (-> k1), the k-space work of the call at the raw
+//                      position (k0 + RY k1, kz), and the mirror image back, in place.
+//   pass 3  tile_inv : mirror of pass 1 with the conjugate-sensitivity coil sum and the update of Eq. 3.
+//
+// All stages of passes 1 and 3 are distributed over the whole block (a stage of N butterflies keeps N lanes busy
+// whatever the radices are; with one warp per row, as before, a 23-point stage of 184 = 8 x 23 used 8 of every 32
+// lanes).  The radix-RY stage comes first because it reads the staged sensitivities column by column as they lie in
+// memory; the ky twiddles belong to the middle pass, which is bound by memory and has issue slots to spare.
+#pragma once
+#include "size_ops.cuh"
+
+namespace gleam {
+
+struct TileArgs {
+    const cf* x; const cf* sens; cf* out;     // image side; x may be null in pass 3 (a zero image)
+    cf* V;                                    // workspace
+    long long v_unit, v_slab, v_k0, v_j;      // its strides (elements); kz is contiguous
+    float eta;
+    int C, T, Ts, n0, G, i0_start, BY;
+    int csplit;                               // the coils of one tile are dealt to this many blocks (pass 3: a cluster)
+    int x_planar, out_planar; long long plane; // two-real-channel layout of x / out (see RowArgs)
+    const cf* aty;                            // A^H y image of the normal-equations form, or null (see RowArgs)
+};
+
+template <class PZ, int RY>
+struct Tile {
+    static constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, S = PZ::S;
+    static constexpr int BF0 = PZ::BF0;                      // butterflies per row of the first kz stage
+    static constexpr int LS1 = PZ::LS1;                      // odd run length: the second stage reads without bank conflicts
+    static constexpr int ROW = (S == 2) ? R0 * LS1 : NZ;     // slots of a row in the exchange tile
+    static constexpr int TH = ((NZ + 31) / 32) * 32;         // one thread per kz column
+    static constexpr int T_ELEMS = (RY * ROW + 1) / 2 * 2, STAGE = RY * NZ, TW = (S == 2) ? NZ : 0;
+    static constexpr int RMAX = cmax(RY, cmax(R0, RL));
+    static constexpr int slot(int kz) { return (S == 2) ? (kz / BF0) * LS1 + kz % BF0 : kz; }
+    static constexpr size_t LIMIT = 227 * 1024;
+    static constexpr size_t FWD_BYTES = sizeof(cf) * (T_ELEMS + STAGE + TW);
+    // Pass 3 stages a tile of the workspace and one of the sensitivities.  Where both and the exchange tile take more
+    // than a third of the SM they take turns in one buffer: a third block per SM hides more latency than the longer
+    // reach of two buffers (8 slices of 320 x 256, 8 coils: 84.7 -> 76.7 us per VJP call).
+    static constexpr bool ONE_STAGE = sizeof(cf) * (T_ELEMS + 2 * STAGE + TW) > LIMIT / 3;
+    static constexpr size_t INV_BYTES = sizeof(cf) * (T_ELEMS + (ONE_STAGE ? 1 : 2) * STAGE + TW);
+    // The register bound lets the blocks that shared memory admits be resident.  RY values of the image or of the coil
+    // sum are kept over the coil loop next to a butterfly (a prime radix also holds its sums and differences).
+    static constexpr bool PRIME = RMAX > 4 && RMAX % 2 == 1 && smallest_odd_factor(RMAX) == RMAX;
+    static constexpr int REGS = 2 * RY + (PRIME ? 4 : 2) * RMAX + 16;
+    static constexpr int blocks(size_t bytes) {
+        const int n = cmin(16, cmin((int)(LIMIT / (bytes + 1024)), 65536 / (TH * ((REGS + 7) / 8 * 8))));
+        return cmax(1, cmin(n, 2048 / TH));
+    }
+};
+
+__device__ __forceinline__ void cluster_arrive_wait() {
+    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+}
+// value of another block's shared memory at the same address as `p` in this block
+__device__ __forceinline__ cf cluster_load(const cf* p, unsigned rank) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    unsigned r; cf v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(r) : "memory");
+    return v;
+}
+
+// which tile and which coils a block has
+struct TileId {
+    int b, t, i0, j, c0, c1;
+    unsigned bt, gi, part;
+    __device__ __forceinline__ explicit TileId(const TileArgs& a) {
+        part = blockIdx.x % (unsigned)a.csplit;
+        const unsigned blk = blockIdx.x / (unsigned)a.csplit;
+        j = (int)(blk % (unsigned)a.BY);
+        gi = (blk / (unsigned)a.BY) % (unsigned)a.G;
+        bt = blk / ((unsigned)a.BY * (unsigned)a.G);
+        b = (int)(bt / (unsigned)a.T); t = (int)(bt - (unsigned)b * a.T);
+        i0 = a.i0_start + (int)gi;
+        c0 = (int)part * a.C / a.csplit; c1 = ((int)part + 1) * a.C / a.csplit;
+    }
+};
+
+// RY rows of NZ values, `row_stride` apart in global memory, to a dense tile in shared memory
+template <int NZ, int RY>
+__device__ __forceinline__ void stage_rows(cf* dst, const cf* src, long long row_stride) {
+    if ((int)threadIdx.x < NZ) {
+        const int h = (int)threadIdx.x / (NZ / 2), p = (int)threadIdx.x - h * (NZ / 2);
+        const cf* s = src + h * row_stride + 2 * p;
+        cf* d = dst + h * NZ + 2 * p;
+#pragma unroll
+        for (int m = 0; m < RY / 2; ++m) { cp_async16(d + 2 * m * NZ, s); s += 2 * row_stride; }
+        if (RY % 2 == 1 && h == 0) cp_async16(d + (RY - 1) * NZ, s);
+    }
+    cp_async_commit();
+}
+
+template <class PZ, int RY>
+__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY>::blocks(Tile<PZ, RY>::FWD_BYTES))
+tile_fwd_kernel(const TileArgs a) {
+    using TL = Tile<PZ, RY>;
+    constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
+    extern __shared__ __align__(16) float2 smem[];
+    cf* sT = smem;
+    cf* sS = smem + TL::T_ELEMS;
+    cf* sTw = sS + TL::STAGE;                                 // kz twiddles, [k][j]
+    const TileId id(a);
+    const int tid = threadIdx.x;
+    const bool col = tid < NZ;
+    const long long N1NZ = (long long)RY * a.BY * NZ, V3 = a.n0 * N1NZ;
+    const long long row_elems = id.i0 * N1NZ + (long long)id.j * NZ, row_stride = (long long)a.BY * NZ;
+    const cf* sp = a.sens + ((long long)(id.b * a.C) * a.Ts + (a.Ts > 1 ? id.t : 0)) * V3 + row_elems;
+    const long long s_stride = (long long)a.Ts * V3;
+    if (id.c0 < id.c1) stage_rows<NZ, RY>(sS, sp + id.c0 * s_stride, row_stride);
+    if (TL::S == 2) for (int i = tid; i < NZ; i += TH) sTw[i] = unit_root_fwd<NZ>(((i / BF0) * (i % BF0)) % NZ);
+    cf xv[RY];
+#pragma unroll
+    for (int m = 0; m < RY; ++m)
+        xv[m] = col ? load_image(a.x, id.bt * V3 + row_elems + m * row_stride + tid, a.x_planar, id.b, a.plane) : make_float2(0.f, 0.f);
+
+    for (int c = id.c0; c < id.c1; ++c) {
+        cp_async_wait<0>();
+        __syncthreads();                 // the sensitivities are visible, every thread has left the tile
+        if (col) {
+            cf v[RY];
+#pragma unroll
+            for (int m = 0; m < RY; ++m) v[m] = cmul(sS[m * NZ + tid], xv[m]);
+            Dft<RY, -1>::run(v);
+#pragma unroll
+            for (int k = 0; k < RY; ++k) sT[k * ROW + TL::slot(tid)] = v[k];
+        }
+        __syncthreads();
+        if (c + 1 < id.c1) stage_rows<NZ, RY>(sS, sp + (c + 1) * s_stride, row_stride);
+        const long long unit = ((long long)(id.b * a.C + c)) * a.T + id.t;
+        cf* Vp = a.V + unit * a.v_unit + id.gi * a.v_slab + id.j * a.v_j;
+        // first kz stage, in place: butterfly j of a row reads and writes the slots {k * LS1 + j}
+#pragma unroll 1
+        for (int t = tid; t < RY * BF0; t += TH) {
+            const int row = t / BF0, j = t - row * BF0;
+            cf* e = sT + row * ROW + j;
+            cf v[R0];
+#pragma unroll
+            for (int m = 0; m < R0; ++m) v[m] = e[m * LS1];
+            Dft<R0, -1>::run(v);
+            if (TL::S == 2) {
+#pragma unroll
+                for (int k = 0; k < R0; ++k) e[k * LS1] = (k == 0) ? v[0] : cmul(v[k], sTw[k * BF0 + j]);
+            } else {
+                cf* o = Vp + row * a.v_k0;
+#pragma unroll
+                for (int k = 0; k < R0; ++k) o[k] = v[k];
+            }
+        }
+        if (TL::S == 2) {
+            __syncthreads();
+            // second kz stage: butterfly j reads the run j * LS1 .. + RL
+#pragma unroll 1
+            for (int t = tid; t < RY * R0; t += TH) {
+                const int row = t / R0, j = t - row * R0;
+                const cf* e = sT + row * ROW + j * LS1;
+                cf u[RL];
+#pragma unroll
+                for (int m = 0; m < RL; ++m) u[m] = e[m];
+                Dft<RL, -1>::run(u);
+                cf* o = Vp + row * a.v_k0 + j;
+#pragma unroll
+                for (int k = 0; k < RL; ++k) o[R0 * k] = u[k];
+            }
+        }
+    }
+    cp_async_wait<0>();
+}
+
+template <class PZ, int RY>
+__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY>::blocks(Tile<PZ, RY>::INV_BYTES))
+tile_inv_kernel(const TileArgs a) {
+    using TL = Tile<PZ, RY>;
+    constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
+    extern __shared__ __align__(16) float2 smem[];
+    cf* sT = smem;
+    cf* sV = smem + TL::T_ELEMS;
+    cf* sS = sV + (TL::ONE_STAGE ? 0 : TL::STAGE);
+    cf* sTw = sS + TL::STAGE;
+    const TileId id(a);
+    const int tid = threadIdx.x;
+    const bool col = tid < NZ;
+    const long long N1NZ = (long long)RY * a.BY * NZ, V3 = a.n0 * N1NZ;
+    const long long row_elems = id.i0 * N1NZ + (long long)id.j * NZ, row_stride = (long long)a.BY * NZ;
+    const cf* sp = a.sens + ((long long)(id.b * a.C) * a.Ts + (a.Ts > 1 ? id.t : 0)) * V3 + row_elems;
+    const long long s_stride = (long long)a.Ts * V3, x_off = id.bt * V3 + row_elems + tid;
+    auto v_ptr = [&](int c) { return a.V + (((long long)(id.b * a.C + c)) * a.T + id.t) * a.v_unit + id.gi * a.v_slab + id.j * a.v_j; };
+    if (id.c0 < id.c1) stage_rows<NZ, RY>(sV, v_ptr(id.c0), a.v_k0);
+    if (TL::S == 2) for (int i = tid; i < NZ; i += TH) sTw[i] = unit_root_fwd<NZ>(((i / BF0) * (i % BF0)) % NZ);
+    cf acc[RY];
+#pragma unroll
+    for (int m = 0; m < RY; ++m)
+        acc[m] = (col && id.part == 0) ? coil_sum_start(a.aty, x_off + m * row_stride) : make_float2(0.f, 0.f);
+
+    for (int c = id.c0; c < id.c1; ++c) {
+        cp_async_wait<0>();
+        __syncthreads();                 // the workspace tile is visible, every thread has left the other tiles
+        if (!TL::ONE_STAGE) stage_rows<NZ, RY>(sS, sp + c * s_stride, row_stride);
+        if (TL::S == 2) {
+#pragma unroll 1
+            for (int t = tid; t < RY * R0; t += TH) {
+                const int row = t / R0, j = t - row * R0;
+                const cf* o = sV + row * NZ + j;
+                cf* e = sT + row * ROW + j * LS1;
+                cf u[RL];
+#pragma unroll
+                for (int k = 0; k < RL; ++k) u[k] = o[R0 * k];
+                Dft<RL, +1>::run(u);
+#pragma unroll
+                for (int m = 0; m < RL; ++m) e[m] = u[m];
+            }
+            __syncthreads();
+            if (TL::ONE_STAGE) stage_rows<NZ, RY>(sS, sp + c * s_stride, row_stride);
+            else if (c + 1 < id.c1) stage_rows<NZ, RY>(sV, v_ptr(c + 1), a.v_k0);
+            else cp_async_commit();
+#pragma unroll 1
+            for (int t = tid; t < RY * BF0; t += TH) {
+                const int row = t / BF0, j = t - row * BF0;
+                cf* e = sT + row * ROW + j;
+                cf v[R0];
+#pragma unroll
+                for (int k = 0; k < R0; ++k) { const cf r = e[k * LS1]; v[k] = (k == 0) ? r : cmulc(r, sTw[k * BF0 + j]); }
+                Dft<R0, +1>::run(v);
+#pragma unroll
+                for (int m = 0; m < R0; ++m) e[m * LS1] = v[m];
+            }
+        } else {
+            for (int t = tid; t < RY; t += TH) {
+                cf v[R0];
+#pragma unroll
+                for (int k = 0; k < R0; ++k) v[k] = sV[t * NZ + k];
+                Dft<R0, +1>::run(v);
+#pragma unroll
+                for (int m = 0; m < R0; ++m) sT[t * NZ + m] = v[m];
+            }
+            __syncthreads();
+            if (c + 1 < id.c1) stage_rows<NZ, RY>(sV, v_ptr(c + 1), a.v_k0);
+            else cp_async_commit();
+        }
+        cp_async_wait<TL::ONE_STAGE ? 0 : 1>();
+        __syncthreads();                 // the sensitivities and the row transforms are visible
+        if (col) {
+            cf v[RY];
+#pragma unroll
+            for (int k = 0; k < RY; ++k) v[k] = sT[k * ROW + TL::slot(tid)];
+            Dft<RY, +1>::run(v);
+#pragma unroll
+            for (int m = 0; m < RY; ++m) {
+                const cf s = sS[m * NZ + tid];
+                acc[m].x = fmaf(s.x, v[m].x, fmaf(s.y, v[m].y, acc[m].x));
+                acc[m].y = fmaf(s.x, v[m].y, fmaf(-s.y, v[m].x, acc[m].y));
+            }
+        }
+        if (TL::ONE_STAGE) {
+            __syncthreads();
+            if (c + 1 < id.c1) stage_rows<NZ, RY>(sV, v_ptr(c + 1), a.v_k0);
+        }
+    }
+    cp_async_wait<0>();
+    if (a.csplit > 1) {
+        // partial coil sums of the other blocks of the cluster, added in block order
+        __syncthreads();
+        if (col && id.part > 0) {
+#pragma unroll
+            for (int m = 0; m < RY; ++m) sT[m * NZ + tid] = acc[m];
+        }
+        cluster_arrive_wait();
+        if (col && id.part == 0) {
+            for (int p = 1; p < a.csplit; ++p) {
+#pragma unroll
+                for (int m = 0; m < RY; ++m) acc[m] = cadd(acc[m], cluster_load(sT + m * NZ + tid, (unsigned)p));
+            }
+        }
+        cluster_arrive_wait();           // no block leaves while its sums are being read
+        if (id.part > 0) return;
+    }
+    if (!col) return;
+#pragma unroll
+    for (int m = 0; m < RY; ++m) {
+        const long long e = x_off + m * row_stride;
+        const cf xv = a.x ? load_image(a.x, e, a.x_planar, id.b, a.plane) : make_float2(0.f, 0.f);
+        store_image(a.out, e, make_float2(fmaf(-a.eta, acc[m].x, xv.x), fmaf(-a.eta, acc[m].y, xv.y)), a.out_planar, id.b, a.plane);
+    }
+}
+
+}  // namespace gleam

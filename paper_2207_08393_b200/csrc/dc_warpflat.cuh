@@ -1,7 +1,6 @@
-// One-pass row kernel (ROW_FUSED arithmetic of dc_warpline.cuh) for two-stage plans whose last stage has
-// fewer butterflies per line than the first (N = R0 * RL, R0 < RL, RL in {8, 16, 32}): in the plain
-// warp-resident form the RL-point butterflies of the last forward stage, the k-space update and the
-// first inverse stage keep only R0 of every RL lanes busy (10 of 16 for N = 160).
+// One-pass row kernel of 2-D problems (arithmetic of dc_warpline.cuh) for two-stage plans N = R0 * RL.  In the plain
+// warp-resident form the RL-point butterflies of the last forward stage, the k-space update and the first inverse
+// stage keep only R0 of every max(R0, RL) lanes busy (10 of 16 for N = 160 = 10 x 16, 8 of 32 for 184 = 8 x 23).
 //
 // Here a warp still owns LW = 32 / RL whole lines, and the first / last image-side stages (S x, R0-point
 // butterflies, twiddles; conj(S) coil sum) keep their fixed lane = (line, butterfly) assignment, so the
@@ -23,12 +22,11 @@ namespace gleam {
 template <class P, bool HAS_Z, bool SMW = false>
 struct WarpFlat {
     static constexpr int N = P::N, R0 = P::R0, RL = P::RL;
-    // R0 < RL is where the plain kernel wastes lanes in the RL-point stages; R0 > RL (368 = 23 x 16) also fits: the
-    // R0-point butterflies then run on all lanes of the image-side stages and the RL-point ones on numbered units
-    static constexpr bool ELIGIBLE = (P::S == 2) && (RL == 8 || RL == 16 || RL == 32) && (R0 != RL) && (N % 2 == 0);
+    static constexpr bool ELIGIBLE = (P::S == 2) && RL >= 2 && RL <= 32 && (N % 2 == 0);
     static constexpr int LW = 32 / RL;                     // lines per warp
     static constexpr int UPC = LW * R0;                    // k-space units per coil
-    static constexpr int USTRIDE = RL + 1;                 // odd: a round's 32 units read without bank conflicts
+    static constexpr int LANES = LW * RL;                  // lanes of the image-side stages (32 if RL is a power of two)
+    static constexpr int USTRIDE = odd_up(RL);             // odd: a round's 32 units read without bank conflicts
     static constexpr int SLOTS_MIN = (32 + UPC - 1) / UPC + 1;     // coils between first forward and inverse stage
     // a ring whose unit count is a multiple of 16 keeps the bank pattern across the wrap; taken when small
     static constexpr int slots_aligned() {
@@ -50,6 +48,11 @@ struct WarpFlat {
     // per line: element offset of its z row (64-bit), sampled count, mask row index
     static constexpr int ELEMS = (OFF_CNT + 2 * LW + 1) / 2 * 2;
     static constexpr size_t WARP_BYTES = sizeof(cf) * ELEMS;      // per warp of the block
+    // Registers: coil sum, twiddles and the sensitivities of the next forward stage are held throughout (2 R0 each),
+    // next to a butterfly of the image side or of the k-space round (a prime radix also holds its sums and differences).
+    static constexpr bool PRIME = RL > 4 && RL % 2 == 1 && smallest_odd_factor(RL) == RL;
+    static constexpr int REGS = cmax(8 * R0 + 24, 6 * R0 + (PRIME ? 4 : 2) * RL + 24);
+    static constexpr int SINGLE_BLOCKS = cmax(4, cmin(RL == 32 ? 12 : 16, 65536 / (32 * ((REGS + 7) / 8 * 8)) / 4 * 4));
 };
 
 // SMW = false: one warp per block, blocks stride over the line groups.
@@ -67,8 +70,9 @@ struct WarpFlat {
 // symmetric in the sign).  Normal-equations form of the step; never together
 // with z).  A template parameter, not a run-time test of a.aty: with the test in the code the plain call measured
 // 11 % slower (17.7 against 16.0 us), although it never takes that branch.
-template <class P, bool HAS_Z, bool SMW, bool HAS_ATY>
-__global__ void __launch_bounds__(SMW ? 512 : 32, SMW ? 1 : (P::R0 > 16 ? 8 : P::RL == 32 ? 12 : 16))
+// ADJ (with z): A^H y, the image is zero; the forward stages are left out and a unit starts from minus its z values.
+template <class P, bool HAS_Z, bool SMW, bool HAS_ATY, bool ADJ>
+__global__ void __launch_bounds__(SMW ? 512 : 32, SMW ? 1 : WarpFlat<P, HAS_Z, SMW>::SINGLE_BLOCKS)
 warpflat_kernel(const RowArgs a, const int nwhole) {
     grid_dependency_wait();
     grid_launch_dependents();
@@ -91,7 +95,8 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
     const int cbase = split ? q * a.C / 4 : 0;                     // first coil and number of coils of this warp
     const int nc = split ? (q + 1) * a.C / 4 - cbase : a.C;
 
-    const int l = lane / RL, j = lane % RL;                 // image-side identity: line of the warp, butterfly
+    const bool img = WF::LANES == 32 || lane < WF::LANES;
+    const int l = img ? lane / RL : LW - 1, j = img ? lane % RL : 0;      // image-side identity: line of the warp, butterfly
 
     if (HAS_Z) {
         for (int i = lane; i < ZS * LW; i += 32) sK[(i / LW) * KTILE + (i % LW) * KSTRIDE + KCAP] = make_float2(0.f, 0.f);
@@ -111,15 +116,15 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
 
     for (long long g = g_first; g < ngroups; g += g_step) {
         const long long row = g * LW + l;
-        const bool row_ok = row < a.nrows;
+        const bool row_ok = img && row < a.nrows;
         const unsigned rowu = row_ok ? (unsigned)row : 0u;       // host side guarantees nrows < 2^31
-        const unsigned bt = rowu / (unsigned)a.rpb;
-        const int ri = (int)(rowu - bt * (unsigned)a.rpb);
+        const unsigned bt = rowu / (unsigned)a.RPB;
+        const int ri = (int)(rowu - bt * (unsigned)a.RPB);
         const int b = (int)(bt / (unsigned)a.T), t = (int)(bt - (unsigned)b * (unsigned)a.T);
-        const long long x_off = ((long long)bt * a.RPB + a.row0 + ri) * N;
+        const long long x_off = ((long long)bt * a.RPB + ri) * N;
         // coil indices below are relative to cbase
-        const long long s_off = (((long long)(b * a.C + cbase) * a.Ts + (a.Ts > 1 ? t : 0)) * a.RPB + a.row0 + ri) * N;
-        const long long k_off = (((long long)(b * a.C + cbase) * a.T + t) * a.RPB + a.row0 + ri) * N;
+        const long long s_off = (((long long)(b * a.C + cbase) * a.Ts + (a.Ts > 1 ? t : 0)) * a.RPB + ri) * N;
+        const long long k_off = (((long long)(b * a.C + cbase) * a.T + t) * a.RPB + ri) * N;
         const long long s_stride = (long long)a.Ts * a.RPB * N;
         const long long k_stride = (long long)a.T * a.RPB * N;
         const cf* sp = a.sens + s_off + j;                       // this lane's sensitivities of coil 0
@@ -132,7 +137,8 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
             const long long xo = __shfl_sync(0xffffffffu, x_off, ll * RL);
             const long long bto = __shfl_sync(0xffffffffu, (long long)bt, ll * RL);
             if (!ok) { if (lane == 0) sC[ll] = -1; continue; }
-            if (!a.x_planar) {
+            if (ADJ) {
+            } else if (!a.x_planar) {
                 for (int i = lane; i < N / 2; i += 32) cp_async16(sX + ll * N + 2 * i, a.x + xo + 2 * i);
             } else {
                 const long long bo = __shfl_sync(0xffffffffu, (long long)b, ll * RL);
@@ -159,7 +165,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 }
             }
             if (lane == 0) sC[ll] = cnt;
-            if (HAS_Z && lane == ll * RL) { sKo[ll] = k_off; sBt[ll] = bt; }
+            if (HAS_Z && img && lane == ll * RL) { sKo[ll] = k_off; sBt[ll] = bt; }
         }
         __syncwarp();
         // z row of coil c for every line of the warp -> slot c % ZS
@@ -194,7 +200,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
 #pragma unroll
         for (int m = 0; m < R0; ++m) acc[m] = (HAS_ATY && row_ok && q == 0) ? a.aty[x_off + j + RL * m] : make_float2(0.f, 0.f);
         cf sf[R0];                       // sensitivities of the next forward image-side stage
-        if (nc > 0) load_sens(sf, 0);
+        if (!ADJ && nc > 0) load_sens(sf, 0);
         int af = 0, ai = 0;              // next coil of the forward / of the inverse image-side stage
 
         for (int br = 0; br < rounds; ++br) {
@@ -205,14 +211,17 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
             while (af < need) {
                 if (HAS_Z) { if (af + ZAHEAD < nc) issue_z(af + ZAHEAD); cp_async_commit(); }
                 if (af == 0) { cp_async_wait<HAS_Z ? 1 : 0>(); __syncwarp(); }      // x (and z of coil 0) have landed
+                if (ADJ) { ++af; continue; }
                 cf v[R0];
 #pragma unroll
                 for (int m = 0; m < R0; ++m) v[m] = cmul(sf[m], x_at(j + RL * m));
                 if (af + 1 < nc) load_sens(sf, af + 1);
                 Dft<R0, -1>::run(v);
                 cf* e = sE + ((af % SLOTS) * UPC + l * R0) * US + j;
+                if (img) {
 #pragma unroll
-                for (int k = 0; k < R0; ++k) e[k * US] = (k == 0) ? v[0] : cmul(v[k], tw0[k]);
+                    for (int k = 0; k < R0; ++k) e[k * US] = (k == 0) ? v[0] : cmul(v[k], tw0[k]);
+                }
                 ++af;
             }
             if (HAS_Z) cp_async_wait<ZAHEAD>();  // everything but a request for the next coil's z is there
@@ -226,9 +235,11 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 const int bl = w / R0, jb = w - bl * R0;
                 cf* e = sE + ((c % SLOTS) * UPC + w) * US;
                 cf u[RL];
+                if (!ADJ) {
 #pragma unroll
-                for (int m = 0; m < RL; ++m) u[m] = e[m];
-                Dft<RL, -1>::run(u);
+                    for (int m = 0; m < RL; ++m) u[m] = e[m];
+                    Dft<RL, -1>::run(u);
+                }
                 if (!HAS_Z) {
                     const float* mm = sM + bl * MS + jb;
 #pragma unroll
@@ -244,9 +255,9 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                         for (int k = 0; k < RL; ++k) {
                             const int r = ri_[R0 * k];
                             const int rr = (r >= 0) ? r : KCAP;
-                            const float wv = mw[rr];
                             const cf q = zk[rr];
-                            u[k] = make_float2(fmaf(wv, u[k].x, -q.x), fmaf(wv, u[k].y, -q.y));
+                            if (ADJ) u[k] = make_float2(-q.x, -q.y);
+                            else { const float wv = mw[rr]; u[k] = make_float2(fmaf(wv, u[k].x, -q.x), fmaf(wv, u[k].y, -q.y)); }
                             if (k % 4 == 3) asm volatile("" ::: "memory");     // four entries in flight at a time: registers
                         }
                     } else if (kc > KCAP) {
@@ -255,8 +266,8 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                         const cf* zrow = a.z + sKo[bl] + c * k_stride;
 #pragma unroll
                         for (int k = 0; k < RL; ++k) {
-                            const float mv = mrow[shift_half(jb + R0 * k, N)];
-                            u[k] = cscale(u[k], mv * mv * (1.0f / N));
+                            if (ADJ) u[k] = make_float2(0.f, 0.f);
+                            else { const float mv = mrow[shift_half(jb + R0 * k, N)]; u[k] = cscale(u[k], mv * mv * (1.0f / N)); }
                             const int r = ri_[R0 * k];
                             if (r >= 0) {
                                 const cf q = zrow[r];
@@ -323,7 +334,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
         if (row_ok) {
 #pragma unroll
             for (int m = 0; m < R0; ++m) {
-                const cf xv = x_at(j + RL * m);
+                const cf xv = ADJ ? make_float2(0.f, 0.f) : x_at(j + RL * m);
                 const cf av = acc[m];
                 const float se = HAS_ATY ? a.eta : -a.eta;          // HAS_ATY: acc holds aty - sum
                 const cf ov = make_float2(fmaf(se, av.x, xv.x), fmaf(se, av.y, xv.y));
@@ -332,7 +343,10 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
             }
         }
         if (a.dot_rows != nullptr) {     // the same in every thread
-            for (int o = RL / 2; o > 0; o >>= 1) dsum += __shfl_down_sync(0xffffffffu, dsum, o, RL);
+            for (int o = pow2_ceil(RL) / 2; o > 0; o >>= 1) {
+                const double d = __shfl_down_sync(0xffffffffu, dsum, o);
+                if (j + o < RL) dsum += d;
+            }
             if (j == 0 && row_ok) a.dot_rows[row] = dsum;
         }
     }

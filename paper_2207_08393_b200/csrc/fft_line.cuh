@@ -7,15 +7,15 @@
 // stage (conjugated butterflies and twiddles, reversed order), so a pointwise operation in
 // k-space sits between them without any reordering.  Transforms are raw: no scaling, no centring.
 //
-// Several lines are processed per thread block.  ROW mode: the line is contiguous in memory and
-// consecutive threads take consecutive butterflies of one line.  COL mode: the line is strided and
-// consecutive threads take the same butterfly of consecutive lines (contiguous in memory).
+// Several strided lines are processed per thread block: consecutive threads take the same butterfly
+// of consecutive lines (contiguous in memory).
 #pragma once
 #include "fft_radix.cuh"
 
 namespace gleam {
 
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
+constexpr int cmin(int a, int b) { return a < b ? a : b; }
 constexpr int odd_up(int a) { return (a % 2 == 0) ? a + 1 : a; }
 
 template <int N_, int R0_, int R1_ = 1, int R2_ = 1>
@@ -47,7 +47,7 @@ template <int N> __device__ const RootTable<N> g_roots = make_root_table<N>();
 
 template <int N> __device__ __forceinline__ cf unit_root_fwd(int e) { return g_roots<N>.v[e]; }
 
-template <class P, bool COL, int L>
+template <class P, int L>
 struct LineFFT {
     static constexpr int N = P::N, R0 = P::R0, R1 = P::R1, RL = P::RL, S = P::S;
     static constexpr int THREADS = ((L * P::MAXBF + 31) / 32) * 32;
@@ -60,8 +60,7 @@ struct LineFFT {
         bool a0, a1, aL;
     };
     __device__ __forceinline__ static void split(int tid, int bf, int& l, int& j, bool& act) {
-        if (COL) { l = tid % L; j = tid / L; }
-        else     { l = tid / bf; j = tid % bf; }
+        l = tid % L; j = tid / L;
         act = (tid < L * bf);
     }
     __device__ __forceinline__ static Ids ids(int tid) {
@@ -73,7 +72,7 @@ struct LineFFT {
         return d;
     }
     __device__ __forceinline__ static int sidx(int l, int off) {
-        return COL ? (off * L + l) : (l * P::LSZ + off);
+        return off * L + l;
     }
 
     struct Tw {
@@ -92,74 +91,11 @@ struct LineFFT {
         }
     }
 
-    // v: n-distribution of the first-stage thread; u: k-distribution of the last-stage thread
-    // flip = 1 swaps the two exchange buffers of a two-stage plan.  A loop that calls only forward()
-    // (or only inverse()) must alternate flip from one call to the next: with a single barrier per
-    // call, the buffer written now must not be the one other threads may still be reading.
-    __device__ __forceinline__ static void forward(cf (&v)[R0], cf (&u)[RL], const Tw& tw, const Ids& d, cf* sm,
-                                                   int flip = 0) {
-        cf* X = sm + ((S == 2 && flip) ? (COL ? L * P::BUF : P::BUF) : 0);
-        cf* Y = sm + (COL ? L * P::BUF : P::BUF);
-        forward_xy(v, u, tw, d, X, Y);
-    }
-    // forward with explicit exchange buffers (two-stage plans use X only)
-    __device__ __forceinline__ static void forward_xy(cf (&v)[R0], cf (&u)[RL], const Tw& tw, const Ids& d, cf* X,
-                                                      cf* Y) {
-        if (S == 1) {
-            Dft<R0, -1>::run(v);
-#pragma unroll
-            for (int k = 0; k < RL; ++k) u[k] = v[k % R0];
-            return;
-        }
-        if (d.a0) {
-            Dft<R0, -1>::run(v);
-#pragma unroll
-            for (int k = 0; k < R0; ++k) {
-                cf t = (k == 0) ? v[0] : cmul(v[k], tw.t0[k]);
-                X[sidx(d.l0, k * P::LS1 + d.j0)] = t;
-            }
-        }
-        __syncthreads();
-        if (S == 3) {
-            if (d.a1) {
-                const int q = d.j1 / P::N2, t = d.j1 % P::N2;
-                cf w[R1];
-#pragma unroll
-                for (int m = 0; m < R1; ++m) w[m] = X[sidx(d.l1, q * P::LS1 + t + P::N2 * m)];
-                Dft<R1, -1>::run(w);
-#pragma unroll
-                for (int k = 0; k < R1; ++k) {
-                    cf r = (k == 0) ? w[0] : cmul(w[k], tw.t1[k]);
-                    Y[sidx(d.l1, (k * R0 + q) * P::LS2 + t)] = r;
-                }
-            }
-            __syncthreads();
-            if (d.aL) {
-#pragma unroll
-                for (int m = 0; m < RL; ++m) u[m] = Y[sidx(d.lL, d.jL * P::LS2 + m)];
-                Dft<RL, -1>::run(u);
-            }
-        } else {
-            if (d.aL) {
-#pragma unroll
-                for (int m = 0; m < RL; ++m) u[m] = X[sidx(d.lL, d.jL * P::LS1 + m)];
-                Dft<RL, -1>::run(u);
-            }
-        }
-    }
-
-    // mirror image of forward(): u (k-distribution) -> v (n-distribution), unscaled inverse.
-    // Buffer use: two-stage plans exchange through Y (X may still be read by forward());
-    // three-stage plans go through X then Y.
-    __device__ __forceinline__ static void inverse(cf (&u)[RL], cf (&v)[R0], const Tw& tw, const Ids& d, cf* sm,
-                                                   int flip = 0) {
+    // u (k-distribution of the last-stage thread) -> v (n-distribution of the first-stage thread), unscaled inverse.
+    // Two-stage plans exchange through Y, three-stage plans go through X then Y.
+    __device__ __forceinline__ static void inverse(cf (&u)[RL], cf (&v)[R0], const Tw& tw, const Ids& d, cf* sm) {
         cf* X = sm;
-        cf* Y = sm + ((S == 2 && flip) ? 0 : (COL ? L * P::BUF : P::BUF));
-        inverse_xy(u, v, tw, d, X, Y);
-    }
-    // inverse with explicit exchange buffers (two-stage plans use Y only)
-    __device__ __forceinline__ static void inverse_xy(cf (&u)[RL], cf (&v)[R0], const Tw& tw, const Ids& d, cf* X,
-                                                      cf* Y) {
+        cf* Y = sm + L * P::BUF;
         if (S == 1) {
 #pragma unroll
             for (int k = 0; k < R0; ++k) v[k] = u[k % RL];

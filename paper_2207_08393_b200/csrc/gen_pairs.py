@@ -1,69 +1,29 @@
-"""Writes pairs.def: every (ky, kz) extent pair of sizes.def that the row-tile kernels of dc_rowtile.cuh can
-take (the compile-time predicate RowTile::ELIGIBLE restated here, plus the shared-memory limit).
+"""Writes pairs.def: the phase-encode extents (n1, n2) whose row-tile kernels split both axes into two register
+stages with a middle radix of at most 24.  The other extents run the same three passes with one row per block
+(single-stage n1), single-stage rows (n2) or a middle radix of 32.
 
     python paper_2207_08393_b200/csrc/gen_pairs.py        # rewrites pairs.def next to this file
-
-ky = n1 uses its two-stage plan (RY, BY) of sizes.def, kz = n2 its two-stage warp-resident plan (Z0, Z1).
 """
 import os
 import re
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-SMEM_LIMIT = 227 * 1024
-GROUPS = 8          # translation units the pairs are spread over
-
-
-def pow2_ceil(v):
-    p = 1
-    while p < v:
-        p *= 2
-    return p
-
-
-def odd_up(a):
-    return a + 1 if a % 2 == 0 else a
 
 
 def plans():
+    """{length: (R0, R1)}, the plans of the contiguous axis."""
     text = open(os.path.join(HERE, "sizes.def")).read()
-    out = {}
-    for m in re.finditer(r"GLEAM_SIZE\((\d+), (\d+), (\d+), (\d+), (\d+), (\d+), (\d+), (\d+), (\d+)\)", text):
-        n, a0, a1, a2 = (int(m.group(i)) for i in range(1, 5))
-        out[n] = (a0, a1, a2)
-    return out
+    return {int(n): (int(a0), int(a1)) for n, a0, a1 in re.findall(r"GLEAM_SIZE\((\d+), (\d+), (\d+),", text)}
 
 
 def main():
     P = plans()
-    pairs = []
-    for n2, (z0, z1, z2) in sorted(P.items()):
-        if z2 != 1 or z1 == 1:
-            continue                                   # kz needs a two-stage plan
-        bf0, bfl = n2 // z0, n2 // z1
-        if max(bf0, bfl) > 32 or n2 % 2:
-            continue                                   # warp-resident lines only
-        tpl = pow2_ceil(max(bf0, bfl)); lw = 32 // tpl
-        exl = z0 * odd_up(n2 // z0)
-        for n1, (ry, by, r2) in sorted(P.items()):
-            if r2 != 1 or by == 1:
-                continue                               # ky needs a two-stage split RY * BY
-            if ry % lw or ry // lw > 32 or by > 24:
-                continue
-            warps = ry // lw
-            per_warp = lw * n2 + lw * exl + (lw * exl) % 2
-            smem = 8 * (ry * n2 + warps * per_warp + 2)
-            if smem > SMEM_LIMIT:
-                continue
-            pairs.append((n1, ry, by, n2, z0, z1))
+    pairs = [(n1, ry, by, n2, z0) for n2, (z0, z1) in sorted(P.items()) if z1 > 1
+             for n1, (ry, by) in sorted(P.items()) if 1 < by <= 24]
     with open(os.path.join(HERE, "pairs.def"), "w") as fh:
-        fh.write("// Generated by gen_pairs.py from sizes.def: (ky, kz) pairs with row-tile kernels.\n")
-        fh.write("// GLEAM_PAIR(n1, RY, BY, n2, kz plan R0, R1): ky = n1 = RY * BY, kz = n2 = R0 * R1.\n")
-        for gi in range(GROUPS):
-            fh.write("#if !defined(GLEAM_PAIR_GROUP) || GLEAM_PAIR_GROUP == %d\n" % gi)
-            for k, p in enumerate(pairs):
-                if k % GROUPS == gi:
-                    fh.write("GLEAM_PAIR(%d, %d, %d, %d, %d, %d)\n" % p)
-            fh.write("#endif\n")
+        fh.write("// Generated by gen_pairs.py from sizes.def.  GLEAM_PAIR(n1, RY, BY, n2, Z0): n1 = RY * BY, first radix Z0 of n2.\n")
+        for p in pairs:
+            fh.write("GLEAM_PAIR(%d, %d, %d, %d, %d)\n" % p)
     print(len(pairs), "pairs")
 
 

@@ -2,17 +2,19 @@
 // the sequence of kernel launches for each problem class.
 //
 //   readout-invariant mask, fft_rank 2 :  [z = R^H y table]  ->  fused row kernel (one pass)
-//   readout-invariant mask, fft_rank 3 :  [z table]  ->  per chunk of readout slabs:
-//                                         rows forward -> columns (mask, residual) -> rows inverse
-//   full mask                           :  rows forward -> strided axes -> rows inverse on a
-//                                         coil-volume workspace
+//   readout-invariant mask, fft_rank 3 :  [z table]  ->  per chunk of readout slabs the three row-tile
+//                                         passes over (ky, kz): forward, middle (mask, residual), inverse
+//   full mask, fft_rank 2               :  the same three passes over (n1, n2)
+//   full mask, fft_rank 3               :  forward pass, middle pass without k-space work, readout axis
+//                                         (mask, residual), middle pass back, inverse pass
 //
 // With a mask that does not depend on the readout index the readout transform commutes with the
 // mask, so A^H(Ax - y) = S^H P^H M (M P S x - R^H y) with P over the phase-encode axes and R over
 // the readout axis only; R^H y is needed at sampled positions alone.
 #include "../../include/gleam.h"
 #include "size_ops.cuh"
-#include "dc_rowtile.cuh"
+#include "dc_mid.cuh"
+#include "dc_axis.cuh"
 #include "dc_fused3d.cuh"
 #include "dc_fused_entry.h"
 #include "dc_entry.h"
@@ -26,118 +28,92 @@
 
 namespace gleam {
 
-#define GLEAM_SIZE(N, A0, A1, A2, LR, B0, B1, B2, LC) extern const SizeOps size_ops_##N;
+#define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) extern const SizeOps size_ops_##N; extern const MidOps mid_ops_##N; extern const AxisOps axis_ops_##N;
 #include "sizes.def"
 #undef GLEAM_SIZE
 
-const PairOps* find_pair(int n1, int n2);     // kernels_pairs.cu
+#define GLEAM_TILE_RYS GLEAM_TILE_R(1) GLEAM_TILE_R(2) GLEAM_TILE_R(4) GLEAM_TILE_R(6) GLEAM_TILE_R(8) GLEAM_TILE_R(10) \
+    GLEAM_TILE_R(12) GLEAM_TILE_R(16) GLEAM_TILE_R(20)
+#define GLEAM_TILE_R(R) const TileOps* find_tile_##R(int n2);     // kernels_tile.cu
+GLEAM_TILE_RYS
+#undef GLEAM_TILE_R
 
 static const SizeOps* find_size(int n) {
     switch (n) {
-#define GLEAM_SIZE(N, A0, A1, A2, LR, B0, B1, B2, LC) case N: return &size_ops_##N;
+#define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) case N: return &size_ops_##N;
 #include "sizes.def"
 #undef GLEAM_SIZE
         default: return nullptr;
     }
 }
+static const MidOps* find_mid(int n) {
+    switch (n) {
+#define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) case N: return &mid_ops_##N;
+#include "sizes.def"
+#undef GLEAM_SIZE
+        default: return nullptr;
+    }
+}
+static const AxisOps* find_axis(int n) {
+    switch (n) {
+#define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) case N: return &axis_ops_##N;
+#include "sizes.def"
+#undef GLEAM_SIZE
+        default: return nullptr;
+    }
+}
+static const TileOps* find_tile(int ry, int n2) {
+    switch (ry) {
+#define GLEAM_TILE_R(R) case R: return find_tile_##R(n2);
+        GLEAM_TILE_RYS
+#undef GLEAM_TILE_R
+        default: return nullptr;
+    }
+}
 
-// Ranks of the sampled phase-encode positions, in the order of the raw (half-shifted) k index q:
-//   zidx[bt][q]  = rank of q among the sampled positions, or -1 where M[sh(q)] == 0
-//   zlist[bt][r] = unshifted source position p = sh(q) of rank r;   zcount[bt] = number sampled.
-// Block (chunk, bt) owns ZMAP_CHUNK consecutive q; it counts the sampled positions before its chunk
-// by itself (no communication between blocks), then scans its own chunk.
-#define ZMAP_THREADS 1024
-#define ZMAP_PER_THREAD 2
-#define ZMAP_CHUNK (ZMAP_THREADS * ZMAP_PER_THREAD)
-#define ZMAP_TILE 8
+// Ranks of the sampled (ky, kz) positions, in the order the middle pass consumes them: groups of equal raw
+// ky mod ry, inside a group by (ky div ry, kz), so that the entries one of its blocks needs are contiguous.
+//   zidx[bt][q]  = rank of the raw (half-shifted) position q among the sampled ones, or -1 where M[sh(q)] == 0
+//   zlist[bt][r] = unshifted source position p = sh(q) of rank r;   zcount[bt] = number sampled
+//   zstart[bt][k0] = first rank of group k0, zstart[bt][ry] the total;   m2c[bt][r] = squared mask weight
+// One warp per raw ky row, in two launches: the sampled positions of every row are counted, then numbered behind
+// those of the rows before it in that order (a warp adds up to n1 counts by itself).  Bound by latency: a mask plane
+// is a few hundred KB.
+#define ZMAP_THREADS 256
 #define ZMAP_MAX_RY 32
+template <bool COUNT>
 __global__ void __launch_bounds__(ZMAP_THREADS) zmap_kernel(const float* __restrict__ mask, int* __restrict__ zidx,
                                                             int* __restrict__ zlist, int* __restrict__ zcount,
                                                             float* __restrict__ m2c, int* __restrict__ zstart,
-                                                            int* __restrict__ chunk_cnt, int count_only,
-                                                            int n1, int n2, int rank, int ry) {
-    __shared__ int warp_sum[ZMAP_THREADS / 32];
-    __shared__ int base_sh;
-    const int pe = (rank == 2) ? n2 : n1 * n2;
-    const long long bt = blockIdx.y;
-    const float* mk = mask + bt * pe;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int q_begin = blockIdx.x * ZMAP_CHUNK;
-    // Rank order.  rank 2: the raw k index.  rank 3: column tiles of ZMAP_TILE raw kz indices, inside
-    // a tile by (raw ky, raw kz): the sampled entries that one tile of the column kernel needs are
-    // then neighbours in the compact z table.  raw_of maps the scan position to the raw position.
-    // ry > 0 (row-tile path): groups of equal ky mod ry, inside a group by (ky div ry, kz): the sampled
-    // entries one block of the row-tile middle pass needs are contiguous; zstart[bt][k0] is the
-    // first rank of group k0, zstart[bt][ry] the total.
-    const bool tiled = (ry == 0) && (rank == 3) && (n2 % ZMAP_TILE == 0);
-    const int per_k0 = (ry > 0) ? (n1 / ry) * n2 : 1;
-    auto raw_of = [&](int q) -> int {
-        if (ry > 0) {
-            const int k0 = q / per_k0, rem = q - k0 * per_k0;
-            return (k0 + ry * (rem / n2)) * n2 + rem % n2;
-        }
-        if (!tiled) return q;
-        const int per_tile = n1 * ZMAP_TILE;
-        const int tile = q / per_tile, rem = q - tile * per_tile;
-        return (rem / ZMAP_TILE) * n2 + tile * ZMAP_TILE + rem % ZMAP_TILE;
-    };
-    auto src_of = [&](int q) -> int {            // unshifted source position of scan position q
-        const int rq = raw_of(q);
-        if (rank == 2) return shift_half(rq, n2);
-        return shift_half(rq / n2, n1) * n2 + shift_half(rq % n2, n2);
-    };
-    // Two launches: the first (count_only) stores the number of sampled positions of every chunk,
-    // the second adds up the chunks before its own and numbers its entries.
-    const int nchunks = gridDim.x;
-    if (count_only) {
+                                                            int* __restrict__ row_cnt, int n1, int n2, int ry) {
+    const int lane = threadIdx.x & 31, row = blockIdx.x * (ZMAP_THREADS / 32) + (threadIdx.x >> 5);   // row = k0 * by + k1
+    if (row >= n1) return;
+    const int by = n1 / ry, k0 = row / by, k1 = row - k0 * by, ky = k0 + ry * k1;
+    const long long bt = blockIdx.y, pe = (long long)n1 * n2;
+    const int src_row = shift_half(ky, n1) * n2;
+    const float* mk = mask + bt * pe + src_row;
+    int* cnt = row_cnt + bt * n1;
+    if (COUNT) {
         int c = 0;
-#pragma unroll
-        for (int e = 0; e < ZMAP_PER_THREAD; ++e) {
-            const int q = q_begin + tid * ZMAP_PER_THREAD + e;
-            c += (q < pe && mk[src_of(q)] != 0.f) ? 1 : 0;
-        }
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (lane == 0) warp_sum[warp] = c;
-        __syncthreads();
-        if (tid == 0) { int t = 0; for (int w = 0; w < ZMAP_THREADS / 32; ++w) t += warp_sum[w]; chunk_cnt[bt * nchunks + blockIdx.x] = t; }
+        for (int kz = lane; kz < n2; kz += 32) c += (mk[kz] != 0.f) ? 1 : 0;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) cnt[row] = c;
         return;
     }
-    if (tid == 0) { int t = 0; for (int w = 0; w < (int)blockIdx.x; ++w) t += chunk_cnt[bt * nchunks + w]; base_sh = t; }
-    __syncthreads();
-    const int base = base_sh;
-    __syncthreads();
-    // this chunk: each thread owns ZMAP_PER_THREAD consecutive q
-    const int q0 = q_begin + tid * ZMAP_PER_THREAD;
-    int src[ZMAP_PER_THREAD]; bool on[ZMAP_PER_THREAD]; int mine = 0;
-#pragma unroll
-    for (int e = 0; e < ZMAP_PER_THREAD; ++e) {
-        const int q = q0 + e;
-        src[e] = (q < pe) ? src_of(q) : 0;
-        on[e] = (q < pe) && (mk[src[e]] != 0.f);
-        mine += on[e] ? 1 : 0;
+    int r = 0;
+    for (int e = lane; e < row; e += 32) r += cnt[e];
+    r = __reduce_add_sync(0xffffffffu, r);
+    if (lane == 0 && k1 == 0) zstart[bt * (ZMAP_MAX_RY + 1) + k0] = r;
+    for (int z0 = 0; z0 < n2; z0 += 32) {
+        const int kz = z0 + lane, sz = shift_half(kz, n2);
+        const float mv = (kz < n2) ? mk[sz] : 0.f;
+        const unsigned bal = __ballot_sync(0xffffffffu, mv != 0.f);
+        const int mine = r + __popc(bal & ((1u << lane) - 1u));
+        if (kz < n2) zidx[bt * pe + (long long)ky * n2 + kz] = (mv != 0.f) ? mine : -1;
+        if (mv != 0.f) { zlist[bt * pe + mine] = src_row + sz; m2c[bt * pe + mine] = mv * mv; }
+        r += __popc(bal);
     }
-    int incl = mine;                                         // inclusive scan inside the warp
-    for (int o = 1; o < 32; o <<= 1) { int t = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += t; }
-    if (lane == 31) warp_sum[warp] = incl;
-    __syncthreads();
-    int wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += warp_sum[w];
-    int r = base + wbase + incl - mine;
-#pragma unroll
-    for (int e = 0; e < ZMAP_PER_THREAD; ++e) {
-        const int q = q0 + e;
-        if (q >= pe) break;
-        if (ry > 0 && q % per_k0 == 0) zstart[bt * (ZMAP_MAX_RY + 1) + q / per_k0] = r;
-        if (on[e]) {
-            const float mv = mk[src[e]];
-            zidx[bt * pe + raw_of(q)] = r; zlist[bt * pe + r] = src[e]; m2c[bt * pe + r] = mv * mv; ++r;
-        }
-        else zidx[bt * pe + raw_of(q)] = -1;
-    }
-    if (q_begin + ZMAP_CHUNK >= pe && tid == ZMAP_THREADS - 1) {                 // last chunk, last thread: total
-        zcount[bt] = r;
-        if (ry > 0) zstart[bt * (ZMAP_MAX_RY + 1) + ry] = r;
-    }
+    if (lane == 0 && row == n1 - 1) { zcount[bt] = r; zstart[bt * (ZMAP_MAX_RY + 1) + ry] = r; }
 }
 
 static inline uint64_t align_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
@@ -148,7 +124,7 @@ struct Layout {
     long long V, units, images;
     bool separable;
     // workspace (byte offsets)
-    uint64_t off_z, off_zidx, off_zlist, off_zcount, off_m2c, off_zstart, off_zchunk, off_W, total;
+    uint64_t off_z, off_zidx, off_zlist, off_zcount, off_m2c, off_zstart, off_zrows, off_W, total;
     int G;  // readout slabs per chunk (rank 3 separable)
     // fused persistent kernel of the separable 3-D path: control words first (at offset 0, the same
     // for forward and VJP calls, so that gleam_dc_check_status finds them), then the ring of R slabs
@@ -217,7 +193,7 @@ static int make_layout(const gleam_dims* d, bool with_y, Layout* L) {
     if (L->images * L->n0 * L->n1 >= (1ll << 31)) return GLEAM_ERR_BAD_DIMS;   // row counters are 32-bit
     L->separable = d->mask_kind == GLEAM_MASK_READOUT_INVARIANT;
     uint64_t off = 0;
-    L->off_z = L->off_zidx = L->off_zlist = L->off_zcount = L->off_m2c = L->off_zstart = L->off_zchunk = L->off_W = 0; L->G = 0;
+    L->off_z = L->off_zidx = L->off_zlist = L->off_zcount = L->off_m2c = L->off_zstart = L->off_zrows = L->off_W = 0; L->G = 0;
     L->fused = false; L->off_ctrl = L->ctrl_bytes = L->off_ring = 0; L->R = L->L2 = L->L3 = 0;
     if (L->separable && L->rank == 3 && fused_enabled() && fused3d_supported(L->n1, L->n2) &&
         L->images * L->n0 < (1ll << 24)) {
@@ -240,7 +216,7 @@ static int make_layout(const gleam_dims* d, bool with_y, Layout* L) {
             L->off_zcount = off; off = align_up(off + (uint64_t)L->images * sizeof(int), 256);
             L->off_m2c = off; off = align_up(off + (uint64_t)L->images * pe * sizeof(float), 256);
             L->off_zstart = off; off = align_up(off + (uint64_t)L->images * (ZMAP_MAX_RY + 1) * sizeof(int), 256);
-            L->off_zchunk = off; off = align_up(off + (uint64_t)L->images * ((pe + ZMAP_CHUNK - 1) / ZMAP_CHUNK) * sizeof(int), 256);
+            L->off_zrows = off; off = align_up(off + (uint64_t)L->images * L->n1 * sizeof(int), 256);
         }
         if (L->rank == 3) {
             const uint64_t slab = (uint64_t)L->units * L->n1 * L->n2 * sizeof(cf);
@@ -307,8 +283,7 @@ cudaError_t prof_mark(int cls, cudaStream_t s) {
 
 bool dot_rows_supported(const gleam_dims* d) {
     if (!d || d->fft_rank != 2 || d->mask_kind != GLEAM_MASK_READOUT_INVARIANT) return false;
-    const SizeOps* op2 = find_size(d->n[2]);
-    return op2 && op2->row_is_warp_resident;
+    return find_size(d->n[2]) != nullptr;
 }
 
 int run(const void* x, const void* y, const void* sens, const float* mask, float eta, void* out,
@@ -318,6 +293,9 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
     if (mode == RUN_PREPARE) {
         if (!y) return GLEAM_ERR_NULL_POINTER;
         x = nullptr; sens = nullptr; out = nullptr;
+    } else if (mode == RUN_ADJOINT) {
+        if (!y || !sens || !out) return GLEAM_ERR_NULL_POINTER;
+        x = nullptr; eta = 1.0f;                             // 0 - 1 * A^H (A 0 - y)
     } else if (!x || !sens || !out) {
         return GLEAM_ERR_NULL_POINTER;
     }
@@ -345,7 +323,7 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
     // aliasing: out may equal x exactly; nothing else may overlap an output or the workspace
     if (layout & ~(GLEAM_X_CHANNELS | GLEAM_OUT_CHANNELS)) return GLEAM_ERR_BAD_DIMS;
     if (mode != RUN_PREPARE) {
-        if (out != x && overlaps(out, img_b, x, img_b)) return GLEAM_ERR_ALIAS;
+        if (x && out != x && overlaps(out, img_b, x, img_b)) return GLEAM_ERR_ALIAS;
         if (out == x && ((layout & GLEAM_X_CHANNELS) != 0) != ((layout & GLEAM_OUT_CHANNELS) != 0)) return GLEAM_ERR_ALIAS;
         if (overlaps(out, img_b, sens, sens_b) || overlaps(out, img_b, mask, mask_b)) return GLEAM_ERR_ALIAS;
         if (y && overlaps(out, img_b, y, ksp_b)) return GLEAM_ERR_ALIAS;
@@ -353,7 +331,7 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
     }
     if (L.total > 0) {
         const void* w = d->workspace;
-        if ((mode != RUN_PREPARE && (overlaps(w, L.total, x, img_b) || overlaps(w, L.total, out, img_b) ||
+        if ((mode != RUN_PREPARE && ((x && overlaps(w, L.total, x, img_b)) || overlaps(w, L.total, out, img_b) ||
                                      overlaps(w, L.total, sens, sens_b))) ||
             overlaps(w, L.total, mask, mask_b) || (y && overlaps(w, L.total, y, ksp_b)) ||
             (aty && overlaps(w, L.total, aty, img_b)))
@@ -363,123 +341,103 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
 
     cudaStream_t s = (cudaStream_t)d->stream;
     char* ws = (char*)d->workspace;
-    const SizeOps* op2 = find_size(L.n2);
-    const SizeOps* op1 = find_size(L.n1);
-    const SizeOps* op0 = (L.rank == 3) ? find_size(L.n0) : nullptr;
+    const bool adjoint = mode == RUN_ADJOINT;
+    const MidOps* mid = find_mid(L.n1);          // split of n1 in the row-tile passes
+    const float g = gsign(L.n2) * gsign(L.n1) * (L.rank == 3 ? gsign(L.n0) : 1.f);
+    cf* z = (L.separable && y) ? (cf*)(ws + L.off_z) : nullptr;
+    int* zidx = (int*)(ws + L.off_zidx);
+    float* m2c = (float*)(ws + L.off_m2c);
+    int* zstart = (int*)(ws + L.off_zstart);
 
-    RowArgs ra{};
-    ra.x = (const cf*)x; ra.sens = (const cf*)sens; ra.out = (cf*)out; ra.eta = eta;
-    ra.C = L.C; ra.T = L.T; ra.Ts = L.Ts; ra.RPB = L.n0 * L.n1;
-    ra.x_planar = (layout & GLEAM_X_CHANNELS) ? 1 : 0; ra.out_planar = (layout & GLEAM_OUT_CHANNELS) ? 1 : 0;
-    ra.plane = (long long)L.T * L.V;
-    ra.aty = (const cf*)aty;
-    ColArgs ca{};
-    ca.C = L.C; ca.T = L.T; ca.rank = L.rank; ca.n0 = L.n0; ca.n1 = L.n1; ca.n2 = L.n2;
-
-    if (L.separable) {
-        cf* z = y ? (cf*)(ws + L.off_z) : nullptr;
-        if (y) {
-            // ranks of the sampled positions, then the z table: inverse transform of y along the
-            // readout axis at the sampled positions only
-            int* zidx = (int*)(ws + L.off_zidx);
+    if (L.separable && y && mode != RUN_APPLY) {     // RUN_APPLY: the tables of an earlier RUN_PREPARE are in the workspace
+        // ranks of the sampled positions (rank 2: the blocks that need them derive them from the mask row), then the
+        // z table: inverse transform of y along the readout axis at the sampled positions only
+        ColArgs cz{};
+        cz.C = L.C; cz.T = L.T; cz.rank = L.rank; cz.n2 = L.n2;
+        cz.y = (const cf*)y; cz.z = z; cz.mask = mask; cz.es = (int)pe; cz.nouter = L.units;
+        if (L.rank == 3) {
             int* zlist = (int*)(ws + L.off_zlist);
             int* zcount = (int*)(ws + L.off_zcount);
-            float* m2c = (float*)(ws + L.off_m2c);
-            int* zstart = (int*)(ws + L.off_zstart);
-            const PairOps* zpair = (L.rank == 3) ? find_pair(L.n1, L.n2) : nullptr;
-            const int zry = (zpair && zpair->ry <= ZMAP_MAX_RY) ? zpair->ry : 0;
-            int* zchunk = (int*)(ws + L.off_zchunk);
-            const dim3 zgrid((unsigned)((pe + ZMAP_CHUNK - 1) / ZMAP_CHUNK), (unsigned)L.images);
-            // rank 2 with a one-pass row kernel that counts the sampled positions itself: nothing
-            // but the z table needs the ranks, and the kernel that writes it derives them per block
-            const bool self_ranks = L.rank == 2 && op2->row_is_warp_resident && pe <= COLZ_SELF_MAX;
-            if (mode != RUN_APPLY && !self_ranks) {      // RUN_APPLY: the tables of an earlier RUN_PREPARE are in the workspace
-                CK(prof_mark(GLEAM_K_PREP_M2, s));
-                if (zgrid.x > 1) {        // a table of one chunk needs no counts of earlier chunks
-                    zmap_kernel<<<zgrid, ZMAP_THREADS, 0, s>>>(mask, zidx, zlist, zcount, m2c, zstart, zchunk, 1, L.n1, L.n2, L.rank, zry);
-                    CK(cudaGetLastError());
-                    CK(prof_mark(GLEAM_K_PREP_M2, s));
-                }
-                zmap_kernel<<<zgrid, ZMAP_THREADS, 0, s>>>(mask, zidx, zlist, zcount, m2c, zstart, zchunk, 0, L.n1, L.n2, L.rank, zry);
-                CK(cudaGetLastError());
-            }
-            ca.zidx = zidx; ca.zlist = zlist; ca.zcount = zcount; ca.m2c = m2c; ca.zstart = zry ? zstart : nullptr;
-            ra.zidx = zidx;
-            ColArgs cz = ca;
-            cz.y = (const cf*)y; cz.z = z; cz.mask = mask;
-            if (self_ranks) { cz.zlist = nullptr; cz.zcount = nullptr; cz.zidx = nullptr; }
-            cz.es = (int)pe; cz.nouter = L.units;
-            const int nro = (L.rank == 2) ? L.n1 : L.n0;
-            float g = gsign(nro) * gsign(L.n2) * (L.rank == 3 ? gsign(L.n1) : 1.f);
-            cz.scale = g / sqrtf((float)nro * (float)pe);
-            if (mode != RUN_APPLY) LAUNCH(GLEAM_K_COL_Z, ((L.rank == 2) ? op1 : op0)->col(COL_Z, cz, s));
+            int* zrows = (int*)(ws + L.off_zrows);
+            const dim3 zgrid((unsigned)((L.n1 + ZMAP_THREADS / 32 - 1) / (ZMAP_THREADS / 32)), (unsigned)L.images);
+            CK(prof_mark(GLEAM_K_PREP_M2, s));
+            zmap_kernel<true><<<zgrid, ZMAP_THREADS, 0, s>>>(mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry);
+            CK(cudaGetLastError());
+            CK(prof_mark(GLEAM_K_PREP_M2, s));
+            zmap_kernel<false><<<zgrid, ZMAP_THREADS, 0, s>>>(mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry);
+            CK(cudaGetLastError());
+            cz.zlist = zlist; cz.zcount = zcount;
         }
-        if (mode == RUN_PREPARE) { CK(prof_mark(-1, s)); return GLEAM_OK; }
-        if (L.rank == 2) {
-            ra.mask = mask; ra.z = z; ra.rpb = L.n1; ra.row0 = 0; ra.nrows = L.images * L.n1;
-            ra.dot_rows = dot_rows;
-            LAUNCH(GLEAM_K_ROW_FUSED, op2->row(ROW_FUSED, ra, s));
+        cz.scale = g / sqrtf((float)(L.rank == 2 ? L.n1 : L.n0) * (float)pe);
+        LAUNCH(GLEAM_K_COL_Z, find_size(L.rank == 2 ? L.n1 : L.n0)->col_z(cz, s));
+    }
+    if (mode == RUN_PREPARE) {                       // a full mask has nothing to prepare
+        if (L.separable) CK(prof_mark(-1, s));
+        return GLEAM_OK;
+    }
+    const int x_planar = (layout & GLEAM_X_CHANNELS) ? 1 : 0, out_planar = (layout & GLEAM_OUT_CHANNELS) ? 1 : 0;
+    const long long plane = (long long)L.T * L.V;
+    if (L.separable && L.rank == 2) {
+        RowArgs ra{};
+        ra.x = (const cf*)x; ra.sens = (const cf*)sens; ra.out = (cf*)out; ra.eta = eta; ra.mask = mask; ra.z = z;
+        ra.C = L.C; ra.T = L.T; ra.Ts = L.Ts; ra.RPB = L.n1; ra.nrows = L.images * L.n1;
+        ra.x_planar = x_planar; ra.out_planar = out_planar; ra.plane = plane;
+        ra.aty = (const cf*)aty; ra.dot_rows = dot_rows;
+        LAUNCH(GLEAM_K_ROW_FUSED, find_size(L.n2)->row(ra, s));
+        CK(prof_mark(-1, s));
+        return GLEAM_OK;
+    }
+    if (L.fused && !y && !aty && layout == 0) {
+        // one persistent kernel walks all slabs; its counters start from zero
+        FusedArgs fa{};
+        fa.x = (const cf*)x; fa.sens = (const cf*)sens; fa.out = (cf*)out; fa.W = (cf*)(ws + L.off_ring);
+        fa.mask = mask; fa.ctrl = (int*)(ws + L.off_ctrl); fa.eta = eta; fa.scale2 = 1.0f / (float)pe;
+        fa.C = L.C; fa.T = L.T; fa.Ts = L.Ts; fa.n0 = L.n0; fa.nslabs = (int)(L.images * L.n0);
+        fa.R = L.R; fa.L2 = L.L2; fa.L3 = L.L3;
+        fa.withhold = fused3d_withhold(); fa.limit_ns = fused3d_limit_ns();
+        CK(cudaMemsetAsync(fa.ctrl, 0, L.ctrl_bytes, s));
+        LAUNCH(GLEAM_K_FUSED3D, fused3d_launch(L.n1, fa, s));
+        CK(prof_mark(-1, s));
+        return GLEAM_OK;
+    }
+
+    // ---- row-tile passes ----
+    const TileOps* tile = find_tile(mid->ry, L.n2);
+    const long long plane_pe = (long long)L.n1 * L.n2, tiles = L.images * L.n0 * mid->by;
+    TileArgs ta{};
+    ta.x = (const cf*)x; ta.sens = (const cf*)sens; ta.out = (cf*)out; ta.V = (cf*)(ws + L.off_W); ta.eta = eta;
+    ta.C = L.C; ta.T = L.T; ta.Ts = L.Ts; ta.n0 = L.n0; ta.BY = mid->by;
+    ta.x_planar = x_planar; ta.out_planar = out_planar; ta.plane = plane; ta.aty = (const cf*)aty;
+    MidArgs ma{};
+    ma.V = ta.V; ma.mask = mask; ma.zin = z; ma.zidx = zidx; ma.m2c = m2c; ma.zstart = zstart; ma.y = (const cf*)y;
+    ma.C = L.C; ma.T = L.T; ma.n0 = L.n0; ma.NZ = L.n2; ma.nunits = L.units;
+    ma.scale = g / sqrtf((float)plane_pe); ma.scale2 = 1.0f / (float)plane_pe;
+    const bool full3 = !L.separable && L.rank == 3;
+    const int slabs = L.separable ? L.G : L.n0;      // per chunk
+    for (int i0 = 0; i0 < L.n0; i0 += slabs) {
+        const int n = (L.n0 - i0 < slabs) ? (L.n0 - i0) : slabs;
+        ta.G = ma.G = n; ta.i0_start = ma.i0_start = i0;
+        // workspace (unit, slab, k0, j, kz); with a readout pass (unit, k0, j, slab, kz), so that the lines along the
+        // readout axis are pieces of one contiguous block
+        ta.v_unit = n * plane_pe;
+        ta.v_slab = full3 ? L.n2 : plane_pe;
+        ta.v_j = full3 ? (long long)L.n0 * L.n2 : L.n2;
+        ta.v_k0 = mid->by * ta.v_j;
+        ma.v_unit = ta.v_unit; ma.v_slab = ta.v_slab; ma.v_k0 = ta.v_k0; ma.v_j = ta.v_j;
+        if (!adjoint) LAUNCH(GLEAM_K_ROW_FWD, tile->fwd(ta, L.images, tiles, s));
+        if (L.separable) {
+            LAUNCH(GLEAM_K_COL_MID_SEP, mid->launch(!z ? MID_SEP : adjoint ? MID_ADJ_Z : MID_SEP_Z, ma, s));
+        } else if (L.rank == 2) {
+            LAUNCH(GLEAM_K_COL_MID_FULL, mid->launch(adjoint ? MID_ADJ_FULL : MID_FULL, ma, s));
         } else {
-            if (L.fused && !y && !aty && layout == 0) {
-                // one persistent kernel walks all slabs; its counters start from zero
-                FusedArgs fa{};
-                fa.x = (const cf*)x; fa.sens = (const cf*)sens; fa.out = (cf*)out; fa.W = (cf*)(ws + L.off_ring);
-                fa.mask = mask; fa.zin = z; fa.zidx = ca.zidx; fa.m2c = ca.m2c; fa.zstart = ca.zstart;
-                fa.ctrl = (int*)(ws + L.off_ctrl); fa.eta = eta; fa.scale2 = 1.0f / (float)pe;
-                fa.C = L.C; fa.T = L.T; fa.Ts = L.Ts; fa.n0 = L.n0; fa.nslabs = (int)(L.images * L.n0);
-                fa.R = L.R; fa.L2 = L.L2; fa.L3 = L.L3;
-                fa.withhold = fused3d_withhold(); fa.limit_ns = fused3d_limit_ns();
-                CK(cudaMemsetAsync(fa.ctrl, 0, L.ctrl_bytes, s));
-                LAUNCH(GLEAM_K_FUSED3D, fused3d_launch(L.n1, fa, s));
-                CK(prof_mark(-1, s));
-                return GLEAM_OK;
-            }
-            cf* W = (cf*)(ws + L.off_W);
-            const PairOps* pair = find_pair(L.n1, L.n2);
-            for (int i0 = 0; i0 < L.n0; i0 += L.G) {
-                const int g = (L.n0 - i0 < L.G) ? (L.n0 - i0) : L.G;
-                if (pair) {
-                    // row-tile kernels: every pass over the workspace is contiguous
-                    TileArgs ta{};
-                    ta.x = (const cf*)x; ta.sens = (const cf*)sens; ta.out = (cf*)out; ta.V = W; ta.mask = mask;
-                    ta.zin = z; ta.zidx = ca.zidx; ta.m2c = ca.m2c; ta.zstart = ca.zstart; ta.eta = eta; ta.scale2 = 1.0f / (float)pe;
-                    ta.C = L.C; ta.T = L.T; ta.Ts = L.Ts; ta.n0 = L.n0; ta.G = g; ta.i0_start = i0; ta.nunits = L.units;
-                    ta.x_planar = ra.x_planar; ta.out_planar = ra.out_planar; ta.plane = ra.plane; ta.aty = ra.aty;
-                    LAUNCH(GLEAM_K_ROW_FWD, pair->fwd(ta, L.images, s));
-                    LAUNCH(GLEAM_K_COL_MID_SEP, pair->mid(ta, s));
-                    LAUNCH(GLEAM_K_ROW_INV, pair->inv(ta, L.images, s));
-                    continue;
-                }
-                ra.W = W; ra.rpb = g * L.n1; ra.row0 = i0 * L.n1; ra.nrows = L.images * ra.rpb;
-                LAUNCH(GLEAM_K_ROW_FWD, op2->row(ROW_FWD, ra, s));
-                ColArgs cm = ca;
-                cm.W = W; cm.mask = mask; cm.scale2 = 1.0f / (float)pe; cm.zin = z; cm.es = L.n2; cm.nouter = L.units * g; cm.G = g; cm.i0_start = i0;
-                LAUNCH(GLEAM_K_COL_MID_SEP, op1->col(COL_MID_SEP, cm, s));
-                LAUNCH(GLEAM_K_ROW_INV, op2->row(ROW_INV, ra, s));
-            }
+            if (!adjoint) LAUNCH(GLEAM_K_COL_FWD, mid->launch(MID_FWD, ma, s));
+            AxisArgs aa{};
+            aa.W = ta.V; aa.y = (const cf*)y; aa.mask = mask; aa.C = L.C; aa.T = L.T; aa.n1 = L.n1; aa.n2 = L.n2; aa.ry = mid->ry;
+            aa.nunits = L.units; aa.scale = g / (float)sqrt((double)L.V); aa.scale2 = (float)(1.0 / (double)L.V);
+            LAUNCH(GLEAM_K_COL_MID_FULL, find_axis(L.n0)->launch(adjoint ? AXIS_ADJ : AXIS_MID, aa, s));
+            LAUNCH(GLEAM_K_COL_INV, mid->launch(MID_INV, ma, s));
         }
-    } else {
-        if (mode == RUN_PREPARE) return GLEAM_OK;      // a full mask has nothing to prepare
-        cf* W = (cf*)(ws + L.off_W);
-        ra.W = W; ra.rpb = L.n0 * L.n1; ra.row0 = 0; ra.nrows = L.images * ra.rpb;
-        LAUNCH(GLEAM_K_ROW_FWD, op2->row(ROW_FWD, ra, s));
-        float g = gsign(L.n2) * gsign(L.n1) * (L.rank == 3 ? gsign(L.n0) : 1.f);
-        const double ntot = (L.rank == 3) ? (double)L.V : (double)L.n1 * L.n2;
-        ColArgs cm = ca;
-        cm.W = W; cm.y = (const cf*)y; cm.mask = mask;
-        cm.scale = g / (float)sqrt(ntot); cm.scale2 = (float)(1.0 / ntot);
-        if (L.rank == 2) {
-            cm.es = L.n2; cm.nouter = L.units;
-            LAUNCH(GLEAM_K_COL_MID_FULL, op1->col(COL_MID_FULL, cm, s));
-        } else {
-            ColArgs c1 = ca;
-            c1.W = W; c1.es = L.n2; c1.nouter = L.units * L.n0;
-            LAUNCH(GLEAM_K_COL_FWD, op1->col(COL_FWD, c1, s));
-            cm.es = L.n1 * L.n2; cm.nouter = L.units;
-            LAUNCH(GLEAM_K_COL_MID_FULL, op0->col(COL_MID_FULL, cm, s));
-            LAUNCH(GLEAM_K_COL_INV, op1->col(COL_INV, c1, s));
-        }
-        LAUNCH(GLEAM_K_ROW_INV, op2->row(ROW_INV, ra, s));
+        LAUNCH(GLEAM_K_ROW_INV, tile->inv(ta, L.images, tiles, s));
     }
     CK(prof_mark(-1, s));
     return GLEAM_OK;
@@ -615,16 +573,7 @@ GLEAM_API int gleam_dc_vjp_layout(const void* grad_out, const void* sens, const 
 }
 
 GLEAM_API int gleam_dc_adjoint(const void* y, const void* sens, const float* mask, void* out, const gleam_dims* dims) {
-    if (!dims || !y || !sens || !mask || !out) return GLEAM_ERR_NULL_POINTER;
-    if (((uintptr_t)out & 15) != 0) return GLEAM_ERR_BAD_DIMS;
-    int rc = gleam::check_device_ptr(out);
-    if (rc != GLEAM_OK) return rc;
-    // all argument checks of the step itself, before the output is cleared
-    rc = gleam::run(out, y, sens, mask, 1.0f, out, dims, gleam::RUN_ALL, nullptr, true);
-    if (rc != GLEAM_OK) return rc;
-    const uint64_t img_b = (uint64_t)dims->batch * dims->frames * dims->n[0] * dims->n[1] * dims->n[2] * sizeof(gleam::cf);
-    if (cudaMemsetAsync(out, 0, img_b, (cudaStream_t)dims->stream) != cudaSuccess) return GLEAM_ERR_CUDA;
-    return gleam::run(out, y, sens, mask, 1.0f, out, dims);     // 0 - 1 * A^H (A 0 - y), in place
+    return gleam::run(nullptr, y, sens, mask, 1.0f, out, dims, gleam::RUN_ADJOINT);
 }
 
 GLEAM_API int gleam_dc_forward_aty(const void* x, const void* aty, const void* sens, const float* mask, float eta,
@@ -683,8 +632,13 @@ GLEAM_API int gleam_dc_fused_wait_stats(const gleam_dims* dims, uint64_t* ns_and
 }
 
 GLEAM_API int32_t gleam_dc_rowtile_split(int32_t n1, int32_t n2) {
-    const gleam::PairOps* p = gleam::find_pair(n1, n2);
-    return p ? p->ry : 0;
+    static const int pairs[][3] = {
+#define GLEAM_PAIR(N1, RY, BY, N2, Z0) {N1, N2, RY},
+#include "pairs.def"
+#undef GLEAM_PAIR
+    };
+    for (const auto& p : pairs) if (p[0] == n1 && p[1] == n2) return p[2];
+    return 0;
 }
 
 GLEAM_API void gleam_dc_set_fused(int32_t on) { gleam::g_fused_on.store(on ? 1 : 0); }
@@ -827,29 +781,26 @@ GLEAM_API int gleam_dc_grad_y(const void* grad_out, const void* sens, const floa
         return GLEAM_ERR_ALIAS;
     cudaStream_t s = (cudaStream_t)dims->stream;
     cf* W = (cf*)((char*)dims->workspace + G.off_W);
-    const SizeOps* op2 = find_size(L.n2);
-    const SizeOps* op1 = find_size(L.n1);
-    const SizeOps* op0 = (L.rank == 3) ? find_size(L.n0) : nullptr;
-    RowArgs ra{};
-    ra.x = (const cf*)grad_out; ra.sens = (const cf*)sens; ra.W = W; ra.eta = 0.f;
-    ra.C = L.C; ra.T = L.T; ra.Ts = L.Ts; ra.RPB = L.n0 * L.n1; ra.rpb = ra.RPB; ra.row0 = 0; ra.nrows = L.images * ra.rpb;
-    LAUNCH(GLEAM_K_ROW_FWD, op2->row(ROW_FWD, ra, s));
-    ColArgs ca{};
-    ca.C = L.C; ca.T = L.T; ca.rank = L.rank; ca.n0 = L.n0; ca.n1 = L.n1; ca.n2 = L.n2; ca.W = W;
+    const MidOps* mid = find_mid(L.n1);
     const float gs = gsign(L.n2) * gsign(L.n1) * (L.rank == 3 ? gsign(L.n0) : 1.f);
     const double ntot = (L.rank == 3) ? (double)L.V : (double)L.n1 * L.n2;
-    ColArgs cy = ca;
-    cy.mask = mask; cy.ky_out = (cf*)grad_y; cy.mask_pe = L.separable ? (int)pe : 0;
-    cy.scale = eta * gs / (float)sqrt(ntot);
+    TileArgs ta{};
+    ta.x = (const cf*)grad_out; ta.sens = (const cf*)sens; ta.V = W; ta.C = L.C; ta.T = L.T; ta.Ts = L.Ts; ta.n0 = L.n0; ta.G = L.n0; ta.BY = mid->by;
+    ta.v_unit = L.V; ta.v_slab = L.n2; ta.v_j = (long long)L.n0 * L.n2; ta.v_k0 = mid->by * ta.v_j;
+    LAUNCH(GLEAM_K_ROW_FWD, find_tile(mid->ry, L.n2)->fwd(ta, L.images, L.images * L.n0 * mid->by, s));
+    MidArgs ma{};
+    ma.V = W; ma.v_unit = ta.v_unit; ma.v_slab = ta.v_slab; ma.v_k0 = ta.v_k0; ma.v_j = ta.v_j;
+    ma.C = L.C; ma.T = L.T; ma.n0 = ma.G = L.n0; ma.NZ = L.n2; ma.nunits = L.units;
     if (L.rank == 2) {
-        cy.es = L.n2; cy.nouter = L.units;
-        LAUNCH(GLEAM_K_COL_FWD, op1->col(COL_GRADY, cy, s));
+        ma.mask = mask; ma.mask_row = L.separable ? 1 : 0; ma.ky_out = (cf*)grad_y; ma.scale = eta * gs / (float)sqrt(ntot);
+        LAUNCH(GLEAM_K_COL_FWD, mid->launch(MID_GRADY, ma, s));
     } else {
-        ColArgs c1 = ca;
-        c1.es = L.n2; c1.nouter = L.units * L.n0;
-        LAUNCH(GLEAM_K_COL_FWD, op1->col(COL_FWD, c1, s));
-        cy.es = L.n1 * L.n2; cy.nouter = L.units;
-        LAUNCH(GLEAM_K_COL_FWD, op0->col(COL_GRADY, cy, s));
+        LAUNCH(GLEAM_K_COL_FWD, mid->launch(MID_FWD, ma, s));
+        AxisArgs aa{};
+        aa.W = W; aa.mask = mask; aa.mask_plane = L.separable ? 1 : 0; aa.ky_out = (cf*)grad_y;
+        aa.C = L.C; aa.T = L.T; aa.n1 = L.n1; aa.n2 = L.n2; aa.ry = mid->ry; aa.nunits = L.units;
+        aa.scale = eta * gs / (float)sqrt(ntot);
+        LAUNCH(GLEAM_K_COL_FWD, find_axis(L.n0)->launch(AXIS_GRADY, aa, s));
     }
     CK(prof_mark(-1, s));
     return GLEAM_OK;

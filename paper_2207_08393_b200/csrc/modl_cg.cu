@@ -4,8 +4,7 @@
 // The normal operator is the data-consistency VJP path of this library with eta = -1/mu:
 //     q = p + (1/mu) A^H A p = H p / mu,          H = A^H A + mu I,
 // so the factor mu moves into the scalars (alpha = <r,r> / (mu <p,q>),  r -= alpha mu q) and no
-// operator kernel changes.  The right-hand side A^H y is the forward call on a zero image with
-// eta = 1.  What remains are image-sized vector updates with inner products per batch example:
+// operator kernel changes.  What remains are image-sized vector updates with inner products per batch example:
 //
 //     cg_init : b = A^H y + mu z  (VJP: b = mu g);  r = p = b;  x = 0;  partial sums of <b,b>
 //     cg_dot  : partial sums of Re <p,q>
@@ -225,9 +224,7 @@ static int modl_cg(const void* z, const void* y, const void* sens, const float* 
     // the operator's own argument checks (y, sens, mask) before anything is enqueued
     CGRUN(run(ws + L.off_r, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ALL, nullptr, true));
     if (y) {
-        // A^H y: the forward call on a zero image with eta = 1
-        CGCK(cudaMemsetAsync(ws + L.off_r, 0, L.img_bytes, s));
-        CGRUN(run(ws + L.off_r, y, sens, mask, 1.0f, ws + L.off_q, &dd));
+        CGRUN(run(nullptr, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ADJOINT));
         CGCK(prof_mark(GLEAM_K_CG_VEC, s));
         cg_init_kernel<true><<<grid, CG_THREADS, 0, s>>>(a);
     } else {

@@ -1,0 +1,57 @@
+"""Row-tile passes, readout pass and coil-numbered one-pass kernel at the sizes where their tilings can go wrong, against
+the CPU oracle: forward, VJP and A^H y of the same inputs."""
+import numpy as np
+import pytest
+
+from oracle.oracle import MASK_FULL, MASK_READOUT_INVARIANT
+from tests.gpu_common import assert_close, run_gpu
+from tests.test_gpu_parity import problem
+
+pytestmark = pytest.mark.gpu
+
+
+def check_all(oracle, d, x, y, sens, mask, eta, what):
+    import torch
+    import paper_2207_08393_b200 as g
+    for yy, ref, name in ((y, oracle.dc_forward(x, y, sens, mask, eta, d, nthreads=8), "forward"),
+                          (None, oracle.dc_vjp(x, sens, mask, eta, d, nthreads=8), "vjp")):
+        got = run_gpu(x, yy, sens, mask, eta, d.fft_rank, d.sens_has_frames, d.mask_kind)
+        assert_close(got, ref, x, what + " " + name)
+    zero = np.zeros_like(x)
+    ref = oracle.dc_forward(zero, y, sens, mask, 1.0, d, nthreads=8)      # 0 - (A^H (A 0 - y))
+    dc = g.DataConsistency(d.batch, d.coils, d.frames, d.fft_rank, d.n, d.sens_has_frames, d.mask_kind)
+    dev = torch.device("cuda:0")
+    out = dc.adjoint(*(torch.from_numpy(a).to(dev) for a in (y, sens, mask)))
+    torch.cuda.synchronize()
+    assert_close(out.cpu().numpy(), ref, ref, what + " adjoint")
+
+
+# n1: rows per block and middle radix (1 x 20, 2 x 23, 12 x 32, 16 x 32, 20 x 32); n2: columns per block (single-stage
+# rows, a last warp with 8 or 14 idle lanes, both stage buffers, one buffer for both, the largest tile)
+@pytest.mark.parametrize("n", [(1, 20, 16), (1, 46, 40), (1, 384, 46), (1, 512, 24), (1, 640, 32), (1, 320, 368), (1, 40, 640), (1, 16, 512)])
+@pytest.mark.parametrize("coils", [1, 5])
+def test_slices_with_an_arbitrary_mask(oracle, n, coils):
+    d, x, y, sens, mask = problem(2, 1, coils, 1, n, MASK_FULL, weighted=(coils == 5), seed=sum(n), density=0.3)
+    check_all(oracle, d, x, y, sens, mask, 0.9, "slice %s" % (n,))
+
+
+# readout pass: columns per block 32 / 16 with a remainder, single-stage and two-stage lengths, radix 32, prime radix
+@pytest.mark.parametrize("n", [(4, 12, 46), (20, 6, 20), (46, 8, 24), (96, 4, 40), (128, 6, 10), (160, 4, 16), (512, 2, 12), (640, 2, 20)])
+def test_volumes_with_an_arbitrary_mask(oracle, n):
+    d, x, y, sens, mask = problem(3, 1, 3, 1, n, MASK_FULL, weighted=(n[0] == 96), seed=sum(n), density=0.3)
+    check_all(oracle, d, x, y, sens, mask, 1.0, "volume %s" % (n,))
+
+
+# coils dealt to clusters of 1, 2 and 4 blocks (few tiles), with coil counts that do not divide; frames and batches
+@pytest.mark.parametrize("B,C,T,n", [(1, 2, 1, (2, 64, 80)), (1, 7, 1, (2, 92, 64)), (2, 4, 2, (2, 24, 128)), (1, 3, 1, (40, 20, 32)), (1, 6, 1, (2, 640, 20))])
+def test_coil_split_of_the_row_tiles(oracle, B, C, T, n):
+    d, x, y, sens, mask = problem(3, B, C, T, n, MASK_READOUT_INVARIANT, sens_has_frames=int(T > 1), seed=sum(n) + C, density=0.2)
+    check_all(oracle, d, x, y, sens, mask, 0.8, "split %s" % (n,))
+
+
+# one-pass kernel: lines per warp 1 ... 8 with idle lanes, prime radices, lines beyond the end, more samples than are staged
+@pytest.mark.parametrize("n2", [46, 92, 184, 368, 384, 512, 640])
+@pytest.mark.parametrize("rows,coils,density", [(2, 2, 0.1), (10, 3, 0.9), (20, 16, 0.2)])
+def test_one_pass_kernel_of_slices(oracle, n2, rows, coils, density):
+    d, x, y, sens, mask = problem(2, 1, coils, 1, (1, rows, n2), MASK_READOUT_INVARIANT, seed=n2 + rows, density=density)
+    check_all(oracle, d, x, y, sens, mask, 0.9, "n2=%d rows=%d" % (n2, rows))
