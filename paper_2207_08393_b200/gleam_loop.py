@@ -24,7 +24,7 @@ class _DCFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x_ch, step):
         out = torch.empty_like(x_ch)
-        _b.gleam_dc_forward_layout(x_ch, step.y, step.sens, step.mask, step.eta, out, step.dc.dims(),
+        _b.gleam_dc_forward_layout(x_ch, step.y, step.sens, step.mask, step.eta, out, step.dc.call_dims(),
                                    _b.GLEAM_X_CHANNELS | _b.GLEAM_OUT_CHANNELS)
         ctx.step = step
         return out
@@ -34,7 +34,7 @@ class _DCFunction(torch.autograd.Function):
         step = ctx.step
         grad_out = grad_out.contiguous()
         grad_in = torch.empty_like(grad_out)
-        _b.gleam_dc_vjp_layout(grad_out, step.sens, step.mask, step.eta, grad_in, step.dc.dims(),
+        _b.gleam_dc_vjp_layout(grad_out, step.sens, step.mask, step.eta, grad_in, step.dc.call_dims(),
                                _b.GLEAM_X_CHANNELS | _b.GLEAM_OUT_CHANNELS)
         return grad_in, None
 
@@ -44,11 +44,11 @@ class _L1Function(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x_ch, step):
-        loss = torch.empty(1, dtype=torch.float64, device=x_ch.device)
+        loss = torch.empty((), dtype=torch.float64, device=x_ch.device)
         grad = torch.empty_like(x_ch)
         _b.gleam_l1_loss(x_ch, step.ref, loss, grad, step.l1_dims(), _b.GLEAM_X_CHANNELS | _b.GLEAM_OUT_CHANNELS)
         ctx.save_for_backward(grad)
-        return loss[0].to(torch.float32)
+        return loss.to(torch.float32)
 
     @staticmethod
     def backward(ctx, g):
@@ -66,10 +66,10 @@ class DataConsistencyStep:
         self.shape = (B, C, T, fft_rank, n)
         self.dc = _b.DataConsistency(B, C, T, fft_rank, n, 0, mask_kind)
         self._l1_ws = torch.empty(max(_b.gleam_l1_loss_workspace_size(), 256), dtype=torch.uint8, device=y.device)
+        self._l1_kept = _b.CallDims(B, 1, T, fft_rank, n)
 
     def l1_dims(self):
-        B, C, T, rank, n = self.shape
-        return _b.make_dims(B, 1, T, rank, n, stream=torch.cuda.current_stream(), workspace=self._l1_ws)
+        return self._l1_kept.get(self._l1_ws)
 
     def apply(self, x_ch):
         return _DCFunction.apply(x_ch, self)
