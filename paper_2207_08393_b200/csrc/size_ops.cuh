@@ -4,8 +4,10 @@
 #include "dc_kernels.cuh"
 #include "dc_warpline.cuh"
 #include "dc_warpflat.cuh"
+#include "dc_coilpar.cuh"
 
 #include <atomic>
+#include <type_traits>
 
 namespace gleam {
 
@@ -179,8 +181,36 @@ GLEAM_FLAT(640, 32, 32)
 #undef GLEAM_FLAT
 template <class P, int RL> using FlatPlan = Plan<P::N, P::N / RL, RL>;
 
+// the plan of every row kernel that takes z
+template <class P> using ZPlan = std::conditional_t<FlatRL<P::N>::z != 0, FlatPlan<P, FlatRL<P::N>::z ? FlatRL<P::N>::z : P::RL>, P>;
+
+// Few lines: the coils of a line group side by side (dc_coilpar.cuh) while all warps are resident at once (16 per SM).
+// Measured per call, numbered or plain kernel -> here: one 64 x 64 slice of 8 coils 12.5 -> 4.3 us (prepared step),
+// 4.7 -> 3.4 us (VJP); 6 x 8 coils of 46 x 240 18.6 -> 7.3 and 11.7 -> 6.2 us; beyond the line 6 x 4 coils of 368 x 80
+// 7.6 -> 11.3 us; with 2 or 3 coils 3.9 -> 4.8 us.  *taken: the call was launched here.
+template <class P, bool HAS_Z, bool ADJ>
+inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken) {
+    using CP = CoilPar<P>;
+    *taken = false;
+    int sms = 0;
+    cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    const int warps = a.C < 16 ? a.C : 16;
+    const long long groups = (a.nrows + CP::LW - 1) / CP::LW;
+    const size_t bytes = CP::bytes(warps, a.C);
+    if (a.C < 4 || bytes > CP::LIMIT || groups <= 0 || groups * warps > 16LL * sms) return cudaSuccess;
+    static PerDevice done;
+    if ((e = ensure_smem(coilpar_kernel<P, HAS_Z, ADJ>, CP::LIMIT, done)) != cudaSuccess) return e;
+    *taken = true;
+    return launch_overlapped(true, coilpar_kernel<P, HAS_Z, ADJ>, dim3((unsigned)groups), dim3(32 * warps), bytes, s, a);
+}
+
 template <class P>
 inline cudaError_t launch_warpline(const RowArgs& a, cudaStream_t s) {
+    bool taken = false;
+    const cudaError_t e = a.z == nullptr ? launch_coilpar<ZPlan<P>, false, false>(a, s, &taken)
+                        : a.x != nullptr ? launch_coilpar<ZPlan<P>, true, false>(a, s, &taken) : launch_coilpar<ZPlan<P>, true, true>(a, s, &taken);
+    if (taken || e != cudaSuccess) return e;
     // the numbering across coils pays once a round of 32 units spans more than one coil
     const bool flat = flat_enabled() && a.C >= 2;
     if constexpr (FlatRL<P::N>::v != 0) if (flat && a.z == nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::v>, false>(a, s);
