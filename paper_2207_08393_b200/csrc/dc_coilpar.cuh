@@ -18,8 +18,8 @@ struct CoilPar {
     static constexpr int LW = 32 / TPL;                           // lines per group
     static constexpr int EXL = (S == 2) ? P::SM_A : 0;            // exchange elements per line
     static constexpr int LINE = LW * N;
-    // float2 units: x, scaled mask^2 (floats) and ranks (ints) per line, exchange per warp, then one line group per coil
-    static constexpr int OFF_M = LINE, OFF_I = OFF_M + (LINE + 1) / 2, OFF_E = OFF_I + (LINE + 1) / 2;
+    // float2 units: x, scaled mask^2 (floats) and unit masks per line, exchange per warp, then one line group per coil
+    static constexpr int OFF_M = LINE, OFF_U = OFF_M + (LINE + 1) / 2, OFF_E = OFF_U + LW * P::BFL;
     static constexpr size_t bytes(int warps, int coils) { return sizeof(cf) * (size_t)(OFF_E + warps * LW * EXL + coils * LINE); }
     static constexpr size_t LIMIT = 200 * 1024;
 };
@@ -35,7 +35,7 @@ coilpar_kernel(const RowArgs a) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, warps = blockDim.x >> 5;
     cf* sX = smem;
     float* sM = reinterpret_cast<float*>(smem + CP::OFF_M);
-    int* sI = reinterpret_cast<int*>(smem + CP::OFF_I);
+    UnitMask* sU = reinterpret_cast<UnitMask*>(smem + CP::OFF_U);
     cf* sE = smem + CP::OFF_E + warp * LW * EXL;
     cf* sV = smem + CP::OFF_E + warps * LW * EXL;
     const long long row0 = (long long)blockIdx.x * LW;
@@ -55,21 +55,14 @@ coilpar_kernel(const RowArgs a) {
     };
     const long long s_stride = (long long)a.Ts * a.RPB * N, k_stride = (long long)a.T * a.RPB * N;
 
-    // ---- x, mask weights and ranks of the lines: one warp per line ----
+    // ---- x, mask weights and unit masks of the lines: one warp per line ----
     for (int ll = warp; ll < LW; ll += warps) {
         long long x_off = 0, s_off = 0, k_off = 0, bt = 0; int b = 0;
         const bool ok = line_of(ll, x_off, s_off, k_off, bt, b);
-        int cnt = 0;
-        for (int k0 = 0; k0 < N; k0 += 32) {
-            const int k = k0 + lane;
-            const float mv = (ok && k < N) ? a.mask[bt * N + shift_half(k, N)] : 0.f;
-            if (!ADJ && k < N) sX[ll * N + k] = ok ? load_image(a.x, x_off + k, a.x_planar, b, a.plane) : make_float2(0.f, 0.f);
-            if (k < N) sM[ll * N + k] = mv * mv * (1.0f / N);
-            if (HAS_Z) {
-                const unsigned bal = __ballot_sync(0xffffffffu, mv != 0.f);
-                if (k < N) sI[ll * N + k] = (mv != 0.f) ? cnt + __popc(bal & ((1u << lane) - 1u)) : -1;
-                cnt += __popc(bal);
-            }
+        if (HAS_Z) line_units<P::BFL, RL>(a.mask + bt * N, ok, lane, sU + ll * P::BFL, ADJ ? nullptr : sM + ll * N);
+        for (int k = lane; k < N; k += 32) {
+            if (!ADJ) sX[ll * N + k] = ok ? load_image(a.x, x_off + k, a.x_planar, b, a.plane) : make_float2(0.f, 0.f);
+            if (!HAS_Z) { const float mv = ok ? a.mask[bt * N + shift_half(k, N)] : 0.f; sM[ll * N + k] = mv * mv * (1.0f / N); }
         }
     }
     const int l = lane / TPL, j = lane % TPL;
@@ -111,18 +104,12 @@ coilpar_kernel(const RowArgs a) {
             }
         }
         if (aL) {
-            const cf* zrow = HAS_Z ? a.z + k_off + c * k_stride : nullptr;
+            if (HAS_Z) {
+                const UnitMask um = sU[l * P::BFL + j];
+                unit_update<P::BFL, RL, ADJ>(u, um.bits, sM + l * N + j, a.z + k_off + c * k_stride + um.first);
+            } else {
 #pragma unroll
-            for (int k = 0; k < RL; ++k) {
-                const int at = l * N + j + P::BFL * k;
-                if (HAS_Z) {
-                    const int r = sI[at];
-                    const cf q = (r >= 0) ? zrow[r] : make_float2(0.f, 0.f);
-                    const float w = sM[at];
-                    u[k] = ADJ ? make_float2(-q.x, -q.y) : make_float2(fmaf(w, u[k].x, -q.x), fmaf(w, u[k].y, -q.y));
-                } else {
-                    u[k] = cscale(u[k], sM[at]);
-                }
+                for (int k = 0; k < RL; ++k) u[k] = cscale(u[k], sM[l * N + j + P::BFL * k]);
             }
         }
         if (P::S == 2) {

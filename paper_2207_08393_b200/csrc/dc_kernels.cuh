@@ -17,13 +17,15 @@
 
 namespace gleam {
 
+__device__ __forceinline__ int shift_half(int k, int n) { int h = n >> 1; return k >= n - h ? k - (n - h) : k + h; }
+
 
 struct RowArgs {
     const cf* x;        // image-domain input (B,T,n0,n1,n2); null with z: a zero image (A^H y)
     const cf* sens;     // (B,C,[T],n0,n1,n2)
     cf* out;            // (B,T,n0,n1,n2)
     const float* mask;  // readout-invariant mask (B,T,n2)
-    const cf* z;        // compact table of shifted, signed, masked R^H y: (B,C,T,n1,[rank < n2]); may be null
+    const cf* z;        // compact table of shifted, signed, masked R^H y: (B,C,T,n1,[rank < n2]), unit order; may be null
     float eta;
     int C, T, Ts;       // coils, frames, sens frames (T or 1)
     int RPB;            // rows of an image (n1)
@@ -69,13 +71,55 @@ struct ColArgs {
     int es;             // element stride of the transformed axis = phase-encode positions per outer index
     long long nouter;   // outer indices
     int C, T, rank, n2;
+    int unit_r0;        // rank 2: the ranks follow the units of the row kernel (below)
     int ztiles;         // blocks launched per outer index (they stride over the tiles of ranks)
     float scale;        // g_ro g_pe / sqrt(N_ro N_pe)
 };
 
+// Rank order of the sampled positions of a 2-D mask row (unit order): the raw k indices k = jb + R0 k1 (k1 < RL) that
+// one last-stage butterfly of the row kernel's plan N = R0 RL holds are neighbours, jb outermost.  A butterfly's z values
+// are then one contiguous run of the compact row, and what it needs to know of the mask is one word: bit k1 is set where
+// k is sampled.  The update reads shared memory at the sampled entries only (it used to read a rank, a weight and a z
+// value for every entry: 8 x 16 coils x 640 rows of 320 at 4x, 152 -> 128 us; 256-point rows at 3x, 58 -> 36 us).
+struct UnitMask { unsigned bits; int first; };       // that word, and the rank of the run's first entry
+// The masks of the R0 units of one line, by one warp: lane jb < R0 reads its RL mask values (and stores their squares,
+// scaled, at raw k in `weight` unless it is null).  Returns the number of sampled positions in every lane.
+template <int R0, int RL>
+__device__ __forceinline__ int line_units(const float* mask_row, bool ok, int lane, UnitMask* units, float* weight) {
+    constexpr int N = R0 * RL;
+    static_assert(R0 <= 32 && RL <= 32, "one lane per unit, one bit per entry");
+    unsigned bits = 0;
+    if (lane < R0) {
+#pragma unroll
+        for (int k1 = 0; k1 < RL; ++k1) {
+            const int k = lane + R0 * k1;
+            const float m = ok ? mask_row[shift_half(k, N)] : 0.f;
+            if (weight != nullptr) weight[k] = m * m * (1.0f / N);
+            bits |= (m != 0.f ? 1u : 0u) << k1;
+        }
+    }
+    int incl = __popc(bits);
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += t; }
+    if (lane < R0) units[lane] = UnitMask{bits, incl - __popc(bits)};
+    return __shfl_sync(0xffffffffu, incl, 31);
+}
+// k-space update of one unit: u = w u - z at the sampled entries, 0 elsewhere (adjoint: -z).  `weight` points at the
+// unit's first entry (stride R0), `z` at its run; both are read at sampled entries only.
+template <int R0, int RL, bool ADJ>
+__device__ __forceinline__ void unit_update(cf (&u)[RL], unsigned bits, const float* weight, const cf* z) {
+#pragma unroll
+    for (int k = 0; k < RL; ++k) {
+        float w = 0.f; cf q = make_float2(0.f, 0.f);
+        if (bits & (1u << k)) {
+            if (!ADJ) w = weight[R0 * k];
+            q = *z++;
+        }
+        u[k] = ADJ ? make_float2(-q.x, -q.y) : make_float2(fmaf(w, u[k].x, -q.x), fmaf(w, u[k].y, -q.y));
+    }
+}
+
 constexpr int COLZ_SELF_MAX = 1024;   // COL_Z ranks a mask row of at most this many positions by itself
 
-__device__ __forceinline__ int shift_half(int k, int n) { int h = n >> 1; return k >= n - h ? k - (n - h) : k + h; }
 
 // --------------------------------------------------------------------------------------------
 // z table: L sampled phase-encode positions of one unit per block, inverse transform along the readout axis.
@@ -102,8 +146,8 @@ col_z_kernel(const ColArgs a) {
     cf v[R0], u[RL];
 
     // Without a rank map from an earlier launch (a.zlist == null; rank 2 with at most COLZ_SELF_MAX phase-encode
-    // positions) the block ranks the sampled positions of its mask row itself: it lists the source positions sh(q) of
-    // the sampled raw k indices q in the order of q -- the order in which the one-pass row kernel counts them.
+    // positions) the block ranks the sampled positions of its mask row itself: it lists their source positions sh(k) in
+    // unit order.
     __shared__ int s_list[COLZ_SELF_MAX];
     __shared__ unsigned s_bal[COLZ_SELF_MAX / 32];
     const bool self_ranks = a.zlist == nullptr;
@@ -111,11 +155,12 @@ col_z_kernel(const ColArgs a) {
     if (self_ranks) {
         const float* mk = a.mask + bt * pe;
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-        const int nchunks = (a.es + 31) / 32;
-        // every warp marks the sampled entries of its chunks of 32 raw indices ...
+        const int nchunks = (a.es + 31) / 32, r0 = a.unit_r0, rl = a.es / r0;
+        auto source = [&](int q) { return shift_half(q / rl + r0 * (q % rl), a.es); };        // of entry q in unit order
+        // every warp marks the sampled entries of its chunks of 32 ...
         for (int c = warp; c < nchunks; c += nwarps) {
             const int q = c * 32 + lane;
-            const bool on = (q < a.es) && (mk[shift_half(q, a.es)] != 0.f);
+            const bool on = (q < a.es) && (mk[source(q)] != 0.f);
             const unsigned bal = __ballot_sync(0xffffffffu, on);
             if (lane == 0) s_bal[c] = bal;
         }
@@ -126,7 +171,7 @@ col_z_kernel(const ColArgs a) {
             for (int e = 0; e < c; ++e) before += __popc(s_bal[e]);
             const unsigned bal = s_bal[c];
             const int q = c * 32 + lane;
-            if ((bal >> lane) & 1u) s_list[before + __popc(bal & ((1u << lane) - 1u))] = shift_half(q, a.es);
+            if ((bal >> lane) & 1u) s_list[before + __popc(bal & ((1u << lane) - 1u))] = source(q);
         }
         for (int e = 0; e < nchunks; ++e) cnt += __popc(s_bal[e]);
         __syncthreads();

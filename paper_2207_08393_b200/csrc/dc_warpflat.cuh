@@ -36,16 +36,16 @@ struct WarpFlat {
     static constexpr int SLOTS = (!SMW && !HAS_Z && slots_aligned() * UPC * USTRIDE * 8 <= 11 * 1024) ? slots_aligned() : SLOTS_MIN;
     static constexpr int ZS = SMW ? SLOTS : SLOTS + 1;     // z rows are requested one forward stage ahead (SMW: in their own stage)
     static constexpr int KCAP = ((N + 3) / 4 + 1) / 2 * 2; // staged z entries per line (more: read from global memory)
-    static constexpr int KSTRIDE = KCAP + 2;               // entry KCAP holds zero (unsampled positions point at it)
+    static constexpr int KSTRIDE = KCAP;
     static constexpr int KTILE = LW * KSTRIDE;
     static constexpr int MS = N + ((LW > 1 && N % 32 == 0) ? 16 : 0);   // mask row stride (floats): lines on different banks
     // shared memory of the warp, in float2 units
     static constexpr int OFF_X = 0, OFF_E = LW * N, OFF_M2 = OFF_E + SLOTS * UPC * USTRIDE + (SLOTS * UPC * USTRIDE) % 2;
-    // mask weights: one float per raw k (no z), or one per sampled rank next to 16-bit ranks of every raw k (with z)
-    static constexpr int OFF_IDX = OFF_M2 + ((HAS_Z ? LW * KSTRIDE : LW * MS) + 3) / 4 * 2;
-    static constexpr int OFF_K = OFF_IDX + (HAS_Z ? (LW * N + 7) / 8 * 2 : 0);
+    // mask weights of every raw k; with z: the units' masks, and the staged z rows
+    static constexpr int OFF_U = OFF_M2 + (LW * MS + 3) / 4 * 2;
+    static constexpr int OFF_K = OFF_U + (HAS_Z ? (LW * R0 + 1) / 2 * 2 : 0);
     static constexpr int OFF_CNT = OFF_K + (HAS_Z ? ZS * KTILE : 0);
-    // per line: element offset of its z row (64-bit), sampled count, mask row index
+    // per line: element offset of its z row (64-bit), sampled count
     static constexpr int ELEMS = (OFF_CNT + 2 * LW + 1) / 2 * 2;
     static constexpr size_t WARP_BYTES = sizeof(cf) * ELEMS;      // per warp of the block
     // Registers: coil sum, twiddles and the sensitivities of the next forward stage are held throughout (2 R0 each),
@@ -85,11 +85,10 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
     cf* sX = wsm + WF::OFF_X;
     cf* sE = wsm + WF::OFF_E;
     float* sM = reinterpret_cast<float*>(wsm + WF::OFF_M2);
-    short* sI = reinterpret_cast<short*>(wsm + WF::OFF_IDX);
+    UnitMask* sU = reinterpret_cast<UnitMask*>(wsm + WF::OFF_U);
     cf* sK = wsm + WF::OFF_K;
     long long* sKo = reinterpret_cast<long long*>(wsm + WF::OFF_CNT);      // per line: offset of the z row of coil cbase
     int* sC = reinterpret_cast<int*>(wsm + WF::OFF_CNT + LW);              // per line: sampled entries, -1 for a line past the end
-    unsigned* sBt = reinterpret_cast<unsigned*>(sC + LW);                   // per line: mask row
     const bool split = SMW && warp >= nwhole;                      // one of four warps that share a group
     const int set = split ? (warp - nwhole) >> 2 : 0, q = split ? (warp - nwhole) & 3 : 0;
     const int cbase = split ? q * a.C / 4 : 0;                     // first coil and number of coils of this warp
@@ -98,11 +97,6 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
     const bool img = WF::LANES == 32 || lane < WF::LANES;
     const int l = img ? lane / RL : LW - 1, j = img ? lane % RL : 0;      // image-side identity: line of the warp, butterfly
 
-    if (HAS_Z) {
-        for (int i = lane; i < ZS * LW; i += 32) sK[(i / LW) * KTILE + (i % LW) * KSTRIDE + KCAP] = make_float2(0.f, 0.f);
-        if (lane < LW) sM[lane * KSTRIDE + KCAP] = 0.f;
-        __syncwarp();
-    }
     // inter-stage twiddles exp(-2 pi i j k / N) of this lane (fetching them again before the image-side stages of
     // every round, to free registers for the k-space round, was measured slower: 18.7 against 16.4 us per call)
     cf tw0[R0];
@@ -136,7 +130,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
             const bool ok = __shfl_sync(0xffffffffu, (int)row_ok, ll * RL) != 0;
             const long long xo = __shfl_sync(0xffffffffu, x_off, ll * RL);
             const long long bto = __shfl_sync(0xffffffffu, (long long)bt, ll * RL);
-            if (!ok) { if (lane == 0) sC[ll] = -1; continue; }
+            if (!ok) { if (HAS_Z && lane == 0) sC[ll] = 0; continue; }
             if (ADJ) {
             } else if (!a.x_planar) {
                 for (int i = lane; i < N / 2; i += 32) cp_async16(sX + ll * N + 2 * i, a.x + xo + 2 * i);
@@ -150,22 +144,16 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                     for (int i = lane; i < N; i += 32) { dst[2 * i] = xf[i]; dst[2 * i + 1] = xf[a.plane + i]; }
                 }
             }
-            int cnt = 0;
-            for (int k0 = 0; k0 < N; k0 += 32) {
-                const int k = k0 + lane;
-                const float mv = (k < N) ? a.mask[bto * N + shift_half(k, N)] : 0.f;
-                if (!HAS_Z) {
-                    if (k < N) sM[ll * MS + k] = mv * mv * (1.0f / N);
-                } else {
-                    const unsigned bal = __ballot_sync(0xffffffffu, mv != 0.f);
-                    const int r = cnt + __popc(bal & ((1u << lane) - 1u));
-                    if (k < N) sI[ll * N + k] = (short)((mv != 0.f) ? r : -1);
-                    if (mv != 0.f && r < KCAP) sM[ll * KSTRIDE + r] = mv * mv * (1.0f / N);
-                    cnt += __popc(bal);
+            if (HAS_Z) {
+                const int cnt = line_units<R0, RL>(a.mask + bto * N, true, lane, sU + ll * R0, ADJ ? nullptr : sM + ll * MS);
+                if (lane == 0) sC[ll] = cnt;
+                if (img && lane == ll * RL) sKo[ll] = k_off;
+            } else {
+                for (int k = lane; k < N; k += 32) {
+                    const float mv = a.mask[bto * N + shift_half(k, N)];
+                    sM[ll * MS + k] = mv * mv * (1.0f / N);
                 }
             }
-            if (lane == 0) sC[ll] = cnt;
-            if (HAS_Z && img && lane == ll * RL) { sKo[ll] = k_off; sBt[ll] = bt; }
         }
         __syncwarp();
         // z row of coil c for every line of the warp -> slot c % ZS
@@ -245,40 +233,12 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
 #pragma unroll
                     for (int k = 0; k < RL; ++k) u[k] = cscale(u[k], mm[R0 * k]);
                 } else {
+                    // z of a line that is staged from shared memory, of others straight from its row
+                    const UnitMask um = sU[bl * R0 + jb];
                     const int kc = sC[bl];
-                    const short* ri_ = sI + bl * N + jb;
-                    if (kc > 0 && kc <= KCAP) {
-                        // staged z and weights by rank: unsampled entries read the zero slots
-                        const float* mw = sM + bl * KSTRIDE;
-                        const cf* zk = sK + (c % ZS) * KTILE + bl * KSTRIDE;
-#pragma unroll
-                        for (int k = 0; k < RL; ++k) {
-                            const int r = ri_[R0 * k];
-                            const int rr = (r >= 0) ? r : KCAP;
-                            const cf q = zk[rr];
-                            if (ADJ) u[k] = make_float2(-q.x, -q.y);
-                            else { const float wv = mw[rr]; u[k] = make_float2(fmaf(wv, u[k].x, -q.x), fmaf(wv, u[k].y, -q.y)); }
-                            if (k % 4 == 3) asm volatile("" ::: "memory");     // four entries in flight at a time: registers
-                        }
-                    } else if (kc > KCAP) {
-                        // more sampled entries than the stage holds: weights and z from global memory
-                        const float* mrow = a.mask + (long long)sBt[bl] * N;
-                        const cf* zrow = a.z + sKo[bl] + c * k_stride;
-#pragma unroll
-                        for (int k = 0; k < RL; ++k) {
-                            if (ADJ) u[k] = make_float2(0.f, 0.f);
-                            else { const float mv = mrow[shift_half(jb + R0 * k, N)]; u[k] = cscale(u[k], mv * mv * (1.0f / N)); }
-                            const int r = ri_[R0 * k];
-                            if (r >= 0) {
-                                const cf q = zrow[r];
-                                u[k] = make_float2(u[k].x - q.x, u[k].y - q.y);
-                            }
-                            asm volatile("" ::: "memory");      // one entry at a time: this rare path must not cost registers
-                        }
-                    } else {       // nothing sampled on this line (or no line)
-#pragma unroll
-                        for (int k = 0; k < RL; ++k) u[k] = make_float2(0.f, 0.f);
-                    }
+                    const float* mw = sM + bl * MS + jb;
+                    if (kc <= KCAP) unit_update<R0, RL, ADJ>(u, kc > 0 ? um.bits : 0u, mw, sK + (c % ZS) * KTILE + bl * KSTRIDE + um.first);
+                    else unit_update<R0, RL, ADJ>(u, um.bits, mw, a.z + sKo[bl] + c * k_stride + um.first);
                 }
                 Dft<RL, +1>::run(u);
                 if (live) {

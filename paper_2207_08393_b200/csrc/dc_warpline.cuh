@@ -36,18 +36,16 @@ struct WarpLine {
     static constexpr int TPL = pow2_ceil(BFMAX);          // lanes per line
     static constexpr int LW = 32 / TPL;                   // lines per warp
     static constexpr int EXL = (S == 2) ? P::SM_A : 0;    // exchange elements per line
-    // per-warp shared memory, in float2 units: S[2], z[2], x, exchange, m2 (floats, N/2 float2 per line), ranks.
-    // Up to KCAP sampled z entries per line are staged (lines with more read z straight from global memory);
-    // slot KCAP of every line's stage holds zero: unsampled entries point at it, which keeps the k-space
-    // update free of branches
+    // per-warp shared memory, in float2 units: S[2], z[2], x, exchange, m2 (floats, N/2 float2 per line), unit masks.
+    // Up to KCAP sampled z entries per line are staged (lines with more read z straight from global memory)
     static constexpr int TILE = LW * N;
     static constexpr int KCAP = ((N + 3) / 4 + 1) / 2 * 2;
-    static constexpr int KSTRIDE = KCAP + 2;
+    static constexpr int KSTRIDE = KCAP;
     static constexpr int KTILE = LW * KSTRIDE;
     static constexpr int OFF_S = 0, OFF_K = 2 * TILE, OFF_X = OFF_K + (HAS_Z ? 2 * KTILE : 0),
                          OFF_EX = OFF_X + TILE, OFF_M2 = OFF_EX + LW * EXL + (LW * EXL) % 2;
-    static constexpr int OFF_IDX = OFF_M2 + TILE / 2;     // ranks of the raw k indices (ints)
-    static constexpr int WARP_ELEMS = OFF_IDX + (HAS_Z ? TILE / 2 : 0) + 2;
+    static constexpr int OFF_U = OFF_M2 + TILE / 2;       // masks of the units (last-stage butterflies) of every line
+    static constexpr int WARP_ELEMS = OFF_U + (HAS_Z ? LW * P::BFL : 0) + 2;
     static constexpr int WARP_ELEMS_ALIGNED = (WARP_ELEMS + 1) / 2 * 2;   // keep 16-byte alignment per warp
 };
 
@@ -68,7 +66,7 @@ warpline_kernel(const RowArgs a) {
     cf* sX = wsm + WL::OFF_X;
     cf* sE = wsm + WL::OFF_EX;
     float* sM = reinterpret_cast<float*>(wsm + WL::OFF_M2);
-    int* sI = reinterpret_cast<int*>(wsm + WL::OFF_IDX);
+    UnitMask* sU = reinterpret_cast<UnitMask*>(wsm + WL::OFF_U);
 
     const int l = lane / TPL, j = lane % TPL;
     const bool a0 = j < P::BF0, aL = j < P::BFL;
@@ -79,10 +77,6 @@ warpline_kernel(const RowArgs a) {
         for (int k = 0; k < R0; ++k) tw0[k] = unit_root_fwd<N>((j * k) % N);
     }
 
-    if (HAS_Z) {
-        for (int i = lane; i < 2 * LW; i += 32) sK[(i / LW) * KTILE + (i % LW) * KSTRIDE + KCAP] = make_float2(0.f, 0.f);
-        __syncwarp();
-    }
     const long long ngroups = (a.nrows + LW - 1) / LW;
     const long long wstride = (long long)gridDim.x * WARPS;
     constexpr bool use_z = HAS_Z;
@@ -143,20 +137,16 @@ warpline_kernel(const RowArgs a) {
                 }
             }
             {
-                // scaled mask^2 in raw k order and, with z, the rank of every sampled k (the order
-                // in which the z table was written)
-                int cnt = 0;
-                for (int k0 = 0; k0 < N; k0 += 32) {
-                    const int k = k0 + lane;
-                    const float mv = (k < N) ? a.mask[bto * N + shift_half(k, N)] : 0.f;
-                    if (k < N) sM[ll * N + k] = mv * mv * (1.0f / N);
-                    if (use_z) {
-                        const unsigned bal = __ballot_sync(0xffffffffu, mv != 0.f);
-                        if (k < N) sI[ll * N + k] = (mv != 0.f) ? cnt + __popc(bal & ((1u << lane) - 1u)) : -1;
-                        cnt += __popc(bal);
+                // scaled mask^2 in raw k order and, with z, the masks of the units
+                if (use_z) {
+                    const int cnt = line_units<P::BFL, RL>(a.mask + bto * N, true, lane, sU + ll * P::BFL, ADJ ? nullptr : sM + ll * N);
+                    if (l == ll) k_cnt = cnt;
+                } else {
+                    for (int k = lane; k < N; k += 32) {
+                        const float mv = a.mask[bto * N + shift_half(k, N)];
+                        sM[ll * N + k] = mv * mv * (1.0f / N);
                     }
                 }
-                if (use_z && l == ll) k_cnt = cnt;
             }
         }
         issue_coil(0, 0);
@@ -214,29 +204,14 @@ warpline_kernel(const RowArgs a) {
             }
             {
                 if (aL) {
-                    const float* mm = sM + l * N;
-                    if (use_z && row_ok && k_cnt <= KCAP) {
-                        // staged z: unsampled entries read the zero slot (lanes without a row hold no rank table)
+                    const float* mm = sM + l * N + j;
+                    if (!use_z) {
 #pragma unroll
-                        for (int k = 0; k < RL; ++k) {
-                            const float w = mm[j + P::BFL * k];
-                            const int r = sI[l * N + j + P::BFL * k];
-                            const cf q = cK[(r >= 0) ? r : KCAP];
-                            u[k] = make_float2(fmaf(w, u[k].x, -q.x), fmaf(w, u[k].y, -q.y));
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < RL; ++k) {
-                            const float w = mm[j + P::BFL * k];
-                            u[k] = cscale(u[k], w);
-                            if (use_z && row_ok) {      // more sampled entries than the stage holds: from global memory
-                                const int r = sI[l * N + j + P::BFL * k];
-                                if (r >= 0 && r < N) {
-                                    const cf q = gK[r];
-                                    u[k] = make_float2(u[k].x - q.x, u[k].y - q.y);
-                                }
-                            }
-                        }
+                        for (int k = 0; k < RL; ++k) u[k] = cscale(u[k], mm[P::BFL * k]);
+                    } else {       // staged z, or straight from the line's row (lanes without a row hold no mask)
+                        const UnitMask um = row_ok ? sU[l * P::BFL + j] : UnitMask{0u, 0};
+                        if (k_cnt <= KCAP) unit_update<P::BFL, RL, ADJ>(u, um.bits, mm, cK + um.first);
+                        else unit_update<P::BFL, RL, ADJ>(u, um.bits, mm, gK + um.first);
                     }
                 }
             }

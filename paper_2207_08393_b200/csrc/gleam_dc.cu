@@ -353,7 +353,7 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
         // ranks of the sampled positions (rank 2: the blocks that need them derive them from the mask row), then the
         // z table: inverse transform of y along the readout axis at the sampled positions only
         ColArgs cz{};
-        cz.C = L.C; cz.T = L.T; cz.rank = L.rank; cz.n2 = L.n2;
+        cz.C = L.C; cz.T = L.T; cz.rank = L.rank; cz.n2 = L.n2; cz.unit_r0 = find_size(L.n2)->unit_r0;
         cz.y = (const cf*)y; cz.z = z; cz.mask = mask; cz.es = (int)pe; cz.nouter = L.units;
         if (L.rank == 3) {
             int* zlist = (int*)(ws + L.off_zlist);

@@ -3,7 +3,7 @@
 
 namespace gleam {
 #define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) \
-    extern const SizeOps size_ops_##N = {N, &SizeImpl<Plan<N, A0, A1>, Plan<N, B0, B1, B2>, LC>::row, \
+    extern const SizeOps size_ops_##N = {N, ZPlan<Plan<N, A0, A1>>::BFL, &SizeImpl<Plan<N, A0, A1>, Plan<N, B0, B1, B2>, LC>::row, \
                                          &SizeImpl<Plan<N, A0, A1>, Plan<N, B0, B1, B2>, LC>::col_z};
 #include "sizes.def"
 #undef GLEAM_SIZE

@@ -25,7 +25,7 @@ struct PerDevice {
 };
 
 struct SizeOps {
-    int N;
+    int N, unit_r0;              // unit_r0: units per line of the row kernels that take z (one plan for all of them)
     cudaError_t (*row)(const RowArgs& a, cudaStream_t s);
     cudaError_t (*col_z)(const ColArgs& a, cudaStream_t s);
 };
@@ -181,7 +181,7 @@ GLEAM_FLAT(640, 32, 32)
 #undef GLEAM_FLAT
 template <class P, int RL> using FlatPlan = Plan<P::N, P::N / RL, RL>;
 
-// the plan of every row kernel that takes z
+// the plan of every row kernel that takes z: the ranks of the sampled positions follow its units
 template <class P> using ZPlan = std::conditional_t<FlatRL<P::N>::z != 0, FlatPlan<P, FlatRL<P::N>::z ? FlatRL<P::N>::z : P::RL>, P>;
 
 // Few lines: the coils of a line group side by side (dc_coilpar.cuh) while all warps are resident at once (16 per SM).
@@ -216,7 +216,7 @@ inline cudaError_t launch_warpline(const RowArgs& a, cudaStream_t s) {
     if constexpr (FlatRL<P::N>::v != 0) if (flat && a.z == nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::v>, false>(a, s);
     if constexpr (FlatRL<P::N>::z != 0) if (flat && a.z != nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::z>, true>(a, s);
     if (a.z == nullptr) return launch_warpline_z<P, false, false>(a, s);
-    return a.x != nullptr ? launch_warpline_z<P, true, false>(a, s) : launch_warpline_z<P, true, true>(a, s);
+    return a.x != nullptr ? launch_warpline_z<ZPlan<P>, true, false>(a, s) : launch_warpline_z<ZPlan<P>, true, true>(a, s);
 }
 
 template <class P, int L>
