@@ -467,12 +467,18 @@ __global__ void __launch_bounds__(GRAD_THREADS) grad_eta_partial_kernel(const cf
     }
     if (threadIdx.x == 0) part[(long long)blockIdx.y * gridDim.x + blockIdx.x] = sh[0];
 }
+// Sum of n <= GRAD_MAX_BLOCKS values by one warp, in a fixed order (every lane's loads are in flight together; one
+// thread adding them one after another took 10 us).
+__device__ __forceinline__ double warp_array_sum(const double* __restrict__ v, int n) {
+    double s = 0.0;
+#pragma unroll
+    for (int e = 0; e < GRAD_MAX_BLOCKS / 32; ++e) { const int i = e * 32 + (int)threadIdx.x; if (i < n) s += v[i]; }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    return s;
+}
 __global__ void grad_eta_final_kernel(const double* __restrict__ part, int nblocks, double* __restrict__ grad_eta) {
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < nblocks; ++i) s += part[(long long)blockIdx.x * nblocks + i];
-        grad_eta[blockIdx.x] = -s;
-    }
+    const double s = warp_array_sum(part + (long long)blockIdx.x * nblocks, nblocks);
+    if (threadIdx.x == 0) grad_eta[blockIdx.x] = -s;
 }
 
 
@@ -505,11 +511,8 @@ __global__ void __launch_bounds__(GRAD_THREADS) l1_partial_kernel(const cf* __re
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 __global__ void l1_final_kernel(const double* __restrict__ part, int nblocks, double inv_n, double* __restrict__ loss) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < nblocks; ++i) s += part[i];
-        *loss = s * inv_n;
-    }
+    const double s = warp_array_sum(part, nblocks);
+    if (threadIdx.x == 0) *loss = s * inv_n;
 }
 
 
