@@ -60,7 +60,10 @@ coilpar_kernel(const RowArgs a) {
         long long x_off = 0, s_off = 0, k_off = 0, bt = 0; int b = 0;
         const bool ok = line_of(ll, x_off, s_off, k_off, bt, b);
         if (HAS_Z) line_units<P::BFL, RL>(a.mask + bt * N, ok, lane, sU + ll * P::BFL, ADJ ? nullptr : sM + ll * N);
-        for (int k = lane; k < N; k += 32) {
+#pragma unroll 8
+        for (int k0 = 0; k0 < N; k0 += 32) {
+            const int k = k0 + lane;
+            if (k >= N) break;
             if (!ADJ) sX[ll * N + k] = ok ? load_image(a.x, x_off + k, a.x_planar, b, a.plane) : make_float2(0.f, 0.f);
             if (!HAS_Z) { const float mv = ok ? a.mask[bt * N + shift_half(k, N)] : 0.f; sM[ll * N + k] = mv * mv * (1.0f / N); }
         }
@@ -136,13 +139,13 @@ coilpar_kernel(const RowArgs a) {
     }
     __syncthreads();
 
-    // ---- conjugate-sensitivity sum over the coils in order, update, Re<x, out> per row ----
+    // ---- conjugate-sensitivity sum over the coils in order, update, Re<x, out> and <out, out> per row ----
     // tasks: (line, segment of its elements), one warp each
-    __shared__ double s_dot[64];
+    __shared__ double s_dot[2][64];
     const int segs = warps > LW ? warps / LW : 1;
     for (int task = warp; task < LW * segs; task += warps) {
         const int ll = task % LW, seg = task / LW;
-        double dsum = 0.0;
+        double dsum = 0.0, nsum = 0.0;
         if (line_of(ll, x_off, s_off, k_off, bt, b)) {
             for (int n = seg * 32 + lane; n < N; n += 32 * segs) {
                 const cf* sp = a.sens + s_off + n;
@@ -156,20 +159,21 @@ coilpar_kernel(const RowArgs a) {
                 const cf xv = ADJ ? make_float2(0.f, 0.f) : sX[ll * N + n];
                 const cf ov = make_float2(fmaf(-a.eta, acc.x, xv.x), fmaf(-a.eta, acc.y, xv.y));
                 store_image(a.out, x_off + n, ov, a.out_planar, b, a.plane);
-                dsum += (double)xv.x * ov.x + (double)xv.y * ov.y;
+                if (a.dot_rows != nullptr) { dsum += (double)xv.x * ov.x + (double)xv.y * ov.y; nsum += (double)ov.x * ov.x + (double)ov.y * ov.y; }
             }
         }
         if (a.dot_rows != nullptr) {
-            for (int o = 16; o > 0; o >>= 1) dsum += __shfl_down_sync(0xffffffffu, dsum, o);
-            if (lane == 0) s_dot[task] = dsum;
+            for (int o = 16; o > 0; o >>= 1) { dsum += __shfl_down_sync(0xffffffffu, dsum, o); nsum += __shfl_down_sync(0xffffffffu, nsum, o); }
+            if (lane == 0) { s_dot[0][task] = dsum; s_dot[1][task] = nsum; }
         }
     }
     if (a.dot_rows != nullptr) {
         __syncthreads();
         if (tid < LW && row0 + tid < a.nrows) {
-            double d = 0.0;
-            for (int seg = 0; seg < segs; ++seg) d += s_dot[seg * LW + tid];
+            double d = 0.0, n = 0.0;
+            for (int seg = 0; seg < segs; ++seg) { d += s_dot[0][seg * LW + tid]; n += s_dot[1][seg * LW + tid]; }
             a.dot_rows[row0 + tid] = d;
+            a.dot_rows[a.nrows + row0 + tid] = n;
         }
     }
 }

@@ -18,9 +18,9 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
         int layout = 0,      // layout: GLEAM_X_CHANNELS | GLEAM_OUT_CHANNELS (two-real-channel image arrays)
         const void* aty = nullptr);   // with y == nullptr: out = x - eta (A^H A x - aty), aty = A^H y as an image
 
-// dot_rows (device, one double per image row, B*T*n1): the one-pass 2-D kernel also stores
-// Re<x_row, out_row> of every row it writes, so that a caller's inner product <x, out> needs no
-// pass of its own.  Only where this returns true (2-D, readout-invariant mask, warp-resident row plan).
+// dot_rows (device, two arrays of one double per image row, B*T*n1): the one-pass 2-D kernel also stores
+// Re<x_row, out_row> and <out_row, out_row> of every row it writes, so that a caller's inner products need no
+// pass of their own.  Only where this returns true (2-D, readout-invariant mask, warp-resident row plan).
 bool dot_rows_supported(const gleam_dims* d);
 
 // GLEAM_OK for a device (or managed) pointer, GLEAM_ERR_NOT_DEVICE_POINTER otherwise

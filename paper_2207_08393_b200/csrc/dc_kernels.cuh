@@ -30,7 +30,7 @@ struct RowArgs {
     int C, T, Ts;       // coils, frames, sens frames (T or 1)
     int RPB;            // rows of an image (n1)
     long long nrows;    // B*T*n1
-    double* dot_rows;   // if not null, Re<x, out> of every image row, (B*T*n1)
+    double* dot_rows;   // if not null, Re<x, out> of every image row, (B*T*n1), followed by <out, out> of every row
     // Two-real-channel layout (B, 2, T, n0, n1, n2) float32 of the image-side arrays (the form the learned
     // prior takes and returns): real index of complex element e of example b = e + b * plane, the imaginary
     // part `plane` further on (plane = T * n0 * n1 * n2).

@@ -149,9 +149,11 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 if (lane == 0) sC[ll] = cnt;
                 if (img && lane == ll * RL) sKo[ll] = k_off;
             } else {
-                for (int k = lane; k < N; k += 32) {
-                    const float mv = a.mask[bto * N + shift_half(k, N)];
-                    sM[ll * MS + k] = mv * mv * (1.0f / N);
+#pragma unroll
+                for (int k0 = 0; k0 < N; k0 += 32) {       // a trip count known at compile time: all loads in flight
+                    const int k = k0 + lane;
+                    const float mv = (k < N) ? a.mask[bto * N + shift_half(k, N)] : 0.f;
+                    if (k < N) sM[ll * MS + k] = mv * mv * (1.0f / N);
                 }
             }
         }
@@ -289,8 +291,8 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 for (int m = 0; m < R0; ++m) acc[m] = cadd(acc[m], o[m * 32 + lane]);
             }
         }
-        // ---- out = x - eta * sum, and Re<x, out> per row for the caller's inner product ----
-        double dsum = 0.0;
+        // ---- out = x - eta * sum, and Re<x, out>, <out, out> per row for the caller's inner products ----
+        double dsum = 0.0, nsum = 0.0;
         if (row_ok) {
 #pragma unroll
             for (int m = 0; m < R0; ++m) {
@@ -299,15 +301,15 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 const float se = HAS_ATY ? a.eta : -a.eta;          // HAS_ATY: acc holds aty - sum
                 const cf ov = make_float2(fmaf(se, av.x, xv.x), fmaf(se, av.y, xv.y));
                 store_image(a.out, x_off + j + RL * m, ov, a.out_planar, b, a.plane);
-                if (a.dot_rows != nullptr) dsum += (double)xv.x * ov.x + (double)xv.y * ov.y;
+                if (a.dot_rows != nullptr) { dsum += (double)xv.x * ov.x + (double)xv.y * ov.y; nsum += (double)ov.x * ov.x + (double)ov.y * ov.y; }
             }
         }
         if (a.dot_rows != nullptr) {     // the same in every thread
             for (int o = pow2_ceil(RL) / 2; o > 0; o >>= 1) {
-                const double d = __shfl_down_sync(0xffffffffu, dsum, o);
-                if (j + o < RL) dsum += d;
+                const double d = __shfl_down_sync(0xffffffffu, dsum, o), n = __shfl_down_sync(0xffffffffu, nsum, o);
+                if (j + o < RL) { dsum += d; nsum += n; }
             }
-            if (j == 0 && row_ok) a.dot_rows[row] = dsum;
+            if (j == 0 && row_ok) { a.dot_rows[row] = dsum; a.dot_rows[a.nrows + row] = nsum; }
         }
     }
 }

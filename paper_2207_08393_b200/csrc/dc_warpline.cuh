@@ -142,9 +142,11 @@ warpline_kernel(const RowArgs a) {
                     const int cnt = line_units<P::BFL, RL>(a.mask + bto * N, true, lane, sU + ll * P::BFL, ADJ ? nullptr : sM + ll * N);
                     if (l == ll) k_cnt = cnt;
                 } else {
-                    for (int k = lane; k < N; k += 32) {
-                        const float mv = a.mask[bto * N + shift_half(k, N)];
-                        sM[ll * N + k] = mv * mv * (1.0f / N);
+#pragma unroll
+                    for (int k0 = 0; k0 < N; k0 += 32) {       // a trip count known at compile time: all loads in flight
+                        const int k = k0 + lane;
+                        const float mv = (k < N) ? a.mask[bto * N + shift_half(k, N)] : 0.f;
+                        if (k < N) sM[ll * N + k] = mv * mv * (1.0f / N);
                     }
                 }
             }
@@ -248,7 +250,7 @@ warpline_kernel(const RowArgs a) {
         }
         cp_async_wait<0>();
         {
-            double dsum = 0.0;       // Re<x, out> over this lane's elements (for the caller's inner product)
+            double dsum = 0.0, nsum = 0.0;       // Re<x, out>, <out, out> over this lane's elements (for the caller's inner products)
             if (a0 && row_ok) {
 #pragma unroll
                 for (int m = 0; m < R0; ++m) {
@@ -258,12 +260,15 @@ warpline_kernel(const RowArgs a) {
                     const cf av = acc[m];
                     const cf ov = make_float2(fmaf(-a.eta, av.x, xv.x), fmaf(-a.eta, av.y, xv.y));
                     store_image(a.out, x_off + j + P::BF0 * m, ov, a.out_planar, b, a.plane);
-                    if (a.dot_rows != nullptr) dsum += (double)xv.x * ov.x + (double)xv.y * ov.y;
+                    if (a.dot_rows != nullptr) { dsum += (double)xv.x * ov.x + (double)xv.y * ov.y; nsum += (double)ov.x * ov.x + (double)ov.y * ov.y; }
                 }
             }
             if (a.dot_rows != nullptr) {     // the same in every thread
-                for (int o = TPL / 2; o > 0; o >>= 1) dsum += __shfl_down_sync(0xffffffffu, dsum, o, TPL);
-                if (j == 0 && row_ok) a.dot_rows[row] = dsum;
+                for (int o = TPL / 2; o > 0; o >>= 1) {
+                    dsum += __shfl_down_sync(0xffffffffu, dsum, o, TPL);
+                    nsum += __shfl_down_sync(0xffffffffu, nsum, o, TPL);
+                }
+                if (j == 0 && row_ok) { a.dot_rows[row] = dsum; a.dot_rows[a.nrows + row] = nsum; }
             }
         }
     }
