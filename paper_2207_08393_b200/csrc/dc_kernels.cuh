@@ -127,7 +127,8 @@ constexpr int COLZ_SELF_MAX = 1024;   // COL_Z ranks a mask row of at most this 
 template <class P, int L>
 __global__ void __launch_bounds__(LineFFT<P, L>::THREADS)
 col_z_kernel(const ColArgs a) {
-    grid_launch_dependents();    // a one-pass row kernel behind this launch may be scheduled early
+    grid_dependency_wait();
+    grid_launch_dependents();
     using E = LineFFT<P, L>;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL;
     extern __shared__ float2 smem[];

@@ -86,6 +86,8 @@ __global__ void __launch_bounds__(ZMAP_THREADS) zmap_kernel(const float* __restr
                                                             int* __restrict__ zlist, int* __restrict__ zcount,
                                                             float* __restrict__ m2c, int* __restrict__ zstart,
                                                             int* __restrict__ row_cnt, int n1, int n2, int ry) {
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int lane = threadIdx.x & 31, row = blockIdx.x * (ZMAP_THREADS / 32) + (threadIdx.x >> 5);   // row = k0 * by + k1
     if (row >= n1) return;
     const int by = n1 / ry, k0 = row / by, k1 = row - k0 * by, ky = k0 + ry * k1;
@@ -361,11 +363,9 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
             int* zrows = (int*)(ws + L.off_zrows);
             const dim3 zgrid((unsigned)((L.n1 + ZMAP_THREADS / 32 - 1) / (ZMAP_THREADS / 32)), (unsigned)L.images);
             CK(prof_mark(GLEAM_K_PREP_M2, s));
-            zmap_kernel<true><<<zgrid, ZMAP_THREADS, 0, s>>>(mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry);
-            CK(cudaGetLastError());
+            CK(launch_overlapped(true, zmap_kernel<true>, zgrid, dim3(ZMAP_THREADS), 0, s, mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry));
             CK(prof_mark(GLEAM_K_PREP_M2, s));
-            zmap_kernel<false><<<zgrid, ZMAP_THREADS, 0, s>>>(mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry);
-            CK(cudaGetLastError());
+            CK(launch_overlapped(true, zmap_kernel<false>, zgrid, dim3(ZMAP_THREADS), 0, s, mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry));
             cz.zlist = zlist; cz.zcount = zcount;
         }
         cz.scale = g / sqrtf((float)(L.rank == 2 ? L.n1 : L.n0) * (float)pe);

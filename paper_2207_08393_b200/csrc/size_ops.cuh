@@ -237,8 +237,7 @@ inline cudaError_t launch_col_z(const ColArgs& a, cudaStream_t s) {
     const long long blocks = a.nouter * tiles;
     if (blocks <= 0) return cudaSuccess;
     if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-    col_z_kernel<P, L><<<(unsigned)blocks, E::THREADS, E::SMEM_BYTES, s>>>(b);
-    return cudaGetLastError();
+    return launch_overlapped(a.zlist != nullptr, col_z_kernel<P, L>, dim3((unsigned)blocks), dim3(E::THREADS), E::SMEM_BYTES, s, b);
 }
 
 template <class P, class PC, int LC>
