@@ -20,6 +20,23 @@ namespace gleam {
 __device__ __forceinline__ int shift_half(int k, int n) { int h = n >> 1; return k >= n - h ? k - (n - h) : k + h; }
 
 
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int NKEEP> __device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(NKEEP) : "memory");
+}
+
 struct RowArgs {
     const cf* x;        // image-domain input (B,T,n0,n1,n2); null with z: a zero image (A^H y)
     const cf* sens;     // (B,C,[T],n0,n1,n2)
@@ -69,10 +86,10 @@ struct ColArgs {
     const int* zcount;  // (B,T)
     const float* mask;  // readout-invariant mask
     int es;             // element stride of the transformed axis = phase-encode positions per outer index
-    long long nouter;   // outer indices
+    int images;         // B*T
     int C, T, rank, n2;
     int unit_r0;        // rank 2: the ranks follow the units of the row kernel (below)
-    int ztiles;         // blocks launched per outer index (they stride over the tiles of ranks)
+    int bpi;            // blocks per image: they share its (coil, tile of ranks) pairs
     float scale;        // g_ro g_pe / sqrt(N_ro N_pe)
 };
 
@@ -122,29 +139,35 @@ constexpr int COLZ_SELF_MAX = 1024;   // COL_Z ranks a mask row of at most this 
 
 
 // --------------------------------------------------------------------------------------------
-// z table: L sampled phase-encode positions of one unit per block, inverse transform along the readout axis.
+// z table: tiles of L sampled phase-encode positions of one unit, inverse transform along the readout axis:
+//     z[r] = (g/sqrt(N_ro N_pe)) (-1)^{n_ro} (-1)^{p} M[p] * Rraw^H( (-1)^{k_ro} y[.., p] ),  p = source of rank r
+// Gathers 8-byte samples; bound by the DRAM sectors they touch (four columns each).  A block walks over tiles of one
+// image and has the next one on its way to shared memory (8-byte cp.async) while it transforms the current one: with a
+// block per tile, loads, transform and stores of a 640-point tile took turns on an SM (4 x 15 coils of 640 x 368 at 7x
+// 46 -> 38 us, 2 x 12 coils of 384 x 320 at 4x 25 -> 15 us, 20 frames of 192 x 160 17 -> 13 us).
+// Two buffers take turns as "incoming tile" and "current tile"; once every thread holds its elements of the current one,
+// its buffer takes the (last) exchange of the transform.  Three-stage plans have a third for their first exchange.
 // --------------------------------------------------------------------------------------------
+template <class P, int L>
+struct ColZ {
+    using E = LineFFT<P, L>;
+    static constexpr int BUFSZ = L * cmax(P::BUF, P::N);
+    static constexpr size_t SMEM_BYTES = sizeof(cf) * (P::S == 3 ? 3 : 2) * BUFSZ;
+    static_assert(E::THREADS % L == 0, "a thread copies one line's samples");
+};
+
 template <class P, int L>
 __global__ void __launch_bounds__(LineFFT<P, L>::THREADS)
 col_z_kernel(const ColArgs a) {
     grid_dependency_wait();
-    grid_launch_dependents();
+    grid_launch_dependents();    // a one-pass row kernel behind this launch may be scheduled early
     using E = LineFFT<P, L>;
-    constexpr int N = P::N, R0 = P::R0, RL = P::RL;
-    extern __shared__ float2 smem[];
-    // the launch has ztiles blocks per outer index, which stride over the tiles of sampled ranks (their number is
-    // only known on the device)
-    const int tiles = a.ztiles;
-    const long long o = blockIdx.x / tiles;           // outer index
-    int i_base = (int)(blockIdx.x % tiles) * L;
-    const int t = (int)(o % a.T), b = (int)(o / ((long long)a.C * a.T));
-    const long long bt = (long long)b * a.T + t, pe = a.es;
-    if (a.zlist != nullptr && i_base >= a.zcount[bt]) return;       // no tile of sampled ranks for this block
-    const typename E::Ids d = E::ids(threadIdx.x);
-    typename E::Tw tw;
-    E::make_tw(d, tw);
-    int i = i_base + d.l0;                            // every stage sees the same line index l = tid % L
-    cf v[R0], u[RL];
+    constexpr int N = P::N, R0 = P::R0, RL = P::RL, BUFSZ = ColZ<P, L>::BUFSZ;
+    extern __shared__ __align__(16) float2 smem[];
+    const int tid = threadIdx.x;
+    const int bt = blockIdx.x / a.bpi, t = bt % a.T, b = bt / a.T;
+    const long long pe = a.es;
+    const float* mk = a.mask + bt * pe;
 
     // Without a rank map from an earlier launch (a.zlist == null; rank 2 with at most COLZ_SELF_MAX phase-encode
     // positions) the block ranks the sampled positions of its mask row itself: it lists their source positions sh(k) in
@@ -154,8 +177,7 @@ col_z_kernel(const ColArgs a) {
     const bool self_ranks = a.zlist == nullptr;
     int cnt = 0;
     if (self_ranks) {
-        const float* mk = a.mask + bt * pe;
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+        const int lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
         const int nchunks = (a.es + 31) / 32, r0 = a.unit_r0, rl = a.es / r0;
         auto source = [&](int q) { return shift_half(q / rl + r0 * (q % rl), a.es); };        // of entry q in unit order
         // every warp marks the sampled entries of its chunks of 32 ...
@@ -179,35 +201,58 @@ col_z_kernel(const ColArgs a) {
     } else {
         cnt = a.zcount[bt];
     }
-    // Lines are the sampled phase-encode positions of this unit's (b,t), by rank r.
-    // z[r] = (g/sqrt(N_ro N_pe)) (-1)^{n_ro} (-1)^{p} M[p] * Rraw^H( (-1)^{k_ro} y[.., p] ),  p = zlist[r]
-    for (; i_base < cnt; i_base += tiles * L, i += tiles * L) {
+    const int ntiles = (cnt + L - 1) / L, items = a.C * ntiles;
+    auto source_of = [&](int i) { return self_ranks ? s_list[i] : a.zlist[bt * pe + i]; };
+    auto unit_of = [&](int item) { return ((long long)b * a.C + item / ntiles) * a.T + t; };
+    const int l = tid % L;                             // every stage sees the same line
+    auto issue = [&](int item, cf* dst) {
+        const int i = (item % ntiles) * L + l;
+        if (i < cnt) {
+            const cf* src = a.y + (unit_of(item) * N + tid / L) * pe + source_of(i);
+            for (int n = tid / L; n < N; n += E::THREADS / L) { cp_async8(dst + n * L + l, src); src += (E::THREADS / L) * pe; }
+        }
+    };
+
+    int item = blockIdx.x % a.bpi;
+    if (item >= items) return;
+    const typename E::Ids d = E::ids(tid);
+    typename E::Tw tw;
+    E::make_tw(d, tw);
+    issue(item, smem);
+    cp_async_commit();
+    for (int it = 0; item < items; item += a.bpi, ++it) {
+        cf* cur = smem + (it % 2) * BUFSZ;
+        cf* nxt = smem + ((it + 1) % 2) * BUFSZ;
+        cf* spare = smem + (P::S == 3 ? 2 : 0) * BUFSZ;
+        cp_async_wait<0>();
+        __syncthreads();               // the tile is visible to all; every thread has left the one before
+        if (item + a.bpi < items) issue(item + a.bpi, nxt);
+        cp_async_commit();
+        const int i = (item % ntiles) * L + l;
         const bool ok = i < cnt;
-        int p = 0, psign = 0; float mv = 0.f;
+        int psign = 0; float mv = 0.f;
         if (ok) {
-            p = self_ranks ? s_list[i] : a.zlist[bt * pe + i];
-            mv = a.mask[bt * pe + p];
+            const int p = source_of(i);
+            mv = mk[p];
             psign = (a.rank == 2) ? (p & 1) : ((p / a.n2 + p % a.n2) & 1);
         }
-        if (d.aL && ok) {
+        cf v[R0], u[RL];
+        if (d.aL) {
+            const float odd = (d.jL & 1) ? -1.f : 1.f;
 #pragma unroll
             for (int k = 0; k < RL; ++k) {
-                const int kk = d.jL + P::BFL * k;
-                const cf yv = a.y[o * (long long)N * pe + (long long)kk * pe + p];
-                u[k] = (kk & 1) ? make_float2(-yv.x, -yv.y) : yv;
+                const cf yv = ok ? cur[(d.jL + P::BFL * k) * L + l] : make_float2(0.f, 0.f);
+                u[k] = cscale(yv, (P::BFL * k) % 2 ? -odd : odd);
             }
         }
-        E::inverse(u, v, tw, d, smem);
+        if (P::S == 2) __syncthreads();
+        E::inverse(u, v, tw, d, spare, cur);
         if (d.a0 && ok) {
-            const float f = (psign ? -a.scale : a.scale) * mv;
+            const float f = ((psign + d.j0) & 1) ? -a.scale * mv : a.scale * mv;
+            cf* dst = a.z + (unit_of(item) * N + d.j0) * pe + i;
 #pragma unroll
-            for (int m = 0; m < R0; ++m) {
-                const int n = d.j0 + P::BF0 * m;
-                const float ff = (n & 1) ? -f : f;
-                a.z[o * (long long)N * pe + (long long)n * pe + i] = cscale(v[m], ff);
-            }
+            for (int m = 0; m < R0; ++m) { *dst = cscale(v[m], (P::BF0 * m) % 2 ? -f : f); dst += P::BF0 * pe; }
         }
-        __syncthreads();                                // exchange buffer is reused by the next tile
     }
 }
 

@@ -32,7 +32,6 @@ struct Plan {
     static constexpr int SM_A = (S >= 2) ? R0 * LS1 : 0;
     static constexpr int SM_B = (S == 3) ? R0 * R1 * LS2 : 0;
     static constexpr int BUF = cmax(SM_A, SM_B);   // one exchange buffer (elements)
-    static constexpr int LSZ = 2 * BUF;            // two buffers per line
 };
 
 // exp(-2 pi i e / N), e = 0..N-1, evaluated at compile time in double precision and stored as a
@@ -51,8 +50,6 @@ template <class P, int L>
 struct LineFFT {
     static constexpr int N = P::N, R0 = P::R0, R1 = P::R1, RL = P::RL, S = P::S;
     static constexpr int THREADS = ((L * P::MAXBF + 31) / 32) * 32;
-    static constexpr int SMEM_ELEMS = L * P::LSZ + 1;
-    static constexpr size_t SMEM_BYTES = sizeof(cf) * SMEM_ELEMS;
 
     // which line / butterfly a thread owns in each stage
     struct Ids {
@@ -93,9 +90,7 @@ struct LineFFT {
 
     // u (k-distribution of the last-stage thread) -> v (n-distribution of the first-stage thread), unscaled inverse.
     // Two-stage plans exchange through Y, three-stage plans go through X then Y.
-    __device__ __forceinline__ static void inverse(cf (&u)[RL], cf (&v)[R0], const Tw& tw, const Ids& d, cf* sm) {
-        cf* X = sm;
-        cf* Y = sm + L * P::BUF;
+    __device__ __forceinline__ static void inverse(cf (&u)[RL], cf (&v)[R0], const Tw& tw, const Ids& d, cf* X, cf* Y) {
         if (S == 1) {
 #pragma unroll
             for (int k = 0; k < R0; ++k) v[k] = u[k % RL];

@@ -356,7 +356,7 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
         // z table: inverse transform of y along the readout axis at the sampled positions only
         ColArgs cz{};
         cz.C = L.C; cz.T = L.T; cz.rank = L.rank; cz.n2 = L.n2; cz.unit_r0 = find_size(L.n2)->unit_r0;
-        cz.y = (const cf*)y; cz.z = z; cz.mask = mask; cz.es = (int)pe; cz.nouter = L.units;
+        cz.y = (const cf*)y; cz.z = z; cz.mask = mask; cz.es = (int)pe; cz.images = (int)L.images;
         if (L.rank == 3) {
             int* zlist = (int*)(ws + L.off_zlist);
             int* zcount = (int*)(ws + L.off_zcount);

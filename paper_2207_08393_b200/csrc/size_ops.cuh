@@ -222,22 +222,35 @@ inline cudaError_t launch_warpline(const RowArgs& a, cudaStream_t s) {
 template <class P, int L>
 inline cudaError_t launch_col_z(const ColArgs& a, cudaStream_t s) {
     using E = LineFFT<P, L>;
-    static PerDevice attr_done;
-    cudaError_t e = ensure_smem(col_z_kernel<P, L>, E::SMEM_BYTES, attr_done, (COLZ_SELF_MAX + COLZ_SELF_MAX / 32) * sizeof(int));
+    using CZ = ColZ<P, L>;
+    static PerDevice attr_done, slots_cache;
+    cudaError_t e = ensure_smem(col_z_kernel<P, L>, CZ::SMEM_BYTES, attr_done, (COLZ_SELF_MAX + COLZ_SELF_MAX / 32) * sizeof(int));
     if (e != cudaSuccess) return e;
-    long long tiles = (a.es + L - 1) / L;
+    int slots = 0;
+    if ((e = resident_slots(col_z_kernel<P, L>, E::THREADS, CZ::SMEM_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
+    if (a.images <= 0) return cudaSuccess;
+    int sms = 0;
+    if ((e = device_sms(&sms)) != cudaSuccess) return e;
+    // Every sample in flight holds a line of L1, so the blocks take no more than 132 KB of the SM's 228 for their tiles
+    // (64 / 100 / 132 / 164 / 196 KB: 640-point slices 40 / 34 / 38 / 42 / 48 us, 320 x 320 x 256 at 12x 223 / 238 /
+    // 234 / 225 / 243 us, 8 x 16 coils of 640 x 320 at 4x 81 / 85 / 76 / 87 / 101 us).
+    constexpr int TILE_KB = 132;
+    static PerDevice carveout_done;
+    std::atomic<int>* flag = carveout_done.slot();
+    if (!flag || !flag->load(std::memory_order_acquire)) {
+        if ((e = cudaFuncSetAttribute(col_z_kernel<P, L>, cudaFuncAttributePreferredSharedMemoryCarveout, TILE_KB * 100 / 228)) != cudaSuccess) return e;
+        if (flag) flag->store(1, std::memory_order_release);
+    }
+    const int per_sm = (int)(TILE_KB * 1024 / CZ::SMEM_BYTES);
+    if (slots > (per_sm > 0 ? per_sm : 1) * sms) slots = (per_sm > 0 ? per_sm : 1) * sms;
+    // the number of sampled ranks is known only on the device: one round of blocks, which share an image's tiles
     ColArgs b = a;
-    // the number of sampled ranks is known only on the device: launch a bounded number of blocks
-    // per outer index and let them stride over the tiles
-    long long cap = 4096 / (a.nouter > 0 ? a.nouter : 1) + 16;
-    // blocks that rank the mask row themselves pay for that once each: about eight per SM in all
-    if (a.zlist == nullptr) cap = (1184 + a.nouter - 1) / (a.nouter > 0 ? a.nouter : 1);
-    if (tiles > cap) tiles = cap;
-    b.ztiles = (int)tiles;
-    const long long blocks = a.nouter * tiles;
-    if (blocks <= 0) return cudaSuccess;
+    const long long most = (long long)a.C * ((a.es + L - 1) / L);
+    long long bpi = slots / a.images;
+    b.bpi = (int)(bpi < 1 ? 1 : bpi > most ? most : bpi);
+    const long long blocks = (long long)a.images * b.bpi;
     if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-    return launch_overlapped(a.zlist != nullptr, col_z_kernel<P, L>, dim3((unsigned)blocks), dim3(E::THREADS), E::SMEM_BYTES, s, b);
+    return launch_overlapped(a.zlist != nullptr, col_z_kernel<P, L>, dim3((unsigned)blocks), dim3(E::THREADS), CZ::SMEM_BYTES, s, b);
 }
 
 template <class P, class PC, int LC>
