@@ -265,6 +265,7 @@ GLEAM_API int gleam_dc_adjoint(const void* y, const void* sens, const float* mas
  */
 #define GLEAM_X_CHANNELS 1u
 #define GLEAM_OUT_CHANNELS 2u
+#define GLEAM_LOSS_FLOAT 4u      /* gleam_l1_loss: loss points at a float, the double mean rounded once */
 GLEAM_API int gleam_dc_forward_layout(const void* x, const void* y, const void* sens, const float* mask, float eta,
                                       void* out, const gleam_dims* dims, uint32_t layout);
 GLEAM_API int gleam_dc_vjp_layout(const void* grad_out, const void* sens, const float* mask, float eta, void* grad_in,

@@ -26,6 +26,7 @@ GLEAM_ERR_TIMEOUT = -9
 
 GLEAM_X_CHANNELS = 1
 GLEAM_OUT_CHANNELS = 2
+GLEAM_LOSS_FLOAT = 4
 
 GLEAM_MASK_FULL = 0
 GLEAM_MASK_READOUT_INVARIANT = 1
@@ -168,15 +169,14 @@ def gleam_dc_length_supported(n: int) -> bool:
 
 
 def _addr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
+    try:
+        return t.data_ptr()
+    except AttributeError:                     # a raw address or None
         return t
-    return int(t.data_ptr())
 
 
 def _check(status: int):
-    if status != GLEAM_OK:
+    if status:
         raise GleamError(status, gleam_status_string(status))
 
 
@@ -195,42 +195,42 @@ def make_dims(batch, coils, frames, fft_rank, n, sens_has_frames=0, mask_kind=GL
 
 def gleam_dc_workspace_size(dims: gleam_dims) -> int:
     out = ctypes.c_uint64(0)
-    _check(load_library().gleam_dc_workspace_size(ctypes.byref(dims), ctypes.byref(out)))
+    _check((_lib or load_library()).gleam_dc_workspace_size(ctypes.byref(dims), ctypes.byref(out)))
     return int(out.value)
 
 
 def gleam_dc_forward(x, y, sens, mask, eta, out, dims: gleam_dims) -> None:
     """out = x - eta A^H (A x - y)  (Eq. 3, eta = 2t).  Enqueues on dims.stream and returns."""
-    _check(load_library().gleam_dc_forward(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta), _addr(out),
+    _check((_lib or load_library()).gleam_dc_forward(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta), _addr(out),
                                             ctypes.byref(dims)))
 
 
 def gleam_dc_vjp(grad_out, sens, mask, eta, grad_in, dims: gleam_dims) -> None:
     """grad_in = grad_out - eta A^H A grad_out  (VJP of Eq. 3 with respect to x)."""
-    _check(load_library().gleam_dc_vjp(_addr(grad_out), _addr(sens), _addr(mask), float(eta), _addr(grad_in),
+    _check((_lib or load_library()).gleam_dc_vjp(_addr(grad_out), _addr(sens), _addr(mask), float(eta), _addr(grad_in),
                                         ctypes.byref(dims)))
 
 
 def gleam_dc_adjoint(y, sens, mask, out, dims: gleam_dims) -> None:
     """out = A^H y, the zero-filled SENSE image."""
-    _check(load_library().gleam_dc_adjoint(_addr(y), _addr(sens), _addr(mask), _addr(out), ctypes.byref(dims)))
+    _check((_lib or load_library()).gleam_dc_adjoint(_addr(y), _addr(sens), _addr(mask), _addr(out), ctypes.byref(dims)))
 
 
 def gleam_dc_prepare(y, mask, dims: gleam_dims) -> None:
     """Computes what Eq. 3 needs from y and the mask alone into dims.workspace (kept by the caller
     until the last gleam_dc_forward_prepared)."""
-    _check(load_library().gleam_dc_prepare(_addr(y), _addr(mask), ctypes.byref(dims)))
+    _check((_lib or load_library()).gleam_dc_prepare(_addr(y), _addr(mask), ctypes.byref(dims)))
 
 
 def gleam_dc_forward_aty(x, aty, sens, mask, eta, out, dims: gleam_dims) -> None:
     """Eq. 3 in normal-equations form: out = x - eta (A^H A x - aty) with aty = A^H y given as an image."""
-    _check(load_library().gleam_dc_forward_aty(_addr(x), _addr(aty), _addr(sens), _addr(mask), float(eta),
+    _check((_lib or load_library()).gleam_dc_forward_aty(_addr(x), _addr(aty), _addr(sens), _addr(mask), float(eta),
                                                _addr(out), ctypes.byref(dims)))
 
 
 def gleam_dc_forward_prepared(x, y, sens, mask, eta, out, dims: gleam_dims) -> None:
     """gleam_dc_forward with the tables of an earlier gleam_dc_prepare(y, mask, dims)."""
-    _check(load_library().gleam_dc_forward_prepared(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta),
+    _check((_lib or load_library()).gleam_dc_forward_prepared(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta),
                                                      _addr(out), ctypes.byref(dims)))
 
 
@@ -247,36 +247,36 @@ def gleam_dc_fused_wait_stats(dims: gleam_dims) -> dict:
     """{kind: (microseconds summed over all blocks, waits that had to spin)} of the last persistent-kernel call."""
     n = len(FUSED_WAIT_KINDS)
     buf = (ctypes.c_uint64 * (2 * n))()
-    _check(load_library().gleam_dc_fused_wait_stats(ctypes.byref(dims), buf, n))
+    _check((_lib or load_library()).gleam_dc_fused_wait_stats(ctypes.byref(dims), buf, n))
     return {FUSED_WAIT_KINDS[i]: (buf[2 * i] * 1e-3, int(buf[2 * i + 1])) for i in range(n)}
 
 
 def gleam_dc_grad_workspace_size(dims: gleam_dims) -> int:
     out = ctypes.c_uint64(0)
-    _check(load_library().gleam_dc_grad_workspace_size(ctypes.byref(dims), ctypes.byref(out)))
+    _check((_lib or load_library()).gleam_dc_grad_workspace_size(ctypes.byref(dims), ctypes.byref(out)))
     return int(out.value)
 
 
 def gleam_dc_grad_eta(grad_out, x, y, sens, mask, grad_eta, dims: gleam_dims) -> None:
     """grad_eta[b] = -Re<g_b, A^H(A x - y)_b> (device float64, one value per batch example)."""
-    _check(load_library().gleam_dc_grad_eta(_addr(grad_out), _addr(x), _addr(y), _addr(sens), _addr(mask),
+    _check((_lib or load_library()).gleam_dc_grad_eta(_addr(grad_out), _addr(x), _addr(y), _addr(sens), _addr(mask),
                                              _addr(grad_eta), ctypes.byref(dims)))
 
 
 def gleam_dc_grad_y(grad_out, sens, mask, eta, grad_y, dims: gleam_dims) -> None:
     """grad_y = eta Omega F S grad_out (complex64, layout of y)."""
-    _check(load_library().gleam_dc_grad_y(_addr(grad_out), _addr(sens), _addr(mask), float(eta), _addr(grad_y),
+    _check((_lib or load_library()).gleam_dc_grad_y(_addr(grad_out), _addr(sens), _addr(mask), float(eta), _addr(grad_y),
                                            ctypes.byref(dims)))
 
 
 def gleam_dc_forward_layout(x, y, sens, mask, eta, out, dims: gleam_dims, layout: int) -> None:
     """gleam_dc_forward with x and / or out in the two-real-channel layout (B, 2, T, n0, n1, n2) float32."""
-    _check(load_library().gleam_dc_forward_layout(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta), _addr(out),
+    _check((_lib or load_library()).gleam_dc_forward_layout(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta), _addr(out),
                                                    ctypes.byref(dims), int(layout)))
 
 
 def gleam_dc_vjp_layout(grad_out, sens, mask, eta, grad_in, dims: gleam_dims, layout: int) -> None:
-    _check(load_library().gleam_dc_vjp_layout(_addr(grad_out), _addr(sens), _addr(mask), float(eta), _addr(grad_in),
+    _check((_lib or load_library()).gleam_dc_vjp_layout(_addr(grad_out), _addr(sens), _addr(mask), float(eta), _addr(grad_in),
                                                ctypes.byref(dims), int(layout)))
 
 
@@ -285,8 +285,8 @@ def gleam_l1_loss_workspace_size() -> int:
 
 
 def gleam_l1_loss(x, ref, loss, grad, dims: gleam_dims, layout: int = 0) -> None:
-    """loss (device float64 scalar) = mean |x - ref|; grad (optional) = (x - ref)/|x - ref|/N."""
-    _check(load_library().gleam_l1_loss(_addr(x), _addr(ref), _addr(loss), _addr(grad), ctypes.byref(dims), int(layout)))
+    """loss (device float64 scalar, float32 with GLEAM_LOSS_FLOAT) = mean |x - ref|; grad (optional) = (x - ref)/|x - ref|/N."""
+    _check((_lib or load_library()).gleam_l1_loss(_addr(x), _addr(ref), _addr(loss), _addr(grad), ctypes.byref(dims), int(layout)))
 
 
 def gleam_measure_fp32_peak(scratch, stream=None) -> float:
@@ -294,7 +294,7 @@ def gleam_measure_fp32_peak(scratch, stream=None) -> float:
     out = ctypes.c_double(0.0)
     if stream is not None and not isinstance(stream, int):
         stream = stream.cuda_stream
-    _check(load_library().gleam_measure_fp32_peak(_addr(scratch), stream or None, ctypes.byref(out)))
+    _check((_lib or load_library()).gleam_measure_fp32_peak(_addr(scratch), stream or None, ctypes.byref(out)))
     return float(out.value)
 
 
@@ -315,7 +315,7 @@ def gleam_dc_debug_fused(withhold_item: int = -1, wait_limit_ns: int = 0) -> Non
 
 def gleam_dc_host_arena_size(dims: gleam_dims) -> int:
     out = ctypes.c_uint64(0)
-    _check(load_library().gleam_dc_host_arena_size(ctypes.byref(dims), ctypes.byref(out)))
+    _check((_lib or load_library()).gleam_dc_host_arena_size(ctypes.byref(dims), ctypes.byref(out)))
     return int(out.value)
 
 
@@ -324,14 +324,14 @@ def gleam_dc_forward_host(x, y, sens, mask, eta, out, dims: gleam_dims, arena, a
     arena is a device uint8 tensor of gleam_dc_host_arena_size(dims) bytes."""
     if arena_bytes is None:
         arena_bytes = arena.numel() * arena.element_size()
-    _check(load_library().gleam_dc_forward_host(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta), _addr(out),
+    _check((_lib or load_library()).gleam_dc_forward_host(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta), _addr(out),
                                                  ctypes.byref(dims), _addr(arena), int(arena_bytes)))
 
 
 def gleam_dc_vjp_host(grad_out, sens, mask, eta, grad_in, dims: gleam_dims, arena, arena_bytes=None) -> None:
     if arena_bytes is None:
         arena_bytes = arena.numel() * arena.element_size()
-    _check(load_library().gleam_dc_vjp_host(_addr(grad_out), _addr(sens), _addr(mask), float(eta), _addr(grad_in),
+    _check((_lib or load_library()).gleam_dc_vjp_host(_addr(grad_out), _addr(sens), _addr(mask), float(eta), _addr(grad_in),
                                              ctypes.byref(dims), _addr(arena), int(arena_bytes)))
 
 
@@ -342,7 +342,7 @@ def gleam_dc_static_scratch_bytes() -> int:
 def gleam_dc_forward_static(x, y, sens, mask, eta, out, dims: gleam_dims) -> None:
     """gleam_dc_forward with the library's own fixed scratch array instead of dims.workspace, for
     callers that cannot allocate device memory.  Calls whose GPU work overlaps race on that array."""
-    _check(load_library().gleam_dc_forward_static(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta),
+    _check((_lib or load_library()).gleam_dc_forward_static(_addr(x), _addr(y), _addr(sens), _addr(mask), float(eta),
                                                    _addr(out), ctypes.byref(dims)))
 
 
@@ -351,7 +351,7 @@ def gleam_dc_launch_count() -> int:
 
 
 def gleam_dc_profile_begin() -> None:
-    _check(load_library().gleam_dc_profile_begin())
+    _check((_lib or load_library()).gleam_dc_profile_begin())
 
 
 def gleam_dc_profile_end() -> dict:
@@ -359,7 +359,7 @@ def gleam_dc_profile_end() -> dict:
     n = len(KERNEL_CLASSES)
     ms = (ctypes.c_float * n)()
     cnt = (ctypes.c_uint32 * n)()
-    _check(load_library().gleam_dc_profile_end(ms, cnt, n))
+    _check((_lib or load_library()).gleam_dc_profile_end(ms, cnt, n))
     return {KERNEL_CLASSES[i]: (float(ms[i]), int(cnt[i])) for i in range(n) if cnt[i]}
 
 
@@ -457,19 +457,19 @@ class DataConsistency:
 
 def gleam_modl_cg_workspace_size(dims: gleam_dims) -> int:
     out = ctypes.c_uint64(0)
-    _check(load_library().gleam_modl_cg_workspace_size(ctypes.byref(dims), ctypes.byref(out)))
+    _check((_lib or load_library()).gleam_modl_cg_workspace_size(ctypes.byref(dims), ctypes.byref(out)))
     return int(out.value)
 
 
 def gleam_modl_cg_forward(z, y, sens, mask, mu, n_iter, out, dims: gleam_dims) -> None:
     """out = (A^H A + mu I)^{-1} (A^H y + mu z) by n_iter conjugate-gradient steps (Eq. 7)."""
-    _check(load_library().gleam_modl_cg_forward(_addr(z), _addr(y), _addr(sens), _addr(mask), float(mu), int(n_iter),
+    _check((_lib or load_library()).gleam_modl_cg_forward(_addr(z), _addr(y), _addr(sens), _addr(mask), float(mu), int(n_iter),
                                                  _addr(out), ctypes.byref(dims)))
 
 
 def gleam_modl_cg_vjp(grad_out, sens, mask, mu, n_iter, grad_z, dims: gleam_dims) -> None:
     """grad_z = mu (A^H A + mu I)^{-1} grad_out by n_iter conjugate-gradient steps."""
-    _check(load_library().gleam_modl_cg_vjp(_addr(grad_out), _addr(sens), _addr(mask), float(mu), int(n_iter),
+    _check((_lib or load_library()).gleam_modl_cg_vjp(_addr(grad_out), _addr(sens), _addr(mask), float(mu), int(n_iter),
                                              _addr(grad_z), ctypes.byref(dims)))
 
 

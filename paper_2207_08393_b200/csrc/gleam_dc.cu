@@ -452,6 +452,7 @@ __global__ void __launch_bounds__(GRAD_THREADS) grad_eta_partial_kernel(const cf
                                                                         const cf* __restrict__ t, long long ne,
                                                                         double* __restrict__ part) {
     // t = x - A^H(Ax - y)  (the step with eta = 1), so A^H(Ax - y) = x - t
+    grid_launch_dependents();
     __shared__ double sh[GRAD_THREADS];
     const long long base = (long long)blockIdx.y * ne;
     double acc = 0.0;
@@ -477,6 +478,7 @@ __device__ __forceinline__ double warp_array_sum(const double* __restrict__ v, i
     return s;
 }
 __global__ void grad_eta_final_kernel(const double* __restrict__ part, int nblocks, double* __restrict__ grad_eta) {
+    grid_dependency_wait();
     const double s = warp_array_sum(part + (long long)blockIdx.x * nblocks, nblocks);
     if (threadIdx.x == 0) grad_eta[blockIdx.x] = -s;
 }
@@ -488,6 +490,7 @@ __global__ void grad_eta_final_kernel(const double* __restrict__ part, int nbloc
 __global__ void __launch_bounds__(GRAD_THREADS) l1_partial_kernel(const cf* __restrict__ x, const cf* __restrict__ r, cf* __restrict__ grad,
                                                                   long long ne, int B, int x_planar, int g_planar, long long plane,
                                                                   float inv_n, double* __restrict__ part) {
+    grid_launch_dependents();
     __shared__ double sh[GRAD_THREADS];
     double acc = 0.0;
     const long long n = ne * B;
@@ -510,9 +513,10 @@ __global__ void __launch_bounds__(GRAD_THREADS) l1_partial_kernel(const cf* __re
     }
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
-__global__ void l1_final_kernel(const double* __restrict__ part, int nblocks, double inv_n, double* __restrict__ loss) {
+__global__ void l1_final_kernel(const double* __restrict__ part, int nblocks, double inv_n, double* __restrict__ loss, int as_float) {
+    grid_dependency_wait();
     const double s = warp_array_sum(part, nblocks);
-    if (threadIdx.x == 0) *loss = s * inv_n;
+    if (threadIdx.x == 0) { if (as_float) *reinterpret_cast<float*>(loss) = (float)(s * inv_n); else *loss = s * inv_n; }
 }
 
 
@@ -684,10 +688,10 @@ GLEAM_API int gleam_l1_loss(const void* x, const void* ref, double* loss, void* 
     Layout L;
     int rc = make_layout(dims, false, &L);
     if (rc != GLEAM_OK) return rc;
-    if (layout & ~(GLEAM_X_CHANNELS | GLEAM_OUT_CHANNELS)) return GLEAM_ERR_BAD_DIMS;
+    if (layout & ~(GLEAM_X_CHANNELS | GLEAM_OUT_CHANNELS | GLEAM_LOSS_FLOAT)) return GLEAM_ERR_BAD_DIMS;
     if (!dims->workspace) return GLEAM_ERR_NULL_POINTER;
     if (dims->workspace_bytes < gleam_l1_loss_workspace_size()) return GLEAM_ERR_WORKSPACE_TOO_SMALL;
-    if (((uintptr_t)x & 7) || ((uintptr_t)ref & 7) || ((uintptr_t)loss & 7) || ((uintptr_t)grad & 7) || ((uintptr_t)dims->workspace & 255)) return GLEAM_ERR_BAD_DIMS;
+    if (((uintptr_t)x & 7) || ((uintptr_t)ref & 7) || ((uintptr_t)loss & ((layout & GLEAM_LOSS_FLOAT) ? 3 : 7)) || ((uintptr_t)grad & 7) || ((uintptr_t)dims->workspace & 255)) return GLEAM_ERR_BAD_DIMS;
     const void* ptrs[5] = {x, ref, loss, grad, dims->workspace};
     for (int i = 0; i < 5; ++i) if (ptrs[i] && (rc = check_device_ptr(ptrs[i])) != GLEAM_OK) return rc;
     const uint64_t img_b = (uint64_t)L.images * L.V * sizeof(cf);
@@ -707,8 +711,7 @@ GLEAM_API int gleam_l1_loss(const void* x, const void* ref, double* loss, void* 
                                                        (layout & GLEAM_OUT_CHANNELS) ? 1 : 0, ne, (float)(1.0 / (double)n), part);
     CK(cudaGetLastError());
     CK(prof_mark(GLEAM_K_CG_VEC, s));
-    l1_final_kernel<<<1, 32, 0, s>>>(part, nblocks, 1.0 / (double)n, loss);
-    CK(cudaGetLastError());
+    CK(launch_overlapped(true, l1_final_kernel, dim3(1), dim3(32), 0, s, (const double*)part, nblocks, 1.0 / (double)n, loss, (layout & GLEAM_LOSS_FLOAT) ? 1 : 0));
     CK(prof_mark(-1, s));
     return GLEAM_OK;
 }
@@ -751,8 +754,7 @@ GLEAM_API int gleam_dc_grad_eta(const void* grad_out, const void* x, const void*
     grad_eta_partial_kernel<<<dim3((unsigned)G.nblocks, (unsigned)dims->batch), GRAD_THREADS, 0, s>>>((const cf*)grad_out, (const cf*)x, t, G.ne, part);
     if (cudaGetLastError() != cudaSuccess) return GLEAM_ERR_CUDA;
     if (prof_mark(GLEAM_K_CG_VEC, s) != cudaSuccess) return GLEAM_ERR_CUDA;
-    grad_eta_final_kernel<<<(unsigned)dims->batch, 32, 0, s>>>(part, G.nblocks, grad_eta);
-    if (cudaGetLastError() != cudaSuccess) return GLEAM_ERR_CUDA;
+    if (launch_overlapped(true, grad_eta_final_kernel, dim3((unsigned)dims->batch), dim3(32), 0, s, (const double*)part, G.nblocks, grad_eta) != cudaSuccess) return GLEAM_ERR_CUDA;
     if (prof_mark(-1, s) != cudaSuccess) return GLEAM_ERR_CUDA;
     return GLEAM_OK;
 }

@@ -44,11 +44,12 @@ class _L1Function(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x_ch, step):
-        loss = torch.empty((), dtype=torch.float64, device=x_ch.device)
+        loss = torch.empty((), dtype=torch.float32, device=x_ch.device)
         grad = torch.empty_like(x_ch)
-        _b.gleam_l1_loss(x_ch, step.ref, loss, grad, step.l1_dims(), _b.GLEAM_X_CHANNELS | _b.GLEAM_OUT_CHANNELS)
+        _b.gleam_l1_loss(x_ch, step.ref, loss, grad, step.l1_dims(),
+                         _b.GLEAM_X_CHANNELS | _b.GLEAM_OUT_CHANNELS | _b.GLEAM_LOSS_FLOAT)
         ctx.save_for_backward(grad)
-        return loss.to(torch.float32)
+        return loss
 
     @staticmethod
     def backward(ctx, g):
