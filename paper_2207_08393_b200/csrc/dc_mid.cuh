@@ -214,13 +214,14 @@ struct MidOps {
     cudaError_t (*launch)(int mode, const MidArgs&, cudaStream_t);
 };
 
-// Blocks that share the coils of a tile: doubled while that leaves no more than three blocks per SM.  Splitting only
-// fills SMs that would be idle (a single 320 x 256 slice with 8 coils, 20 tiles: 44 -> 29 us per call for 4 blocks a
-// tile); with more tiles the start-up of the additional blocks and the sum over the cluster cost more than the finer
-// grain gains (12 coils of 96 x 240 x 184, 1440 tiles: 512 us unsplit, 549 us for 2, 615 us for 4 blocks a tile).
-inline int coil_split(long long tiles, int sms, int C) {
+// Blocks that share the coils of a tile: doubled while that leaves no more than 640 threads per SM.  Splitting only
+// fills SMs that would be idle (a 160 x 160 slice with 16 coils, 16 tiles: 47 us per VJP call unsplit, 33 / 25 / 21 us
+// for 2 / 4 / 8 blocks a tile); beyond that the start-up of the additional blocks costs more than the finer grain gains
+// (limits of 512 / 640 / 768 / 1024 threads: 2 x 16 coils of 640 x 320 109 / 94 / 94 / 94 us, 5 coils of 24 x 128 x 128
+// 37 / 37 / 43 / 43 us, 9 coils of 320 x 48 x 24 49 / 49 / 49 / 64 us).
+inline int coil_split(long long tiles, int threads, int sms, int C) {
     int cs = 1;
-    while (cs < 4 && 2 * cs <= C && 2 * cs * tiles <= 3LL * sms) cs *= 2;
+    while (cs < MAX_CSPLIT && 2 * cs <= C && 2 * cs * tiles * threads <= 640LL * sms) cs *= 2;
     return cs;
 }
 
@@ -234,7 +235,7 @@ struct TileImpl {
         int sms = 0;
         if ((e = device_sms(&sms)) != cudaSuccess) return e;
         TileArgs a = a0;
-        a.csplit = coil_split(tiles, sms, a.C);
+        a.csplit = coil_split(tiles, TL::TH, sms, a.C);
         const long long blocks = images * a.G * a.BY * a.csplit;
         if (blocks <= 0) return cudaSuccess;
         if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
@@ -248,7 +249,7 @@ struct TileImpl {
         int sms = 0;
         if ((e = device_sms(&sms)) != cudaSuccess) return e;
         TileArgs a = a0;
-        a.csplit = coil_split(tiles, sms, a.C);
+        a.csplit = coil_split(tiles, TL::TH, sms, a.C);
         const long long blocks = images * a.G * a.BY * a.csplit;
         if (blocks <= 0) return cudaSuccess;
         if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;

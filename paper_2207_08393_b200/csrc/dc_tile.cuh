@@ -58,6 +58,7 @@ struct Tile {
     }
 };
 
+constexpr int MAX_CSPLIT = 8;                // blocks that may share the coils of a tile
 __device__ __forceinline__ void cluster_arrive_wait() {
     asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
 }
@@ -66,7 +67,7 @@ __device__ __forceinline__ cf cluster_load(const cf* p, unsigned rank) {
     const unsigned a = (unsigned)__cvta_generic_to_shared(p);
     unsigned r; cf v;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(r) : "memory");
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(r));
     return v;
 }
 
@@ -266,30 +267,42 @@ tile_inv_kernel(const TileArgs a) {
         }
     }
     cp_async_wait<0>();
+    auto finish = [&](int m, cf sum) {       // out = x - eta * sum of row m
+        const long long e = x_off + m * row_stride;
+        const cf xv = a.x ? load_image(a.x, e, a.x_planar, id.b, a.plane) : make_float2(0.f, 0.f);
+        store_image(a.out, e, make_float2(fmaf(-a.eta, sum.x, xv.x), fmaf(-a.eta, sum.y, xv.y)), a.out_planar, id.b, a.plane);
+    };
     if (a.csplit > 1) {
-        // partial coil sums of the other blocks of the cluster, added in block order
+        // The partial coil sums of the cluster's blocks, added in block order; the blocks share the rows.  All loads of a
+        // row are requested before the first is used (one after another they took 10 us).
         __syncthreads();
-        if (col && id.part > 0) {
+        if (col) {
 #pragma unroll
             for (int m = 0; m < RY; ++m) sT[m * NZ + tid] = acc[m];
         }
         cluster_arrive_wait();
-        if (col && id.part == 0) {
-            for (int p = 1; p < a.csplit; ++p) {
+        if (col) {
+#pragma unroll 2
+            for (int m = (int)id.part; m < RY; m += a.csplit) {
+                cf t[MAX_CSPLIT];
 #pragma unroll
-                for (int m = 0; m < RY; ++m) acc[m] = cadd(acc[m], cluster_load(sT + m * NZ + tid, (unsigned)p));
+                for (int p = 0; p < MAX_CSPLIT; ++p) t[p] = (p < a.csplit) ? cluster_load(sT + m * NZ + tid, (unsigned)p) : make_float2(0.f, 0.f);
+                cf sum = t[0];
+#pragma unroll
+                for (int p = 1; p < MAX_CSPLIT; ++p) sum = cadd(sum, t[p]);
+                finish(m, sum);
             }
         }
         cluster_arrive_wait();           // no block leaves while its sums are being read
-        if (id.part > 0) return;
+        return;
     }
     if (!col) return;
+    cf xv[RY];
 #pragma unroll
-    for (int m = 0; m < RY; ++m) {
-        const long long e = x_off + m * row_stride;
-        const cf xv = a.x ? load_image(a.x, e, a.x_planar, id.b, a.plane) : make_float2(0.f, 0.f);
-        store_image(a.out, e, make_float2(fmaf(-a.eta, acc[m].x, xv.x), fmaf(-a.eta, acc[m].y, xv.y)), a.out_planar, id.b, a.plane);
-    }
+    for (int m = 0; m < RY; ++m) xv[m] = a.x ? load_image(a.x, x_off + m * row_stride, a.x_planar, id.b, a.plane) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < RY; ++m)
+        store_image(a.out, x_off + m * row_stride, make_float2(fmaf(-a.eta, acc[m].x, xv[m].x), fmaf(-a.eta, acc[m].y, xv[m].y)), a.out_planar, id.b, a.plane);
 }
 
 }  // namespace gleam
