@@ -160,7 +160,10 @@ template <class P, int L>
 __global__ void __launch_bounds__(LineFFT<P, L>::THREADS)
 col_z_kernel(const ColArgs a) {
     grid_dependency_wait();
-    grid_launch_dependents();    // a one-pass row kernel behind this launch may be scheduled early
+    // The row kernel behind this launch is scheduled when its blocks end.  Scheduled at their start, its single-warp
+    // blocks piled up on the SMs with room and stayed there (8 x 16 coils of 128 x 120, forward 48 against 29 us); only
+    // next to a handful of blocks the earlier start is the better one (64 x 64, 8 coils: 7.4 against 8.1 us).
+    if (gridDim.x <= 64) grid_launch_dependents();
     using E = LineFFT<P, L>;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL, BUFSZ = ColZ<P, L>::BUFSZ;
     extern __shared__ __align__(16) float2 smem[];

@@ -138,7 +138,6 @@ constexpr int CG_BATCH = 2;
 template <bool FROM_ROWS, bool LAST>
 __global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) {
     grid_dependency_wait();
-    grid_launch_dependents();
     const long long base = (long long)blockIdx.y * a.ne2, stride = (long long)gridDim.x * CG_THREADS;
     long long i = (long long)blockIdx.x * CG_THREADS + threadIdx.x;
     float4 pv[CG_BATCH], xv[CG_BATCH], qv[LAST ? 1 : CG_BATCH], rv[LAST ? 1 : CG_BATCH];

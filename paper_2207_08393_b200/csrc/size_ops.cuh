@@ -187,7 +187,10 @@ template <class P> using ZPlan = std::conditional_t<FlatRL<P::N>::z != 0, FlatPl
 // Few lines: the coils of a line group side by side (dc_coilpar.cuh) while all warps are resident at once (16 per SM).
 // Measured per call, numbered or plain kernel -> here: one 64 x 64 slice of 8 coils 12.5 -> 4.3 us (prepared step),
 // 4.7 -> 3.4 us (VJP); 6 x 8 coils of 46 x 240 18.6 -> 7.3 and 11.7 -> 6.2 us; beyond the line 6 x 4 coils of 368 x 80
-// 7.6 -> 11.3 us; with 2 or 3 coils 3.9 -> 4.8 us.  *taken: the call was launched here.
+// 7.6 -> 11.3 us; with 2 or 3 coils 3.9 -> 4.8 us.  Larger problems first take two to four coils per warp: prepared step
+// of 8 x 16 coils of 128 x 24 24 -> 5.9 us, 4 x 7 coils of 384 x 32 12.7 -> 5.5 us, 6 x 10 coils of 128 x 160 16 -> 11 us;
+// not below 8 warps without z (14 x 17 frames of 64 x 128, VJP 11 -> 16 us with 4) and not for last radices beyond 16
+// (16 coils of 320 x 320, 19.5 -> 26 us).  *taken: the call was launched here.
 template <class P, bool HAS_Z, bool ADJ>
 inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken) {
     using CP = CoilPar<P>;
@@ -195,8 +198,11 @@ inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken)
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
-    const int warps = a.C < 16 ? a.C : 16;
+    // fewest warps that still pay: each takes several coils then, so that more line groups are resident at once
+    constexpr int LEAST = !HAS_Z ? 8 : P::RL <= 16 ? 4 : 16;
+    int warps = a.C < 16 ? a.C : 16;
     const long long groups = (a.nrows + CP::LW - 1) / CP::LW;
+    while (groups * warps > 16LL * sms && (warps + 1) / 2 >= LEAST) warps = (warps + 1) / 2;
     const size_t bytes = CP::bytes(warps, a.C);
     if (a.C < 4 || bytes > CP::LIMIT || groups <= 0 || groups * warps > 16LL * sms) return cudaSuccess;
     static PerDevice done;
@@ -229,20 +235,6 @@ inline cudaError_t launch_col_z(const ColArgs& a, cudaStream_t s) {
     int slots = 0;
     if ((e = resident_slots(col_z_kernel<P, L>, E::THREADS, CZ::SMEM_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
     if (a.images <= 0) return cudaSuccess;
-    int sms = 0;
-    if ((e = device_sms(&sms)) != cudaSuccess) return e;
-    // Every sample in flight holds a line of L1, so the blocks take no more than 132 KB of the SM's 228 for their tiles
-    // (64 / 100 / 132 / 164 / 196 KB: 640-point slices 40 / 34 / 38 / 42 / 48 us, 320 x 320 x 256 at 12x 223 / 238 /
-    // 234 / 225 / 243 us, 8 x 16 coils of 640 x 320 at 4x 81 / 85 / 76 / 87 / 101 us).
-    constexpr int TILE_KB = 132;
-    static PerDevice carveout_done;
-    std::atomic<int>* flag = carveout_done.slot();
-    if (!flag || !flag->load(std::memory_order_acquire)) {
-        if ((e = cudaFuncSetAttribute(col_z_kernel<P, L>, cudaFuncAttributePreferredSharedMemoryCarveout, TILE_KB * 100 / 228)) != cudaSuccess) return e;
-        if (flag) flag->store(1, std::memory_order_release);
-    }
-    const int per_sm = (int)(TILE_KB * 1024 / CZ::SMEM_BYTES);
-    if (slots > (per_sm > 0 ? per_sm : 1) * sms) slots = (per_sm > 0 ? per_sm : 1) * sms;
     // the number of sampled ranks is known only on the device: one round of blocks, which share an image's tiles
     ColArgs b = a;
     const long long most = (long long)a.C * ((a.es + L - 1) / L);
