@@ -38,6 +38,7 @@ coilpar_kernel(const RowArgs a) {
     UnitMask* sU = reinterpret_cast<UnitMask*>(smem + CP::OFF_U);
     cf* sE = smem + CP::OFF_E + warp * LW * EXL;
     cf* sV = smem + CP::OFF_E + warps * LW * EXL;
+    __shared__ bool s_few[LW];                             // the line's sampled entries are as few as other kernels stage
     const long long row0 = (long long)blockIdx.x * LW;
 
     // offsets of a line of this group (identical arithmetic wherever a line index is needed)
@@ -59,7 +60,10 @@ coilpar_kernel(const RowArgs a) {
     for (int ll = warp; ll < LW; ll += warps) {
         long long x_off = 0, s_off = 0, k_off = 0, bt = 0; int b = 0;
         const bool ok = line_of(ll, x_off, s_off, k_off, bt, b);
-        if (HAS_Z) line_units<P::BFL, RL>(a.mask + bt * N, ok, lane, sU + ll * P::BFL, ADJ ? nullptr : sM + ll * N);
+        if (HAS_Z) {
+            const int cnt = line_units<P::BFL, RL>(a.mask + bt * N, ok, lane, sU + ll * P::BFL, ADJ ? nullptr : sM + ll * N);
+            if (lane == 0) s_few[ll] = cnt <= z_stage(N);
+        }
 #pragma unroll 8
         for (int k0 = 0; k0 < N; k0 += 32) {
             const int k = k0 + lane;
@@ -109,7 +113,7 @@ coilpar_kernel(const RowArgs a) {
         if (aL) {
             if (HAS_Z) {
                 const UnitMask um = sU[l * P::BFL + j];
-                unit_update<P::BFL, RL, ADJ>(u, um.bits, sM + l * N + j, a.z + k_off + c * k_stride + um.first);
+                unit_update<P::BFL, RL, ADJ>(u, um.bits, sM + l * N + j, a.z + k_off + c * k_stride + um.first, s_few[l]);
             } else {
 #pragma unroll
                 for (int k = 0; k < RL; ++k) u[k] = cscale(u[k], sM[l * N + j + P::BFL * k]);

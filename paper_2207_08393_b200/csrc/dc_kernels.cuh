@@ -121,9 +121,10 @@ __device__ __forceinline__ int line_units(const float* mask_row, bool ok, int la
     return __shfl_sync(0xffffffffu, incl, 31);
 }
 // k-space update of one unit: u = w u - z at the sampled entries, 0 elsewhere (adjoint: -z).  `weight` points at the
-// unit's first entry (stride R0), `z` at its run; both are read at sampled entries only.
+// unit's first entry (stride R0), `z` at its run; both are read at sampled entries only.  `fused`: one rounding for the
+// two operations (lines whose z values are few enough to be staged), else one each, whichever kernel the line is in.
 template <int R0, int RL, bool ADJ>
-__device__ __forceinline__ void unit_update(cf (&u)[RL], unsigned bits, const float* weight, const cf* z) {
+__device__ __forceinline__ void unit_update(cf (&u)[RL], unsigned bits, const float* weight, const cf* z, bool fused) {
 #pragma unroll
     for (int k = 0; k < RL; ++k) {
         float w = 0.f; cf q = make_float2(0.f, 0.f);
@@ -131,9 +132,13 @@ __device__ __forceinline__ void unit_update(cf (&u)[RL], unsigned bits, const fl
             if (!ADJ) w = weight[R0 * k];
             q = *z++;
         }
-        u[k] = ADJ ? make_float2(-q.x, -q.y) : make_float2(fmaf(w, u[k].x, -q.x), fmaf(w, u[k].y, -q.y));
+        if (ADJ) u[k] = make_float2(-q.x, -q.y);
+        else if (fused) u[k] = make_float2(fmaf(w, u[k].x, -q.x), fmaf(w, u[k].y, -q.y));
+        else u[k] = make_float2(__fsub_rn(__fmul_rn(w, u[k].x), q.x), __fsub_rn(__fmul_rn(w, u[k].y), q.y));
     }
 }
+// sampled entries of a line of N points that are staged
+constexpr int z_stage(int N) { return ((N + 3) / 4 + 1) / 2 * 2; }
 
 constexpr int COLZ_SELF_MAX = 1024;   // COL_Z ranks a mask row of at most this many positions by itself
 

@@ -35,7 +35,7 @@ struct WarpFlat {
     }
     static constexpr int SLOTS = (!SMW && !HAS_Z && slots_aligned() * UPC * USTRIDE * 8 <= 11 * 1024) ? slots_aligned() : SLOTS_MIN;
     static constexpr int ZS = SMW ? SLOTS : SLOTS + 1;     // z rows are requested one forward stage ahead (SMW: in their own stage)
-    static constexpr int KCAP = ((N + 3) / 4 + 1) / 2 * 2; // staged z entries per line (more: read from global memory)
+    static constexpr int KCAP = z_stage(N); // staged z entries per line (more: read from global memory)
     static constexpr int KSTRIDE = KCAP;
     static constexpr int KTILE = LW * KSTRIDE;
     static constexpr int MS = N + ((LW > 1 && N % 32 == 0) ? 16 : 0);   // mask row stride (floats): lines on different banks
@@ -239,8 +239,8 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                     const UnitMask um = sU[bl * R0 + jb];
                     const int kc = sC[bl];
                     const float* mw = sM + bl * MS + jb;
-                    if (kc <= KCAP) unit_update<R0, RL, ADJ>(u, kc > 0 ? um.bits : 0u, mw, sK + (c % ZS) * KTILE + bl * KSTRIDE + um.first);
-                    else unit_update<R0, RL, ADJ>(u, um.bits, mw, a.z + sKo[bl] + c * k_stride + um.first);
+                    if (kc <= KCAP) unit_update<R0, RL, ADJ>(u, kc > 0 ? um.bits : 0u, mw, sK + (c % ZS) * KTILE + bl * KSTRIDE + um.first, true);
+                    else unit_update<R0, RL, ADJ>(u, um.bits, mw, a.z + sKo[bl] + c * k_stride + um.first, false);
                 }
                 Dft<RL, +1>::run(u);
                 if (live) {

@@ -22,7 +22,7 @@ struct WarpLine {
     // per-warp shared memory, in float2 units: S[2], z[2], x, exchange, m2 (floats, N/2 float2 per line), unit masks.
     // Up to KCAP sampled z entries per line are staged (lines with more read z straight from global memory)
     static constexpr int TILE = LW * N;
-    static constexpr int KCAP = ((N + 3) / 4 + 1) / 2 * 2;
+    static constexpr int KCAP = z_stage(N);
     static constexpr int KSTRIDE = KCAP;
     static constexpr int KTILE = LW * KSTRIDE;
     static constexpr int OFF_S = 0, OFF_K = 2 * TILE, OFF_X = OFF_K + (HAS_Z ? 2 * KTILE : 0),
@@ -195,8 +195,8 @@ warpline_kernel(const RowArgs a) {
                         for (int k = 0; k < RL; ++k) u[k] = cscale(u[k], mm[P::BFL * k]);
                     } else {       // staged z, or straight from the line's row (lanes without a row hold no mask)
                         const UnitMask um = row_ok ? sU[l * P::BFL + j] : UnitMask{0u, 0};
-                        if (k_cnt <= KCAP) unit_update<P::BFL, RL, ADJ>(u, um.bits, mm, cK + um.first);
-                        else unit_update<P::BFL, RL, ADJ>(u, um.bits, mm, gK + um.first);
+                        if (k_cnt <= KCAP) unit_update<P::BFL, RL, ADJ>(u, um.bits, mm, cK + um.first, true);
+                        else unit_update<P::BFL, RL, ADJ>(u, um.bits, mm, gK + um.first, false);
                     }
                 }
             }

@@ -114,7 +114,7 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s) {
     if (groups <= 0) return cudaSuccess;
     // One round of 8 to 16 groups per SM: one block per SM that holds all its warps.  4 k + 1 (or 4 k + 2) groups per
     // SM: the groups beyond 4 k are split by coils over four warps each, one per scheduler.  (Measured on cine-shaped
-    // problems, per call: 13 groups per SM 18.7 -> 16.6 us, 12 per SM 18.7 -> 15.3 us; up to 7 per SM single-warp
+    // problems, per call: 13 groups per SM 18.7 -> 16.6 us, with z 22.7 -> 21.5 us, 12 per SM 18.7 -> 15.3 us; up to 7 per SM single-warp
     // blocks are faster, 11.3 against 12.7 us.)
     if constexpr (P::RL <= 16 && P::R0 <= 12 && !WF::PRIME) {   // larger butterflies need more registers than 16 warps per SM leave
         using WS = WarpFlat<P, HAS_Z, true>;
@@ -126,9 +126,7 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s) {
             if (per - nsplit + 4 * nsplit > 16) nsplit = 0;
             const int nwhole = per - nsplit, warps = nwhole + 4 * nsplit;
             const size_t bytes = WS::WARP_BYTES * (size_t)warps;
-            // with z the split groups were measured slower than single-warp blocks (13 groups per SM: 25.2 against
-            // 24.7 us per call), whole groups alone faster (12 per SM: 22.5 against 24.5 us)
-            if (warps <= 16 && bytes <= 227 * 1024 && !(HAS_Z && nsplit > 0)) {
+            if (warps <= 16 && bytes <= 227 * 1024) {
                 // the attribute is set once, to what the largest block of this kernel can ask for
                 constexpr size_t SMEM_CAP = 227 * 1024;
                 if ((e = ensure_smem(warpflat_kernel<P, HAS_Z, true, HAS_ATY, ADJ>, 16 * WS::WARP_BYTES < SMEM_CAP ? 16 * WS::WARP_BYTES : SMEM_CAP, attrs_done)) != cudaSuccess) return e;
