@@ -157,10 +157,12 @@ inline bool flat_enabled() {
 // quarters of them busy in both stages.  Measured, VJP / prepared step, 8 x 16 coils x 512 rows, plain -> numbered:
 // 46: 100 / 113 -> 23 / 33 us; 92: 107 / 127 -> 36 / 49; 184: 127 / 144 -> 68 / 81; 384: 150 / 217 -> 89 / 125;
 // 512: 153 / 252 -> 124 / 157; 640: 391 / 822 -> 155 / 200 (three-stage block kernel before); 64 as 4 x 16 and 32 as
-// 4 x 8 for the VJP: 19 -> 16, 23 -> 15 us; but 120: 37 / 45 -> 42 / 69, 240: 60 / 90 -> 69 / 95, 256: 60 / 94 -> 64 / 94.
+// 4 x 8 for the VJP: 19 -> 16, 23 -> 15 us; but 120: 37 / 44 -> 42 / 56, 240: 60 / 72 -> 69 / 88.  With z, 256 gains where a
+// line has more samples than are staged (at 3.2x 156 -> 101 us, at 6x equal), 32 28 -> 24 us; 64 as 4 x 16 29 -> 23 us, but
+// 2 x 10 coils x 256 rows 4.9 -> 6.9 us; 368 as 23 x 16 154 -> 143 us, but 4 x 15 coils x 640 rows 97 -> 109 us.
 template <int N> struct FlatRL { static constexpr int v = 0, z = 0; };
 #define GLEAM_FLAT(N, V, Z) template <> struct FlatRL<N> { static constexpr int v = V, z = Z; };
-GLEAM_FLAT(32, 8, 0)
+GLEAM_FLAT(32, 8, 8)
 GLEAM_FLAT(46, 23, 23)
 GLEAM_FLAT(48, 8, 8)
 GLEAM_FLAT(64, 16, 0)
@@ -171,6 +173,7 @@ GLEAM_FLAT(128, 16, 16)
 GLEAM_FLAT(160, 16, 16)
 GLEAM_FLAT(184, 23, 23)
 GLEAM_FLAT(192, 0, 32)
+GLEAM_FLAT(256, 0, 16)
 GLEAM_FLAT(320, 32, 32)
 GLEAM_FLAT(368, 16, 23)
 GLEAM_FLAT(384, 32, 32)
