@@ -37,6 +37,7 @@ struct Axis {
 template <class P, int KC, int MODE>
 __global__ void __launch_bounds__(Axis<P, KC>::THREADS, Axis<P, KC>::BLOCKS)
 axis_kernel(const AxisArgs a) {
+    grid_dependency_wait();
     using AX = Axis<P, KC>;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL, BF0 = P::BF0, BFL = P::BFL, LS1 = P::LS1;
     extern __shared__ __align__(16) float2 smem[];
@@ -162,8 +163,7 @@ struct AxisImpl {
         const long long blocks = a.nunits * a.n1 * ((a.n2 + KC - 1) / KC);
         if (blocks <= 0) return cudaSuccess;
         if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-        axis_kernel<P, KC, MODE><<<(unsigned)blocks, AX::THREADS, AX::BYTES + (a.y ? AX::Y_BYTES : 0), s>>>(a);
-        return cudaGetLastError();
+        return launch_overlapped(true, axis_kernel<P, KC, MODE>, dim3((unsigned)blocks), dim3(AX::THREADS), AX::BYTES + (a.y ? AX::Y_BYTES : 0), s, a);
     }
     static cudaError_t launch(int mode, const AxisArgs& a, cudaStream_t s) {
         switch (mode) {

@@ -43,6 +43,7 @@ template <int BY> constexpr int mid_blocks() {
 template <int RY, int BY, int MODE>
 __global__ void __launch_bounds__(256, mid_blocks<BY>())
 mid_kernel(const MidArgs a) {
+    grid_dependency_wait();
     constexpr int N1 = RY * BY;
     constexpr bool FORWARD = MODE != MID_INV && MODE != MID_ADJ_Z && MODE != MID_ADJ_FULL;
     constexpr bool INVERSE = MODE != MID_FWD && MODE != MID_GRADY;
@@ -239,8 +240,7 @@ struct TileImpl {
         const long long blocks = images * a.G * a.BY * a.csplit;
         if (blocks <= 0) return cudaSuccess;
         if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-        tile_fwd_kernel<PZ, RY><<<(unsigned)blocks, TL::TH, TL::FWD_BYTES, s>>>(a);
-        return cudaGetLastError();
+        return launch_overlapped(true, tile_fwd_kernel<PZ, RY>, dim3((unsigned)blocks), dim3(TL::TH), TL::FWD_BYTES, s, a);
     }
     static cudaError_t inv(const TileArgs& a0, long long images, long long tiles, cudaStream_t s) {
         static PerDevice done;
@@ -253,21 +253,16 @@ struct TileImpl {
         const long long blocks = images * a.G * a.BY * a.csplit;
         if (blocks <= 0) return cudaSuccess;
         if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3(TL::TH); cfg.dynamicSmemBytes = TL::INV_BYTES; cfg.stream = s;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)a.csplit; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        cfg.attrs = at; cfg.numAttrs = a.csplit > 1 ? 1 : 0;
-        return cudaLaunchKernelEx(&cfg, tile_inv_kernel<PZ, RY>, a);
+        return launch_overlapped_cluster((unsigned)a.csplit, tile_inv_kernel<PZ, RY>, dim3((unsigned)blocks), dim3(TL::TH), TL::INV_BYTES, s, a);
     }
 };
 
 template <int RY, int BY>
 struct MidImpl {
+    static constexpr int ZCAP = 2048;          // z values of one k0 group that are staged
     template <int MODE> static cudaError_t go(const MidArgs& a0, cudaStream_t s) {
         MidArgs a = a0;
-        const int threads = a.NZ < 256 ? ((a.NZ + 31) / 32) * 32 : 256;
+        const int parts = (a.NZ + 255) / 256, threads = ((a.NZ + parts - 1) / parts + 31) / 32 * 32;   // equal shares of a row
         const long long blocks = a.nunits * a.G * RY;
         if (blocks <= 0) return cudaSuccess;
         if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
@@ -282,12 +277,15 @@ struct MidImpl {
             if (a.y) bytes += (size_t)BY * threads * sizeof(cf);
         }
         if (Z) {
-            a.zcap = BY * a.NZ < 1024 ? BY * a.NZ : 1024;
+            a.zcap = BY * a.NZ < ZCAP ? BY * a.NZ : ZCAP;
             bytes += (size_t)(a.zcap + 1) * (sizeof(cf) + sizeof(float)) + 8;
         }
-        static_assert(!Z || BY * 256 * sizeof(float) + 1025 * 12 + 8 + (BY + 1) * 8 <= 48 * 1024, "over the default shared memory limit");
-        mid_kernel<RY, BY, MODE><<<dim3((unsigned)blocks, (unsigned)((a.NZ + threads - 1) / threads)), threads, bytes, s>>>(a);
-        return cudaGetLastError();
+        if (Z) {
+            static PerDevice done;
+            cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * sizeof(float) + (ZCAP + 1) * 12 + 8, done);
+            if (e != cudaSuccess) return e;
+        }
+        return launch_overlapped(true, mid_kernel<RY, BY, MODE>, dim3((unsigned)blocks, (unsigned)parts), dim3(threads), bytes, s, a);
     }
     static cudaError_t launch(int mode, const MidArgs& a, cudaStream_t s) {
         switch (mode) {

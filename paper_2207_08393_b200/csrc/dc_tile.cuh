@@ -104,6 +104,7 @@ __device__ __forceinline__ void stage_rows(cf* dst, const cf* src, long long row
 template <class PZ, int RY>
 __global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY>::blocks(Tile<PZ, RY>::FWD_BYTES))
 tile_fwd_kernel(const TileArgs a) {
+    grid_dependency_wait();
     using TL = Tile<PZ, RY>;
     constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
     extern __shared__ __align__(16) float2 smem[];
@@ -180,6 +181,7 @@ tile_fwd_kernel(const TileArgs a) {
 template <class PZ, int RY>
 __global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY>::blocks(Tile<PZ, RY>::INV_BYTES))
 tile_inv_kernel(const TileArgs a) {
+    grid_dependency_wait();
     using TL = Tile<PZ, RY>;
     constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
     extern __shared__ __align__(16) float2 smem[];

@@ -11,12 +11,12 @@ namespace gleam {
 // grid_dependency_wait() as its first statement, which holds it until that kernel has completed and
 // its writes are visible, so only the launch latency and the block start-up overlap.
 // grid_launch_dependents() right after the wait lets the next such kernel be scheduled as soon as
-// every block of this one has started; without it the next one is scheduled as the blocks of this one end.  Measured on B200: a gain for launches whose blocks all run
-// at once and end together (cine: 8 % per step); a loss of up to 20 % where the launch before has a
-// long tail (blocks that take a second group of lines), because the early blocks then sit on the
-// SMs next to the tail for tens of microseconds -- so callers allow it for one-round launches, and for the short
-// launches that build the tables of the sampled positions (24 x 80 x 64, 8 coils, A^H y 30 -> 25 us).  The row-tile
-// passes measured up to 27 % slower with it: early blocks fill the SMs unevenly.
+// every block of this one has started; without it the next one is scheduled as the blocks of this one end.  Measured
+// on B200: the early start is a gain between launches whose blocks all run at once and end together (cine: 8 % per
+// step), and in the short launches that build the tables of the sampled positions; elsewhere early blocks fill the SMs
+// unevenly or sit next to a long tail (up to 27 % in the row-tile passes, 20 % in multi-round launches of the row
+// kernels), and those kernels wait without letting the next one in.  Multi-round launches of the one-pass row kernels
+// are not started this way at all: their grid is the number of resident blocks and needs the SMs empty.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -27,15 +27,35 @@ inline bool overlap_enabled() {
     return v == 1;
 }
 
+// cluster > 1: blocks in clusters of that many
+inline void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], bool allow, dim3 grid, dim3 block,
+                                 size_t smem, cudaStream_t s, unsigned cluster) {
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    unsigned n = 0;
+    if (allow && overlap_enabled()) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster; at[n].val.clusterDim.y = 1; at[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = at; cfg.numAttrs = n;
+}
 template <class... KArgs, class... Args>
 inline cudaError_t launch_overlapped(bool allow, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                      cudaStream_t s, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = (allow && overlap_enabled()) ? 1 : 0;
+    cudaLaunchAttribute at[2];
+    launch_config(cfg, at, allow, grid, block, smem, s, 1);
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <class... KArgs, class... Args>
+inline cudaError_t launch_overlapped_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                             cudaStream_t s, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    launch_config(cfg, at, true, grid, block, smem, s, cluster);
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
