@@ -75,7 +75,6 @@ template <class P, bool HAS_Z, bool SMW, bool HAS_ATY, bool ADJ>
 __global__ void __launch_bounds__(SMW ? 512 : 32, SMW ? 1 : WarpFlat<P, HAS_Z, SMW>::SINGLE_BLOCKS)
 warpflat_kernel(const RowArgs a, const int nwhole) {
     grid_dependency_wait();
-    grid_launch_dependents();
     using WF = WarpFlat<P, HAS_Z, SMW>;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL, LW = WF::LW, UPC = WF::UPC, US = WF::USTRIDE, SLOTS = WF::SLOTS;
     constexpr int KCAP = WF::KCAP, KSTRIDE = WF::KSTRIDE, KTILE = WF::KTILE, ZS = WF::ZS, MS = WF::MS;
@@ -103,6 +102,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
 #pragma unroll
     for (int k = 0; k < R0; ++k) tw0[k] = unit_root_fwd<N>((j * k) % N);
     const long long ngroups = (a.nrows + LW - 1) / LW;
+    if (SMW || (long long)gridDim.x >= ngroups) grid_launch_dependents();      // a single round: the next launch may come in
     const int total = UPC * nc, rounds = (total + 31) / 32;
     const long long g_first = !SMW ? (long long)blockIdx.x
                             : split ? (long long)(nwhole + set) * gridDim.x + blockIdx.x : (long long)warp * gridDim.x + blockIdx.x;

@@ -37,7 +37,6 @@ template <class P, int WARPS, bool HAS_Z, bool ADJ>
 __global__ void __launch_bounds__(WARPS * 32)
 warpline_kernel(const RowArgs a) {
     grid_dependency_wait();
-    grid_launch_dependents();
     using WL = WarpLine<P, HAS_Z>;
     constexpr int KCAP = WL::KCAP, KTILE = WL::KTILE, KSTRIDE = WL::KSTRIDE;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL, TPL = WL::TPL, LW = WL::LW, TILE = WL::TILE;
@@ -62,6 +61,7 @@ warpline_kernel(const RowArgs a) {
 
     const long long ngroups = (a.nrows + LW - 1) / LW;
     const long long wstride = (long long)gridDim.x * WARPS;
+    if (wstride >= ngroups) grid_launch_dependents();      // a single round: the next launch may come in
     constexpr bool use_z = HAS_Z;
 
     for (long long g = (long long)blockIdx.x * WARPS + warp; g < ngroups; g += wstride) {

@@ -452,6 +452,7 @@ __global__ void __launch_bounds__(GRAD_THREADS) grad_eta_partial_kernel(const cf
                                                                         const cf* __restrict__ t, long long ne,
                                                                         double* __restrict__ part) {
     // t = x - A^H(Ax - y)  (the step with eta = 1), so A^H(Ax - y) = x - t
+    grid_dependency_wait();
     grid_launch_dependents();
     __shared__ double sh[GRAD_THREADS];
     const long long base = (long long)blockIdx.y * ne;
@@ -490,6 +491,7 @@ __global__ void grad_eta_final_kernel(const double* __restrict__ part, int nbloc
 __global__ void __launch_bounds__(GRAD_THREADS) l1_partial_kernel(const cf* __restrict__ x, const cf* __restrict__ r, cf* __restrict__ grad,
                                                                   long long ne, int B, int x_planar, int g_planar, long long plane,
                                                                   float inv_n, double* __restrict__ part) {
+    grid_dependency_wait();
     grid_launch_dependents();
     __shared__ double sh[GRAD_THREADS];
     double acc = 0.0;
@@ -707,9 +709,8 @@ GLEAM_API int gleam_l1_loss(const void* x, const void* ref, double* loss, void* 
     cudaStream_t s = (cudaStream_t)dims->stream;
     double* part = (double*)dims->workspace;
     CK(prof_mark(GLEAM_K_CG_VEC, s));
-    l1_partial_kernel<<<nblocks, GRAD_THREADS, 0, s>>>((const cf*)x, (const cf*)ref, (cf*)grad, ne, L.B, (layout & GLEAM_X_CHANNELS) ? 1 : 0,
-                                                       (layout & GLEAM_OUT_CHANNELS) ? 1 : 0, ne, (float)(1.0 / (double)n), part);
-    CK(cudaGetLastError());
+    CK(launch_overlapped(true, l1_partial_kernel, dim3((unsigned)nblocks), dim3(GRAD_THREADS), 0, s, (const cf*)x, (const cf*)ref, (cf*)grad, ne, L.B, (layout & GLEAM_X_CHANNELS) ? 1 : 0,
+                                                       (layout & GLEAM_OUT_CHANNELS) ? 1 : 0, ne, (float)(1.0 / (double)n), part));
     CK(prof_mark(GLEAM_K_CG_VEC, s));
     CK(launch_overlapped(true, l1_final_kernel, dim3(1), dim3(32), 0, s, (const double*)part, nblocks, 1.0 / (double)n, loss, (layout & GLEAM_LOSS_FLOAT) ? 1 : 0));
     CK(prof_mark(-1, s));
@@ -751,8 +752,7 @@ GLEAM_API int gleam_dc_grad_eta(const void* grad_out, const void* x, const void*
     cudaStream_t s = (cudaStream_t)dims->stream;
     double* part = (double*)(ws + G.off_part);
     if (prof_mark(GLEAM_K_CG_VEC, s) != cudaSuccess) return GLEAM_ERR_CUDA;
-    grad_eta_partial_kernel<<<dim3((unsigned)G.nblocks, (unsigned)dims->batch), GRAD_THREADS, 0, s>>>((const cf*)grad_out, (const cf*)x, t, G.ne, part);
-    if (cudaGetLastError() != cudaSuccess) return GLEAM_ERR_CUDA;
+    if (launch_overlapped(true, grad_eta_partial_kernel, dim3((unsigned)G.nblocks, (unsigned)dims->batch), dim3(GRAD_THREADS), 0, s, (const cf*)grad_out, (const cf*)x, t, G.ne, part) != cudaSuccess) return GLEAM_ERR_CUDA;
     if (prof_mark(GLEAM_K_CG_VEC, s) != cudaSuccess) return GLEAM_ERR_CUDA;
     if (launch_overlapped(true, grad_eta_final_kernel, dim3((unsigned)dims->batch), dim3(32), 0, s, (const double*)part, G.nblocks, grad_eta) != cudaSuccess) return GLEAM_ERR_CUDA;
     if (prof_mark(-1, s) != cudaSuccess) return GLEAM_ERR_CUDA;

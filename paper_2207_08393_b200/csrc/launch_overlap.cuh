@@ -15,8 +15,7 @@ namespace gleam {
 // on B200: the early start is a gain between launches whose blocks all run at once and end together (cine: 8 % per
 // step), and in the short launches that build the tables of the sampled positions; elsewhere early blocks fill the SMs
 // unevenly or sit next to a long tail (up to 27 % in the row-tile passes, 20 % in multi-round launches of the row
-// kernels), and those kernels wait without letting the next one in.  Multi-round launches of the one-pass row kernels
-// are not started this way at all: their grid is the number of resident blocks and needs the SMs empty.
+// kernels), and those kernels wait without letting the next one in.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -29,7 +28,7 @@ inline bool overlap_enabled() {
 
 // cluster > 1: blocks in clusters of that many
 inline void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], bool allow, dim3 grid, dim3 block,
-                                 size_t smem, cudaStream_t s, unsigned cluster) {
+                               size_t smem, cudaStream_t s, unsigned cluster) {
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
     unsigned n = 0;
     if (allow && overlap_enabled()) {

@@ -102,6 +102,7 @@ __device__ __forceinline__ float4 axpy4(float c, float4 x, float4 y) {
 
 template <bool HAS_Q>
 __global__ void __launch_bounds__(CG_THREADS) cg_init_kernel(const CgArgs a) {
+    grid_dependency_wait();
     const long long base = (long long)blockIdx.y * a.ne2;
     double acc = 0.0;
     for (long long i = (long long)blockIdx.x * CG_THREADS + threadIdx.x; i < a.ne2; i += (long long)gridDim.x * CG_THREADS) {
@@ -118,6 +119,7 @@ __global__ void __launch_bounds__(CG_THREADS) cg_init_kernel(const CgArgs a) {
 }
 
 __global__ void __launch_bounds__(CG_THREADS) cg_dot_kernel(const CgArgs a) {
+    grid_dependency_wait();
     const long long base = (long long)blockIdx.y * a.ne2;
     Sums acc{0.0, 0.0, 0.0};
     for (long long i = (long long)blockIdx.x * CG_THREADS + threadIdx.x; i < a.ne2; i += (long long)gridDim.x * CG_THREADS) {
@@ -274,20 +276,18 @@ static int modl_cg(const void* z, const void* y, const void* sens, const float* 
     if (y) {
         CGRUN(run(nullptr, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ADJOINT));
         CGCK(prof_mark(GLEAM_K_CG_VEC, s));
-        cg_init_kernel<true><<<grid, CG_THREADS, 0, s>>>(a);
+        CGCK(launch_overlapped(true, cg_init_kernel<true>, grid, dim3(CG_THREADS), 0, s, a));
     } else {
         CGCK(prof_mark(GLEAM_K_CG_VEC, s));
-        cg_init_kernel<false><<<grid, CG_THREADS, 0, s>>>(a);
+        CGCK(launch_overlapped(true, cg_init_kernel<false>, grid, dim3(CG_THREADS), 0, s, a));
     }
-    CGCK(cudaGetLastError());
     for (int k = 0; k < n_iter; ++k) {
         a.parity = k & 1;
         CGRUN(run(a.p, nullptr, sens, mask, -1.0f / mu, ws + L.off_q, &dd, RUN_ALL, dot_rows));     // q = H p / mu
         const bool last = k + 1 == n_iter;
         if (!from_rows) {
             CGCK(prof_mark(GLEAM_K_CG_VEC, s));
-            cg_dot_kernel<<<grid, CG_THREADS, 0, s>>>(a);
-            CGCK(cudaGetLastError());
+            CGCK(launch_overlapped(true, cg_dot_kernel, grid, dim3(CG_THREADS), 0, s, a));
         }
         CGCK(prof_mark(GLEAM_K_CG_VEC, s));
         if (from_rows && last) CGCK(launch_overlapped(true, cg_step_kernel<true, true>, grid, dim3(CG_THREADS), 0, s, a));

@@ -55,3 +55,19 @@ def test_coil_split_of_the_row_tiles(oracle, B, C, T, n):
 def test_one_pass_kernel_of_slices(oracle, n2, rows, coils, density):
     d, x, y, sens, mask = problem(2, 1, coils, 1, (1, rows, n2), MASK_READOUT_INVARIANT, seed=n2 + rows, density=density)
     check_all(oracle, d, x, y, sens, mask, 0.9, "n2=%d rows=%d" % (n2, rows))
+
+
+# the same: several coils per warp of a block (24, 32 points), masks of one sample and of all of them, more groups of lines
+# than one round holds
+@pytest.mark.parametrize("B,C,rows,n2,density", [(8, 16, 32, 24, 0.3), (2, 15, 46, 32, 0.02), (1, 7, 10, 32, 1.0), (1, 5, 6, 256, 0.01),
+                                                 (2, 3, 20, 256, 1.0), (8, 2, 640, 368, 0.2)])
+def test_one_pass_kernel_by_the_number_of_lines(oracle, B, C, rows, n2, density):
+    d, x, y, sens, mask = problem(2, B, C, 1, (1, rows, n2), MASK_READOUT_INVARIANT, seed=n2 + C, density=density)
+    check_all(oracle, d, x, y, sens, mask, 0.9, "n2=%d rows=%d coils=%d" % (n2, rows, C))
+
+
+# volumes: no staged samples left over, fewer and more samples per group of middle lines than are staged
+@pytest.mark.parametrize("n,density", [((2, 46, 320), 1.0), ((4, 46, 92), 0.5), ((2, 640, 24), 0.01)])
+def test_samples_of_the_middle_pass(oracle, n, density):
+    d, x, y, sens, mask = problem(3, 1, 3, 1, n, MASK_READOUT_INVARIANT, seed=sum(n), density=density)
+    check_all(oracle, d, x, y, sens, mask, 0.7, "middle pass %s" % (n,))
