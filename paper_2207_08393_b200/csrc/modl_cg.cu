@@ -14,19 +14,24 @@
 // Where the operator is a one-pass 2-D kernel, that kernel also stores Re<p_row, q_row> and <q_row, q_row> of every
 // image row it writes (it holds both in registers at its update step) and cg_dot is not launched.
 //
-// One launch per step: with the search directions conjugate, <r,q> = <p,q>, so
-//     rr' = <r,r> - 2 alpha mu <r,q> + (alpha mu)^2 <q,q> = (alpha mu)^2 <q,q> - rr
-// is known before the new residual exists, and the direction can be updated in the pass that forms it.  Only beta
-// takes this value: alpha is built from the sum <r,r> of the residual itself, so every step minimises along its
-// direction whatever rounding does to beta (which it moves by parts in 1e7 of the old rr).  Bound by launches and
-// L2: 20 frames of 192 x 160, solve and VJP with 10 steps: 664 -> 558 us (40 vector launches -> 22, started while the
+// One launch per step: the norm of the new residual follows from sums that are known before it exists,
+//     rr' = <r,r> - 2 alpha mu <r,q> + (alpha mu)^2 <q,q>,        <r,q> = <p,q> - beta_old <p_old,q>,
+// and the direction is updated in the pass that forms the residual.  <p_old,q> is zero for exactly conjugate directions, but
+// not for steps that were rounded to 32 bits (beta first of all).  H is Hermitian, so it is
+//     <q_old,p> = <q_old,r> + beta_old <q_old,p_old>,
+// and the same identity for the step before, now with the norm that was summed, gives <q_old,r> = (rr_old - (alpha mu)^2
+// <q_old,q_old> - rr) / (2 alpha mu): four scalars of the step before (CgCarry) and no further sum.  Without that term the
+// error of beta grows with the condition number (against 64 bits, 10 steps: 20 frames of 192 x 160 with mu = 1e-3 9.5e-7,
+// with it 1.9e-7, as with a norm that is summed first).  Only beta takes this value: alpha is built from the sum <r,r> of
+// the residual itself, so every step minimises along its direction whatever rounding does to beta.  Bound by launches and
+// L2: 20 frames of 192 x 160, solve and VJP with 10 steps: 664 -> 567 us (40 vector launches -> 22, started while the
 // operator drains).
 //
 // Inner products: every thread accumulates in double precision, a block reduces in a fixed order
 // and stores one partial sum; the kernel that needs the scalar adds the partial sums of its example
 // in a fixed order at its start (every block the same sum).  Producer and consumer are different
 // launches on one stream: no atomics, no fences, no block waits for another one, and the result
-// does not depend on the order in which blocks run.  <r,r> alternates between two partial-sum
+// does not depend on the order in which blocks run.  <r,r> and the carried scalars alternate between two
 // arrays (step parity): cg_step reads one and writes the other.
 #include "dc_entry.h"
 #include "launch_overlap.cuh"
@@ -39,20 +44,28 @@ namespace gleam {
 constexpr int CG_THREADS = 256;
 constexpr int CG_MAX_BLOCKS = 592;          // partial sums per example (4 blocks per SM on 148 SMs)
 
+// What a step leaves for the next one's <p_old,q>: rr - (alpha mu)^2 <q,q>, 1 / (2 alpha mu), beta, <p,q>
+// (alpha mu as the residual took it).
+struct CgCarry { double u, v, beta, pq; };
+
 struct CgArgs {
     const float4* z;         // z (forward) or grad_out (VJP), two complex values per element
     const float4* q;         // A^H y at cg_init, H p / mu afterwards
     float4* r; float4* p; float4* x;
     double* part_rr;         // (2, B, CG_MAX_BLOCKS): <r,r> partial sums of even / odd steps
+    CgCarry* carry;          // (2, B), even / odd steps
     double* part_pq;         // (B, CG_MAX_BLOCKS) twice: <p,q> and <q,q> partial sums written by cg_dot
     const double* dot_rows;  // (B, rows_per_example) twice: Re<p,q> and <q,q> per image row from the operator, or null
     int rows_per_example;
     long long ne2;           // float4 elements per example
     float mu;
+    double inv_mu;
     int parity;              // step k & 1: part_rr[parity] holds <r_k, r_k>
 };
 
-// Sums of three values over the block in a fixed order; the same values in every thread.
+// Sums of three values over the block in a fixed order, in the threads of the first warp.  64-bit arithmetic runs at a
+// fraction of the 32-bit rate, so what is the same for all threads is left to one warp (20 frames of 192 x 160, solve and
+// VJP with 10 steps: 584 -> 567 us).
 struct Sums { double a, b, c; };
 __device__ __forceinline__ Sums block_sums(Sums v) {
     __shared__ Sums warp_sum[CG_THREADS / 32];
@@ -64,8 +77,10 @@ __device__ __forceinline__ Sums block_sums(Sums v) {
     if (lane == 0) warp_sum[warp] = v;
     __syncthreads();
     Sums t{0.0, 0.0, 0.0};
+    if (warp == 0) {
 #pragma unroll
-    for (int w = 0; w < CG_THREADS / 32; ++w) { t.a += warp_sum[w].a; t.b += warp_sum[w].b; t.c += warp_sum[w].c; }
+        for (int w = 0; w < CG_THREADS / 32; ++w) { t.a += warp_sum[w].a; t.b += warp_sum[w].b; t.c += warp_sum[w].c; }
+    }
     return t;
 }
 
@@ -116,6 +131,7 @@ __global__ void __launch_bounds__(CG_THREADS) cg_init_kernel(const CgArgs a) {
     }
     const Sums t = block_sums(Sums{acc, 0.0, 0.0});
     if (threadIdx.x == 0) rr_slot(a, 0)[blockIdx.x] = t.a;
+    if (threadIdx.x == 0 && blockIdx.x == 0) a.carry[blockIdx.y] = CgCarry{0.0, 0.0, 0.0, 0.0};      // p = r
 }
 
 __global__ void __launch_bounds__(CG_THREADS) cg_dot_kernel(const CgArgs a) {
@@ -153,6 +169,8 @@ __global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) 
         }
     };
     fetch();
+    __shared__ double carry[4];              // CgCarry of the step before
+    if (!LAST && threadIdx.x < 4) carry[threadIdx.x] = __ldcg(reinterpret_cast<const double*>(a.carry + (size_t)a.parity * gridDim.y + blockIdx.y) + threadIdx.x);
     Sums s;
     s.a = array_share(rr_slot(a, a.parity), (int)gridDim.x);
     const double* pq = FROM_ROWS ? a.dot_rows + (size_t)blockIdx.y * a.rows_per_example : a.part_pq + (size_t)blockIdx.y * CG_MAX_BLOCKS;
@@ -160,10 +178,23 @@ __global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) 
     s.b = array_share(pq, npq);
     s.c = LAST ? 0.0 : array_share(pq + (size_t)gridDim.y * (FROM_ROWS ? a.rows_per_example : CG_MAX_BLOCKS), npq);
     s = block_sums(s);
-    // an example whose residual is exactly zero stays as it is
-    const double alpha = (s.a > 0.0 && s.b > 0.0) ? s.a / ((double)a.mu * s.b) : 0.0, amu = alpha * (double)a.mu;
-    const double rr_new = amu * amu * s.c - s.a;
-    const float af = (float)alpha, cf_ = (float)-amu, beta = (s.a > 0.0 && rr_new > 0.0) ? (float)(rr_new / s.a) : 0.f;
+    __shared__ float scalars[3];
+    if (threadIdx.x == 0) {
+        // an example whose residual is exactly zero stays as it is; one division on the way to the vectors
+        const bool live = s.a > 0.0 && s.b > 0.0;
+        const double inv = 1.0 / s.b, amu = live ? s.a * inv : 0.0;
+        const float cf_ = (float)-amu;
+        float beta = 0.f;
+        if (!LAST) {
+            const CgCarry c{carry[0], carry[1], carry[2], carry[3]};
+            const double old = c.beta * ((c.u - s.a) * c.v + c.beta * c.pq);        // beta_old <p_old,q>
+            const double ratio = amu * s.c * inv - 1.0 + 2.0 * old * inv;           // rr' / rr
+            if (live && ratio > 0.0) beta = (float)ratio;
+        }
+        scalars[0] = (float)(amu * a.inv_mu); scalars[1] = cf_; scalars[2] = beta;
+    }
+    __syncthreads();
+    const float af = scalars[0], cf_ = scalars[1], beta = scalars[2];
     double acc = 0.0;
     while (i < a.ne2) {
 #pragma unroll
@@ -184,12 +215,16 @@ __global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) 
     if (LAST) return;
     const Sums t = block_sums(Sums{acc, 0.0, 0.0});
     if (threadIdx.x == 0) rr_slot(a, a.parity ^ 1)[blockIdx.x] = t.a;
+    if (threadIdx.x == 0 && blockIdx.x == 0) {
+        const double amu = -(double)cf_;
+        a.carry[(size_t)(a.parity ^ 1) * gridDim.y + blockIdx.y] = CgCarry{s.a - amu * amu * s.c, amu > 0.0 ? 0.5 / amu : 0.0, (double)beta, s.b};
+    }
 }
 
 static inline uint64_t up256(uint64_t v) { return (v + 255) / 256 * 256; }
 
 struct CgLayout {
-    uint64_t dc_bytes, img_bytes, off_q, off_r, off_p, off_rr, off_pq, off_rows, total;
+    uint64_t dc_bytes, img_bytes, off_q, off_r, off_p, off_rr, off_carry, off_pq, off_rows, total;
     long long ne2;
     int B;
 };
@@ -210,6 +245,7 @@ static int cg_layout(const gleam_dims* d, CgLayout* L) {
     L->off_r = off; off = up256(off + L->img_bytes);
     L->off_p = off; off = up256(off + L->img_bytes);
     L->off_rr = off; off = up256(off + 2u * (uint64_t)d->batch * CG_MAX_BLOCKS * sizeof(double));
+    L->off_carry = off; off = up256(off + 2u * (uint64_t)d->batch * sizeof(CgCarry));
     L->off_pq = off; off = up256(off + 2u * (uint64_t)d->batch * CG_MAX_BLOCKS * sizeof(double));
     L->off_rows = off; off = up256(off + 2u * (uint64_t)d->batch * d->frames * d->n[1] * sizeof(double));
     L->total = off;
@@ -261,7 +297,8 @@ static int modl_cg(const void* z, const void* y, const void* sens, const float* 
     a.z = (const float4*)z; a.q = (const float4*)(ws + L.off_q);
     a.r = (float4*)(ws + L.off_r); a.p = (float4*)(ws + L.off_p); a.x = (float4*)out;
     a.part_rr = (double*)(ws + L.off_rr); a.part_pq = (double*)(ws + L.off_pq);
-    a.ne2 = L.ne2; a.mu = mu; a.parity = 0;
+    a.carry = (CgCarry*)(ws + L.off_carry);
+    a.ne2 = L.ne2; a.mu = mu; a.inv_mu = 1.0 / (double)mu; a.parity = 0;
     long long nb = (L.ne2 + (long long)CG_THREADS * 4 - 1) / ((long long)CG_THREADS * 4);
     if (nb < 1) nb = 1;
     if (nb > CG_MAX_BLOCKS) nb = CG_MAX_BLOCKS;

@@ -163,3 +163,46 @@ def test_error_codes():
     g.gleam_modl_cg_forward(z, y, s, m, 0.05, 10, z, d)          # exact alias is allowed
     torch.cuda.synchronize()
 
+
+
+def textbook_steps(z, sens, mask, mu, n_iter, dtype):
+    """Textbook conjugate gradients on the VJP's system in numpy, vectors in ``dtype``, scalars in double; one coil
+    expansion, transforms along the last axis only (a readout-invariant mask).  All iterates."""
+    real = np.float32 if dtype == np.complex64 else np.float64
+    s, m = sens[0].astype(dtype), np.fft.ifftshift(mask[0].astype(real), axes=-1)[:, None, :]
+    inner = lambda a, b: float(np.sum(a.real.astype(np.float64) * b.real + a.imag.astype(np.float64) * b.imag))
+    r = (real(mu) * z[0].astype(dtype)).astype(dtype)
+    x, p, rr, out = np.zeros_like(r), r.copy(), inner(r, r), []
+    for _ in range(n_iter):
+        k = np.fft.fft(s[:, None] * p[None], norm="ortho") * (m * m)[None]
+        q = (p + real(1 / mu) * np.sum(s.conj()[:, None] * np.fft.ifft(k.astype(dtype), norm="ortho").astype(dtype), axis=0)).astype(dtype)
+        alpha = rr / (mu * inner(p, q))
+        x = (x + real(alpha) * p).astype(dtype)
+        r = (r - real(alpha * mu) * q).astype(dtype)
+        rr, last = inner(r, r), rr
+        p = (r + real(rr / last) * p).astype(dtype)
+        out.append(x)
+    return out
+
+
+@pytest.mark.parametrize("kind", [MASK_READOUT_INVARIANT, MASK_FULL])      # sums from the operator's rows / from their own kernel
+def test_step_lengths_of_an_ill_conditioned_system(kind):
+    """mu = 1e-4, condition number about 1e4: an error of beta is amplified by it, so the iterates show whether beta is
+    as good as one from a residual norm that is summed first.  Bound: twice the error, against 64 bits, of textbook steps
+    with vectors in single precision (the rounding of the vectors differs between the two; 7 to 10 times without the
+    conjugacy term)."""
+    rng = np.random.default_rng(1)
+    C, T, n1, n2, mu = 8, 4, 96, 160, float(np.float32(1e-4))
+    u1, u2, a = np.linspace(-1, 1, n1)[:, None], np.linspace(-1, 1, n2)[None, :], 2 * np.pi * np.arange(C)[:, None, None] / C
+    sens = np.exp(-(u1 - np.cos(a)) ** 2 - (u2 - np.sin(a)) ** 2) * np.exp(1j * (a + u1))
+    sens = (sens / np.sqrt(np.sum(np.abs(sens) ** 2, axis=0)))[None, :, None].astype(np.complex64)      # (B, C, n0, n1, n2)
+    mask = (rng.uniform(size=(1, T, n2)) < 0.1).astype(np.float32)
+    z = crandn(rng, 1, T, 1, n1, n2)
+    single = textbook_steps(z[:, :, 0], sens[:, :, 0], mask, mu, 20, np.complex64)
+    double = textbook_steps(z[:, :, 0], sens[:, :, 0], mask, mu, 20, np.complex128)
+    given = mask if kind == MASK_READOUT_INVARIANT else np.ascontiguousarray(np.broadcast_to(mask[:, :, None, None, :], (1, T, 1, n1, n2)))
+    for k in (10, 15, 20):
+        ref = double[k - 1]
+        err = lambda v: np.linalg.norm(v.astype(np.complex128) - ref) / np.linalg.norm(ref)
+        got = run_gpu_modl(z, None, sens, given, mu, k, 2, 0, kind)
+        assert err(got[0, :, 0]) <= 2 * err(single[k - 1]), (k, err(got[0, :, 0]), err(single[k - 1]))
