@@ -371,24 +371,24 @@ def _current_stream_handle() -> int:
 
 
 class CallDims:
-    """The ``gleam_dims`` of one problem shape and workspace, kept per stream: a call on the same stream takes the
-    finished structure instead of filling one (5 us).  A structure is never changed once it is in use, so threads may
-    share the holder; ``get`` starts over when the workspace tensor was replaced."""
+    """The ``gleam_dims`` of one problem shape, kept per stream and workspace memory: a call that finds its structure does
+    not fill one (5 us).  Kept by the address and size of the workspace as they are at the call, from which alone a
+    structure follows: a tensor that was given other storage (``resize_``, ``set_``) gets another one.  A structure is
+    never changed once it is in use, so threads may share the holder."""
 
-    LIMIT = 64                                 # streams remembered; beyond that the table starts over
+    LIMIT = 64                                 # structures remembered; beyond that the table starts over
 
     def __init__(self, *shape):
-        self._shape, self._table = shape, (None, {})
+        self._shape, self._known = shape, {}
 
     def get(self, workspace, stream=None) -> gleam_dims:
         handle = _current_stream_handle() if stream is None else stream if isinstance(stream, int) else stream.cuda_stream
-        owner, known = self._table
-        if owner is not workspace or len(known) > self.LIMIT:
-            known = {}
-            self._table = (workspace, known)
-        d = known.get(handle)
+        key = (handle, workspace.data_ptr(), workspace.nbytes)
+        d = self._known.get(key)
         if d is None:
-            d = known[handle] = make_dims(*self._shape, stream=handle, workspace=workspace)
+            if len(self._known) >= self.LIMIT:
+                self._known = {}
+            d = self._known[key] = make_dims(*self._shape, stream=handle, workspace=key[1], workspace_bytes=key[2])
         return d
 
 
