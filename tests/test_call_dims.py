@@ -1,4 +1,5 @@
 """The structure a call takes follows the workspace's memory and the stream, whatever was kept from earlier calls (CPU)."""
+import pytest
 import torch
 
 from paper_2207_08393_b200 import binding
@@ -39,3 +40,15 @@ def test_another_tensor_and_the_bound():
     for i in range(4 * kept.LIMIT):
         check(kept, a if i % 2 else b, i)
     assert len(kept._known) <= kept.LIMIT
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_current_stream_without_the_undocumented_functions(monkeypatch, missing):
+    class Stream:
+        cuda_stream = 41
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.setattr(torch._C, name, lambda *a: 43, raising=False)
+    assert binding._current_stream_handle() == 43
+    monkeypatch.delattr(torch._C, missing)
+    assert binding._current_stream_handle() == 41
