@@ -696,12 +696,12 @@ GLEAM_API int gleam_l1_loss(const void* x, const void* ref, double* loss, void* 
     if (((uintptr_t)x & 7) || ((uintptr_t)ref & 7) || ((uintptr_t)loss & ((layout & GLEAM_LOSS_FLOAT) ? 3 : 7)) || ((uintptr_t)grad & 7) || ((uintptr_t)dims->workspace & 255)) return GLEAM_ERR_BAD_DIMS;
     const void* ptrs[5] = {x, ref, loss, grad, dims->workspace};
     for (int i = 0; i < 5; ++i) if (ptrs[i] && (rc = check_device_ptr(ptrs[i])) != GLEAM_OK) return rc;
-    const uint64_t img_b = (uint64_t)L.images * L.V * sizeof(cf);
+    const uint64_t img_b = (uint64_t)L.images * L.V * sizeof(cf), loss_b = (layout & GLEAM_LOSS_FLOAT) ? sizeof(float) : sizeof(double);
     if (grad && grad != x && (overlaps(grad, img_b, x, img_b) || overlaps(grad, img_b, ref, img_b))) return GLEAM_ERR_ALIAS;
     if (grad == x && ((layout & GLEAM_X_CHANNELS) != 0) != ((layout & GLEAM_OUT_CHANNELS) != 0)) return GLEAM_ERR_ALIAS;
     if (overlaps(dims->workspace, gleam_l1_loss_workspace_size(), x, img_b) || overlaps(dims->workspace, gleam_l1_loss_workspace_size(), ref, img_b) ||
-        (grad && overlaps(dims->workspace, gleam_l1_loss_workspace_size(), grad, img_b)) || overlaps(loss, 8, x, img_b) ||
-        (grad && overlaps(loss, 8, grad, img_b)))
+        (grad && overlaps(dims->workspace, gleam_l1_loss_workspace_size(), grad, img_b)) || overlaps(loss, loss_b, x, img_b) ||
+        (grad && overlaps(loss, loss_b, grad, img_b)))
         return GLEAM_ERR_ALIAS;
     const long long ne = (long long)L.T * L.V, n = ne * L.B;
     long long nb = (n + GRAD_THREADS * 8 - 1) / (GRAD_THREADS * 8);

@@ -116,3 +116,28 @@ def test_l1_loss_and_gradient_match_oracle(oracle, shape):
         g.gleam_l1_loss(tx, tr, loss, None, dims, layout)              # loss alone
         torch.cuda.synchronize()
         assert abs(float(loss[0]) - ref_loss) <= 1e-6 * ref_loss
+
+
+def test_l1_loss_as_a_float_next_to_the_images():
+    """A float loss is four bytes: it may lie directly before (or behind) an image; a double there overlaps it."""
+    import torch
+    import paper_2207_08393_b200 as g
+    from paper_2207_08393_b200 import binding
+    dev, n, layout = torch.device("cuda:0"), (1, 12, 16), g.GLEAM_X_CHANNELS | g.GLEAM_OUT_CHANNELS
+    size = 2 * 12 * 16
+    buf = torch.randn(2 + 2 * size + 2, dtype=torch.float32, device=dev)       # [., loss, x, grad, loss, .]
+    x, grad = buf[2:2 + size], buf[2 + size:2 + 2 * size]
+    ref = torch.randn(12 * 16, dtype=torch.complex64, device=dev)
+    ws = torch.empty(g.gleam_l1_loss_workspace_size(), dtype=torch.uint8, device=dev)
+    dims = g.make_dims(1, 1, 1, 2, n, stream=torch.cuda.current_stream(), workspace=ws)
+    expect = float((torch.complex(x[:size // 2], x[size // 2:]) - ref).abs().double().mean())
+    for at in (1, 2 + 2 * size):
+        g.gleam_l1_loss(x, ref, buf[at:], grad, dims, layout | binding.GLEAM_LOSS_FLOAT)
+        assert abs(float(buf[at]) - expect) <= 1e-6 * expect
+    for at in (2, 1 + 2 * size):                           # inside x / grad
+        with pytest.raises(g.GleamError) as e:
+            g.gleam_l1_loss(x, ref, buf[at:], grad, dims, layout | binding.GLEAM_LOSS_FLOAT)
+        assert e.value.status == binding.GLEAM_ERR_ALIAS
+    with pytest.raises(g.GleamError) as e:                 # eight bytes in grad's last element
+        g.gleam_l1_loss(x, ref, buf[2 * size:], grad, dims, layout)
+    assert e.value.status == binding.GLEAM_ERR_ALIAS
