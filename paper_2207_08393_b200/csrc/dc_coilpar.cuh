@@ -22,6 +22,8 @@ struct CoilPar {
     static constexpr int OFF_M = LINE, OFF_U = OFF_M + (LINE + 1) / 2, OFF_E = OFF_U + LW * P::BFL;
     static constexpr size_t bytes(int warps, int coils) { return sizeof(cf) * (size_t)(OFF_E + warps * LW * EXL + coils * LINE); }
     static constexpr size_t LIMIT = 200 * 1024;
+    // shared memory of an SM, and what a block takes beyond `bytes`: the kernel's static arrays and the 1 KB reserved
+    static constexpr size_t SM_BYTES = 228 * 1024, BLOCK_BYTES = 1024 + 2 * 64 * sizeof(double) + 192;
 };
 
 template <class P, bool HAS_Z, bool ADJ>

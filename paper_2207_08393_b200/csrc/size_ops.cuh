@@ -184,13 +184,23 @@ template <class P, int RL> using FlatPlan = Plan<P::N, P::N / RL, RL>;
 // the plan of every row kernel that takes z: the ranks of the sampled positions follow its units
 template <class P> using ZPlan = std::conditional_t<FlatRL<P::N>::z != 0, FlatPlan<P, FlatRL<P::N>::z ? FlatRL<P::N>::z : P::RL>, P>;
 
-// Few lines: the coils of a line group side by side (dc_coilpar.cuh) while all warps are resident at once (16 per SM).
+// Few lines: the coils of a line group side by side (dc_coilpar.cuh), as long as that takes no more than 16 warps per SM
+// and so many rounds of resident blocks (shared memory holds one line group per coil, registers 16 warps per SM).
 // Measured per call, numbered or plain kernel -> here: one 64 x 64 slice of 8 coils 12.5 -> 4.3 us (prepared step),
-// 4.7 -> 3.4 us (VJP); 6 x 8 coils of 46 x 240 18.6 -> 7.3 and 11.7 -> 6.2 us; beyond the line 6 x 4 coils of 368 x 80
-// 7.6 -> 11.3 us; with 2 or 3 coils 3.9 -> 4.8 us.  Larger problems first take two to four coils per warp: prepared step
-// of 8 x 16 coils of 128 x 24 24 -> 5.9 us, 4 x 7 coils of 384 x 32 12.7 -> 5.5 us, 6 x 10 coils of 128 x 160 16 -> 11 us;
+// 4.7 -> 3.4 us (VJP); 6 x 8 coils of 46 x 240 18.6 -> 7.3 and 11.7 -> 6.2 us; beyond 16 warps per SM 6 x 4 coils of
+// 368 x 80 7.6 -> 11.3 us; with 2 or 3 coils 3.9 -> 4.8 us.  Larger problems first take several coils per warp: prepared
+// step of 8 x 16 coils of 128 x 24 24 -> 5.9 us, 4 x 7 coils of 384 x 32 12.7 -> 5.5 us, 6 x 10 coils of 128 x 160 16 -> 11 us;
 // not below 8 warps without z (14 x 17 frames of 64 x 128, VJP 11 -> 16 us with 4) and not for last radices beyond 16
 // (16 coils of 320 x 320, 19.5 -> 26 us).  *taken: the call was launched here.
+//
+// Rounds.  A second one costs as much as the first, so it pays only where a coil costs the other kernel much.  Prepared
+// step / VJP, other kernel -> two rounds: 16 x 23 points, 12 coils of 184 x 368 23.2 / 26.6 -> 18.0 / 16.6 us, 9 coils of 240
+// x 368 18.9 / 20.6 -> 18.2 / 16.5; 256 points, 2 x 16 coils of 512 x 256 35.2 -> 31.5, 12 coils of 640 x 256 27.5 -> 22.5; 240
+// points, 14 coils of 320 x 240 24.2 / 18.7 -> 18.1 / 15.2; 160 points, 12 coils of 384 x 160 18.0 / 11.4 -> 11.8 / 9.5.  It does
+// not with 32 lanes or few image-side butterflies, where the numbered kernel is at its best: 7 coils of 320 x 320 11.6 / 7.8
+// -> 15.2 / 12.6, 7 coils of 320 x 512 14.4 / 10.8 -> 19.9 / 16.4, 12 coils of 192 x 640 25.8 / 19.0 -> 24.5 / 23.4; 12 coils of
+// 184 x 184 13.1 / 9.6 -> 14.7 / 12.0, of 192 x 92 8.9 / 7.0 -> 13.1 / 10.6.  With z and last radices up to 16, fewer warps that
+// make it one round come first: 12 coils of 384 x 240 15.8 -> 13.9, of 384 x 160 11.8 -> 9.6.
 template <class P, bool HAS_Z, bool ADJ>
 inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken) {
     using CP = CoilPar<P>;
@@ -198,15 +208,37 @@ inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken)
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
+    constexpr int WARPS = 16;
+    constexpr int ROUNDS = (P::RL == 32 || (P::RL == 23 && P::R0 <= 8)) ? 1 : 2;
     // fewest warps that still pay: each takes several coils then, so that more line groups are resident at once
-    constexpr int LEAST = !HAS_Z ? 8 : P::RL <= 16 ? 4 : 16;
-    int warps = a.C < 16 ? a.C : 16;
+    constexpr int LEAST = !HAS_Z ? 8 : P::RL <= 16 ? 4 : WARPS;
+    int warps = a.C < WARPS ? a.C : WARPS;
     const long long groups = (a.nrows + CP::LW - 1) / CP::LW;
-    while (groups * warps > 16LL * sms && (warps + 1) / 2 >= LEAST) warps = (warps + 1) / 2;
-    const size_t bytes = CP::bytes(warps, a.C);
-    if (a.C < 4 || bytes > CP::LIMIT || groups <= 0 || groups * warps > 16LL * sms) return cudaSuccess;
-    static PerDevice done;
+    while (groups * warps > (long long)WARPS * sms && (warps + 1) / 2 >= LEAST) warps = (warps + 1) / 2;
+    if (a.C < 4 || groups <= 0 || groups * warps > (long long)WARPS * sms) return cudaSuccess;
+    static PerDevice done, by_warps[WARPS + 1];
     if ((e = ensure_smem(coilpar_kernel<P, HAS_Z, ADJ>, CP::LIMIT, done)) != cudaSuccess) return e;
+    long long rounds = 0;
+    auto count_rounds = [&](int w) -> cudaError_t {
+        int slots = 0;                                       // by threads and registers; shared memory depends on the coils
+        if ((e = resident_slots(coilpar_kernel<P, HAS_Z, ADJ>, 32 * w, 0, by_warps[w], &slots)) != cudaSuccess) return e;
+        const long long by_smem = (long long)sms * (CP::SM_BYTES / (CP::bytes(w, a.C) + CP::BLOCK_BYTES));
+        const long long resident = slots < by_smem ? slots : by_smem;
+        rounds = resident > 0 ? (groups + resident - 1) / resident : groups;
+        return cudaSuccess;
+    };
+    if ((e = count_rounds(warps)) != cudaSuccess) return e;
+    if (HAS_Z && P::RL <= 16 && rounds > 1) {
+        const int most = warps;
+        const long long with_most = rounds;
+        while (rounds > 1 && (warps + 1) / 2 >= LEAST) {
+            warps = (warps + 1) / 2;
+            if ((e = count_rounds(warps)) != cudaSuccess) return e;
+        }
+        if (rounds > 1) { warps = most; rounds = with_most; }
+    }
+    const size_t bytes = CP::bytes(warps, a.C);
+    if (bytes > CP::LIMIT || rounds > ROUNDS) return cudaSuccess;
     *taken = true;
     return launch_overlapped(true, coilpar_kernel<P, HAS_Z, ADJ>, dim3((unsigned)groups), dim3(32 * warps), bytes, s, a);
 }

@@ -1,0 +1,80 @@
+"""Which kernels and launch shapes the rules of the dispatch choose, read from the captured launches of a call, and the
+results of the calls whose choice lies next to a line, against the CPU oracle."""
+import pytest
+
+from oracle.oracle import MASK_READOUT_INVARIANT
+from tests.test_gpu_parity import problem
+from tests.test_gpu_tiles import check_all
+
+pytestmark = pytest.mark.gpu
+
+
+def captured(fn):
+    """The kernel launches of fn(), in order: name, blocks, threads, resident blocks on this GPU, and whether the launch
+    may start before the one before it has ended."""
+    import torch
+    from cuda.bindings import driver
+    def ok(r):
+        assert int(r[0]) == 0, r[0]
+        return r[1:] if len(r) > 2 else r[1] if len(r) == 2 else None
+    fn()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        fn()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    count = ok(driver.cuGraphGetNodes(raw))[1]
+    nodes = ok(driver.cuGraphGetNodes(raw, count))[0]
+    edges = ok(driver.cuGraphGetEdges_v2(raw))[3]
+    before, after, data = ok(driver.cuGraphGetEdges_v2(raw, edges))[:3]
+    follows = {int(b): (int(a), int(e.type) == int(driver.CUgraphDependencyType.CU_GRAPH_DEPENDENCY_TYPE_PROGRAMMATIC))
+               for a, b, e in zip(before, after, data)}
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    launches = {}
+    for n in nodes:
+        p = ok(driver.cuGraphKernelNodeGetParams(n))
+        f = p.func if int(p.func) else ok(driver.cuKernelGetFunction(p.kern))
+        per_sm = ok(driver.cuOccupancyMaxActiveBlocksPerMultiprocessor(f, p.blockDimX, p.sharedMemBytes))
+        launches[int(n)] = dict(name=ok(driver.cuFuncGetName(f)).decode(), blocks=p.gridDimX * p.gridDimY, threads=p.blockDimX,
+                                resident=per_sm * sms, early=follows.get(int(n), (0, False))[1])
+    order = [n for n in launches if n not in follows]
+    nexts = {a: b for b, (a, _) in follows.items()}
+    while order[-1] in nexts:
+        order.append(nexts[order[-1]])
+    assert len(order) == len(launches)
+    return [launches[n] for n in order]
+
+
+def holder(shape):
+    import torch
+    import paper_2207_08393_b200 as g
+    B, C, T, n1, n2 = shape
+    n, dev = (1, n1, n2), torch.device("cuda:0")
+    x = torch.zeros((B, T) + n, dtype=torch.complex64, device=dev)
+    y = torch.zeros((B, C, T) + n, dtype=torch.complex64, device=dev)
+    s = torch.zeros((B, C) + n, dtype=torch.complex64, device=dev)
+    m = torch.ones((B, T, n2), dtype=torch.float32, device=dev)
+    return g.DataConsistency(B, C, T, 2, n), x, y, s, m
+
+
+# (batch, coils, frames, n1, n2), rounds that the kernel with the coils side by side may take
+@pytest.mark.parametrize("shape,most", [
+    ((1, 7, 1, 320, 512), 1), ((1, 7, 1, 320, 320), 1), ((1, 6, 1, 320, 384), 1), ((1, 12, 1, 192, 640), 1),
+    ((1, 12, 1, 184, 184), 1), ((1, 12, 1, 192, 92), 1), ((1, 40, 1, 512, 256), 2), ((2, 16, 1, 512, 256), 2),
+    ((1, 12, 1, 184, 368), 2), ((1, 14, 1, 320, 240), 2), ((1, 8, 1, 64, 64), 1)])
+def test_rounds_of_the_coils_side_by_side(shape, most):
+    dc, x, y, s, m = holder(shape)
+    for fn in (lambda: dc.vjp(x, s, m, 1.0), lambda: dc.forward(x, y, s, m, 1.0), lambda: dc.adjoint(y, s, m)):
+        row = captured(fn)[-1]
+        if "coilpar_kernel" in row["name"]:
+            assert -(-row["blocks"] // row["resident"]) <= most, row
+        else:
+            assert shape[3:] != (64, 64), row              # few lines
+
+
+@pytest.mark.parametrize("shape", [(1, 7, 1, 320, 320), (1, 12, 1, 192, 92), (1, 12, 1, 184, 368), (1, 14, 1, 320, 240),
+                                   (1, 12, 1, 384, 160), (1, 40, 1, 160, 256)])
+def test_results_next_to_the_lines(oracle, shape):
+    B, C, T, n1, n2 = shape
+    d, x, y, sens, mask = problem(2, B, C, T, (1, n1, n2), MASK_READOUT_INVARIANT, weighted=(C == 14), seed=n1 + n2, density=0.3)
+    check_all(oracle, d, x, y, sens, mask, 0.9, "%s" % (shape,))
