@@ -351,6 +351,14 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
     float* m2c = (float*)(ws + L.off_m2c);
     int* zstart = (int*)(ws + L.off_zstart);
 
+    const int x_planar = (layout & GLEAM_X_CHANNELS) ? 1 : 0, out_planar = (layout & GLEAM_OUT_CHANNELS) ? 1 : 0;
+    const long long plane = (long long)L.T * L.V;
+    RowArgs ra{};                                    // rank 2, readout-invariant mask: the one-pass launch
+    ra.x = (const cf*)x; ra.sens = (const cf*)sens; ra.out = (cf*)out; ra.eta = eta; ra.mask = mask; ra.z = z;
+    ra.C = L.C; ra.T = L.T; ra.Ts = L.Ts; ra.RPB = L.n1; ra.nrows = L.images * L.n1;
+    ra.x_planar = x_planar; ra.out_planar = out_planar; ra.plane = plane;
+    ra.aty = (const cf*)aty; ra.dot_rows = dot_rows;
+
     if (L.separable && y && mode != RUN_APPLY) {     // RUN_APPLY: the tables of an earlier RUN_PREPARE are in the workspace
         // ranks of the sampled positions (rank 2: the blocks that need them derive them from the mask row), then the
         // z table: inverse transform of y along the readout axis at the sampled positions only
@@ -369,21 +377,14 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
             cz.zlist = zlist; cz.zcount = zcount;
         }
         cz.scale = g / sqrtf((float)(L.rank == 2 ? L.n1 : L.n0) * (float)pe);
-        LAUNCH(GLEAM_K_COL_Z, find_size(L.rank == 2 ? L.n1 : L.n0)->col_z(cz, s));
+        LAUNCH(GLEAM_K_COL_Z, find_size(L.rank == 2 ? L.n1 : L.n0)->col_z(cz, L.rank == 2 ? &ra : nullptr, find_size(L.n2)->row, s));
     }
     if (mode == RUN_PREPARE) {                       // a full mask has nothing to prepare
         if (L.separable) CK(prof_mark(-1, s));
         return GLEAM_OK;
     }
-    const int x_planar = (layout & GLEAM_X_CHANNELS) ? 1 : 0, out_planar = (layout & GLEAM_OUT_CHANNELS) ? 1 : 0;
-    const long long plane = (long long)L.T * L.V;
     if (L.separable && L.rank == 2) {
-        RowArgs ra{};
-        ra.x = (const cf*)x; ra.sens = (const cf*)sens; ra.out = (cf*)out; ra.eta = eta; ra.mask = mask; ra.z = z;
-        ra.C = L.C; ra.T = L.T; ra.Ts = L.Ts; ra.RPB = L.n1; ra.nrows = L.images * L.n1;
-        ra.x_planar = x_planar; ra.out_planar = out_planar; ra.plane = plane;
-        ra.aty = (const cf*)aty; ra.dot_rows = dot_rows;
-        LAUNCH(GLEAM_K_ROW_FUSED, find_size(L.n2)->row(ra, s));
+        LAUNCH(GLEAM_K_ROW_FUSED, find_size(L.n2)->row(ra, s, nullptr));
         CK(prof_mark(-1, s));
         return GLEAM_OK;
     }

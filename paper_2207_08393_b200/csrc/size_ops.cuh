@@ -24,10 +24,13 @@ struct PerDevice {
     }
 };
 
+// Launches the row kernel; with `single` nothing is launched, it tells whether the launch would be one round of blocks.
+typedef cudaError_t (*RowLaunch)(const RowArgs& a, cudaStream_t s, bool* single);
+
 struct SizeOps {
     int N, unit_r0;              // unit_r0: units per line of the row kernels that take z (one plan for all of them)
-    cudaError_t (*row)(const RowArgs& a, cudaStream_t s);
-    cudaError_t (*col_z)(const ColArgs& a, cudaStream_t s);
+    RowLaunch row;
+    cudaError_t (*col_z)(const ColArgs& a, const RowArgs* row, RowLaunch row_launch, cudaStream_t s);
 };
 
 // static_bytes: statically declared shared memory of the kernel, which counts against the same
@@ -73,7 +76,7 @@ inline cudaError_t resident_slots(K kernel, int threads, size_t smem, PerDevice&
 // persistent launch of the warp-resident row kernel: one block per resident slot, warps stride
 // over the line groups
 template <class P, bool HAS_Z, bool ADJ>
-inline cudaError_t launch_warpline_z(const RowArgs& a, cudaStream_t s) {
+inline cudaError_t launch_warpline_z(const RowArgs& a, cudaStream_t s, bool* single) {
     using WL = WarpLine<P, HAS_Z>;
     constexpr int WARPS = 1;
     constexpr size_t SMEM = sizeof(cf) * WARPS * WL::WARP_ELEMS_ALIGNED;
@@ -85,6 +88,7 @@ inline cudaError_t launch_warpline_z(const RowArgs& a, cudaStream_t s) {
     if ((e = resident_slots(warpline_kernel<P, WARPS, HAS_Z, ADJ>, WARPS * 32, SMEM, slots_cache, &slots)) != cudaSuccess) return e;
     const long long groups = (a.nrows + WL::LW - 1) / WL::LW;
     long long blocks = (groups + WARPS - 1) / WARPS;
+    if (single) { *single = blocks <= slots; return cudaSuccess; }
     if (blocks <= 0) return cudaSuccess;
     if (blocks > slots) blocks = slots;
     return launch_overlapped(true, warpline_kernel<P, WARPS, HAS_Z, ADJ>, dim3((unsigned)blocks),
@@ -100,7 +104,7 @@ inline bool split_enabled() {
 
 // the one-pass kernel with the k-space units numbered across the coils (dc_warpflat.cuh)
 template <class P, bool HAS_Z, bool HAS_ATY, bool ADJ>
-inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s) {
+inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* single) {
     static_assert(WarpFlat<P, HAS_Z>::ELIGIBLE, "not a plan the coil-numbered kernel takes");
     using WF = WarpFlat<P, HAS_Z, false>;
     static PerDevice attr_done;
@@ -110,6 +114,7 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s) {
     int slots = 0;
     if ((e = resident_slots(warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ>, 32, WF::WARP_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
     const long long groups = (a.nrows + WF::LW - 1) / WF::LW;
+    if (single) { *single = groups <= slots; return cudaSuccess; }       // one block per SM below is one round, too
     if (groups <= 0) return cudaSuccess;
     // One round of 8 to 16 groups per SM: one block per SM that holds all its warps.  4 k + 1 (or 4 k + 2) groups per
     // SM: the groups beyond 4 k are split by coils over four warps each, one per scheduler.  (Measured on cine-shaped
@@ -138,10 +143,10 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s) {
     return launch_overlapped(true, warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ>, dim3((unsigned)blocks), dim3(32), WF::WARP_BYTES, s, a, 1);
 }
 template <class P, bool HAS_Z>
-inline cudaError_t launch_warpflat_z(const RowArgs& a, cudaStream_t s) {
-    if constexpr (!HAS_Z) { if (a.aty != nullptr) return launch_warpflat_zy<P, false, true, false>(a, s); }
-    else { if (a.x == nullptr) return launch_warpflat_zy<P, true, false, true>(a, s); }
-    return launch_warpflat_zy<P, HAS_Z, false, false>(a, s);
+inline cudaError_t launch_warpflat_z(const RowArgs& a, cudaStream_t s, bool* single) {
+    if constexpr (!HAS_Z) { if (a.aty != nullptr) return launch_warpflat_zy<P, false, true, false>(a, s, single); }
+    else { if (a.x == nullptr) return launch_warpflat_zy<P, true, false, true>(a, s, single); }
+    return launch_warpflat_zy<P, HAS_Z, false, false>(a, s, single);
 }
 // GLEAM_NO_FLAT=1 keeps the plain warp-resident kernel for those lengths (tuning aid, read once).
 inline bool flat_enabled() {
@@ -202,7 +207,7 @@ template <class P> using ZPlan = std::conditional_t<FlatRL<P::N>::z != 0, FlatPl
 // 184 x 184 13.1 / 9.6 -> 14.7 / 12.0, of 192 x 92 8.9 / 7.0 -> 13.1 / 10.6.  With z and last radices up to 16, fewer warps that
 // make it one round come first: 12 coils of 384 x 240 15.8 -> 13.9, of 384 x 160 11.8 -> 9.6.
 template <class P, bool HAS_Z, bool ADJ>
-inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken) {
+inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken, bool* single) {
     using CP = CoilPar<P>;
     *taken = false;
     int sms = 0;
@@ -240,25 +245,27 @@ inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken)
     const size_t bytes = CP::bytes(warps, a.C);
     if (bytes > CP::LIMIT || rounds > ROUNDS) return cudaSuccess;
     *taken = true;
+    if (single) { *single = rounds <= 1; return cudaSuccess; }
     return launch_overlapped(true, coilpar_kernel<P, HAS_Z, ADJ>, dim3((unsigned)groups), dim3(32 * warps), bytes, s, a);
 }
 
 template <class P>
-inline cudaError_t launch_warpline(const RowArgs& a, cudaStream_t s) {
+inline cudaError_t launch_warpline(const RowArgs& a, cudaStream_t s, bool* single) {
     bool taken = false;
-    const cudaError_t e = a.z == nullptr ? launch_coilpar<ZPlan<P>, false, false>(a, s, &taken)
-                        : a.x != nullptr ? launch_coilpar<ZPlan<P>, true, false>(a, s, &taken) : launch_coilpar<ZPlan<P>, true, true>(a, s, &taken);
+    const cudaError_t e = a.z == nullptr ? launch_coilpar<ZPlan<P>, false, false>(a, s, &taken, single)
+                        : a.x != nullptr ? launch_coilpar<ZPlan<P>, true, false>(a, s, &taken, single) : launch_coilpar<ZPlan<P>, true, true>(a, s, &taken, single);
     if (taken || e != cudaSuccess) return e;
     // the numbering across coils pays once a round of 32 units spans more than one coil
     const bool flat = flat_enabled() && a.C >= 2;
-    if constexpr (FlatRL<P::N>::v != 0) if (flat && a.z == nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::v>, false>(a, s);
-    if constexpr (FlatRL<P::N>::z != 0) if (flat && a.z != nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::z>, true>(a, s);
-    if (a.z == nullptr) return launch_warpline_z<P, false, false>(a, s);
-    return a.x != nullptr ? launch_warpline_z<ZPlan<P>, true, false>(a, s) : launch_warpline_z<ZPlan<P>, true, true>(a, s);
+    if constexpr (FlatRL<P::N>::v != 0) if (flat && a.z == nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::v>, false>(a, s, single);
+    if constexpr (FlatRL<P::N>::z != 0) if (flat && a.z != nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::z>, true>(a, s, single);
+    if (a.z == nullptr) return launch_warpline_z<P, false, false>(a, s, single);
+    return a.x != nullptr ? launch_warpline_z<ZPlan<P>, true, false>(a, s, single) : launch_warpline_z<ZPlan<P>, true, true>(a, s, single);
 }
 
+// row, row_launch: the row launch of such a call (2-D problems), or null
 template <class P, int L>
-inline cudaError_t launch_col_z(const ColArgs& a, cudaStream_t s) {
+inline cudaError_t launch_col_z(const ColArgs& a, const RowArgs* row, RowLaunch row_launch, cudaStream_t s) {
     using E = LineFFT<P, L>;
     using CZ = ColZ<P, L>;
     static PerDevice attr_done, slots_cache;
@@ -274,21 +281,29 @@ inline cudaError_t launch_col_z(const ColArgs& a, cudaStream_t s) {
     b.bpi = (int)(bpi < 1 ? 1 : bpi > most ? most : bpi);
     const long long blocks = (long long)a.images * b.bpi;
     if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-    // Scheduled as the launch before it ends, except behind a row launch of one round, which lets the next launch in at
-    // its start: early blocks of the table then crowd the SMs that had room (2 x 12 coils of 384 x 320, forward 29.5
-    // against 31.8 us; 20 frames x 8 of 192 x 160, 30.6 against 32.4).  Such a round holds some 16 warps per SM of about
-    // 320 points each; larger calls gain (4 x 15 of 640 x 368: 130 -> 123.5 us), and so do grids of a few blocks.
-    int sms = 0;
-    if ((e = device_sms(&sms)) != cudaSuccess) return e;
-    const bool overlap = a.zlist != nullptr || blocks <= 64 || (long long)a.images * a.es * a.n2 > 16LL * 320 * sms;
+    // Scheduled as the launch before it ends, except where that may be a row launch of one round, which lets the next
+    // launch in at its start (asked of the row launch of such a call, with and without z): early blocks of the table then
+    // crowd the SMs that had room.  Forward and VJP in turn, without -> with the attribute: one round, 2 x 16 coils of 640 x
+    // 320 91 -> 116 us, 4 x 8 of 384 x 384 66 -> 85, 3 x 15 of 640 x 368 (the VJP alone is one round) 162 -> 169, 20 frames x
+    // 8 of 192 x 160 54 -> 62; several rounds, 24 frames 71.9 -> 69.8, 4 x 15 of 640 x 368 226.5 -> 224.0, 4 x 8 coils x 8 frames
+    // of 128 x 92 52.1 -> 50.2 (a launch's latency, hidden; enqueued call by call, equal in a replayed graph).  Grids of a few
+    // blocks gain, too.
+    bool overlap = true;
+    if (row != nullptr && blocks > 64) {
+        RowArgs plain = *row;
+        plain.z = nullptr; plain.aty = nullptr;
+        bool with_z = false, without = false;
+        if ((e = row_launch(*row, s, &with_z)) != cudaSuccess || (e = row_launch(plain, s, &without)) != cudaSuccess) return e;
+        overlap = !with_z && !without;
+    }
     return launch_overlapped(overlap, col_z_kernel<P, L>, dim3((unsigned)blocks), dim3(E::THREADS), CZ::SMEM_BYTES, s, b);
 }
 
 template <class P, class PC, int LC>
 struct SizeImpl {
     static_assert(WarpLine<P>::ELIGIBLE, "row plans have at most two stages of at most 32 butterflies");
-    static cudaError_t row(const RowArgs& a, cudaStream_t s) { return launch_warpline<P>(a, s); }
-    static cudaError_t col_z(const ColArgs& a, cudaStream_t s) { return launch_col_z<PC, LC>(a, s); }
+    static cudaError_t row(const RowArgs& a, cudaStream_t s, bool* single) { return launch_warpline<P>(a, s, single); }
+    static cudaError_t col_z(const ColArgs& a, const RowArgs* row, RowLaunch row_launch, cudaStream_t s) { return launch_col_z<PC, LC>(a, row, row_launch, s); }
 };
 
 }  // namespace gleam
