@@ -146,19 +146,30 @@ constexpr int COLZ_SELF_MAX = 1024;   // COL_Z ranks a mask row of at most this 
 // --------------------------------------------------------------------------------------------
 // z table: tiles of L sampled phase-encode positions of one unit, inverse transform along the readout axis:
 //     z[r] = (g/sqrt(N_ro N_pe)) (-1)^{n_ro} (-1)^{p} M[p] * Rraw^H( (-1)^{k_ro} y[.., p] ),  p = source of rank r
-// Gathers 8-byte samples; bound by the DRAM sectors they touch (four columns each).  A block walks over tiles of one
-// image and has the next one on its way to shared memory (8-byte cp.async) while it transforms the current one: with a
-// block per tile, loads, transform and stores of a 640-point tile took turns on an SM (4 x 15 coils of 640 x 368 at 7x
-// 46 -> 38 us, 2 x 12 coils of 384 x 320 at 4x 25 -> 15 us, 20 frames of 192 x 160 17 -> 13 us).
-// Two buffers take turns as "incoming tile" and "current tile"; once every thread holds its elements of the current one,
-// its buffer takes the (last) exchange of the transform.  Three-stage plans have a third for their first exchange.
+// Gathers 8-byte samples; bound by the DRAM sectors and pages they touch and by the requests in flight.  A block walks over
+// tiles of one image; a sample goes straight to the register of the butterfly that takes it, and other blocks fill the time
+// a tile waits.  Butterflies of 20 and 23 points leave one to three blocks per SM, so there the next tile is on its way to
+// shared memory (8-byte cp.async) while the current one is transformed; elsewhere that costs more than it gives.  Cold L2, us,
+// staged -> direct: 256 x 256 x 160 at 7x, 6 coils 108 -> 98, 240 x 320 x 184 182 -> 162, 64 x 240 x 184 45 -> 41, 8 x 16 coils of
+// 640 x 320 at 4x 90 -> 80, 4 x 8 coils x 4 of 256 x 256 39 -> 31; but 8 x 16 coils of 320 x 320 43 -> 45, 46 x 184 x 160 31 -> 39,
+// 184 x 240 x 184 at 3x 211 -> 242, 368 x 320 x 320 at 3x 287 -> 326.
+// Staged, two buffers take turns as "incoming tile" and "current tile"; once every thread holds its elements of the
+// current one, its buffer takes the exchange of the transform.
 // --------------------------------------------------------------------------------------------
 template <class P, int L>
 struct ColZ {
     using E = LineFFT<P, L>;
-    static constexpr int BUFSZ = L * cmax(P::BUF, P::N);
-    static constexpr size_t SMEM_BYTES = sizeof(cf) * (P::S == 3 ? 3 : 2) * BUFSZ;
-    static_assert(E::THREADS % L == 0, "a thread copies one line's samples");
+    static constexpr bool STAGED = P::S == 2 && P::RL >= 20;
+    static constexpr int BUFSZ = L * (STAGED ? cmax(P::BUF, P::N) : P::BUF);
+    static constexpr size_t SMEM_BYTES = sizeof(cf) * (STAGED ? 2 : P::S == 3 ? 2 : 1) * BUFSZ;
+    static_assert(E::THREADS % L == 0, "a thread has one line in every stage");
+    static_assert(!STAGED || P::S == 2, "the exchange takes the current tile's buffer");
+    // Volumes: candidate tiles (of which the sampled ones have work) per block, 0 for one round of blocks that share all
+    // tiles.  Blocks are dealt out in order, which keeps the tiles in work next to each other in y; those of a single round
+    // drift apart.  Cold L2, one round -> 8 tiles per block: 320 x 320 x 256 at 12x 249 -> 234 us, at 7x 314 -> 295, but at 3.5x,
+    // where a DRAM page holds more of a tile, 354 -> 376; 240 x 320 x 184 (direct) 166 -> 154.  23-point plans do not gain
+    // (184 x 240 x 184 at 5x 162 -> 174).  Slices rank their mask row in every block and stay with one round.
+    static constexpr int TILES = P::RL == 23 ? 0 : 8;
 };
 
 template <class P, int L>
@@ -171,6 +182,7 @@ col_z_kernel(const ColArgs a) {
     if (gridDim.x <= 64) grid_launch_dependents();
     using E = LineFFT<P, L>;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL, BUFSZ = ColZ<P, L>::BUFSZ;
+    constexpr bool STAGED = ColZ<P, L>::STAGED;
     extern __shared__ __align__(16) float2 smem[];
     const int tid = threadIdx.x;
     const int bt = blockIdx.x / a.bpi, t = bt % a.T, b = bt / a.T;
@@ -219,6 +231,7 @@ col_z_kernel(const ColArgs a) {
             const cf* src = a.y + (unit_of(item) * N + tid / L) * pe + source_of(i);
             for (int n = tid / L; n < N; n += E::THREADS / L) { cp_async8(dst + n * L + l, src); src += (E::THREADS / L) * pe; }
         }
+        cp_async_commit();
     };
 
     int item = blockIdx.x % a.bpi;
@@ -226,35 +239,35 @@ col_z_kernel(const ColArgs a) {
     const typename E::Ids d = E::ids(tid);
     typename E::Tw tw;
     E::make_tw(d, tw);
-    issue(item, smem);
-    cp_async_commit();
+    if (STAGED) issue(item, smem);
     for (int it = 0; item < items; item += a.bpi, ++it) {
-        cf* cur = smem + (it % 2) * BUFSZ;
-        cf* nxt = smem + ((it + 1) % 2) * BUFSZ;
-        cf* spare = smem + (P::S == 3 ? 2 : 0) * BUFSZ;
-        cp_async_wait<0>();
-        __syncthreads();               // the tile is visible to all; every thread has left the one before
-        if (item + a.bpi < items) issue(item + a.bpi, nxt);
-        cp_async_commit();
+        cf* cur = smem + (STAGED ? (it % 2) * BUFSZ : 0);
+        if (STAGED) {
+            cp_async_wait<0>();
+            __syncthreads();           // the tile is visible to all; every thread has left the one before
+            if (item + a.bpi < items) issue(item + a.bpi, smem + ((it + 1) % 2) * BUFSZ);
+        }
         const int i = (item % ntiles) * L + l;
         const bool ok = i < cnt;
-        int psign = 0; float mv = 0.f;
+        int p = 0, psign = 0; float mv = 0.f;
         if (ok) {
-            const int p = source_of(i);
+            p = source_of(i);
             mv = mk[p];
             psign = (a.rank == 2) ? (p & 1) : ((p / a.n2 + p % a.n2) & 1);
         }
         cf v[R0], u[RL];
         if (d.aL) {
             const float odd = (d.jL & 1) ? -1.f : 1.f;
+            const cf* src = a.y + (unit_of(item) * N + d.jL) * pe + p;
 #pragma unroll
             for (int k = 0; k < RL; ++k) {
-                const cf yv = ok ? cur[(d.jL + P::BFL * k) * L + l] : make_float2(0.f, 0.f);
+                const cf yv = !ok ? make_float2(0.f, 0.f) : STAGED ? cur[(d.jL + P::BFL * k) * L + l] : __ldg(src);
                 u[k] = cscale(yv, (P::BFL * k) % 2 ? -odd : odd);
+                src += P::BFL * pe;
             }
         }
-        if (P::S == 2) __syncthreads();
-        E::inverse(u, v, tw, d, spare, cur);
+        if (P::S == 2) __syncthreads();        // the exchange buffer is free
+        E::inverse(u, v, tw, d, smem + BUFSZ, cur);
         if (d.a0 && ok) {
             const float f = ((psign + d.j0) & 1) ? -a.scale * mv : a.scale * mv;
             cf* dst = a.z + (unit_of(item) * N + d.j0) * pe + i;

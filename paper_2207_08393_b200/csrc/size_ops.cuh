@@ -274,10 +274,12 @@ inline cudaError_t launch_col_z(const ColArgs& a, const RowArgs* row, RowLaunch 
     int slots = 0;
     if ((e = resident_slots(col_z_kernel<P, L>, E::THREADS, CZ::SMEM_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
     if (a.images <= 0) return cudaSuccess;
-    // the number of sampled ranks is known only on the device: one round of blocks, which share an image's tiles
+    // The number of sampled ranks is known only on the device.  The blocks of an image share its tiles: one round of
+    // blocks, more for volumes (ColZ::TILES).
     ColArgs b = a;
     const long long most = (long long)a.C * ((a.es + L - 1) / L);
     long long bpi = slots / a.images;
+    if (a.rank == 3 && CZ::TILES > 0 && bpi < most / cmax(CZ::TILES, 1)) bpi = most / cmax(CZ::TILES, 1);
     b.bpi = (int)(bpi < 1 ? 1 : bpi > most ? most : bpi);
     const long long blocks = (long long)a.images * b.bpi;
     if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;

@@ -96,3 +96,13 @@ def test_early_start_of_the_z_table(shape, early):
     tables = [i for i, k in enumerate(launches) if "col_z_kernel" in k["name"]]
     assert len(tables) == 2 and len(launches) == 5
     assert launches[tables[1]]["early"] == early, launches[tables[1]]
+
+
+# z table: more sampled tiles than blocks (a block walks over several, also with the last tile part full) and fewer, one-, two-
+# and three-stage readouts, staged and direct tiles
+@pytest.mark.parametrize("rank,coils,n,density", [
+    (3, 4, (4, 256, 160), 0.9), (3, 9, (16, 184, 184), 0.95), (3, 3, (46, 96, 120), 0.97), (3, 2, (64, 46, 24), 0.03), (3, 8, (368, 10, 46), 0.5),
+    (2, 40, (1, 640, 96), 1.0), (2, 40, (1, 184, 160), 0.9), (2, 3, (1, 320, 368), 0.9), (2, 24, (1, 16, 512), 0.8)])
+def test_z_table_tiles_and_blocks(oracle, rank, coils, n, density):
+    d, x, y, sens, mask = problem(rank, 1, coils, 1, n, MASK_READOUT_INVARIANT, weighted=(coils % 2 == 1), seed=sum(n), density=density)
+    check_all(oracle, d, x, y, sens, mask, 0.8, "z table %s" % (n,))
