@@ -7,7 +7,7 @@
 //   P1(s, j)   rows ky = j + BY m of every coil: S_c x, radix-RY transform across the rows, kz
 //              transform of each result row, store  W[slot][c][k0][j][kz]
 //   P2(s, k0)  the BY contiguous rows of (c, k0): twiddle w_N1^(j k0), radix-BY transform over j,
-//              mask^2 / (N1 NZ) (and - z in the forward call), inverse, conjugate twiddle, in place
+//              mask^2 / (N1 NZ), inverse, conjugate twiddle, in place
 //   P3(s, j)   mirror of P1: kz inverse, inverse radix-RY, conj(S_c) coil sum, out = x - eta sum
 // P2(s,.) needs all P1(s,.), P3(s,.) needs all P2(s,.); W is a ring of R slabs, so P1(s,.) also
 // needs all P3(s-R,.).  Items are drawn from one global counter in the order
@@ -38,8 +38,6 @@ struct FusedArgs {
     const cf* x; const cf* sens; cf* out;     // image side
     cf* W;                                    // ring (R, C, RY, BY, NZ)
     const float* mask;                        // (B,T,N1,NZ)
-    const cf* zin; const int* zidx;           // forward call: compact z table, rank map
-    const float* m2c; const int* zstart;      //               squared weights by rank, first rank of each ky-mod-RY group
     int* ctrl;                                // [0] next item, [1] error word; per-slab counters from ctrl + 64
     float eta, scale2;
     int C, T, Ts, n0;
@@ -131,7 +129,7 @@ struct Shared {                      // control block behind the tiles
 
 }  // namespace fused
 
-template <int BY, bool HAS_Z>
+template <int BY>
 __global__ void __launch_bounds__(fused::THREADS, 1)
 fused3d_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap tm_sens, const __grid_constant__ CUtensorMap tm_x,
                const __grid_constant__ CUtensorMap tm_ring, const __grid_constant__ CUtensorMap tm_mask) {

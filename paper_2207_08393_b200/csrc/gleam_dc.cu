@@ -150,10 +150,9 @@ static void fused_ring(int* R, int* L2, int* L3) {
     }
     *R = v[0]; *L2 = v[1]; *L3 = v[2];
 }
-// The persistent kernel is opt-in: measured on the 320 x 320 x 256 volume it only draws level with the three
-// whole-volume passes (1.81 ms against 1.77-1.93 ms per VJP call), so the default keeps those.  GLEAM_FUSED=1 in the environment
-// or gleam_dc_set_fused(1) selects it; the choice changes the workspace layout, so it is made before
-// gleam_dc_workspace_size.
+// The persistent kernel is opt-in: on the 320 x 320 x 256 volume a VJP call takes 1.81 ms with it and 1.79 ms with the three
+// whole-volume passes, so the default keeps those.  GLEAM_FUSED=1 in the environment or gleam_dc_set_fused(1) selects it;
+// the choice changes the workspace layout, so it is made before gleam_dc_workspace_size.
 static std::atomic<int> g_fused_on{-1};
 static bool fused_enabled() {
     int v = g_fused_on.load(std::memory_order_relaxed);
@@ -161,9 +160,9 @@ static bool fused_enabled() {
     return v == 1;
 }
 
-// Target size of the 3-D chunk workspace.  A chunk of about 48 MB would stay inside L2 between the
-// three kernels of a chunk, but at their present speed the kernels are bound by instruction issue,
-// not by bandwidth, and fewer, larger launches measure faster; the default therefore covers the
+// Target size of the 3-D chunk workspace.  A chunk of about 48 MB would stay inside L2 between the three passes, but the
+// launches of such a chunk are too short to fill the GPU: large launches stream at 0.84 to 0.90 of copy bandwidth, and
+// chunks sized for L2 measured slower (VJP of 320 x 320 x 256 1790 -> 2026 us and more).  The default therefore covers the
 // whole volume up to 2 GB.  GLEAM_CHUNK_MB overrides it (tuning aid, read once).
 static uint64_t chunk_target_bytes() {
     static uint64_t v = 0;

@@ -53,18 +53,13 @@ static cudaError_t launch_fused(const FusedArgs& a, cudaStream_t s) {
     if ((me = make_map(&tm_mask, a.mask, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, NZ, RY, BY, images, NZ, RY * NZ, N1 * NZ, NZ, BY)) != cudaSuccess) return me;
     static PerDevice attr_done, sm_cache;
     cudaError_t e;
-    if (a.zin) {
-        if ((e = ensure_smem(fused3d_kernel<BY, true>, fused::SMEM_BYTES, attr_done)) != cudaSuccess) return e;
-    }
-    static PerDevice attr_done_v;
-    if ((e = ensure_smem(fused3d_kernel<BY, false>, fused::SMEM_BYTES, attr_done_v)) != cudaSuccess) return e;
+    if ((e = ensure_smem(fused3d_kernel<BY>, fused::SMEM_BYTES, attr_done)) != cudaSuccess) return e;
     int blocks = 0;
-    if ((e = resident_slots(fused3d_kernel<BY, false>, fused::THREADS, fused::SMEM_BYTES, sm_cache, &blocks)) != cudaSuccess) return e;
+    if ((e = resident_slots(fused3d_kernel<BY>, fused::THREADS, fused::SMEM_BYTES, sm_cache, &blocks)) != cudaSuccess) return e;
     const long long items = (long long)(a.nslabs + a.L3) * (2 * BY + fused::RY);
     if (blocks > items) blocks = (int)items;
     if (blocks < 1) return cudaSuccess;
-    if (a.zin) fused3d_kernel<BY, true><<<blocks, fused::THREADS, fused::SMEM_BYTES, s>>>(a, tm_sens, tm_x, tm_ring, tm_mask);
-    else fused3d_kernel<BY, false><<<blocks, fused::THREADS, fused::SMEM_BYTES, s>>>(a, tm_sens, tm_x, tm_ring, tm_mask);
+    fused3d_kernel<BY><<<blocks, fused::THREADS, fused::SMEM_BYTES, s>>>(a, tm_sens, tm_x, tm_ring, tm_mask);
     return cudaGetLastError();
 }
 
