@@ -31,7 +31,12 @@ struct Axis {
     static constexpr size_t BYTES = sizeof(cf) * (X_ELEMS + (P::S == 2 ? N : 0));
     static constexpr size_t Y_BYTES = sizeof(cf) * P::RL * THREADS;
     static constexpr int REGS = (2 * cmax(P::R0, P::RL) + P::RL + 32 + 7) / 8 * 8;
-    static constexpr int BLOCKS = cmax(1, cmin(cmin(16, 2048 / THREADS), 65536 / (THREADS * REGS)));
+    // Blocks that the register bound keeps resident.  Butterflies of 15 and 16 points get two blocks of 256 threads and 128
+    // registers: with three (80 registers) weights and addresses are spilled and fewer loads are in flight (forward / VJP, us a
+    // pass: 256 x 256 x 160, 8 coils 799 / 503 -> 466 / 388, 240 x 96 x 96 150 / 115 -> 114 / 98, 192 x 96 x 128 145 / 119 -> 127 /
+    // 107, 160 x 160 x 128, 6 coils 160 / 125 -> 142 / 114).  Smaller ones want the blocks (with one fewer 96 x 160 x 128 82 / 70
+    // -> 111 / 97, 64 x 160 x 128 39 / 33 -> 43 / 35); a 640-point block of 512 threads has 128 registers at most and spills 148 B.
+    static constexpr int BLOCKS = cmax(1, cmin(cmin(cmax(P::R0, P::RL) > 12 ? 2 : 16, 2048 / THREADS), 65536 / (THREADS * REGS)));
 };
 
 template <class P, int KC, int MODE>

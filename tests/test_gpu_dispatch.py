@@ -10,7 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 def captured(fn):
-    """The kernel launches of fn(), in order: name, blocks, threads, resident blocks on this GPU, and whether the launch
+    """The kernel launches of fn(), in order: name, blocks, threads, resident blocks on this GPU, bytes of local memory (spilled
+    registers), and whether the launch
     may start before the one before it has ended (from the third edge on: the binding gives its buffer of edge data back
     before it is read, and the allocator writes over the first two entries)."""
     import torch
@@ -37,7 +38,8 @@ def captured(fn):
         f = p.func if int(p.func) else ok(driver.cuKernelGetFunction(p.kern))
         per_sm = ok(driver.cuOccupancyMaxActiveBlocksPerMultiprocessor(f, p.blockDimX, p.sharedMemBytes))
         launches[int(n)] = dict(name=ok(driver.cuFuncGetName(f)).decode(), blocks=p.gridDimX * p.gridDimY, threads=p.blockDimX,
-                                resident=per_sm * sms, early=follows.get(int(n), (0, False))[1])
+                                resident=per_sm * sms, spilled=ok(driver.cuFuncGetAttribute(driver.CUfunction_attribute.CU_FUNC_ATTRIBUTE_LOCAL_SIZE_BYTES, f)),
+                                early=follows.get(int(n), (0, False))[1])
     order = [n for n in launches if n not in follows]
     nexts = {a: b for b, (a, _) in follows.items()}
     while order[-1] in nexts:
@@ -106,3 +108,18 @@ def test_early_start_of_the_z_table(shape, early):
 def test_z_table_tiles_and_blocks(oracle, rank, coils, n, density):
     d, x, y, sens, mask = problem(rank, 1, coils, 1, n, MASK_READOUT_INVARIANT, weighted=(coils % 2 == 1), seed=sum(n), density=density)
     check_all(oracle, d, x, y, sens, mask, 0.8, "z table %s" % (n,))
+
+
+@pytest.mark.parametrize("n0", [48, 64, 128, 160, 184, 192, 240, 256])
+def test_readout_pass_keeps_its_columns_in_registers(n0):
+    import torch
+    import paper_2207_08393_b200 as g
+    n, dev = (n0, 4, 24), torch.device("cuda:0")
+    x = torch.zeros((1, 1) + n, dtype=torch.complex64, device=dev)
+    y = torch.zeros((1, 2, 1) + n, dtype=torch.complex64, device=dev)
+    s = torch.zeros((1, 2) + n, dtype=torch.complex64, device=dev)
+    m = torch.ones((1, 1) + n, dtype=torch.float32, device=dev)
+    dc = g.DataConsistency(1, 2, 1, 3, n, 0, g.GLEAM_MASK_FULL)
+    for fn in (lambda: dc.forward(x, y, s, m, 1.0), lambda: dc.vjp(x, s, m, 1.0), lambda: dc.adjoint(y, s, m)):
+        passes = [k for k in captured(fn) if "axis_kernel" in k["name"]]
+        assert len(passes) == 1 and passes[0]["spilled"] == 0, passes
