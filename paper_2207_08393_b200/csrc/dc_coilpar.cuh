@@ -26,6 +26,8 @@ struct CoilPar {
     static constexpr size_t SM_BYTES = 228 * 1024, BLOCK_BYTES = 1024 + 2 * 64 * sizeof(double) + 192;
 };
 
+// Sixteen warps have 128 registers each: butterflies of 32 points beside 16 or 20 spill 170 to 320 B (512 and 640 points, 172 B
+// and 324 B without z), one reason why those lengths come here for a single round only.
 template <class P, bool HAS_Z, bool ADJ>
 __global__ void __launch_bounds__(512)
 coilpar_kernel(const RowArgs a) {

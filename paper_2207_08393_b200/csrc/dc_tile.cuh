@@ -50,6 +50,7 @@ struct Tile {
     static constexpr size_t INV_BYTES = sizeof(cf) * (T_ELEMS + (ONE_STAGE ? 1 : 2) * STAGE + TW);
     // The register bound lets the blocks that shared memory admits be resident.  RY values of the image or of the coil
     // sum are kept over the coil loop next to a butterfly (a prime radix also holds its sums and differences).
+    // A block has a thread per column, so 640-point rows have at most 96 registers and spill up to 180 B whatever the bound.
     static constexpr bool PRIME = RMAX > 4 && RMAX % 2 == 1 && smallest_odd_factor(RMAX) == RMAX;
     static constexpr int REGS = 2 * RY + (PRIME ? 4 : 2) * RMAX + 16;
     static constexpr int blocks(size_t bytes) {

@@ -71,6 +71,8 @@ struct WarpFlat {
 // with z).  A template parameter, not a run-time test of a.aty: with the test in the code the plain call measured
 // 11 % slower (17.7 against 16.0 us), although it never takes that branch.
 // ADJ (with z): A^H y, the image is zero; the forward stages are left out and a unit starts from minus its z values.
+// Registers: sixteen warps of one block have 128 each, which the step with z of 160 points exceeds by 52 B (spilled to
+// local memory; single-warp blocks without the spill are slower all the same, see launch_warpflat_zy).
 template <class P, bool HAS_Z, bool SMW, bool HAS_ATY, bool ADJ>
 __global__ void __launch_bounds__(SMW ? 512 : 32, SMW ? 1 : WarpFlat<P, HAS_Z, SMW>::SINGLE_BLOCKS)
 warpflat_kernel(const RowArgs a, const int nwhole) {

@@ -162,8 +162,12 @@ inline bool flat_enabled() {
 // 46: 100 / 113 -> 23 / 33 us; 92: 107 / 127 -> 36 / 49; 184: 127 / 144 -> 68 / 81; 384: 150 / 217 -> 89 / 125;
 // 512: 153 / 252 -> 124 / 157; 640: 391 / 822 -> 155 / 200 (three-stage block kernel before); 64 as 4 x 16 and 32 as
 // 4 x 8 for the VJP: 19 -> 16, 23 -> 15 us; but 120: 37 / 44 -> 42 / 56, 240: 60 / 72 -> 69 / 88.  With z, 256 gains where a
-// line has more samples than are staged (at 3.2x 156 -> 101 us, at 6x equal), 32 28 -> 24 us; 64 as 4 x 16 29 -> 23 us, but
-// 2 x 10 coils x 256 rows 4.9 -> 6.9 us; 368 as 23 x 16 154 -> 143 us, but 4 x 15 coils x 640 rows 97 -> 109 us.
+// line has more samples than are staged (at 3.2x 156 -> 101 us, at 6x equal), 32 28 -> 24 us.
+// With z one plan has to serve every problem of a length, since the ranks of the samples follow it.  Prepared steps, this
+// plan against the other: 368 as 16 x 23 against 23 x 16, 19 problems of 320 to 5120 rows and 4 to 16 coils: faster in 15 (8 coils
+// of 640 rows 21 against 28 us, 15 of 2560 93 against 106), slower by up to 13 % where 23 x 16 just fills its last round (15 of
+// 1920 rows 74 against 65, 16 of 2048 77 against 69).  64 as 8 x 8 against 4 x 16: faster while the coils go side by side (2 x 16
+// coils of 512 rows 8.6 against 16.8 us), slower beyond (8 x 16 coils of 512 28.5 against 21.4, 24 x 8 of 128 15.6 against 10.7).
 template <int N> struct FlatRL { static constexpr int v = 0, z = 0; };
 #define GLEAM_FLAT(N, V, Z) template <> struct FlatRL<N> { static constexpr int v = V, z = Z; };
 GLEAM_FLAT(32, 8, 8)

@@ -132,4 +132,4 @@ def test_every_eligible_extent_pair_has_row_tile_kernels(lib):
                 count += 1
     assert count == len(listed)
     assert g.gleam_dc_rowtile_split(320, 256) == 16 and g.gleam_dc_rowtile_split(128, 128) > 0
-    assert g.gleam_dc_rowtile_split(640, 256) == 0            # three-stage plan: general middle pass
+    assert g.gleam_dc_rowtile_split(640, 256) == 0            # 20 x 32: middle radix beyond 24
