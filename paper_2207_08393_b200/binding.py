@@ -374,25 +374,26 @@ def _current_stream_handle() -> int:
 
 
 class CallDims:
-    """The ``gleam_dims`` of one problem shape, kept per stream and workspace memory: a call that finds its structure does
-    not fill one (5 us).  Kept by the address and size of the workspace as they are at the call, from which alone a
-    structure follows: a tensor that was given other storage (``resize_``, ``set_``) gets another one.  A structure is
-    never changed once it is in use, so threads may share the holder."""
+    """The ``gleam_dims`` of one problem shape, kept per stream: a call that finds its structure does not fill one (5 us).
+    A structure counts only for the workspace memory it was filled with, compared at every call by address and size: a
+    tensor that was given other storage (``resize_``, ``set_``) gets another structure.  A structure is never changed
+    once it is in use, so threads may share the holder."""
 
-    LIMIT = 64                                 # structures remembered; beyond that the table starts over
+    LIMIT = 64                                 # streams remembered; beyond that the table starts over
 
     def __init__(self, *shape):
-        self._shape, self._known = shape, {}
+        self._shape, self._known = shape, {}   # {stream: (address, bytes, structure)}
 
     def get(self, workspace, stream=None) -> gleam_dims:
         handle = _current_stream_handle() if stream is None else stream if isinstance(stream, int) else stream.cuda_stream
-        key = (handle, workspace.data_ptr(), workspace.nbytes)
-        d = self._known.get(key)
-        if d is None:
+        kept = self._known.get(handle)
+        if kept is None or kept[0] != workspace.data_ptr() or kept[1] != workspace.nbytes:
             if len(self._known) >= self.LIMIT:
                 self._known = {}
-            d = self._known[key] = make_dims(*self._shape, stream=handle, workspace=key[1], workspace_bytes=key[2])
-        return d
+            address, size = workspace.data_ptr(), workspace.nbytes
+            kept = address, size, make_dims(*self._shape, stream=handle, workspace=address, workspace_bytes=size)
+            self._known[handle] = kept
+        return kept[2]
 
 
 class DataConsistency:
