@@ -8,7 +8,7 @@ gradient data-consistency step).  One operator application in single precision d
 perturbations of their vectors by at most about the condition number of A^H A + mu I
 (<= (1 + mu) / mu = 21 for the paper's mu = 0.05 with unit-norm sensitivities), and since the
 inner products are accumulated in double precision the steps do not add to it: 21 * 1e-7 = 2e-6
-(measured on the full-size workloads: 1.8e-6 after 10 and after 30 steps), a factor 10 of margin.
+(measured on the full-size workloads: 1.9e-6 after 10 and after 30 steps), a factor 10 of margin.
 """
 import numpy as np
 import pytest
