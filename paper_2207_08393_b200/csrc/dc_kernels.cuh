@@ -261,7 +261,7 @@ col_z_kernel(const ColArgs a) {
             const cf* src = a.y + (unit_of(item) * N + d.jL) * pe + p;
 #pragma unroll
             for (int k = 0; k < RL; ++k) {
-                const cf yv = !ok ? make_float2(0.f, 0.f) : STAGED ? cur[(d.jL + P::BFL * k) * L + l] : __ldg(src);
+                const cf yv = !ok ? make_float2(0.f, 0.f) : STAGED ? cur[(d.jL + P::BFL * k) * L + l] : *src;
                 u[k] = cscale(yv, (P::BFL * k) % 2 ? -odd : odd);
                 src += P::BFL * pe;
             }
