@@ -185,7 +185,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
         auto load_sens = [&](cf (&dst)[R0], int c) {
             const cf* p = sp + c * s_stride;
 #pragma unroll
-            for (int m = 0; m < R0; ++m) dst[m] = row_ok ? __ldg(p + RL * m) : make_float2(0.f, 0.f);
+            for (int m = 0; m < R0; ++m) dst[m] = row_ok ? p[RL * m] : make_float2(0.f, 0.f);
         };
 
         cf acc[R0];

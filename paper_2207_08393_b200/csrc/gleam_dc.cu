@@ -82,10 +82,10 @@ static const TileOps* find_tile(int ry, int n2) {
 #define ZMAP_THREADS 256
 #define ZMAP_MAX_RY 32
 template <bool COUNT>
-__global__ void __launch_bounds__(ZMAP_THREADS) zmap_kernel(const float* __restrict__ mask, int* __restrict__ zidx,
-                                                            int* __restrict__ zlist, int* __restrict__ zcount,
-                                                            float* __restrict__ m2c, int* __restrict__ zstart,
-                                                            int* __restrict__ row_cnt, int n1, int n2, int ry) {
+__global__ void __launch_bounds__(ZMAP_THREADS) zmap_kernel(const float* mask, int* zidx,
+                                                            int* zlist, int* zcount,
+                                                            float* m2c, int* zstart,
+                                                            int* row_cnt, int n1, int n2, int ry) {
     grid_dependency_wait();
     grid_launch_dependents();
     const int lane = threadIdx.x & 31, row = blockIdx.x * (ZMAP_THREADS / 32) + (threadIdx.x >> 5);   // row = k0 * by + k1
@@ -448,9 +448,9 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
 // <g, a> per batch example, double accumulation in a fixed order: block partial sums, then one block per example.
 #define GRAD_THREADS 256
 #define GRAD_MAX_BLOCKS 512
-__global__ void __launch_bounds__(GRAD_THREADS) grad_eta_partial_kernel(const cf* __restrict__ g, const cf* __restrict__ x,
-                                                                        const cf* __restrict__ t, long long ne,
-                                                                        double* __restrict__ part) {
+__global__ void __launch_bounds__(GRAD_THREADS) grad_eta_partial_kernel(const cf* g, const cf* x,
+                                                                        const cf* t, long long ne,
+                                                                        double* part) {
     // t = x - A^H(Ax - y)  (the step with eta = 1), so A^H(Ax - y) = x - t
     grid_dependency_wait();
     grid_launch_dependents();
@@ -471,14 +471,14 @@ __global__ void __launch_bounds__(GRAD_THREADS) grad_eta_partial_kernel(const cf
 }
 // Sum of n <= GRAD_MAX_BLOCKS values by one warp, in a fixed order (every lane's loads are in flight together; one
 // thread adding them one after another took 10 us).
-__device__ __forceinline__ double warp_array_sum(const double* __restrict__ v, int n) {
+__device__ __forceinline__ double warp_array_sum(const double* v, int n) {
     double s = 0.0;
 #pragma unroll
     for (int e = 0; e < GRAD_MAX_BLOCKS / 32; ++e) { const int i = e * 32 + (int)threadIdx.x; if (i < n) s += v[i]; }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     return s;
 }
-__global__ void grad_eta_final_kernel(const double* __restrict__ part, int nblocks, double* __restrict__ grad_eta) {
+__global__ void grad_eta_final_kernel(const double* part, int nblocks, double* grad_eta) {
     grid_dependency_wait();
     const double s = warp_array_sum(part + (long long)blockIdx.x * nblocks, nblocks);
     if (threadIdx.x == 0) grad_eta[blockIdx.x] = -s;
@@ -488,9 +488,9 @@ __global__ void grad_eta_final_kernel(const double* __restrict__ part, int nbloc
 // ---- complex l1 loss between an image and a reference (training loss of the paper's networks) ----
 // loss = mean |x - r|; grad = (x - r) / |x - r| / N (zero where x = r).  Block partial sums in double, summed
 // by one thread in block order: deterministic.
-__global__ void __launch_bounds__(GRAD_THREADS) l1_partial_kernel(const cf* __restrict__ x, const cf* __restrict__ r, cf* __restrict__ grad,
+__global__ void __launch_bounds__(GRAD_THREADS) l1_partial_kernel(const cf* x, const cf* r, cf* grad,
                                                                   long long ne, int B, int x_planar, int g_planar, long long plane,
-                                                                  float inv_n, double* __restrict__ part) {
+                                                                  float inv_n, double* part) {
     grid_dependency_wait();
     grid_launch_dependents();
     __shared__ double sh[GRAD_THREADS];
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(GRAD_THREADS) l1_partial_kernel(const cf* __re
     }
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
-__global__ void l1_final_kernel(const double* __restrict__ part, int nblocks, double inv_n, double* __restrict__ loss, int as_float) {
+__global__ void l1_final_kernel(const double* part, int nblocks, double inv_n, double* loss, int as_float) {
     grid_dependency_wait();
     const double s = warp_array_sum(part, nblocks);
     if (threadIdx.x == 0) { if (as_float) *reinterpret_cast<float*>(loss) = (float)(s * inv_n); else *loss = s * inv_n; }
