@@ -1,5 +1,7 @@
 """Which kernels and launch shapes the rules of the dispatch choose, read from the captured launches of a call, and the
 results of the calls whose choice lies next to a line, against the CPU oracle."""
+import ctypes
+
 import pytest
 
 from oracle.oracle import MASK_READOUT_INVARIANT
@@ -11,9 +13,7 @@ pytestmark = pytest.mark.gpu
 
 def captured(fn):
     """The kernel launches of fn(), in order: name, blocks, threads, resident blocks on this GPU, bytes of local memory (spilled
-    registers), and whether the launch
-    may start before the one before it has ended (from the third edge on: the binding gives its buffer of edge data back
-    before it is read, and the allocator writes over the first two entries)."""
+    registers), and whether the launch may start before the one before it has ended."""
     import torch
     from cuda.bindings import driver
     def ok(r):
@@ -27,10 +27,16 @@ def captured(fn):
     raw = driver.CUgraph(graph.raw_cuda_graph())
     count = ok(driver.cuGraphGetNodes(raw))[1]
     nodes = ok(driver.cuGraphGetNodes(raw, count))[0]
-    edges = ok(driver.cuGraphGetEdges_v2(raw))[3]
-    before, after, data = ok(driver.cuGraphGetEdges_v2(raw, edges))[:3]
-    follows = {int(b): (int(a), int(e.type) == int(driver.CUgraphDependencyType.CU_GRAPH_DEPENDENCY_TYPE_PROGRAMMATIC))
-               for a, b, e in zip(before, after, data)}
+    # through ctypes: the package gives its buffer of edge data back before they are read
+    class Edge(ctypes.Structure):
+        _fields_ = [("from_port", ctypes.c_ubyte), ("to_port", ctypes.c_ubyte), ("type", ctypes.c_ubyte), ("reserved", ctypes.c_ubyte * 5)]
+    get_edges, edges = ctypes.CDLL("libcuda.so.1").cuGraphGetEdges_v2, ctypes.c_size_t(0)
+    get_edges.argtypes = [ctypes.c_void_p] * 4 + [ctypes.POINTER(ctypes.c_size_t)]
+    assert get_edges(graph.raw_cuda_graph(), None, None, None, edges) == 0
+    before, after, data = (ctypes.c_void_p * edges.value)(), (ctypes.c_void_p * edges.value)(), (Edge * edges.value)()
+    assert edges.value == 0 or get_edges(graph.raw_cuda_graph(), before, after, data, edges) == 0
+    programmatic = int(driver.CUgraphDependencyType.CU_GRAPH_DEPENDENCY_TYPE_PROGRAMMATIC)
+    follows = {b: (a, e.type == programmatic) for a, b, e in zip(before, after, data)}
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     launches = {}
     for n in nodes:
@@ -98,6 +104,7 @@ def test_early_start_of_the_z_table(shape, early):
     tables = [i for i, k in enumerate(launches) if "col_z_kernel" in k["name"]]
     assert len(tables) == 2 and len(launches) == 5
     assert launches[tables[1]]["early"] == early, launches[tables[1]]
+    assert all(k["early"] for i, k in enumerate(launches) if i > 0 and i not in tables)
 
 
 # z table: more sampled tiles than blocks (a block walks over several, also with the last tile part full) and fewer, one-, two-
