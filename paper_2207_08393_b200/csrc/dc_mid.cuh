@@ -141,7 +141,7 @@ mid_kernel(const MidArgs a) {
 #pragma unroll
             for (int j = 1; j < BY; ++j) c[j] = cmul(c[j], twiddle(j));
         }
-        Dft<BY, -1>::run(c);
+        Dft<BY, -1, true>::run(c);
     }
     if (MODE == MID_SEP) {
 #pragma unroll
@@ -189,7 +189,7 @@ mid_kernel(const MidArgs a) {
         return;
     }
     if (INVERSE) {
-        Dft<BY, +1>::run(c);
+        Dft<BY, +1, true>::run(c);
         if (RY > 1) {
 #pragma unroll
             for (int j = 1; j < BY; ++j) c[j] = cmulc(c[j], twiddle(j));

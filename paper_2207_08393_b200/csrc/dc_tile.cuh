@@ -133,7 +133,7 @@ tile_fwd_kernel(const TileArgs a) {
             cf v[RY];
 #pragma unroll
             for (int m = 0; m < RY; ++m) v[m] = cmul(sS[m * NZ + tid], xv[m]);
-            Dft<RY, -1>::run(v);
+            Dft<RY, -1, true>::run(v);
 #pragma unroll
             for (int k = 0; k < RY; ++k) sT[k * ROW + TL::slot(tid)] = v[k];
         }
@@ -149,7 +149,7 @@ tile_fwd_kernel(const TileArgs a) {
             cf v[R0];
 #pragma unroll
             for (int m = 0; m < R0; ++m) v[m] = e[m * LS1];
-            Dft<R0, -1>::run(v);
+            Dft<R0, -1, true>::run(v);
             if (TL::S == 2) {
 #pragma unroll
                 for (int k = 0; k < R0; ++k) e[k * LS1] = (k == 0) ? v[0] : cmul(v[k], sTw[k * BF0 + j]);
@@ -169,7 +169,7 @@ tile_fwd_kernel(const TileArgs a) {
                 cf u[RL];
 #pragma unroll
                 for (int m = 0; m < RL; ++m) u[m] = e[m];
-                Dft<RL, -1>::run(u);
+                Dft<RL, -1, true>::run(u);
                 cf* o = Vp + row * a.v_k0 + j;
 #pragma unroll
                 for (int k = 0; k < RL; ++k) o[R0 * k] = u[k];
@@ -218,7 +218,7 @@ tile_inv_kernel(const TileArgs a) {
                 cf u[RL];
 #pragma unroll
                 for (int k = 0; k < RL; ++k) u[k] = o[R0 * k];
-                Dft<RL, +1>::run(u);
+                Dft<RL, +1, true>::run(u);
 #pragma unroll
                 for (int m = 0; m < RL; ++m) e[m] = u[m];
             }
@@ -233,7 +233,7 @@ tile_inv_kernel(const TileArgs a) {
                 cf v[R0];
 #pragma unroll
                 for (int k = 0; k < R0; ++k) { const cf r = e[k * LS1]; v[k] = (k == 0) ? r : cmulc(r, sTw[k * BF0 + j]); }
-                Dft<R0, +1>::run(v);
+                Dft<R0, +1, true>::run(v);
 #pragma unroll
                 for (int m = 0; m < R0; ++m) e[m * LS1] = v[m];
             }
@@ -242,7 +242,7 @@ tile_inv_kernel(const TileArgs a) {
                 cf v[R0];
 #pragma unroll
                 for (int k = 0; k < R0; ++k) v[k] = sV[t * NZ + k];
-                Dft<R0, +1>::run(v);
+                Dft<R0, +1, true>::run(v);
 #pragma unroll
                 for (int m = 0; m < R0; ++m) sT[t * NZ + m] = v[m];
             }
@@ -256,7 +256,7 @@ tile_inv_kernel(const TileArgs a) {
             cf v[RY];
 #pragma unroll
             for (int k = 0; k < RY; ++k) v[k] = sT[k * ROW + TL::slot(tid)];
-            Dft<RY, +1>::run(v);
+            Dft<RY, +1, true>::run(v);
 #pragma unroll
             for (int m = 0; m < RY; ++m) {
                 const cf s = sS[m * NZ + tid];

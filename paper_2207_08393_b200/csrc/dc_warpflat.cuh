@@ -79,6 +79,9 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
     grid_dependency_wait();
     using WF = WarpFlat<P, HAS_Z, SMW>;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL, LW = WF::LW, UPC = WF::UPC, US = WF::USTRIDE, SLOTS = WF::SLOTS;
+    // Folded twiddles: plain and normal-equations calls 87 -> 85 and 88 -> 86 us (8 x 16 coils of 640 x 320), 30 -> 28 (8 x 8
+    // of 512 x 256); the block of many warps without A^H y measured slower with them (20 frames of 192 x 160, 16.4 -> 16.8).
+    constexpr bool FOLD = !HAS_Z && (!SMW || HAS_ATY);
     constexpr int KCAP = WF::KCAP, KSTRIDE = WF::KSTRIDE, KTILE = WF::KTILE, ZS = WF::ZS, MS = WF::MS;
     extern __shared__ __align__(16) float2 smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -208,7 +211,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
 #pragma unroll
                 for (int m = 0; m < R0; ++m) v[m] = cmul(sf[m], x_at(j + RL * m));
                 if (af + 1 < nc) load_sens(sf, af + 1);
-                Dft<R0, -1>::run(v);
+                Dft<R0, -1, FOLD>::run(v);
                 cf* e = sE + ((af % SLOTS) * UPC + l * R0) * US + j;
                 if (img) {
 #pragma unroll
@@ -230,7 +233,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 if (!ADJ) {
 #pragma unroll
                     for (int m = 0; m < RL; ++m) u[m] = e[m];
-                    Dft<RL, -1>::run(u);
+                    Dft<RL, -1, FOLD>::run(u);
                 }
                 if (!HAS_Z) {
                     const float* mm = sM + bl * MS + jb;
@@ -244,7 +247,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                     if (kc <= KCAP) unit_update<R0, RL, ADJ>(u, kc > 0 ? um.bits : 0u, mw, sK + (c % ZS) * KTILE + bl * KSTRIDE + um.first, true);
                     else unit_update<R0, RL, ADJ>(u, um.bits, mw, a.z + sKo[bl] + c * k_stride + um.first, false);
                 }
-                Dft<RL, +1>::run(u);
+                Dft<RL, +1, FOLD>::run(u);
                 if (live) {
 #pragma unroll
                     for (int m = 0; m < RL; ++m) e[m] = u[m];
@@ -262,7 +265,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                     const cf r = e[k * US];
                     v[k] = (k == 0) ? r : cmulc(r, tw0[k]);
                 }
-                Dft<R0, +1>::run(v);
+                Dft<R0, +1, FOLD>::run(v);
 #pragma unroll
                 for (int m = 0; m < R0; ++m) {
                     if (HAS_ATY) {      // acc = aty - sum

@@ -167,7 +167,7 @@ warpline_kernel(const RowArgs a) {
                 if (a0) {
 #pragma unroll
                     for (int m = 0; m < R0; ++m) v[m] = cmul(cS[j + P::BF0 * m], x_at(j + P::BF0 * m));
-                    Dft<R0, -1>::run(v);
+                    Dft<R0, -1, !HAS_Z>::run(v);
                 }
                 if (P::S == 2) {
                     if (a0) {
@@ -179,7 +179,7 @@ warpline_kernel(const RowArgs a) {
                     if (aL) {
 #pragma unroll
                         for (int m = 0; m < RL; ++m) u[m] = sE[l * WL::EXL + j * P::LS1 + m];
-                        Dft<RL, -1>::run(u);
+                        Dft<RL, -1, !HAS_Z>::run(u);
                     }
                     __syncwarp();
                 } else {
@@ -203,7 +203,7 @@ warpline_kernel(const RowArgs a) {
             {
                 if (P::S == 2) {
                     if (aL) {
-                        Dft<RL, +1>::run(u);
+                        Dft<RL, +1, !HAS_Z>::run(u);
 #pragma unroll
                         for (int m = 0; m < RL; ++m) sE[l * WL::EXL + j * P::LS1 + m] = u[m];
                     }
@@ -220,7 +220,7 @@ warpline_kernel(const RowArgs a) {
                     for (int k = 0; k < R0; ++k) v[k] = u[k % RL];
                 }
                 if (a0) {
-                    Dft<R0, +1>::run(v);
+                    Dft<R0, +1, !HAS_Z>::run(v);
 #pragma unroll
                     for (int m = 0; m < R0; ++m) {
                         const cf sv = cS[j + P::BF0 * m];

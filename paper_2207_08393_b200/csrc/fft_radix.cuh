@@ -128,18 +128,19 @@ constexpr int ct_factor(int r) {     // outer factor A of the split R = A * B
 }
 constexpr bool is_prime_like(int r) { return r == 2 || r == 4 || (r % 2 == 1 && smallest_odd_factor(r) == r); }
 
-template <int R, int DIR> struct Dft;
+// FOLD: constant twiddles folded into the multiply-adds of the butterfly behind them (DftFolded).
+template <int R, int DIR, bool FOLD = false> struct Dft;
 
-template <int DIR> struct Dft<1, DIR> { static GLEAM_HD void run(cf (&)[1]) {} };
+template <int DIR, bool FOLD> struct Dft<1, DIR, FOLD> { static GLEAM_HD void run(cf (&)[1]) {} };
 
-template <int DIR> struct Dft<2, DIR> {
+template <int DIR, bool FOLD> struct Dft<2, DIR, FOLD> {
     static GLEAM_HD void run(cf (&v)[2]) {
         const cf a = v[0], b = v[1];
         v[0] = cadd(a, b); v[1] = csub(a, b);
     }
 };
 
-template <int DIR> struct Dft<4, DIR> {
+template <int DIR, bool FOLD> struct Dft<4, DIR, FOLD> {
     static GLEAM_HD void run(cf (&v)[4]) {
         const cf s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
         const cf s13 = cadd(v[1], v[3]), d13 = csub(v[1], v[3]);
@@ -217,6 +218,74 @@ template <int R, int DIR> struct DftComposite {
     }
 };
 
+// Constant twiddle w = exp(DIR 2 pi i E / R) as w a = f rot(a) with a real factor f (the larger of cosine and sine, with its
+// sign): rot takes one multiply-add per component, and f goes into the multiply-adds of the butterfly that follows.
+template <int E_, int R, int DIR> struct FoldedTwiddle {
+    static constexpr int E = ((E_ % R) + R) % R;
+    static constexpr bool UNIT = (4 * E) % R == 0;                       // a multiple of a quarter turn
+    static constexpr double C = ct::cos2pi(E, R), S = DIR * ct::sin2pi(E, R);
+    static constexpr bool COS = (C < 0 ? -C : C) >= (S < 0 ? -S : S);
+    static constexpr bool DIAG = (8 * E) % R == 0 && !UNIT;              // |cosine| = |sine|
+    static constexpr double F = UNIT ? 1.0 : COS ? C : S;
+    static constexpr float T = float(COS ? S / C : C / S);
+    static GLEAM_HD cf rot(cf a) {
+        if constexpr (E == 0) return a;
+        else if constexpr (2 * E == R) return make_float2(-a.x, -a.y);
+        else if constexpr (4 * E == R) return mul_i_dir<DIR>(a);
+        else if constexpr (UNIT) return mul_i_dir<-DIR>(a);
+        else if constexpr (DIAG) return T > 0 ? make_float2(a.x - a.y, a.y + a.x) : make_float2(a.x + a.y, a.y - a.x);
+        else if constexpr (COS) return make_float2(fmaf(-T, a.y, a.x), fmaf(T, a.x, a.y));
+        else return make_float2(fmaf(T, a.x, -a.y), fmaf(T, a.y, a.x));
+    }
+};
+// y + f a with a constant f
+template <class F> GLEAM_HD cf cadd_folded(cf y, cf a, F) {
+    constexpr double f = F::value();
+    if constexpr (f == 1.0) return cadd(y, a);
+    else if constexpr (f == -1.0) return csub(y, a);
+    else return caxpy(float(f), a, y);
+}
+// four values with constant twiddles exp(DIR 2 pi i E n / R), n = 0..3, then their 4-point transform
+template <int E, int R, int DIR> struct TwiddledDft4 {
+    static GLEAM_HD void run(cf y0, cf y1, cf y2, cf y3, cf (&o)[4]) {
+        using W1 = FoldedTwiddle<E, R, DIR>; using W2 = FoldedTwiddle<2 * E, R, DIR>; using W3 = FoldedTwiddle<3 * E, R, DIR>;
+        struct P2 { static constexpr double value() { return W2::F; } }; struct M2 { static constexpr double value() { return -W2::F; } };
+        struct P3 { static constexpr double value() { return W3::F / W1::F; } }; struct M3 { static constexpr double value() { return -W3::F / W1::F; } };
+        struct P1 { static constexpr double value() { return W1::F; } }; struct M1 { static constexpr double value() { return -W1::F; } };
+        const cf a1 = W1::rot(y1), a2 = W2::rot(y2), a3 = W3::rot(y3);
+        const cf s02 = cadd_folded(y0, a2, P2{}), d02 = cadd_folded(y0, a2, M2{});
+        const cf s13 = cadd_folded(a1, a3, P3{}), d13 = cadd_folded(a1, a3, M3{});       // over W1::F
+        o[0] = cadd_folded(s02, s13, P1{}); o[2] = cadd_folded(s02, s13, M1{});
+        constexpr float f = float(DIR * W1::F);
+        o[1] = make_float2(fmaf(-f, d13.y, d02.x), fmaf(f, d13.x, d02.y));
+        o[3] = make_float2(fmaf(f, d13.y, d02.x), fmaf(-f, d13.x, d02.y));
+    }
+};
+
+// The same with the twiddles folded: 4 B points (8, 16, 32) take 52, 144 and 376 operations instead of 56, 160 and 432, and
+// round less (error of 8 / 16 / 32 points against 64 bits 5.11e-8 / 6.11e-8 / 7.27e-8 -> 4.98e-8 / 5.94e-8 / 6.97e-8).
+template <int R, int DIR> struct DftFolded {
+    static constexpr int A = ct_factor(R);
+    static constexpr int B = R / A;
+    static_assert(A == 4, "the others have coprime factors");
+    static GLEAM_HD void run(cf (&v)[R]) {
+        cf y[A][B];
+        static_for<0, A>([&](auto n1i) {
+            constexpr int n1 = decltype(n1i)::value;
+            cf t[B];
+            static_for<0, B>([&](auto n2i) { constexpr int n2 = decltype(n2i)::value; t[n2] = v[A * n2 + n1]; });
+            Dft<B, DIR, true>::run(t);
+            static_for<0, B>([&](auto k2i) { constexpr int k2 = decltype(k2i)::value; y[n1][k2] = t[k2]; });
+        });
+        static_for<0, B>([&](auto k2i) {
+            constexpr int k2 = decltype(k2i)::value;
+            cf t[A];
+            TwiddledDft4<k2, R, DIR>::run(y[0][k2], y[1][k2], y[2][k2], y[3][k2], t);
+            static_for<0, A>([&](auto k1i) { constexpr int k1 = decltype(k1i)::value; v[k2 + B * k1] = t[k1]; });
+        });
+    }
+};
+
 // composite R = A * B with coprime factors (6, 10, 12, 15, 20, ...): prime-factor index maps,
 //   n = (B n1 + A n2) mod R,   k = the residue with k mod A = k1 and k mod B = k2,
 // turn the transform into A-point and B-point transforms with no twiddle factors in between
@@ -226,7 +295,7 @@ constexpr int crt_index(int k1, int A, int k2, int B) {
     for (int k = 0; k < A * B; ++k) if (k % A == k1 && k % B == k2) return k;
     return 0;
 }
-template <int R, int DIR> struct DftCoprime {
+template <int R, int DIR, bool FOLD> struct DftCoprime {
     static constexpr int A = ct_factor(R);
     static constexpr int B = R / A;
     static GLEAM_HD void run(cf (&v)[R]) {
@@ -235,23 +304,24 @@ template <int R, int DIR> struct DftCoprime {
             constexpr int n1 = decltype(n1i)::value;
             cf t[B];
             static_for<0, B>([&](auto n2i) { constexpr int n2 = decltype(n2i)::value; t[n2] = v[(B * n1 + A * n2) % R]; });
-            Dft<B, DIR>::run(t);
+            Dft<B, DIR, FOLD>::run(t);
             static_for<0, B>([&](auto k2i) { constexpr int k2 = decltype(k2i)::value; y[n1][k2] = t[k2]; });
         });
         static_for<0, B>([&](auto k2i) {
             constexpr int k2 = decltype(k2i)::value;
             cf t[A];
             static_for<0, A>([&](auto n1i) { constexpr int n1 = decltype(n1i)::value; t[n1] = y[n1][k2]; });
-            Dft<A, DIR>::run(t);
+            Dft<A, DIR, FOLD>::run(t);
             static_for<0, A>([&](auto k1i) { constexpr int k1 = decltype(k1i)::value; v[crt_index(k1, A, k2, B)] = t[k1]; });
         });
     }
 };
 
-template <int R, int DIR> struct Dft {
+template <int R, int DIR, bool FOLD> struct Dft {
     static GLEAM_HD void run(cf (&v)[R]) {
         if constexpr (R % 2 == 1 && smallest_odd_factor(R) == R) DftPrime<R, DIR>::run(v);
-        else if constexpr (ct_gcd(ct_factor(R), R / ct_factor(R)) == 1) DftCoprime<R, DIR>::run(v);
+        else if constexpr (ct_gcd(ct_factor(R), R / ct_factor(R)) == 1) DftCoprime<R, DIR, FOLD>::run(v);
+        else if constexpr (FOLD) DftFolded<R, DIR>::run(v);
         else DftComposite<R, DIR>::run(v);
     }
 };
