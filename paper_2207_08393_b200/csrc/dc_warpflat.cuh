@@ -28,13 +28,20 @@ struct WarpFlat {
     static constexpr int LANES = LW * RL;                  // lanes of the image-side stages (32 if RL is a power of two)
     static constexpr int USTRIDE = odd_up(RL);             // odd: a round's 32 units read without bank conflicts
     static constexpr int SLOTS_MIN = (32 + UPC - 1) / UPC + 1;     // coils between first forward and inverse stage
+    // Where the z values of a unit wait for its butterfly: in the unit's own slots of the ring, which it has just read (RING_Z),
+    // or in a staging area per coil, requested a forward stage earlier.  The first takes any number of samples, leaves the
+    // staging area's shared memory to further blocks and makes the update free of branches, but the butterfly alone has to
+    // cover the latency: not where so large ones leave 8 warps per SM or fewer.  Prepared step, staged -> ring: 8 x 16 coils
+    // of 640 x 320 at 4x 137 -> 112 us, at 2.9x 138 -> 118, 8 x 8 of 512 x 256 52 -> 46, 2 x 12 of 384 x 320 26.1 -> 20.9, 20
+    // frames x 8 of 192 x 160 21.9 -> 20.8; but 4 x 15 of 640 x 368 92 -> 98, 8 of 640 x 640 24 -> 26.5.
+    static constexpr bool RING_Z = !(RL > 16 && R0 >= 16);
     // a ring whose unit count is a multiple of 16 keeps the bank pattern across the wrap; taken when small
     static constexpr int slots_aligned() {
         for (int s = SLOTS_MIN; s <= SLOTS_MIN + 3; ++s) if ((s * UPC) % 16 == 0) return s;
         return SLOTS_MIN;
     }
-    static constexpr int SLOTS = (!SMW && !HAS_Z && slots_aligned() * UPC * USTRIDE * 8 <= 11 * 1024) ? slots_aligned() : SLOTS_MIN;
-    static constexpr int ZS = SMW ? SLOTS : SLOTS + 1;     // z rows are requested one forward stage ahead (SMW: in their own stage)
+    static constexpr int SLOTS = (!SMW && (!HAS_Z || RING_Z) && slots_aligned() * UPC * USTRIDE * 8 <= 11 * 1024) ? slots_aligned() : SLOTS_MIN;
+    static constexpr int ZS = RING_Z ? 0 : SMW ? SLOTS : SLOTS + 1;     // staged: one forward stage ahead (SMW: in their own stage)
     static constexpr int KCAP = z_stage(N); // staged z entries per line (more: read from global memory)
     static constexpr int KSTRIDE = KCAP;
     static constexpr int KTILE = LW * KSTRIDE;
@@ -135,7 +142,11 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
             const bool ok = __shfl_sync(0xffffffffu, (int)row_ok, ll * RL) != 0;
             const long long xo = __shfl_sync(0xffffffffu, x_off, ll * RL);
             const long long bto = __shfl_sync(0xffffffffu, (long long)bt, ll * RL);
-            if (!ok) { if (HAS_Z && lane == 0) sC[ll] = 0; continue; }
+            if (!ok) {                                               // no z is read for a line past the end
+                if (HAS_Z && lane == 0) sC[ll] = 0;
+                if (HAS_Z && lane < R0) sU[ll * R0 + lane] = UnitMask{0u, 0};
+                continue;
+            }
             if (ADJ) {
             } else if (!a.x_planar) {
                 for (int i = lane; i < N / 2; i += 32) cp_async16(sX + ll * N + 2 * i, a.x + xo + 2 * i);
@@ -174,8 +185,9 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 for (int i = lane; i < (kc + 1) / 2; i += 32) cp_async16(sK + (c % ZS) * KTILE + ll * KSTRIDE + 2 * i, ks + 2 * i);
             }
         };
+        constexpr bool STAGED_Z = HAS_Z && !WF::RING_Z;
         constexpr int ZAHEAD = SMW ? 0 : 1;      // forward stages between the request for a z row and the stage of its coil
-        if (HAS_Z && ZAHEAD) issue_z(0);
+        if (STAGED_Z && ZAHEAD) issue_z(0);
         cp_async_commit();
 
         const bool x_planes = a.x_planar && (N % 4 == 0);          // x staged as two planes of floats
@@ -204,8 +216,8 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
             const int done = (br == rounds - 1) ? nc : upto / UPC;       // coils complete after this round
             // ---- forward image-side stage: S x, R0-point butterflies, twiddles, into the ring ----
             while (af < need) {
-                if (HAS_Z) { if (af + ZAHEAD < nc) issue_z(af + ZAHEAD); cp_async_commit(); }
-                if (af == 0) { cp_async_wait<HAS_Z ? 1 : 0>(); __syncwarp(); }      // x (and z of coil 0) have landed
+                if (STAGED_Z) { if (af + ZAHEAD < nc) issue_z(af + ZAHEAD); cp_async_commit(); }
+                if (af == 0) { cp_async_wait<STAGED_Z ? 1 : 0>(); __syncwarp(); }      // x (and z of coil 0) have landed
                 if (ADJ) { ++af; continue; }
                 cf v[R0];
 #pragma unroll
@@ -219,7 +231,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 }
                 ++af;
             }
-            if (HAS_Z) cp_async_wait<ZAHEAD>();  // everything but a request for the next coil's z is there
+            if (STAGED_Z) cp_async_wait<ZAHEAD>();  // everything but a request for the next coil's z is there
             __syncwarp();
             // ---- k-space round: units 32 br .. 32 br + 31, one per lane ----
             {
@@ -233,12 +245,43 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 if (!ADJ) {
 #pragma unroll
                     for (int m = 0; m < RL; ++m) u[m] = e[m];
-                    Dft<RL, -1, FOLD>::run(u);
                 }
+                if (HAS_Z && WF::RING_Z) {
+                    // every entry at its place, zero where nothing was sampled; a lane reads back only what it requested
+                    const UnitMask um = sU[bl * R0 + jb];
+                    if (live) {
+                        const cf* zs = a.z + sKo[bl] + c * k_stride + um.first;
+#pragma unroll
+                        for (int k = 0; k < RL; ++k) if (!(um.bits & (1u << k))) e[k] = make_float2(0.f, 0.f);
+                        for (unsigned left = um.bits; left != 0; left &= left - 1) cp_async8(e + (__ffs((int)left) - 1), zs++);
+                    }
+                    cp_async_commit();
+                }
+                if (!ADJ) Dft<RL, -1, FOLD>::run(u);
                 if (!HAS_Z) {
                     const float* mm = sM + bl * MS + jb;
 #pragma unroll
                     for (int k = 0; k < RL; ++k) u[k] = cscale(u[k], mm[R0 * k]);
+                } else if (WF::RING_Z) {
+                    cp_async_wait<0>();
+                    const float* mw = sM + bl * MS + jb;
+                    const bool few = sC[bl] <= KCAP;         // one rounding or two, as in the other kernels
+                    if (ADJ) {
+#pragma unroll
+                        for (int k = 0; k < RL; ++k) { const cf q = e[k]; u[k] = make_float2(-q.x, -q.y); }
+                    } else if (__all_sync(0xffffffffu, few)) {
+#pragma unroll
+                        for (int k = 0; k < RL; ++k) { const cf q = e[k]; const float w = mw[R0 * k]; u[k] = make_float2(fmaf(w, u[k].x, -q.x), fmaf(w, u[k].y, -q.y)); }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < RL; ++k) {
+                            const cf q = e[k];
+                            const float w = mw[R0 * k];
+                            const cf one = make_float2(fmaf(w, u[k].x, -q.x), fmaf(w, u[k].y, -q.y));
+                            const cf two = make_float2(__fsub_rn(__fmul_rn(w, u[k].x), q.x), __fsub_rn(__fmul_rn(w, u[k].y), q.y));
+                            u[k] = few ? one : two;
+                        }
+                    }
                 } else {
                     // z of a line that is staged from shared memory, of others straight from its row
                     const UnitMask um = sU[bl * R0 + jb];

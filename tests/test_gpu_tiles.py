@@ -71,3 +71,28 @@ def test_one_pass_kernel_by_the_number_of_lines(oracle, B, C, rows, n2, density)
 def test_samples_of_the_middle_pass(oracle, n, density):
     d, x, y, sens, mask = problem(3, 1, 3, 1, n, MASK_READOUT_INVARIANT, seed=sum(n), density=density)
     check_all(oracle, d, x, y, sens, mask, 0.7, "middle pass %s" % (n,))
+
+
+# one-pass kernel with measurements: frames without samples, with few, with more than a quarter and with all of them, whose
+# lines share a warp (4, 2 and 1 lines per warp, rows that leave lines past the end), one and several rounds of units,
+# one block per SM (18 frames of 120 rows); unsampled measurements are NaN
+@pytest.mark.parametrize("n2,rows,C,T", [(32, 10, 3, 5), (48, 6, 2, 5), (80, 2, 3, 5), (96, 6, 3, 4), (128, 10, 3, 5), (160, 120, 3, 18), (184, 6, 3, 4),
+                                         (192, 4, 2, 4), (256, 6, 3, 4), (320, 10, 3, 4), (384, 2, 3, 4), (512, 2, 3, 4)])
+def test_measurements_of_frames_of_unlike_density(oracle, n2, rows, C, T):
+    d, x, y, sens, mask = problem(2, 1, C, T, (1, rows, n2), MASK_READOUT_INVARIANT, seed=n2 + rows, weighted=True)
+    rng = np.random.default_rng(n2)
+    for t in range(T):
+        keep = rng.uniform(size=n2) < (0.0, 0.1, 0.5, 1.0)[t % 4]
+        mask[:, t] *= keep
+        y[:, :, t][..., ~keep] = np.nan
+    clean = np.nan_to_num(y)
+    assert_close(run_gpu(x, y, sens, mask, 0.9, 2, 0, MASK_READOUT_INVARIANT), oracle.dc_forward(x, clean, sens, mask, 0.9, d, nthreads=8), x, "n2=%d" % n2)
+    import torch
+    import paper_2207_08393_b200 as g
+    dev = torch.device("cuda:0")
+    dc = g.DataConsistency(1, C, T, 2, (1, rows, n2))
+    tx, ty, ts, tm = (torch.from_numpy(a).to(dev) for a in (x, y, sens, mask))
+    got = dc.adjoint(ty, ts, tm)
+    torch.cuda.synchronize()
+    ref = oracle.dc_forward(np.zeros_like(x), clean, sens, mask, 1.0, d, nthreads=8)
+    assert_close(got.cpu().numpy(), ref, ref, "n2=%d adjoint" % n2)
