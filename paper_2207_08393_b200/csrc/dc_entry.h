@@ -16,7 +16,8 @@ enum { RUN_ALL = 0, RUN_PREPARE = 1, RUN_APPLY = 2, RUN_ADJOINT = 3 };
 int run(const void* x, const void* y, const void* sens, const float* mask, float eta, void* out,
         const gleam_dims* d, int mode = RUN_ALL, double* dot_rows = nullptr, bool check_only = false,
         int layout = 0,      // layout: GLEAM_X_CHANNELS | GLEAM_OUT_CHANNELS (two-real-channel image arrays)
-        const void* aty = nullptr);   // with y == nullptr: out = x - eta (A^H A x - aty), aty = A^H y as an image
+        const void* aty = nullptr,    // with y == nullptr: out = x - eta (A^H A x - aty), aty = A^H y as an image
+        int* dot_count = nullptr);    // set (also by check_only) to the number of sums per example in each half of dot_rows
 
 // dot_rows (device, two arrays of one double per image row, B*T*n1): the one-pass 2-D kernel also stores
 // Re<x_row, out_row> and <out_row, out_row> of every row it writes, so that a caller's inner products need no

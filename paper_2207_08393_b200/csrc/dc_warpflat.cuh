@@ -80,15 +80,18 @@ struct WarpFlat {
 // ADJ (with z): A^H y, the image is zero; the forward stages are left out and a unit starts from minus its z values.
 // Registers: sixteen warps of one block have 128 each, which the step with z of 160 points exceeds by 52 B (spilled to
 // local memory; single-warp blocks without the spill are slower all the same, see launch_warpflat_zy).
-template <class P, bool HAS_Z, bool SMW, bool HAS_ATY, bool ADJ>
+// DOT: the inner products of dot_rows (conjugate gradients; calls without z and A^H y).  A template parameter for the same
+// reason as HAS_ATY: with the block sums behind a run-time test the plain call of 20 frames of 192 x 160 took 17.3 us, not 16.4.
+template <class P, bool HAS_Z, bool SMW, bool HAS_ATY, bool ADJ, bool DOT>
 __global__ void __launch_bounds__(SMW ? 512 : 32, SMW ? 1 : WarpFlat<P, HAS_Z, SMW>::SINGLE_BLOCKS)
 warpflat_kernel(const RowArgs a, const int nwhole) {
     grid_dependency_wait();
     using WF = WarpFlat<P, HAS_Z, SMW>;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL, LW = WF::LW, UPC = WF::UPC, US = WF::USTRIDE, SLOTS = WF::SLOTS;
     // Folded twiddles: plain and normal-equations calls 87 -> 85 and 88 -> 86 us (8 x 16 coils of 640 x 320), 30 -> 28 (8 x 8
-    // of 512 x 256); the block of many warps without A^H y measured slower with them (20 frames of 192 x 160, 16.4 -> 16.8).
-    constexpr bool FOLD = !HAS_Z && (!SMW || HAS_ATY);
+    // of 512 x 256); the block of many warps without A^H y measured slower with them (20 frames of 192 x 160, 16.4 -> 16.8),
+    // and so did the 23-point image side (4 x 15 of 640 x 368, 78.7 -> 79.0 and 80.1 -> 80.9).
+    constexpr bool FOLD = !HAS_Z && (!SMW || HAS_ATY) && R0 != 23;
     constexpr int KCAP = WF::KCAP, KSTRIDE = WF::KSTRIDE, KTILE = WF::KTILE, ZS = WF::ZS, MS = WF::MS;
     extern __shared__ __align__(16) float2 smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -119,6 +122,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
     const long long g_first = !SMW ? (long long)blockIdx.x
                             : split ? (long long)(nwhole + set) * gridDim.x + blockIdx.x : (long long)warp * gridDim.x + blockIdx.x;
     const long long g_step = !SMW ? (long long)gridDim.x : ngroups;              // SMW: a single round
+    if (SMW && DOT && a.dot_blocks && g_first >= ngroups && lane < 3) reinterpret_cast<double*>(sX)[lane] = 0.0;
 
     for (long long g = g_first; g < ngroups; g += g_step) {
         const long long row = g * LW + l;
@@ -349,15 +353,33 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 const float se = HAS_ATY ? a.eta : -a.eta;          // HAS_ATY: acc holds aty - sum
                 const cf ov = make_float2(fmaf(se, av.x, xv.x), fmaf(se, av.y, xv.y));
                 store_image(a.out, x_off + j + RL * m, ov, a.out_planar, b, a.plane);
-                if (a.dot_rows != nullptr) { dsum += (double)xv.x * ov.x + (double)xv.y * ov.y; nsum += (double)ov.x * ov.x + (double)ov.y * ov.y; }
+                if (DOT) { dsum += (double)xv.x * ov.x + (double)xv.y * ov.y; nsum += (double)ov.x * ov.x + (double)ov.y * ov.y; }
             }
         }
-        if (a.dot_rows != nullptr) {     // the same in every thread
+        if (SMW && DOT && a.dot_blocks) {
+            for (int o = 16; o > 0; o >>= 1) { dsum += __shfl_down_sync(0xffffffffu, dsum, o); nsum += __shfl_down_sync(0xffffffffu, nsum, o); }
+            __syncwarp();                // the image has been read
+            if (lane == 0) { double* p = reinterpret_cast<double*>(sX); p[0] = dsum; p[1] = nsum; p[2] = (double)b; }
+        } else if (DOT) {
             for (int o = pow2_ceil(RL) / 2; o > 0; o >>= 1) {
                 const double d = __shfl_down_sync(0xffffffffu, dsum, o), n = __shfl_down_sync(0xffffffffu, nsum, o);
                 if (j + o < RL) { dsum += d; nsum += n; }
             }
             if (j == 0 && row_ok) { a.dot_rows[row] = dsum; a.dot_rows[a.nrows + row] = nsum; }
+        }
+    }
+    if (SMW && DOT && a.dot_blocks) {    // one pair of sums per block and example, in a fixed order
+        __syncthreads();
+        if (warp == 0) {
+            const int warps = blockDim.x >> 5;
+            const double* p = reinterpret_cast<const double*>(smem + (lane < warps ? lane : 0) * WF::ELEMS + WF::OFF_X);
+            const bool has = lane < nwhole || (lane < warps && ((lane - nwhole) & 3) == 0);
+            for (int ex = 0; ex < a.dot_blocks; ++ex) {
+                const bool mine = has && p[2] == (double)ex;
+                double d = mine ? p[0] : 0.0, n = mine ? p[1] : 0.0;
+                for (int o = 8; o > 0; o >>= 1) { d += __shfl_down_sync(0xffffffffu, d, o); n += __shfl_down_sync(0xffffffffu, n, o); }
+                if (lane == 0) { double* out = a.dot_rows + (long long)ex * a.T * a.RPB + blockIdx.x; out[0] = d; out[a.nrows] = n; }
+            }
         }
     }
 }

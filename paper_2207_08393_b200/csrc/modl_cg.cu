@@ -55,8 +55,8 @@ struct CgArgs {
     double* part_rr;         // (2, B, CG_MAX_BLOCKS): <r,r> partial sums of even / odd steps
     CgCarry* carry;          // (2, B), even / odd steps
     double* part_pq;         // (B, CG_MAX_BLOCKS) twice: <p,q> and <q,q> partial sums written by cg_dot
-    const double* dot_rows;  // (B, rows_per_example) twice: Re<p,q> and <q,q> per image row from the operator, or null
-    int rows_per_example;
+    const double* dot_rows;  // (B, rows_per_example) twice: Re<p,q> and <q,q> per image row or block from the operator, or null
+    int rows_per_example, dot_count;         // dot_count of them are in use
     long long ne2;           // float4 elements per example
     float mu;
     double inv_mu;
@@ -84,20 +84,42 @@ __device__ __forceinline__ Sums block_sums(Sums v) {
     return t;
 }
 
-// This thread's share of the sum of n values written by an earlier launch, in a fixed order; v is 16-byte aligned.
-// Eight pairs are requested at a time: 20 frames of 192 rows are one round of loads.
-__device__ __forceinline__ double array_share(const double* v, int n) {
+// This thread's share of the sum of n values written by an earlier launch, in a fixed order, as thread `first` of `threads`;
+// v is 16-byte aligned.  Eight pairs are requested at a time: 20 frames of 192 rows are one round of loads of a block.
+__device__ __forceinline__ double array_share(const double* v, int n, int first, int threads) {
     double t = 0.0;
     const int pairs = n / 2;
-    for (int i0 = threadIdx.x; i0 < pairs; i0 += 8 * CG_THREADS) {
+    for (int i0 = first; i0 < pairs; i0 += 8 * threads) {
         double2 w[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) w[e] = (i0 + e * CG_THREADS < pairs) ? __ldcg(reinterpret_cast<const double2*>(v) + i0 + e * CG_THREADS) : make_double2(0.0, 0.0);
+        for (int e = 0; e < 8; ++e) w[e] = (i0 + e * threads < pairs) ? __ldcg(reinterpret_cast<const double2*>(v) + i0 + e * threads) : make_double2(0.0, 0.0);
 #pragma unroll
         for (int e = 0; e < 8; ++e) t += w[e].x + w[e].y;
     }
-    if (n % 2 && threadIdx.x == 0) t += __ldcg(v + n - 1);
+    if (n % 2 && first == 0) t += __ldcg(v + n - 1);
     return t;
+}
+// Sums of the arrays a (na values), b and c (nb values each; c may be null), valid in the first thread.  Short arrays are
+// dealt to the warps, so that a warp has one value to add across its lanes (6 coils of 320 x 320, 10 steps: 117 -> 110 us);
+// long ones take every thread (10 frames of 192 rows: 306 -> 298).
+constexpr int CG_DEALT = 768;
+__device__ __forceinline__ Sums array_sums(const double* a, int na, const double* b, const double* c, int nb) {
+    constexpr int W = CG_THREADS / 32, WA = 2, WB = (W - WA) / 2;           // warps of a, of b and of c
+    __shared__ double warp_sum[W];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int which = warp < WA ? 0 : warp < WA + WB ? 1 : 2, first = which == 0 ? 0 : which == 1 ? WA : WA + WB;
+    const double* v = which == 0 ? a : which == 1 ? b : c;
+    double t = v == nullptr ? 0.0 : array_share(v, which == 0 ? na : nb, (warp - first) * 32 + lane, (which == 0 ? WA : WB) * 32);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) warp_sum[warp] = t;
+    __syncthreads();
+    Sums s{0.0, 0.0, 0.0};
+    if (threadIdx.x == 0) {
+        for (int w = 0; w < WA; ++w) s.a += warp_sum[w];
+        for (int w = WA; w < WA + WB; ++w) s.b += warp_sum[w];
+        for (int w = WA + WB; w < W; ++w) s.c += warp_sum[w];
+    }
+    return s;
 }
 
 __device__ __forceinline__ double* rr_slot(const CgArgs& a, int which) {
@@ -153,7 +175,7 @@ __global__ void __launch_bounds__(CG_THREADS) cg_dot_kernel(const CgArgs a) {
 
 // CG_BATCH elements of every vector are requested before the sums are formed, so that their latency covers that of the sums.
 constexpr int CG_BATCH = 2;
-template <bool FROM_ROWS, bool LAST>
+template <bool FROM_ROWS, bool DEALT, bool LAST>
 __global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) {
     grid_dependency_wait();
     const long long base = (long long)blockIdx.y * a.ne2, stride = (long long)gridDim.x * CG_THREADS;
@@ -171,13 +193,18 @@ __global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) 
     fetch();
     __shared__ double carry[4];              // CgCarry of the step before
     if (!LAST && threadIdx.x < 4) carry[threadIdx.x] = __ldcg(reinterpret_cast<const double*>(a.carry + (size_t)a.parity * gridDim.y + blockIdx.y) + threadIdx.x);
-    Sums s;
-    s.a = array_share(rr_slot(a, a.parity), (int)gridDim.x);
     const double* pq = FROM_ROWS ? a.dot_rows + (size_t)blockIdx.y * a.rows_per_example : a.part_pq + (size_t)blockIdx.y * CG_MAX_BLOCKS;
-    const int npq = FROM_ROWS ? a.rows_per_example : (int)gridDim.x;
-    s.b = array_share(pq, npq);
-    s.c = LAST ? 0.0 : array_share(pq + (size_t)gridDim.y * (FROM_ROWS ? a.rows_per_example : CG_MAX_BLOCKS), npq);
-    s = block_sums(s);
+    const int npq = FROM_ROWS ? a.dot_count : (int)gridDim.x;
+    const double* qq = pq + (size_t)gridDim.y * (FROM_ROWS ? a.rows_per_example : CG_MAX_BLOCKS);
+    Sums s;
+    if (DEALT) {
+        s = array_sums(rr_slot(a, a.parity), (int)gridDim.x, pq, LAST ? nullptr : qq, npq);
+    } else {
+        s.a = array_share(rr_slot(a, a.parity), (int)gridDim.x, threadIdx.x, CG_THREADS);
+        s.b = array_share(pq, npq, threadIdx.x, CG_THREADS);
+        s.c = LAST ? 0.0 : array_share(qq, npq, threadIdx.x, CG_THREADS);
+        s = block_sums(s);
+    }
     __shared__ float scalars[3];
     if (threadIdx.x == 0) {
         // an example whose residual is exactly zero stays as it is; one division on the way to the vectors
@@ -299,17 +326,24 @@ static int modl_cg(const void* z, const void* y, const void* sens, const float* 
     a.part_rr = (double*)(ws + L.off_rr); a.part_pq = (double*)(ws + L.off_pq);
     a.carry = (CgCarry*)(ws + L.off_carry);
     a.ne2 = L.ne2; a.mu = mu; a.inv_mu = 1.0 / (double)mu; a.parity = 0;
-    long long nb = (L.ne2 + (long long)CG_THREADS * 4 - 1) / ((long long)CG_THREADS * 4);
-    if (nb < 1) nb = 1;
-    if (nb > CG_MAX_BLOCKS) nb = CG_MAX_BLOCKS;
-    const dim3 grid((unsigned)nb, (unsigned)L.B);
     // the one-pass 2-D operator kernel delivers <p,q> per image row
     const bool from_rows = dot_rows_supported(d);
     double* dot_rows = from_rows ? (double*)(ws + L.off_rows) : nullptr;
     a.dot_rows = dot_rows; a.rows_per_example = d->frames * d->n[1];
 
     // the operator's own argument checks (y, sens, mask) before anything is enqueued
-    CGRUN(run(ws + L.off_r, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ALL, nullptr, true));
+    CGRUN(run(ws + L.off_r, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ALL, dot_rows, true, 0, nullptr, &a.dot_count));
+    // Four elements a thread, or two where that is one block per SM, or a round of blocks (a few more) that have few sums to
+    // add at their start, unless four are one block per SM already (those come in while the operator drains).  10 steps, four
+    // -> two: 8 coils x 16 frames of 64 x 64 99 -> 90 us, 20 of 192 x 160 (a sum per block) 259 -> 250, 2 x 6 x 12 of 128 x 128
+    // 186 -> 160; but 3 x 5 x 8 of 128 x 96 128 -> 136 (144 -> 288 blocks), 4 x 15 of 640 x 368 900 -> 910 (920 blocks).
+    auto blocks_of = [&](int each) {
+        const long long n = (L.ne2 + (long long)CG_THREADS * each - 1) / ((long long)CG_THREADS * each);
+        return n < 1 ? 1 : n > CG_MAX_BLOCKS ? CG_MAX_BLOCKS : n;
+    };
+    const long long fine = blocks_of(2) * L.B, coarse = blocks_of(4) * L.B, one = CG_MAX_BLOCKS / 4;
+    const bool two = fine <= one || (coarse > one && (!from_rows || a.dot_count <= CG_DEALT) && fine <= 5 * one);
+    const dim3 grid((unsigned)blocks_of(two ? 2 : 4), (unsigned)L.B);
     if (y) {
         CGRUN(run(nullptr, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ADJOINT));
         CGCK(prof_mark(GLEAM_K_CG_VEC, s));
@@ -327,10 +361,10 @@ static int modl_cg(const void* z, const void* y, const void* sens, const float* 
             CGCK(launch_overlapped(true, cg_dot_kernel, grid, dim3(CG_THREADS), 0, s, a));
         }
         CGCK(prof_mark(GLEAM_K_CG_VEC, s));
-        if (from_rows && last) CGCK(launch_overlapped(true, cg_step_kernel<true, true>, grid, dim3(CG_THREADS), 0, s, a));
-        else if (from_rows) CGCK(launch_overlapped(true, cg_step_kernel<true, false>, grid, dim3(CG_THREADS), 0, s, a));
-        else if (last) CGCK(launch_overlapped(true, cg_step_kernel<false, true>, grid, dim3(CG_THREADS), 0, s, a));
-        else CGCK(launch_overlapped(true, cg_step_kernel<false, false>, grid, dim3(CG_THREADS), 0, s, a));
+        auto step = !from_rows ? (last ? cg_step_kernel<false, true, true> : cg_step_kernel<false, true, false>)
+                  : a.dot_count <= CG_DEALT ? (last ? cg_step_kernel<true, true, true> : cg_step_kernel<true, true, false>)
+                                            : (last ? cg_step_kernel<true, false, true> : cg_step_kernel<true, false, false>);
+        CGCK(launch_overlapped(true, step, grid, dim3(CG_THREADS), 0, s, a));
         CGCK(cudaGetLastError());
     }
     CGCK(prof_mark(-1, s));

@@ -103,18 +103,18 @@ inline bool split_enabled() {
 }
 
 // the one-pass kernel with the k-space units numbered across the coils (dc_warpflat.cuh)
-template <class P, bool HAS_Z, bool HAS_ATY, bool ADJ>
+template <class P, bool HAS_Z, bool HAS_ATY, bool ADJ, bool DOT>
 inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* single) {
     static_assert(WarpFlat<P, HAS_Z>::ELIGIBLE, "not a plan the coil-numbered kernel takes");
     using WF = WarpFlat<P, HAS_Z, false>;
     static PerDevice attr_done;
     static PerDevice slots_cache;
-    cudaError_t e = ensure_smem(warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ>, WF::WARP_BYTES, attr_done);
+    cudaError_t e = ensure_smem(warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ, DOT>, WF::WARP_BYTES, attr_done);
     if (e != cudaSuccess) return e;
     int slots = 0;
-    if ((e = resident_slots(warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ>, 32, WF::WARP_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
+    if ((e = resident_slots(warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ, DOT>, 32, WF::WARP_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
     const long long groups = (a.nrows + WF::LW - 1) / WF::LW;
-    if (single) { *single = groups <= slots; return cudaSuccess; }       // one block per SM below is one round, too
+    if (single) *single = groups <= slots;                   // one block per SM below is one round, too
     if (groups <= 0) return cudaSuccess;
     // One round of 8 to 16 groups per SM: one block per SM that holds all its warps.  4 k + 1 (or 4 k + 2) groups per
     // SM: the groups beyond 4 k are split by coils over four warps each, one per scheduler.  (Measured on cine-shaped
@@ -131,22 +131,31 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* si
             const int nwhole = per - nsplit, warps = nwhole + 4 * nsplit;
             const size_t bytes = WS::WARP_BYTES * (size_t)warps;
             if (warps <= 16 && bytes <= 227 * 1024) {
+                // a sum per block and example, for few examples: the lines of a group belong to one (a line of it decides which)
+                const long long rows = (long long)a.T * a.RPB;
+                const bool whole = DOT && rows >= sms && rows % WF::LW == 0 && a.nrows <= 3 * rows;
+                if (whole && a.dot_count) *a.dot_count = sms;
+                if (single) return cudaSuccess;
+                RowArgs b = a;
+                b.dot_blocks = whole ? (int)(a.nrows / rows) : 0;
                 // the attribute is set once, to what the largest block of this kernel can ask for
                 constexpr size_t SMEM_CAP = 227 * 1024;
-                if ((e = ensure_smem(warpflat_kernel<P, HAS_Z, true, HAS_ATY, ADJ>, 16 * WS::WARP_BYTES < SMEM_CAP ? 16 * WS::WARP_BYTES : SMEM_CAP, attrs_done)) != cudaSuccess) return e;
-                return launch_overlapped(true, warpflat_kernel<P, HAS_Z, true, HAS_ATY, ADJ>, dim3((unsigned)sms), dim3(32 * warps), bytes, s, a, nwhole);
+                if ((e = ensure_smem(warpflat_kernel<P, HAS_Z, true, HAS_ATY, ADJ, DOT>, 16 * WS::WARP_BYTES < SMEM_CAP ? 16 * WS::WARP_BYTES : SMEM_CAP, attrs_done)) != cudaSuccess) return e;
+                return launch_overlapped(true, warpflat_kernel<P, HAS_Z, true, HAS_ATY, ADJ, DOT>, dim3((unsigned)sms), dim3(32 * warps), bytes, s, b, nwhole);
             }
         }
     }
+    if (single) return cudaSuccess;
     long long blocks = groups;
     if (blocks > slots) blocks = slots;
-    return launch_overlapped(true, warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ>, dim3((unsigned)blocks), dim3(32), WF::WARP_BYTES, s, a, 1);
+    return launch_overlapped(true, warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ, DOT>, dim3((unsigned)blocks), dim3(32), WF::WARP_BYTES, s, a, 1);
 }
 template <class P, bool HAS_Z>
 inline cudaError_t launch_warpflat_z(const RowArgs& a, cudaStream_t s, bool* single) {
-    if constexpr (!HAS_Z) { if (a.aty != nullptr) return launch_warpflat_zy<P, false, true, false>(a, s, single); }
-    else { if (a.x == nullptr) return launch_warpflat_zy<P, true, false, true>(a, s, single); }
-    return launch_warpflat_zy<P, HAS_Z, false, false>(a, s, single);
+    if constexpr (!HAS_Z) { if (a.aty != nullptr) return launch_warpflat_zy<P, false, true, false, false>(a, s, single); }
+    else { if (a.x == nullptr) return launch_warpflat_zy<P, true, false, true, false>(a, s, single); }
+    if constexpr (!HAS_Z) { if (a.dot_rows != nullptr) return launch_warpflat_zy<P, false, false, false, true>(a, s, single); }
+    return launch_warpflat_zy<P, HAS_Z, false, false, false>(a, s, single);
 }
 // GLEAM_NO_FLAT=1 keeps the plain warp-resident kernel for those lengths (tuning aid, read once).
 inline bool flat_enabled() {
