@@ -59,7 +59,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         obj = os.path.join(BUILD, "kernels_group%d.o" % g)
         jobs.append((["nvcc"] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +
                      ["-DGLEAM_GROUP=%d" % g, "-c", os.path.join(CSRC, "kernels_group.cu"), "-o", obj], obj))
-        for name in ("mid", "axis"):
+        for name in ("mid", "axis", "brick"):
             obj = os.path.join(BUILD, "kernels_%s%d.o" % (name, g))
             jobs.append((["nvcc"] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +
                          ["-DGLEAM_GROUP=%d" % g, "-c", os.path.join(CSRC, "kernels_%s.cu" % name), "-o", obj], obj))

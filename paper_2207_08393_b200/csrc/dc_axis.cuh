@@ -1,5 +1,5 @@
-// Readout axis of 3-D problems with an arbitrary mask: transform, k-space work, inverse transform, in place on the
-// workspace that the middle passes of dc_mid.cuh leave as (unit, q, n0, n2), the rows q in their order (raw
+// Readout axis of 3-D problems with an arbitrary mask whose lengths dc_brick.cuh does not take: transform, k-space work,
+// inverse transform, in place on the workspace that the middle passes of dc_mid.cuh leave as (unit, q, n0, n2), the rows q in their order (raw
 // ky = q / BY + RY * (q % BY)).  A block takes KC neighbouring kz columns of one (unit, q): n0 pieces of 8 KC bytes
 // that lie n2 apart, so a tile's pieces share DRAM pages (with the volume's natural order they lie a plane apart:
 // 96 x 160 x 128, 6 coils: 306 us for both calls against 150 us here).  Bound by HBM: 16 bytes per element, 24 with

@@ -5,8 +5,9 @@
 //   readout-invariant mask, fft_rank 3 :  [z table]  ->  per chunk of readout slabs the three row-tile
 //                                         passes over (ky, kz): forward, middle (mask, residual), inverse
 //   full mask, fft_rank 2               :  the same three passes over (n1, n2)
-//   full mask, fft_rank 3               :  forward pass, middle pass without k-space work, readout axis
-//                                         (mask, residual), middle pass back, inverse pass
+//   full mask, fft_rank 3               :  forward pass, the rest of the transform with mask and residual and back in
+//                                         one pass (dc_brick.cuh; lengths that do not fit it: middle pass without
+//                                         k-space work, readout axis, middle pass back), inverse pass
 //
 // With a mask that does not depend on the readout index the readout transform commutes with the
 // mask, so A^H(Ax - y) = S^H P^H M (M P S x - R^H y) with P over the phase-encode axes and R over
@@ -15,6 +16,7 @@
 #include "size_ops.cuh"
 #include "dc_mid.cuh"
 #include "dc_axis.cuh"
+#include "dc_brick.cuh"
 #include "dc_fused3d.cuh"
 #include "dc_fused_entry.h"
 #include "dc_entry.h"
@@ -28,7 +30,7 @@
 
 namespace gleam {
 
-#define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) extern const SizeOps size_ops_##N; extern const MidOps mid_ops_##N; extern const AxisOps axis_ops_##N;
+#define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) extern const SizeOps size_ops_##N; extern const MidOps mid_ops_##N; extern const AxisOps axis_ops_##N; extern const BrickLaunch brick_##N;
 #include "sizes.def"
 #undef GLEAM_SIZE
 
@@ -57,6 +59,14 @@ static const MidOps* find_mid(int n) {
 static const AxisOps* find_axis(int n) {
     switch (n) {
 #define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) case N: return &axis_ops_##N;
+#include "sizes.def"
+#undef GLEAM_SIZE
+        default: return nullptr;
+    }
+}
+static BrickLaunch find_brick(int n) {
+    switch (n) {
+#define GLEAM_SIZE(N, A0, A1, B0, B1, B2, LC) case N: return brick_##N;
 #include "sizes.def"
 #undef GLEAM_SIZE
         default: return nullptr;
@@ -436,12 +446,21 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
         } else if (L.rank == 2) {
             LAUNCH(GLEAM_K_COL_MID_FULL, mid->launch(adjoint ? MID_ADJ_FULL : MID_FULL, ma, s));
         } else {
-            if (!adjoint) LAUNCH(GLEAM_K_COL_FWD, mid->launch(MID_FWD, ma, s));
-            AxisArgs aa{};
-            aa.W = ta.V; aa.y = (const cf*)y; aa.mask = mask; aa.C = L.C; aa.T = L.T; aa.n1 = L.n1; aa.n2 = L.n2; aa.ry = mid->ry;
-            aa.nunits = L.units; aa.scale = g / (float)sqrt((double)L.V); aa.scale2 = (float)(1.0 / (double)L.V);
-            LAUNCH(GLEAM_K_COL_MID_FULL, find_axis(L.n0)->launch(adjoint ? AXIS_ADJ : AXIS_MID, aa, s));
-            LAUNCH(GLEAM_K_COL_INV, mid->launch(MID_INV, ma, s));
+            BrickArgs br{};
+            br.V = ta.V; br.y = (const cf*)y; br.mask = mask; br.adjoint = adjoint ? 1 : 0;
+            br.C = L.C; br.T = L.T; br.n1 = L.n1; br.n2 = L.n2; br.ry = mid->ry; br.nunits = L.units;
+            br.scale = g / (float)sqrt((double)L.V); br.scale2 = (float)(1.0 / (double)L.V);
+            bool taken = false;
+            CK(prof_mark(GLEAM_K_COL_MID_FULL, s));
+            CK(find_brick(L.n0)(br, s, &taken));
+            if (!taken) {
+                AxisArgs aa{};
+                aa.W = ta.V; aa.y = br.y; aa.mask = mask; aa.C = L.C; aa.T = L.T; aa.n1 = L.n1; aa.n2 = L.n2; aa.ry = mid->ry;
+                aa.nunits = L.units; aa.scale = br.scale; aa.scale2 = br.scale2;
+                if (!adjoint) LAUNCH(GLEAM_K_COL_FWD, mid->launch(MID_FWD, ma, s));
+                LAUNCH(GLEAM_K_COL_MID_FULL, find_axis(L.n0)->launch(adjoint ? AXIS_ADJ : AXIS_MID, aa, s));
+                LAUNCH(GLEAM_K_COL_INV, mid->launch(MID_INV, ma, s));
+            }
         }
         LAUNCH(GLEAM_K_ROW_INV, tile->inv(ta, L.images, tiles, s));
     }

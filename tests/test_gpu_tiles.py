@@ -42,6 +42,16 @@ def test_volumes_with_an_arbitrary_mask(oracle, n):
     check_all(oracle, d, x, y, sens, mask, 1.0, "volume %s" % (n,))
 
 
+# bricks of k0 group x readout x columns: every middle radix, 16 and 8 columns with a remainder, radix 32 and prime radices of the
+# readout, the largest brick that fits an SM and the next one that does not, batches and frames
+@pytest.mark.parametrize("B,T,n", [(1, 1, (24, 24, 20)), (2, 2, (46, 40, 24)), (1, 1, (48, 48, 46)), (1, 2, (96, 160, 10)), (1, 1, (92, 46, 12)),
+                                   (1, 1, (120, 120, 6)), (1, 1, (40, 192, 40)), (1, 1, (64, 240, 24)), (1, 1, (384, 48, 4)), (1, 1, (368, 128, 2)),
+                                   (1, 1, (160, 320, 12)), (1, 1, (184, 320, 2)), (1, 1, (32, 384, 4))])
+def test_bricks_of_volumes_with_an_arbitrary_mask(oracle, B, T, n):
+    d, x, y, sens, mask = problem(3, B, 2, T, n, MASK_FULL, weighted=(n[0] == 96), seed=sum(n), density=0.2)
+    check_all(oracle, d, x, y, sens, mask, 0.8, "brick %s" % (n,))
+
+
 # coils dealt to clusters of 1, 2 and 4 blocks (few tiles), with coil counts that do not divide; frames and batches
 @pytest.mark.parametrize("B,C,T,n", [(1, 2, 1, (2, 64, 80)), (1, 7, 1, (2, 92, 64)), (2, 4, 2, (2, 24, 128)), (1, 3, 1, (40, 20, 32)), (1, 6, 1, (2, 640, 20))])
 def test_coil_split_of_the_row_tiles(oracle, B, C, T, n):
