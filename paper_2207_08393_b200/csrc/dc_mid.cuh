@@ -272,7 +272,7 @@ struct MidImpl {
         size_t bytes = (Z || FULL || MODE == MID_SEP) ? (size_t)BY * threads * sizeof(float) : 0;
         if (FULL) {
             static PerDevice done;
-            cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * (sizeof(cf) + sizeof(float)), done);
+            cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * (sizeof(cf) + sizeof(float)), done, BY * sizeof(cf));
             if (e != cudaSuccess) return e;
             if (a.y) bytes += (size_t)BY * threads * sizeof(cf);
         }
@@ -282,7 +282,7 @@ struct MidImpl {
         }
         if (Z) {
             static PerDevice done;
-            cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * sizeof(float) + (ZCAP + 1) * 12 + 8, done);
+            cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * sizeof(float) + (ZCAP + 1) * 12 + 8, done, BY * sizeof(cf));
             if (e != cudaSuccess) return e;
         }
         return launch_overlapped(true, mid_kernel<RY, BY, MODE>, dim3((unsigned)blocks, (unsigned)parts), dim3(threads), bytes, s, a);

@@ -35,6 +35,13 @@ def test_slices_with_an_arbitrary_mask(oracle, n, coils):
     check_all(oracle, d, x, y, sens, mask, 0.9, "slice %s" % (n,))
 
 
+# middle radix 16 with full blocks: weights and measurements take 48 KB of shared memory, the twiddles come on top
+@pytest.mark.parametrize("n", [(1, 160, 240), (1, 256, 256), (1, 160, 512)])
+def test_slices_whose_middle_pass_takes_48_kb(oracle, n):
+    d, x, y, sens, mask = problem(2, 1, 2, 1, n, MASK_FULL, seed=sum(n), density=0.3)
+    check_all(oracle, d, x, y, sens, mask, 0.9, "slice %s" % (n,))
+
+
 # readout pass: columns per block 32 / 16 with a remainder, single-stage and two-stage lengths, radix 32, prime radix
 @pytest.mark.parametrize("n", [(4, 12, 46), (20, 6, 20), (46, 8, 24), (96, 4, 40), (128, 6, 10), (160, 4, 16), (512, 2, 12), (640, 2, 20)])
 def test_volumes_with_an_arbitrary_mask(oracle, n):
