@@ -38,8 +38,14 @@ struct Brick {
     static constexpr int LS = W == 16 ? RL : odd_up(RL);       // run of a second-stage butterfly; with 8 columns two runs share the banks
     static constexpr int ROW = R0 * LS;                        // slots of a readout line
     static constexpr size_t BYTES = bytes(W, LS);
-    // Radix 32 spills (3 coils of 384 x 96 x 96, forward 269 -> 307 us); single-stage readouts occur in small tests only.
-    static constexpr bool FITS = P::S == 2 && RL <= 23 && BYTES <= LIMIT;
+    // Where the three passes are slower, over 187 volumes of all pairs of lengths (three passes / brick, forward and VJP together
+    // unless stated).  Not for single-stage readouts, which occur in small tests only; radix 32 (spills: 3 coils of 384 x 96 x 96,
+    // forward 269 -> 307 us); 16 x 15 and 16 x 16 points (two large butterflies in few registers: 0.90 to 1.14, mean 1.0);
+    // 23 points of ky next to smaller ones of the readout (0.94 to 1.31, mean 1.04).  23-point readouts gain most, 1.02 to 2.0.
+    // A^H y has the readout pass and one middle pass to replace: 0.92 to 1.33 with 80 to 128 points, 1.04 to 2.5 with
+    // 23-point stages, 0.78 to 1.2 elsewhere.
+    static constexpr bool FITS = P::S == 2 && RL <= 23 && !(R0 == 16 && (RL == 15 || RL == 16)) && (BY != 23 || RL == 23) && BYTES <= LIMIT;
+    static constexpr bool ADJOINT = RL == 23 || (N >= 80 && N <= 128);
     static constexpr int slot(int i0) { return (i0 / BF0) * LS + i0 % BF0; }
     // The readout stages of UC columns of one k1 belong to one warp, which needs no block barrier between them.
     static constexpr int UC = W == 16 && BY < 10 ? 8 : W;
@@ -252,6 +258,7 @@ struct BrickImpl {
         using BR = Brick<P, BY>;
         if constexpr (!BR::FITS) return cudaSuccess;
         else {
+            if (a.adjoint && !BR::ADJOINT) return cudaSuccess;
             static PerDevice done;
             cudaError_t e = ensure_smem(brick_kernel<P, BY>, BR::BYTES, done);
             if (e != cudaSuccess) return e;

@@ -39,11 +39,12 @@ struct Tile {
     // Slots of a row in the exchange tile.  Congruent to BF0 modulo 16: threads take the butterflies of the first kz stage row
     // after row, and each then has the bank of its thread number.  With rows of R0 runs (odd, packed) two rows of a half warp
     // met on the same banks in its reads and writes.  Packed -> congruent, VJP call, us: 8 coils of 64 x 128 x 128 79.9 -> 73.2,
-    // 96 x 96 x 96 76.7 -> 72.0, 64 x 240 x 192 226 -> 217, 48 x 320 x 240 281 -> 272, 48 x 320 x 320 386 -> 375, 12 of 96 x 240 x 184
-    // 514 -> 494.  Not for short rows and first radices below 8, where the second stage crosses rows more often than that
-    // gains: 64 x 92 x 92 62.7 -> 63.9, 80 x 64 x 46 40.8 -> 41.8, 64 x 96 x 40 30.1 -> 30.2.
+    // 96 x 96 x 96 76.7 -> 72.0, 64 x 240 x 192 226 -> 217, 48 x 320 x 240 281 -> 272, 48 x 320 x 320 386 -> 375.
+    // Not for short rows and first radices below 8, where the second stage crosses rows more often than that
+    // gains: 64 x 92 x 92 62.7 -> 63.9, 80 x 64 x 46 40.8 -> 41.8, 64 x 96 x 40 30.1 -> 30.2.  Nor for 23-point stages: forward of
+    // 15 coils of 128 x 160 x 184 746 -> 793, of 14 of 24 x 24 x 368 76 -> 81.
     static constexpr int PACKED = R0 * LS1;
-    static constexpr int ROW = S != 2 ? NZ : (R0 < 8 || NZ < 64) ? PACKED : PACKED + ((BF0 - PACKED) % 16 + 16) % 16;
+    static constexpr int ROW = S != 2 ? NZ : (R0 < 8 || NZ < 64 || RL == 23) ? PACKED : PACKED + ((BF0 - PACKED) % 16 + 16) % 16;
     static constexpr int TH = ((NZ + 31) / 32) * 32;         // one thread per kz column
     static constexpr int T_ELEMS = (RY * ROW + 1) / 2 * 2, STAGE = RY * NZ, TW = (S == 2) ? NZ : 0;
     static constexpr int RMAX = cmax(RY, cmax(R0, RL));
