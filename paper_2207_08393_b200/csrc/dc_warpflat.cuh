@@ -117,9 +117,11 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
 #pragma unroll
     for (int k = 0; k < R0; ++k) tw0[k] = unit_root_fwd<N>((j * k) % N);
     const long long ngroups = (a.nrows + LW - 1) / LW;
-    // A single round: the next launch may come in.  Not behind A^H y: the small blocks leave room for the next launch's on some
-    // SMs only, and the steps that follow in a chain keep that uneven split (3 x 9 coils of 384 x 256, A^H y and 6 steps 136 us).
-    if (SMW || (!ADJ && (long long)gridDim.x >= ngroups)) grid_launch_dependents();
+    // A single round: the next launch may come in.  Not behind single-warp blocks with z: they leave room for the next launch's
+    // blocks on some SMs only, and the launches behind it in a chain keep that uneven split (enqueued calls, let in -> not: A^H y
+    // and 6 steps of 3 x 9 coils of 384 x 256 136 -> 103 us, 5 prepared steps and VJPs of 2 x 16 of 512 x 384 378 -> 325, of 3 x 12
+    // of 384 x 320 252 -> 218; equal elsewhere).
+    if (SMW || (!HAS_Z && (long long)gridDim.x >= ngroups)) grid_launch_dependents();
     const int total = UPC * nc, rounds = (total + 31) / 32;
     const long long g_first = !SMW ? (long long)blockIdx.x
                             : split ? (long long)(nwhole + set) * gridDim.x + blockIdx.x : (long long)warp * gridDim.x + blockIdx.x;
