@@ -13,6 +13,7 @@
 // Both are copied 16 bytes at a time past L1.
 #pragma once
 #include "size_ops.cuh"
+#include "dc_entry.h"
 
 namespace gleam {
 
@@ -266,6 +267,7 @@ struct BrickImpl {
             if (blocks > 2147483647LL) return cudaSuccess;
             *taken = true;
             if (blocks <= 0) return cudaSuccess;
+            if ((e = prof_mark(GLEAM_K_COL_MID_FULL, s)) != cudaSuccess) return e;
             return launch_overlapped(true, brick_kernel<P, BY>, dim3((unsigned)blocks), dim3(BR::THREADS), BR::BYTES, s, a);
         }
     }

@@ -450,8 +450,7 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
             br.V = ta.V; br.y = (const cf*)y; br.mask = mask; br.adjoint = adjoint ? 1 : 0;
             br.C = L.C; br.T = L.T; br.n1 = L.n1; br.n2 = L.n2; br.ry = mid->ry; br.nunits = L.units;
             br.scale = g / (float)sqrt((double)L.V); br.scale2 = (float)(1.0 / (double)L.V);
-            bool taken = false;
-            CK(prof_mark(GLEAM_K_COL_MID_FULL, s));
+            bool taken = false;                      // a call that the bricks do not take is counted by its three passes alone
             CK(find_brick(L.n0)(br, s, &taken));
             if (!taken) {
                 AxisArgs aa{};

@@ -130,3 +130,24 @@ def test_readout_pass_keeps_its_columns_in_registers(n0):
     for fn in (lambda: dc.forward(x, y, s, m, 1.0), lambda: dc.vjp(x, s, m, 1.0), lambda: dc.adjoint(y, s, m)):
         passes = [k for k in captured(fn) if "axis_kernel" in k["name"]]
         assert len(passes) == 1 and passes[0]["spilled"] == 0, passes
+
+
+# arbitrary masks of volumes: sizes that the bricks take, and ones that they decline (16 x 15 points, single-stage readout or ky,
+# radix 32 of ky, 23 points of ky alone, A^H y of 40 points)
+@pytest.mark.parametrize("n,brick,adjoint", [((96, 160, 10), True, True), ((40, 48, 12), True, False), ((240, 24, 6), False, False),
+                                             ((20, 48, 6), False, False), ((96, 8, 12), False, False), ((64, 384, 4), False, False), ((48, 92, 6), False, False)])
+def test_counted_launches_are_the_launches(n, brick, adjoint):
+    import torch
+    import paper_2207_08393_b200 as g
+    dev = torch.device("cuda:0")
+    x = torch.zeros((1, 1) + n, dtype=torch.complex64, device=dev)
+    y = torch.zeros((1, 2, 1) + n, dtype=torch.complex64, device=dev)
+    s = torch.zeros((1, 2) + n, dtype=torch.complex64, device=dev)
+    m = torch.ones((1, 1) + n, dtype=torch.float32, device=dev)
+    dc = g.DataConsistency(1, 2, 1, 3, n, 0, g.GLEAM_MASK_FULL)
+    for fn, taken in ((lambda: dc.forward(x, y, s, m, 1.0), brick), (lambda: dc.vjp(x, s, m, 1.0), brick), (lambda: dc.adjoint(y, s, m), adjoint)):
+        launches = captured(fn)
+        before = g.gleam_dc_launch_count()
+        fn()
+        assert g.gleam_dc_launch_count() - before == len(launches), launches
+        assert any("brick_kernel" in k["name"] for k in launches) == taken, launches
