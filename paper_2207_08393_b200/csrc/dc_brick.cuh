@@ -188,7 +188,8 @@ brick_kernel(const BrickArgs a) {
 #pragma unroll
                 for (int k = 0; k < RL; ++k) bits |= (mv[k] != 0.f ? 1u : 0u) << k;
                 if (a.n2 % 4 == 0) {                             // pairs stay pairs under the half shift
-                    bits |= __shfl_xor_sync(0xffffffffu, bits, 1);       // both lanes have read their slots
+                    __syncwarp();                                // both lanes have read their slots (a shuffle orders no memory)
+                    bits |= __shfl_xor_sync(0xffffffffu, bits, 1);
                     const int odd = lane & 1;
 #pragma unroll
                     for (int k2 = 0; k2 < RL; k2 += 2) {         // shared between the lanes of the pair
