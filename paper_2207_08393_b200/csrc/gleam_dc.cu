@@ -369,8 +369,8 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
     ra.aty = (const cf*)aty; ra.dot_rows = dot_rows; ra.dot_count = dot_count;
     if (dot_count) *dot_count = L.T * L.n1;          // one per row unless the launch says otherwise
     if (check_only) {
-        bool single = false;
-        if (dot_rows) { ra.z = nullptr; CK(find_size(L.n2)->row(ra, s, &single)); }
+        bool lets_in = false;                        // not asked for, but nothing is launched
+        if (dot_rows) { ra.z = nullptr; CK(find_size(L.n2)->row(ra, s, &lets_in)); }
         return GLEAM_OK;
     }
 

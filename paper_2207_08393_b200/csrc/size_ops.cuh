@@ -24,8 +24,9 @@ struct PerDevice {
     }
 };
 
-// Launches the row kernel; with `single` nothing is launched, it tells whether the launch would be one round of blocks.
-typedef cudaError_t (*RowLaunch)(const RowArgs& a, cudaStream_t s, bool* single);
+// Launches the row kernel; with `lets_in` nothing is launched, it tells whether the launch would let the next one in at its start
+// (grid_launch_dependents; a single round of blocks).
+typedef cudaError_t (*RowLaunch)(const RowArgs& a, cudaStream_t s, bool* lets_in);
 
 struct SizeOps {
     int N, unit_r0;              // unit_r0: units per line of the row kernels that take z (one plan for all of them)
@@ -76,7 +77,7 @@ inline cudaError_t resident_slots(K kernel, int threads, size_t smem, PerDevice&
 // persistent launch of the warp-resident row kernel: one block per resident slot, warps stride
 // over the line groups
 template <class P, bool HAS_Z, bool ADJ>
-inline cudaError_t launch_warpline_z(const RowArgs& a, cudaStream_t s, bool* single) {
+inline cudaError_t launch_warpline_z(const RowArgs& a, cudaStream_t s, bool* lets_in) {
     using WL = WarpLine<P, HAS_Z>;
     constexpr int WARPS = 1;
     constexpr size_t SMEM = sizeof(cf) * WARPS * WL::WARP_ELEMS_ALIGNED;
@@ -88,7 +89,7 @@ inline cudaError_t launch_warpline_z(const RowArgs& a, cudaStream_t s, bool* sin
     if ((e = resident_slots(warpline_kernel<P, WARPS, HAS_Z, ADJ>, WARPS * 32, SMEM, slots_cache, &slots)) != cudaSuccess) return e;
     const long long groups = (a.nrows + WL::LW - 1) / WL::LW;
     long long blocks = (groups + WARPS - 1) / WARPS;
-    if (single) { *single = blocks <= slots; return cudaSuccess; }
+    if (lets_in) { *lets_in = blocks <= slots; return cudaSuccess; }
     if (blocks <= 0) return cudaSuccess;
     if (blocks > slots) blocks = slots;
     return launch_overlapped(true, warpline_kernel<P, WARPS, HAS_Z, ADJ>, dim3((unsigned)blocks),
@@ -104,7 +105,7 @@ inline bool split_enabled() {
 
 // the one-pass kernel with the k-space units numbered across the coils (dc_warpflat.cuh)
 template <class P, bool HAS_Z, bool HAS_ATY, bool ADJ, bool DOT>
-inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* single) {
+inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* lets_in) {
     static_assert(WarpFlat<P, HAS_Z>::ELIGIBLE, "not a plan the coil-numbered kernel takes");
     using WF = WarpFlat<P, HAS_Z, false>;
     static PerDevice attr_done;
@@ -114,7 +115,7 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* si
     int slots = 0;
     if ((e = resident_slots(warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ, DOT>, 32, WF::WARP_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
     const long long groups = (a.nrows + WF::LW - 1) / WF::LW;
-    if (single) *single = groups <= slots;                   // one block per SM below is one round, too
+    if (lets_in) *lets_in = !HAS_Z && groups <= slots;       // single-warp blocks; one block per SM: below
     if (groups <= 0) return cudaSuccess;
     // One round of 8 to 16 groups per SM: one block per SM that holds all its warps.  4 k + 1 (or 4 k + 2) groups per
     // SM: the groups beyond 4 k are split by coils over four warps each, one per scheduler.  (Measured on cine-shaped
@@ -135,7 +136,7 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* si
                 const long long rows = (long long)a.T * a.RPB;
                 const bool whole = DOT && rows >= sms && rows % WF::LW == 0 && a.nrows <= 3 * rows;
                 if (whole && a.dot_count) *a.dot_count = sms;
-                if (single) return cudaSuccess;
+                if (lets_in) { *lets_in = true; return cudaSuccess; }
                 RowArgs b = a;
                 b.dot_blocks = whole ? (int)(a.nrows / rows) : 0;
                 // the attribute is set once, to what the largest block of this kernel can ask for
@@ -145,17 +146,17 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* si
             }
         }
     }
-    if (single) return cudaSuccess;
+    if (lets_in) return cudaSuccess;
     long long blocks = groups;
     if (blocks > slots) blocks = slots;
     return launch_overlapped(true, warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ, DOT>, dim3((unsigned)blocks), dim3(32), WF::WARP_BYTES, s, a, 1);
 }
 template <class P, bool HAS_Z>
-inline cudaError_t launch_warpflat_z(const RowArgs& a, cudaStream_t s, bool* single) {
-    if constexpr (!HAS_Z) { if (a.aty != nullptr) return launch_warpflat_zy<P, false, true, false, false>(a, s, single); }
-    else { if (a.x == nullptr) return launch_warpflat_zy<P, true, false, true, false>(a, s, single); }
-    if constexpr (!HAS_Z) { if (a.dot_rows != nullptr) return launch_warpflat_zy<P, false, false, false, true>(a, s, single); }
-    return launch_warpflat_zy<P, HAS_Z, false, false, false>(a, s, single);
+inline cudaError_t launch_warpflat_z(const RowArgs& a, cudaStream_t s, bool* lets_in) {
+    if constexpr (!HAS_Z) { if (a.aty != nullptr) return launch_warpflat_zy<P, false, true, false, false>(a, s, lets_in); }
+    else { if (a.x == nullptr) return launch_warpflat_zy<P, true, false, true, false>(a, s, lets_in); }
+    if constexpr (!HAS_Z) { if (a.dot_rows != nullptr) return launch_warpflat_zy<P, false, false, false, true>(a, s, lets_in); }
+    return launch_warpflat_zy<P, HAS_Z, false, false, false>(a, s, lets_in);
 }
 // GLEAM_NO_FLAT=1 keeps the plain warp-resident kernel for those lengths (tuning aid, read once).
 inline bool flat_enabled() {
@@ -220,7 +221,7 @@ template <class P> using ZPlan = std::conditional_t<FlatRL<P::N>::z != 0, FlatPl
 // 184 x 184 13.1 / 9.6 -> 14.7 / 12.0, of 192 x 92 8.9 / 7.0 -> 13.1 / 10.6.  With z and last radices up to 16, fewer warps that
 // make it one round come first: 12 coils of 384 x 240 15.8 -> 13.9, of 384 x 160 11.8 -> 9.6.
 template <class P, bool HAS_Z, bool ADJ>
-inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken, bool* single) {
+inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken, bool* lets_in) {
     using CP = CoilPar<P>;
     *taken = false;
     int sms = 0;
@@ -258,22 +259,22 @@ inline cudaError_t launch_coilpar(const RowArgs& a, cudaStream_t s, bool* taken,
     const size_t bytes = CP::bytes(warps, a.C);
     if (bytes > CP::LIMIT || rounds > ROUNDS) return cudaSuccess;
     *taken = true;
-    if (single) { *single = rounds <= 1; return cudaSuccess; }
+    if (lets_in) { *lets_in = rounds <= 1; return cudaSuccess; }
     return launch_overlapped(true, coilpar_kernel<P, HAS_Z, ADJ>, dim3((unsigned)groups), dim3(32 * warps), bytes, s, a);
 }
 
 template <class P>
-inline cudaError_t launch_warpline(const RowArgs& a, cudaStream_t s, bool* single) {
+inline cudaError_t launch_warpline(const RowArgs& a, cudaStream_t s, bool* lets_in) {
     bool taken = false;
-    const cudaError_t e = a.z == nullptr ? launch_coilpar<ZPlan<P>, false, false>(a, s, &taken, single)
-                        : a.x != nullptr ? launch_coilpar<ZPlan<P>, true, false>(a, s, &taken, single) : launch_coilpar<ZPlan<P>, true, true>(a, s, &taken, single);
+    const cudaError_t e = a.z == nullptr ? launch_coilpar<ZPlan<P>, false, false>(a, s, &taken, lets_in)
+                        : a.x != nullptr ? launch_coilpar<ZPlan<P>, true, false>(a, s, &taken, lets_in) : launch_coilpar<ZPlan<P>, true, true>(a, s, &taken, lets_in);
     if (taken || e != cudaSuccess) return e;
     // the numbering across coils pays once a round of 32 units spans more than one coil
     const bool flat = flat_enabled() && a.C >= 2;
-    if constexpr (FlatRL<P::N>::v != 0) if (flat && a.z == nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::v>, false>(a, s, single);
-    if constexpr (FlatRL<P::N>::z != 0) if (flat && a.z != nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::z>, true>(a, s, single);
-    if (a.z == nullptr) return launch_warpline_z<P, false, false>(a, s, single);
-    return a.x != nullptr ? launch_warpline_z<ZPlan<P>, true, false>(a, s, single) : launch_warpline_z<ZPlan<P>, true, true>(a, s, single);
+    if constexpr (FlatRL<P::N>::v != 0) if (flat && a.z == nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::v>, false>(a, s, lets_in);
+    if constexpr (FlatRL<P::N>::z != 0) if (flat && a.z != nullptr) return launch_warpflat_z<FlatPlan<P, FlatRL<P::N>::z>, true>(a, s, lets_in);
+    if (a.z == nullptr) return launch_warpline_z<P, false, false>(a, s, lets_in);
+    return a.x != nullptr ? launch_warpline_z<ZPlan<P>, true, false>(a, s, lets_in) : launch_warpline_z<ZPlan<P>, true, true>(a, s, lets_in);
 }
 
 // row, row_launch: the row launch of such a call (2-D problems), or null
@@ -296,20 +297,22 @@ inline cudaError_t launch_col_z(const ColArgs& a, const RowArgs* row, RowLaunch 
     b.bpi = (int)(bpi < 1 ? 1 : bpi > most ? most : bpi);
     const long long blocks = (long long)a.images * b.bpi;
     if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-    // Scheduled as the launch before it ends, except where that may be a row launch of one round, which lets the next
-    // launch in at its start (asked of the row launch of such a call, with and without z): early blocks of the table then
-    // crowd the SMs that had room.  Forward and VJP in turn, without -> with the attribute: one round, 2 x 16 coils of 640 x
+    // Scheduled as the launch before it ends, except where that may be a row launch which lets the next launch in at its start
+    // (asked of the row launch of such a call, without z and with it): early blocks of the table then crowd the SMs that had
+    // room.  Forward and VJP in turn, without -> with the attribute: one round, 2 x 16 coils of 640 x
     // 320 91 -> 116 us, 4 x 8 of 384 x 384 66 -> 85, 3 x 15 of 640 x 368 (the VJP alone is one round) 162 -> 169, 20 frames x
     // 8 of 192 x 160 54 -> 62; several rounds, 24 frames 71.9 -> 69.8, 4 x 15 of 640 x 368 226.5 -> 224.0, 4 x 8 coils x 8 frames
-    // of 128 x 92 52.1 -> 50.2 (a launch's latency, hidden; enqueued call by call, equal in a replayed graph).  Grids of a few
-    // blocks gain, too.
+    // of 128 x 92 52.1 -> 50.2 (a launch's latency, hidden; enqueued call by call, equal in a replayed graph).  Where only
+    // single-warp blocks with z are one round, which let nothing in, 11 x 6 coils of 320 x 256, two forwards and a VJP 110.9 ->
+    // 106.2.  Grids of a few blocks gain, too.
     bool overlap = true;
     if (row != nullptr && blocks > 64) {
         RowArgs plain = *row;
         plain.z = nullptr; plain.aty = nullptr;
-        bool with_z = false, without = false;
-        if ((e = row_launch(*row, s, &with_z)) != cudaSuccess || (e = row_launch(plain, s, &without)) != cudaSuccess) return e;
-        overlap = !with_z && !without;
+        bool lets_in = false;
+        if ((e = row_launch(plain, s, &lets_in)) != cudaSuccess) return e;
+        if (!lets_in && (e = row_launch(*row, s, &lets_in)) != cudaSuccess) return e;
+        overlap = !lets_in;
     }
     return launch_overlapped(overlap, col_z_kernel<P, L>, dim3((unsigned)blocks), dim3(E::THREADS), CZ::SMEM_BYTES, s, b);
 }
@@ -317,7 +320,7 @@ inline cudaError_t launch_col_z(const ColArgs& a, const RowArgs* row, RowLaunch 
 template <class P, class PC, int LC>
 struct SizeImpl {
     static_assert(WarpLine<P>::ELIGIBLE, "row plans have at most two stages of at most 32 butterflies");
-    static cudaError_t row(const RowArgs& a, cudaStream_t s, bool* single) { return launch_warpline<P>(a, s, single); }
+    static cudaError_t row(const RowArgs& a, cudaStream_t s, bool* lets_in) { return launch_warpline<P>(a, s, lets_in); }
     static cudaError_t col_z(const ColArgs& a, const RowArgs* row, RowLaunch row_launch, cudaStream_t s) { return launch_col_z<PC, LC>(a, row, row_launch, s); }
 };
 

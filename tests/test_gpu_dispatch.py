@@ -89,14 +89,16 @@ def test_results_next_to_the_lines(oracle, shape):
     check_all(oracle, d, x, y, sens, mask, 0.9, "%s" % (shape,))
 
 
-# the z table starts early unless a row launch of one round, which lets it in at its start, may lie before it: line groups
-# against the resident blocks of 148 SMs, with and without z
+# the z table starts early unless a row launch of one round that lets it in at its start may lie before it (single-warp blocks
+# with numbered units and z do not): line groups against the resident blocks of 148 SMs, with and without z
 @pytest.mark.parametrize("shape,early", [
     ((2, 16, 1, 640, 320), False),           # one round each
     ((3, 15, 1, 640, 368), False),           # 1920 groups with z, 960 without: the VJP call is one round
     ((5, 8, 1, 640, 240), False),            # 1600 groups, 1628 blocks
     ((3, 16, 1, 640, 320), True),            # 1920 groups, 1480 and 1776 blocks
     ((1, 8, 24, 192, 160), True),            # 2304 groups, 2072 blocks
+    ((11, 6, 1, 320, 256), True),            # 1760 groups, 1776 blocks with z (numbered units), 1628 without
+    ((4, 8, 8, 64, 64), False),              # 512 groups of the plain kernel with z, 1024 of numbered units without
     ((1, 8, 1, 64, 64), True)])              # a few blocks
 def test_early_start_of_the_z_table(shape, early):
     dc, x, y, s, m = holder(shape)
