@@ -41,7 +41,8 @@ struct WarpFlat {
         return SLOTS_MIN;
     }
     static constexpr int SLOTS = (!SMW && (!HAS_Z || RING_Z) && slots_aligned() * UPC * USTRIDE * 8 <= 11 * 1024) ? slots_aligned() : SLOTS_MIN;
-    static constexpr int ZS = RING_Z ? 0 : SMW ? SLOTS : SLOTS + 1;     // staged: one forward stage ahead (SMW: in their own stage)
+    static constexpr int ZS = RING_Z ? 0 : SLOTS + 1;      // staged: one forward stage ahead
+    static_assert(!SMW || RING_Z, "blocks of many warps stage no z");
     static constexpr int KCAP = z_stage(N); // staged z entries per line (more: read from global memory)
     static constexpr int KSTRIDE = KCAP;
     static constexpr int KTILE = LW * KSTRIDE;
@@ -102,7 +103,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
     UnitMask* sU = reinterpret_cast<UnitMask*>(wsm + WF::OFF_U);
     cf* sK = wsm + WF::OFF_K;
     long long* sKo = reinterpret_cast<long long*>(wsm + WF::OFF_CNT);      // per line: offset of the z row of coil cbase
-    int* sC = reinterpret_cast<int*>(wsm + WF::OFF_CNT + LW);              // per line: sampled entries, -1 for a line past the end
+    int* sC = reinterpret_cast<int*>(wsm + WF::OFF_CNT + LW);              // per line: sampled entries (none in a line past the end)
     const bool split = SMW && warp >= nwhole;                      // one of four warps that share a group
     const int set = split ? (warp - nwhole) >> 2 : 0, q = split ? (warp - nwhole) & 3 : 0;
     const int cbase = split ? q * a.C / 4 : 0;                     // first coil and number of coils of this warp
@@ -188,14 +189,13 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
             for (int ll = 0; ll < LW; ++ll) {
                 const long long ko = sKo[ll];
                 const int kc = sC[ll];
-                if (kc <= 0 || kc > KCAP) continue;
+                if (kc > KCAP) continue;
                 const cf* ks = a.z + ko + c * k_stride;
                 for (int i = lane; i < (kc + 1) / 2; i += 32) cp_async16(sK + (c % ZS) * KTILE + ll * KSTRIDE + 2 * i, ks + 2 * i);
             }
         };
         constexpr bool STAGED_Z = HAS_Z && !WF::RING_Z;
-        constexpr int ZAHEAD = SMW ? 0 : 1;      // forward stages between the request for a z row and the stage of its coil
-        if (STAGED_Z && ZAHEAD) issue_z(0);
+        if (STAGED_Z) issue_z(0);
         cp_async_commit();
 
         const bool x_planes = a.x_planar && (N % 4 == 0);          // x staged as two planes of floats
@@ -224,7 +224,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
             const int done = (br == rounds - 1) ? nc : upto / UPC;       // coils complete after this round
             // ---- forward image-side stage: S x, R0-point butterflies, twiddles, into the ring ----
             while (af < need) {
-                if (STAGED_Z) { if (af + ZAHEAD < nc) issue_z(af + ZAHEAD); cp_async_commit(); }
+                if (STAGED_Z) { if (af + 1 < nc) issue_z(af + 1); cp_async_commit(); }
                 if (af == 0) { cp_async_wait<STAGED_Z ? 1 : 0>(); __syncwarp(); }      // x (and z of coil 0) have landed
                 if (ADJ) { ++af; continue; }
                 cf v[R0];
@@ -239,7 +239,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                 }
                 ++af;
             }
-            if (STAGED_Z) cp_async_wait<ZAHEAD>();  // everything but a request for the next coil's z is there
+            if (STAGED_Z) cp_async_wait<1>();    // everything but a request for the next coil's z is there
             __syncwarp();
             // ---- k-space round: units 32 br .. 32 br + 31, one per lane ----
             {
@@ -295,7 +295,7 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
                     const UnitMask um = sU[bl * R0 + jb];
                     const int kc = sC[bl];
                     const float* mw = sM + bl * MS + jb;
-                    if (kc <= KCAP) unit_update<R0, RL, ADJ>(u, kc > 0 ? um.bits : 0u, mw, sK + (c % ZS) * KTILE + bl * KSTRIDE + um.first, true);
+                    if (kc <= KCAP) unit_update<R0, RL, ADJ>(u, um.bits, mw, sK + (c % ZS) * KTILE + bl * KSTRIDE + um.first, true);
                     else unit_update<R0, RL, ADJ>(u, um.bits, mw, a.z + sKo[bl] + c * k_stride + um.first, false);
                 }
                 Dft<RL, +1, FOLD>::run(u);

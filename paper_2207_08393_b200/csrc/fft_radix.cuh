@@ -226,6 +226,7 @@ template <int E_, int R, int DIR> struct FoldedTwiddle {
     static constexpr double C = ct::cos2pi(E, R), S = DIR * ct::sin2pi(E, R);
     static constexpr bool COS = (C < 0 ? -C : C) >= (S < 0 ? -S : S);
     static constexpr bool DIAG = (8 * E) % R == 0 && !UNIT;              // |cosine| = |sine|
+    static_assert(!DIAG || COS, "rot takes a diagonal's sign from S / C");
     static constexpr double F = UNIT ? 1.0 : COS ? C : S;
     static constexpr float T = float(COS ? S / C : C / S);
     static GLEAM_HD cf rot(cf a) {
