@@ -165,6 +165,43 @@ def test_error_codes():
 
 
 
+# sums of the operator: per block and example where one block per SM holds several line groups (two and three examples in a
+# block, groups split by coils over four warps, whole ones), per row otherwise (single-warp blocks, four examples, groups with lines
+# of two examples); more and fewer sums than a step deals to its warps
+@pytest.mark.parametrize("shape,threads,dealt", [
+    ((1, 3, 10, 192, 160), 32, False),        # 960 groups of two lines: a sum per row, 1920 of them
+    ((2, 5, 8, 160, 160), 384, True),         # 1280 groups, 9 per SM, the last one by four warps
+    ((3, 4, 6, 160, 160), 512, True),         # 1440 groups, 10 per SM, two of them by four warps
+    ((2, 2, 11, 160, 160), 384, True),        # 1760 groups, 12 per SM
+    ((3, 3, 5, 160, 160), 288, True),         # 1200 groups, 9 per SM, too few coils to split
+    ((4, 3, 8, 80, 160), 288, True),          # four examples: a sum per row, 640 of them
+    ((3, 4, 31, 46, 48), 256, False)])        # 1070 groups of four lines, 1426 rows per example
+def test_sums_of_the_operator_and_examples_of_unlike_scale(oracle, shape, threads, dealt):
+    import torch
+    import paper_2207_08393_b200 as g
+    from tests.test_gpu_dispatch import captured
+    B, C, T, n1, n2 = shape
+    d, z, y, sens, mask = problem(2, B, C, T, (1, n1, n2), MASK_READOUT_INVARIANT, seed=sum(shape), density=0.3)
+    scale = np.array([1.0, 300.0, 0.01, 20.0], dtype=np.float32)[:B]
+    z *= scale[:, None, None, None, None]
+    y *= scale[:, None, None, None, None, None]
+    got = run_gpu_modl(z, y, sens, mask, 0.05, 4, 2, 0, MASK_READOUT_INVARIANT)
+    gotv = run_gpu_modl(z, None, sens, mask, 0.05, 4, 2, 0, MASK_READOUT_INVARIANT)
+    ref = oracle.modl_cg_forward(z, y, sens, mask, 0.05, 4, d, nthreads=8)
+    refv = oracle.modl_cg_vjp(z, sens, mask, 0.05, 4, d, nthreads=8)
+    for b in range(B):
+        close(got[b], ref[b], "%s example %d solve" % (shape, b))
+        close(gotv[b], refv[b], "%s example %d vjp" % (shape, b))
+    dev = torch.device("cuda:0")
+    cg = g.ModlCG(B, C, T, 2, (1, n1, n2))
+    tz, ts, tm = (torch.from_numpy(a).to(dev) for a in (z, sens, mask))
+    launches = captured(lambda: cg.solve_vjp(tz, ts, tm, 0.05))
+    operator = [k for k in launches if "warpflat_kernel" in k["name"]]
+    steps = [k for k in launches if "cg_step_kernel" in k["name"]]
+    assert len(operator) == len(steps) == 10 and all(k["threads"] == threads for k in operator), operator[0]
+    assert all("cg_step_kernelILb1ELb%d" % dealt in k["name"] for k in steps), steps[0]
+
+
 def textbook_steps(z, sens, mask, mu, n_iter, dtype):
     """Textbook conjugate gradients on the VJP's system in numpy, vectors in ``dtype``, scalars in double; one coil
     expansion, transforms along the last axis only (a readout-invariant mask).  All iterates."""

@@ -49,14 +49,36 @@ def test_volumes_with_an_arbitrary_mask(oracle, n):
     check_all(oracle, d, x, y, sens, mask, 1.0, "volume %s" % (n,))
 
 
-# bricks of k0 group x readout x columns: every middle radix, 16 and 8 columns with a remainder, radix 32 and prime radices of the
-# readout, the largest brick that fits an SM and the next one that does not, batches and frames
+# bricks of k0 group x readout x columns: every middle radix, 16, 8 and 4 columns with a remainder, prime radices of the readout, the
+# largest bricks, batches and frames; and sizes next to them that take three passes: radix 32 of the readout or of ky, bricks that
+# do not fit an SM (368 points with radices 20 and 23 of ky)
 @pytest.mark.parametrize("B,T,n", [(1, 1, (24, 24, 20)), (2, 2, (46, 40, 24)), (1, 1, (48, 48, 46)), (1, 2, (96, 160, 10)), (1, 1, (92, 46, 12)),
                                    (1, 1, (120, 120, 6)), (1, 1, (40, 192, 40)), (1, 1, (64, 240, 24)), (1, 1, (384, 48, 4)), (1, 1, (368, 128, 2)),
-                                   (1, 1, (160, 320, 12)), (1, 1, (184, 320, 2)), (1, 1, (32, 384, 4))])
+                                   (1, 1, (160, 320, 12)), (1, 1, (184, 320, 2)), (1, 1, (32, 384, 4)), (1, 1, (320, 120, 10)),
+                                   (1, 1, (368, 320, 2)), (1, 1, (368, 46, 4))])
 def test_bricks_of_volumes_with_an_arbitrary_mask(oracle, B, T, n):
     d, x, y, sens, mask = problem(3, B, 2, T, n, MASK_FULL, weighted=(n[0] == 96), seed=sum(n), density=0.2)
     check_all(oracle, d, x, y, sens, mask, 0.8, "brick %s" % (n,))
+
+
+# bricks: unsampled measurements are NaN.  Pairs of neighbouring kz are copied where one of them was sampled (last length a multiple
+# of 4), else one at a time; 16, 8 and 4 columns, A^H y by the bricks and by its own passes (40 points)
+@pytest.mark.parametrize("n", [(96, 160, 12), (46, 40, 24), (40, 48, 20), (48, 48, 46), (96, 96, 10), (184, 320, 4), (128, 64, 40)])
+def test_bricks_do_not_use_unsampled_measurements(oracle, n):
+    import torch
+    import paper_2207_08393_b200 as g
+    d, x, y, sens, mask = problem(3, 1, 2, 1, n, MASK_FULL, weighted=True, seed=sum(n))
+    mask *= np.random.default_rng(n[0]).uniform(size=mask.shape) < 0.3
+    clean = y.copy()
+    y[np.broadcast_to(mask[:, None] == 0, y.shape)] = np.nan
+    clean[np.isnan(y)] = 0
+    got = run_gpu(x, y, sens, mask, 0.8, 3, 0, MASK_FULL)
+    assert_close(got, oracle.dc_forward(x, clean, sens, mask, 0.8, d, nthreads=8), x, "brick %s" % (n,))
+    dc = g.DataConsistency(1, 2, 1, 3, n, 0, g.GLEAM_MASK_FULL)
+    got = dc.adjoint(*(torch.from_numpy(a).to(torch.device("cuda:0")) for a in (y, sens, mask)))
+    torch.cuda.synchronize()
+    ref = oracle.dc_forward(np.zeros_like(x), clean, sens, mask, 1.0, d, nthreads=8)
+    assert_close(got.cpu().numpy(), ref, ref, "brick %s adjoint" % (n,))
 
 
 # coils dealt to clusters of 1, 2 and 4 blocks (few tiles), with coil counts that do not divide; frames and batches
