@@ -65,10 +65,11 @@ def call_roofline(w, with_y):
     return nbytes, flops
 
 
-def kernel_work(cls, w, launches_per_call, density=1.0):
+def kernel_work(cls, w, launches_per_call, density=1.0, brick_ky=1):
     """Algorithmic (bytes, flops) of ONE launch of a kernel class for workload w.
     Per voxel*coil figures are listed beside each case; density = sampled fraction of the
-    phase-encode positions (the readout transform of y runs at those only)."""
+    phase-encode positions (the readout transform of y runs at those only).  brick_ky: points of the ky stage that
+    col_mid_full does next to the readout (volumes with an arbitrary mask whose lengths the bricks take)."""
     W = w.voxel_coils / launches_per_call        # voxel*coils one launch processes
     C = w.coils
     l2 = math.log2
@@ -85,7 +86,7 @@ def kernel_work(cls, w, launches_per_call, density=1.0):
         return W * 16 * density, W * (5 * l2(nro)) * density
     if cls == "col_mid_full":
         nro = w.n[1] if w.fft_rank == 2 else w.n[0]
-        return W * 24, W * (10 * l2(nro) + 6)
+        return W * 24, W * (10 * l2(nro * brick_ky) + 6)
     if cls in ("col_fwd", "col_inv"):
         return W * 16, W * (5 * l2(w.n[1]))
     if cls == "fused3d":        # one launch = the whole call: read S (8) + x (8/C), write out (8/C); both transforms over (n1, n2)
@@ -395,10 +396,13 @@ def run_ours(args, w):
         step_eager()
     prof = g.gleam_dc_profile_end()
     kernels = {}
+    # arbitrary 3-D masks: without middle passes of its own (col_fwd, col_inv) the ky stage is part of col_mid_full
+    ry = g.gleam_dc_rowtile_split(w.n[1], w.n[2])
+    brick_ky = w.n[1] // ry if full_mask and w.fft_rank == 3 and ry > 0 and "col_fwd" not in prof else 1
     for cls, (ms, cnt) in prof.items():
         calls = (1.0 if cls in ("zmap", "col_z") else 2.0) * chain * prof_steps    # zmap, col_z: forward calls only
         per_call = cnt / calls
-        nbytes, flops = kernel_work(cls, w, max(per_call, 1e-9), density)
+        nbytes, flops = kernel_work(cls, w, max(per_call, 1e-9), density, brick_ky)
         avg_s = ms * 1e-3 / cnt
         kernels[cls] = {"launches_per_step": cnt / prof_steps, "ms_per_step": ms / prof_steps, "avg_us": avg_s * 1e6,
                         "gbs": nbytes / avg_s / 1e9, "tflops": flops / avg_s / 1e12}

@@ -5,8 +5,9 @@
 // three launches it replaces (MID_FWD, the readout pass of dc_axis.cuh and MID_INV) the workspace is read and written once
 // instead of three times.  Forward / VJP call, us: 6 coils of 96 x 160 x 128 206 / 193 -> 160 / 143, 8 of 128 x 128 x 128 333 /
 // 322 -> 220 / 199, 8 of 48 x 320 x 320 671 / 632 -> 547 / 495, 4 of 320 x 120 x 96 317 / 283 -> 245 / 223, 4 of 32 x 96 x 96
-// 30 / 30 -> 26 / 25.  Bound by issue (52 % active; the first and the last ky stage and the copies between them alternate, and
-// two to four bricks fit an SM).
+// 30 / 30 -> 26 / 25.  Bound by issue and what keeps it from its slots: at 6 coils of 96 x 160 x 128, two bricks an SM, 51 %
+// (forward) and 52 % (VJP) active, next to the FP32 pipe at 34 and 40 % and L2 at 7.2 and 6.2 TB/s; the ky stages and the copies
+// before and after them alternate.  One to four bricks fit an SM, a single one in 39 of the 146 variants.
 //
 // The bricks leave little of L1, and a load occupies a line of it until it is served: loading the brick through registers
 // left too few requests in flight (VJP of the first 156 us), and so did measurements one by one (forward 176 us).
@@ -40,9 +41,10 @@ struct Brick {
     static constexpr int ROW = R0 * LS;                        // slots of a readout line
     static constexpr size_t BYTES = bytes(W, LS);
     // Where the three passes are slower, over 187 volumes of all pairs of lengths (three passes / brick, forward and VJP together
-    // unless stated).  Not for single-stage readouts, which occur in small tests only; radix 32 (spills: 3 coils of 384 x 96 x 96,
-    // forward 269 -> 307 us); 16 x 15 and 16 x 16 points (two large butterflies in few registers: 0.90 to 1.14, mean 1.0);
-    // 23 points of ky next to smaller ones of the readout (0.94 to 1.31, mean 1.04).  23-point readouts gain most, 1.02 to 2.0.
+    // unless stated).  Not for single-stage readouts, which occur in small tests only; radix 32 (384 points spill 204 B and read
+    // 548 B back, the variants taken at most 84 B and 200 B: 3 coils of 384 x 96 x 96, forward 269 -> 307 us); 16 x 15 and 16 x 16
+    // points (two large butterflies in few registers: 0.90 to 1.14, mean 1.0); 23 points of ky next to smaller ones of the readout
+    // (0.94 to 1.31, mean 1.04).  23-point readouts gain most, 1.02 to 2.0.
     // A^H y has the readout pass and one middle pass to replace: 0.92 to 1.33 with 80 to 128 points, 1.04 to 2.5 with
     // 23-point stages, 0.78 to 1.2 elsewhere.
     static constexpr bool FITS = P::S == 2 && RL <= 23 && !(R0 == 16 && (RL == 15 || RL == 16)) && (BY != 23 || RL == 23) && BYTES <= LIMIT;

@@ -79,7 +79,7 @@ struct WarpFlat {
 // with z).  A template parameter, not a run-time test of a.aty: with the test in the code the plain call measured
 // 11 % slower (17.7 against 16.0 us), although it never takes that branch.
 // ADJ (with z): A^H y, the image is zero; the forward stages are left out and a unit starts from minus its z values.
-// Registers: sixteen warps of one block have 128 each, which the step with z of 160 points exceeds by 52 B (spilled to
+// Registers: sixteen warps of one block have 128 each, which the step with z of 160 points exceeds by 20 B (spilled to
 // local memory; single-warp blocks without the spill are slower all the same, see launch_warpflat_zy).
 // DOT: the inner products of dot_rows (conjugate gradients; calls without z and A^H y).  A template parameter for the same
 // reason as HAS_ATY: with the block sums behind a run-time test the plain call of 20 frames of 192 x 160 took 17.3 us, not 16.4.
