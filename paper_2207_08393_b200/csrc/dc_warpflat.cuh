@@ -19,6 +19,12 @@
 namespace gleam {
 
 
+enum FlatForm {
+    FLAT_SINGLE = 0,     // one warp per block, blocks stride over the line groups
+    FLAT_SM = 1,         // one block of many warps per SM, a single round
+    FLAT_TAIL = 2        // blocks of four warps that stride over the groups; a block's warps share each group of the last, partial round
+};
+
 template <class P, bool HAS_Z, bool SMW = false>
 struct WarpFlat {
     static constexpr int N = P::N, R0 = P::R0, RL = P::RL;
@@ -72,6 +78,8 @@ struct WarpFlat {
 // coil sums are added in warp order through shared memory.  A quarter of the extra work lands on every scheduler.
 // One block per SM also keeps a dependent launch from moving in next to the running one warp by warp, which
 // would fill the schedulers unevenly.
+// FLAT_TAIL (several rounds, the last one nearly empty): blocks of four warps, each with groups of its own in the full rounds;
+// then a block's warps share one group after another as above.  The rule and its measurements: launch_warpflat_zy.
 // HAS_ATY: the coil sum is kept as aty - sum, starting from the given A^H y image as loaded (no instruction depends on
 // the load before the first inverse stage, so its latency is hidden even when a warp has a single group; the coil
 // terms are subtracted and the update adds eta times the result: the same bits as sum - aty, since rounding is
@@ -83,10 +91,12 @@ struct WarpFlat {
 // local memory; single-warp blocks without the spill are slower all the same, see launch_warpflat_zy).
 // DOT: the inner products of dot_rows (conjugate gradients; calls without z and A^H y).  A template parameter for the same
 // reason as HAS_ATY: with the block sums behind a run-time test the plain call of 20 frames of 192 x 160 took 17.3 us, not 16.4.
-template <class P, bool HAS_Z, bool SMW, bool HAS_ATY, bool ADJ, bool DOT>
-__global__ void __launch_bounds__(SMW ? 512 : 32, SMW ? 1 : WarpFlat<P, HAS_Z, SMW>::SINGLE_BLOCKS)
+template <class P, bool HAS_Z, int FORM, bool HAS_ATY, bool ADJ, bool DOT>
+__global__ void __launch_bounds__(FORM == FLAT_SM ? 512 : FORM == FLAT_TAIL ? 128 : 32,
+                                  FORM == FLAT_SM ? 1 : WarpFlat<P, HAS_Z, FORM == FLAT_SM>::SINGLE_BLOCKS / (FORM == FLAT_TAIL ? 4 : 1))
 warpflat_kernel(const RowArgs a, const int nwhole) {
     grid_dependency_wait();
+    constexpr bool SMW = FORM == FLAT_SM, TAIL = FORM == FLAT_TAIL;
     using WF = WarpFlat<P, HAS_Z, SMW>;
     constexpr int N = P::N, R0 = P::R0, RL = P::RL, LW = WF::LW, UPC = WF::UPC, US = WF::USTRIDE, SLOTS = WF::SLOTS;
     // Folded twiddles: plain and normal-equations calls 87 -> 85 and 88 -> 86 us (8 x 16 coils of 640 x 320), 30 -> 28 (8 x 8
@@ -104,10 +114,11 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
     cf* sK = wsm + WF::OFF_K;
     long long* sKo = reinterpret_cast<long long*>(wsm + WF::OFF_CNT);      // per line: offset of the z row of coil cbase
     int* sC = reinterpret_cast<int*>(wsm + WF::OFF_CNT + LW);              // per line: sampled entries (none in a line past the end)
-    const bool split = SMW && warp >= nwhole;                      // one of four warps that share a group
-    const int set = split ? (warp - nwhole) >> 2 : 0, q = split ? (warp - nwhole) & 3 : 0;
-    const int cbase = split ? q * a.C / 4 : 0;                     // first coil and number of coils of this warp
-    const int nc = split ? (q + 1) * a.C / 4 - cbase : a.C;
+    bool split = SMW && warp >= nwhole;                            // one of four warps that share a group
+    const int set = split ? (warp - nwhole) >> 2 : 0;
+    int q = split ? (warp - nwhole) & 3 : 0;
+    int cbase = split ? q * a.C / 4 : 0;                           // first coil and number of coils of this warp
+    int nc = split ? (q + 1) * a.C / 4 - cbase : a.C;
 
     const bool img = WF::LANES == 32 || lane < WF::LANES;
     const int l = img ? lane / RL : LW - 1, j = img ? lane % RL : 0;      // image-side identity: line of the warp, butterfly
@@ -122,14 +133,22 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
     // blocks on some SMs only, and the launches behind it in a chain keep that uneven split (enqueued calls, let in -> not: A^H y
     // and 6 steps of 3 x 9 coils of 384 x 256 136 -> 103 us, 5 prepared steps and VJPs of 2 x 16 of 512 x 384 378 -> 325, of 3 x 12
     // of 384 x 320 252 -> 218; equal elsewhere).
-    if (SMW || (!HAS_Z && (long long)gridDim.x >= ngroups)) grid_launch_dependents();
-    const int total = UPC * nc, rounds = (total + 31) / 32;
-    const long long g_first = !SMW ? (long long)blockIdx.x
+    if (SMW || (!TAIL && !HAS_Z && (long long)gridDim.x >= ngroups)) grid_launch_dependents();
+    int total = UPC * nc, rounds = (total + 31) / 32;
+    const long long g_first = TAIL ? 4LL * blockIdx.x + warp : !SMW ? (long long)blockIdx.x
                             : split ? (long long)(nwhole + set) * gridDim.x + blockIdx.x : (long long)warp * gridDim.x + blockIdx.x;
-    const long long g_step = !SMW ? (long long)gridDim.x : ngroups;              // SMW: a single round
+    long long g_step = SMW ? ngroups : TAIL ? 4LL * gridDim.x : (long long)gridDim.x;      // SMW: a single round
+    const long long g_whole = TAIL ? ngroups / g_step * g_step : ngroups;        // TAIL: groups of the full rounds
     if (SMW && DOT && a.dot_blocks && g_first >= ngroups && lane < 3) reinterpret_cast<double*>(sX)[lane] = 0.0;
 
-    for (long long g = g_first; g < ngroups; g += g_step) {
+    for (long long g = g_first; g < ngroups || (TAIL && !split); g += g_step) {
+        if (TAIL && !split && g >= g_whole) {            // from here on the block's four warps share a group
+            split = true;
+            q = warp; cbase = q * a.C / 4; nc = (q + 1) * a.C / 4 - cbase;
+            total = UPC * nc; rounds = (total + 31) / 32;
+            g = g_whole + blockIdx.x; g_step = gridDim.x;
+            if (g >= ngroups) break;
+        }
         const long long row = g * LW + l;
         const bool row_ok = img && row < a.nrows;
         const unsigned rowu = row_ok ? (unsigned)row : 0u;       // host side guarantees nrows < 2^31
@@ -346,6 +365,23 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
 #pragma unroll
                 for (int m = 0; m < R0; ++m) acc[m] = cadd(acc[m], o[m * 32 + lane]);
             }
+        }
+        if (TAIL && split) {
+            // as above; the second barrier: a warp's ring is free again once its sums have been read
+            if (q > 0) {
+#pragma unroll
+                for (int m = 0; m < R0; ++m) sE[m * 32 + lane] = acc[m];
+            }
+            __syncthreads();
+            if (q == 0) {
+                for (int w = 1; w < 4; ++w) {
+                    const cf* o = smem + w * WF::ELEMS + WF::OFF_E;
+#pragma unroll
+                    for (int m = 0; m < R0; ++m) acc[m] = cadd(acc[m], o[m * 32 + lane]);
+                }
+            }
+            __syncthreads();
+            if (q > 0) continue;
         }
         // ---- out = x - eta * sum, and Re<x, out>, <out, out> per row for the caller's inner products ----
         double dsum = 0.0, nsum = 0.0;

@@ -110,10 +110,10 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* le
     using WF = WarpFlat<P, HAS_Z, false>;
     static PerDevice attr_done;
     static PerDevice slots_cache;
-    cudaError_t e = ensure_smem(warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ, DOT>, WF::WARP_BYTES, attr_done);
+    cudaError_t e = ensure_smem(warpflat_kernel<P, HAS_Z, FLAT_SINGLE, HAS_ATY, ADJ, DOT>, WF::WARP_BYTES, attr_done);
     if (e != cudaSuccess) return e;
     int slots = 0;
-    if ((e = resident_slots(warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ, DOT>, 32, WF::WARP_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
+    if ((e = resident_slots(warpflat_kernel<P, HAS_Z, FLAT_SINGLE, HAS_ATY, ADJ, DOT>, 32, WF::WARP_BYTES, slots_cache, &slots)) != cudaSuccess) return e;
     const long long groups = (a.nrows + WF::LW - 1) / WF::LW;
     if (lets_in) *lets_in = !HAS_Z && groups <= slots;       // single-warp blocks; one block per SM: below
     if (groups <= 0) return cudaSuccess;
@@ -144,15 +144,36 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* le
                 b.dot_blocks = whole ? (int)(a.nrows / rows) : 0;
                 // the attribute is set once, to what the largest block of this kernel can ask for
                 constexpr size_t SMEM_CAP = 227 * 1024;
-                if ((e = ensure_smem(warpflat_kernel<P, HAS_Z, true, HAS_ATY, ADJ, DOT>, 16 * WS::WARP_BYTES < SMEM_CAP ? 16 * WS::WARP_BYTES : SMEM_CAP, attrs_done)) != cudaSuccess) return e;
-                return launch_overlapped(true, warpflat_kernel<P, HAS_Z, true, HAS_ATY, ADJ, DOT>, dim3((unsigned)sms), dim3(32 * warps), bytes, s, b, nwhole);
+                if ((e = ensure_smem(warpflat_kernel<P, HAS_Z, FLAT_SM, HAS_ATY, ADJ, DOT>, 16 * WS::WARP_BYTES < SMEM_CAP ? 16 * WS::WARP_BYTES : SMEM_CAP, attrs_done)) != cudaSuccess) return e;
+                return launch_overlapped(true, warpflat_kernel<P, HAS_Z, FLAT_SM, HAS_ATY, ADJ, DOT>, dim3((unsigned)sms), dim3(32 * warps), bytes, s, b, nwhole);
             }
         }
     }
     if (lets_in) return cudaSuccess;
+    // A last round that fills no more than a quarter of the warps: blocks of four warps that share each group of it, a quarter
+    // of the coils each (FLAT_TAIL).  Such a round costs a warp's whole run time however few groups it has: 4 x 15 coils of 640 x
+    // 368 are 1280 groups on 1184 warps, VJP 77.6 -> 63.6 us, and 2560 with z, prepared step 92 -> 84.  Where no more than 8
+    // warps are on an SM (368, 512, 640 points; 6 to 16 coils) it makes a VJP behind one full round 1.05-1.30 times as fast and a
+    // prepared step behind one to three 1.04-1.33.  With more warps an SM the single-warp blocks, which finish one by one, fill
+    // the last round themselves (VJP, 7 to 12 coils of 320 and 384 points, 0.82-0.93 times as fast in fours); only prepared steps
+    // gain there, 1.04-1.29 with 12 to 16 coils and a last round that is not too full (0.95-0.98 with fewer or more groups).
+    // Two groups a block: 368 points 1.09, most others slower.  A group of few units is one round whoever shares it.
+    constexpr bool FEW_WARPS = WF::SINGLE_BLOCKS <= 8;
+    if constexpr ((FEW_WARPS || HAS_Z) && 4 * WF::WARP_BYTES <= 227 * 1024) {
+        if (groups > slots && a.C >= (FEW_WARPS ? 6 : 12) && WF::UPC * a.C > 64) {
+            static PerDevice tail_attr_done, tail_cache;
+            constexpr size_t BYTES = 4 * WF::WARP_BYTES;
+            int resident = 0;
+            if ((e = ensure_smem(warpflat_kernel<P, HAS_Z, FLAT_TAIL, HAS_ATY, ADJ, DOT>, BYTES, tail_attr_done)) != cudaSuccess) return e;
+            if ((e = resident_slots(warpflat_kernel<P, HAS_Z, FLAT_TAIL, HAS_ATY, ADJ, DOT>, 128, BYTES, tail_cache, &resident)) != cudaSuccess) return e;
+            const long long full = groups / (4LL * resident), tail = groups % (4LL * resident);
+            if (4 * resident >= slots && tail > 0 && (FEW_WARPS ? tail <= resident : 5 * tail <= 3 * resident) && (full == 1 || (FEW_WARPS && HAS_Z)))
+                return launch_overlapped(true, warpflat_kernel<P, HAS_Z, FLAT_TAIL, HAS_ATY, ADJ, DOT>, dim3((unsigned)resident), dim3(128), BYTES, s, a, 4);
+        }
+    }
     long long blocks = groups;
     if (blocks > slots) blocks = slots;
-    return launch_overlapped(true, warpflat_kernel<P, HAS_Z, false, HAS_ATY, ADJ, DOT>, dim3((unsigned)blocks), dim3(32), WF::WARP_BYTES, s, a, 1);
+    return launch_overlapped(true, warpflat_kernel<P, HAS_Z, FLAT_SINGLE, HAS_ATY, ADJ, DOT>, dim3((unsigned)blocks), dim3(32), WF::WARP_BYTES, s, a, 1);
 }
 template <class P, bool HAS_Z>
 inline cudaError_t launch_warpflat_z(const RowArgs& a, cudaStream_t s, bool* lets_in) {

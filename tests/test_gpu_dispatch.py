@@ -5,6 +5,7 @@ import ctypes
 import pytest
 
 from oracle.oracle import MASK_READOUT_INVARIANT
+from tests.gpu_common import assert_close
 from tests.test_gpu_parity import problem
 from tests.test_gpu_tiles import check_all
 
@@ -107,6 +108,36 @@ def test_early_start_of_the_z_table(shape, early):
     assert len(tables) == 2 and len(launches) == 5
     assert launches[tables[1]]["early"] == early, launches[tables[1]]
     assert all(k["early"] for i, k in enumerate(launches) if i > 0 and i not in tables)
+
+
+# last round of the row kernel: groups shared by the four warps of a block (even and odd numbers of coils, one and two lines a
+# group, a last group with a line past the end, behind one and two full rounds), calls that keep single-warp blocks next to the lines
+@pytest.mark.parametrize("shape,shared", [
+    ((4, 6, 1, 640, 368), ("vjp", "aty", "prepared", "adjoint")),       # 1280 groups of two lines and 2560 of one, 1184 warps
+    ((2, 13, 1, 640, 512), ("vjp", "aty", "prepared")),                 # 1280 groups, weighted mask (A^H y: more warps an SM)
+    ((7, 6, 1, 368, 512), ("prepared",)),                               # 2576 groups: two full rounds
+    ((2, 7, 3, 320, 640), ()),                                          # 1920 groups: three a block
+    ((2, 7, 1, 640, 640), ("vjp", "aty", "prepared", "adjoint")),       # 1280 groups
+    ((4, 5, 1, 640, 368), ()),                                          # too few coils
+    ((27, 12, 3, 46, 256), ("prepared", "adjoint")),                    # 1863 groups of two lines, 1776 warps
+    ((23, 13, 5, 46, 96), ("prepared",)),                               # 2645 groups, 2368 warps
+    ((27, 10, 3, 46, 256), ())])                                        # too few coils for 12 warps an SM
+def test_last_round_of_the_row_kernel(oracle, shape, shared):
+    import torch
+    B, C, T, n1, n2 = shape
+    d, x, y, sens, mask = problem(2, B, C, T, (1, n1, n2), MASK_READOUT_INVARIANT, weighted=(C == 13), seed=sum(shape), density=0.3)
+    check_all(oracle, d, x, y, sens, mask, 0.9, "%s" % (shape,))
+    dc, tx, ty, ts, tm = holder(shape)
+    zero = torch.zeros_like(tx)
+    for name, fn in (("vjp", lambda: dc.vjp(tx, ts, tm, 1.0)), ("aty", lambda: dc.forward_aty(tx, zero, ts, tm, 1.0)),
+                     ("prepared", lambda: dc.forward_prepared(tx, ty, ts, tm, 1.0)), ("adjoint", lambda: dc.adjoint(ty, ts, tm))):
+        row = [k for k in captured(fn) if "warpflat_kernel" in k["name"] or "warpline_kernel" in k["name"]][-1]
+        assert (row["threads"] == 128) == (name in shared), (name, row)
+    dev = torch.device("cuda:0")
+    t = [torch.from_numpy(a).to(dev) for a in (x, y, sens, mask)]
+    aty = dc.adjoint(t[1], t[2], t[3])
+    got = dc.forward_aty(t[0], aty, t[2], t[3], 0.9).cpu().numpy()
+    assert_close(got, oracle.dc_forward(x, y, sens, mask, 0.9, d, nthreads=8), x, "%s normal equations" % (shape,))
 
 
 # z table: more sampled tiles than blocks (a block walks over several, also with the last tile part full) and fewer, one-, two-

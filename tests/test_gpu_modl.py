@@ -175,7 +175,8 @@ def test_error_codes():
     ((2, 2, 11, 160, 160), 384, True),        # 1760 groups, 12 per SM
     ((3, 3, 5, 160, 160), 288, True),         # 1200 groups, 9 per SM, too few coils to split
     ((4, 3, 8, 80, 160), 288, True),          # four examples: a sum per row, 640 of them
-    ((3, 4, 31, 46, 48), 256, False)])        # 1070 groups of four lines, 1426 rows per example
+    ((3, 4, 31, 46, 48), 256, False),         # 1070 groups of four lines, 1426 rows per example
+    ((2, 6, 1, 640, 512), 128, True)])       # 1280 groups on 1184 warps: the last ones by four warps each
 def test_sums_of_the_operator_and_examples_of_unlike_scale(oracle, shape, threads, dealt):
     import torch
     import paper_2207_08393_b200 as g
