@@ -38,6 +38,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 namespace gleam {
 
@@ -173,17 +174,16 @@ __global__ void __launch_bounds__(CG_THREADS) cg_dot_kernel(const CgArgs a) {
     }
 }
 
-// CG_BATCH elements of every vector are requested before the sums are formed, so that their latency covers that of the sums.
-constexpr int CG_BATCH = 2;
-template <bool FROM_ROWS, bool DEALT, bool LAST>
-__global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) {
+// BATCH elements of every vector are requested before the sums are formed, so that their latency covers that of the sums.
+template <bool FROM_ROWS, bool DEALT, bool LAST, int BATCH>
+__global__ void __launch_bounds__(CG_THREADS, BATCH == 2 ? 4 : BATCH == 3 ? 3 : 2) cg_step_kernel(const CgArgs a) {
     grid_dependency_wait();
     const long long base = (long long)blockIdx.y * a.ne2, stride = (long long)gridDim.x * CG_THREADS;
     long long i = (long long)blockIdx.x * CG_THREADS + threadIdx.x;
-    float4 pv[CG_BATCH], xv[CG_BATCH], qv[LAST ? 1 : CG_BATCH], rv[LAST ? 1 : CG_BATCH];
+    float4 pv[BATCH], xv[BATCH], qv[LAST ? 1 : BATCH], rv[LAST ? 1 : BATCH];
     auto fetch = [&]() {
 #pragma unroll
-        for (int e = 0; e < CG_BATCH; ++e) {
+        for (int e = 0; e < BATCH; ++e) {
             const long long at = base + i + e * stride;
             if (i + e * stride >= a.ne2) break;
             pv[e] = a.p[at]; xv[e] = a.x[at];
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) 
     double acc = 0.0;
     while (i < a.ne2) {
 #pragma unroll
-        for (int e = 0; e < CG_BATCH; ++e) {
+        for (int e = 0; e < BATCH; ++e) {
             const long long at = base + i + e * stride;
             if (i + e * stride >= a.ne2) break;
             a.x[at] = axpy4(af, pv[e], xv[e]);
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(CG_THREADS, 4) cg_step_kernel(const CgArgs a) 
                 acc += norm2(r);
             }
         }
-        i += CG_BATCH * stride;
+        i += BATCH * stride;
         fetch();
     }
     if (LAST) return;
@@ -333,17 +333,22 @@ static int modl_cg(const void* z, const void* y, const void* sens, const float* 
 
     // the operator's own argument checks (y, sens, mask) before anything is enqueued
     CGRUN(run(ws + L.off_r, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ALL, dot_rows, true, 0, nullptr, &a.dot_count));
-    // Four elements a thread, or two where that is one block per SM, or a round of blocks (a few more) that have few sums to
-    // add at their start, unless four are one block per SM already (those come in while the operator drains).  10 steps, four
-    // -> two: 8 coils x 16 frames of 64 x 64 99 -> 90 us, 20 of 192 x 160 (a sum per block) 259 -> 250, 2 x 6 x 12 of 128 x 128
-    // 186 -> 160; but 3 x 5 x 8 of 128 x 96 128 -> 136 (144 -> 288 blocks), 4 x 15 of 640 x 368 900 -> 910 (920 blocks).
-    auto blocks_of = [&](int each) {
-        const long long n = (L.ne2 + (long long)CG_THREADS * each - 1) / ((long long)CG_THREADS * each);
-        return n < 1 ? 1 : n > CG_MAX_BLOCKS ? CG_MAX_BLOCKS : n;
-    };
-    const long long fine = blocks_of(2) * L.B, coarse = blocks_of(4) * L.B, one = CG_MAX_BLOCKS / 4;
-    const bool two = fine <= one || (coarse > one && (!from_rows || a.dot_count <= CG_DEALT) && fine <= 5 * one);
-    const dim3 grid((unsigned)blocks_of(two ? 2 : 4), (unsigned)L.B);
+    // Elements a thread of the vector launches, and how many of them a step requests at once.  All of them where that is one
+    // round of resident blocks: a thread that comes back for a few more waits for memory once more after the sums (20 frames of
+    // 192 x 160: 4096 of 307,200 elements were left over by 592 blocks of two a thread; 10 steps 240 -> 227 us with three).  Two
+    // while the blocks are one per SM, then four (two blocks per SM), three (three) and, beyond that, four in two rounds.
+    // Measured against two and four elements in rounds of two, 10 steps: 5 coils of 384 x 640 251 -> 219, of 640 x 320 129 -> 119,
+    // 6 x 18 of 384 x 80 220 -> 203, 3 x 5 of 320 x 256 135 -> 125, 8 x 24 x 3 of 64 x 128 203 -> 199; 4 x 4 of 92 x 640 209 -> 213.
+    // Where the operator sums per block (one block of many warps per SM) and the step is no more than a block per SM, those
+    // of fewer registers come in while the operator drains: two at once (3 x 5 x 8 of 128 x 96 119 against 125).
+    auto blocks_of = [&](int each) { const long long n = (L.ne2 + (long long)CG_THREADS * each - 1) / ((long long)CG_THREADS * each); return n < 1 ? 1 : n; };
+    const long long one = CG_MAX_BLOCKS / 4;                 // a block per SM
+    const bool sums_per_block = from_rows && a.dot_count != a.rows_per_example;
+    int each = 4, batch = 2;
+    if (blocks_of(2) * L.B <= one) each = batch = 2;
+    else if (blocks_of(4) * L.B <= 2 * one) batch = (sums_per_block && blocks_of(4) * L.B <= one) ? 2 : 4;
+    else if (blocks_of(3) * L.B <= 3 * one) each = batch = 3;
+    const dim3 grid((unsigned)(blocks_of(each) < CG_MAX_BLOCKS ? blocks_of(each) : CG_MAX_BLOCKS), (unsigned)L.B);
     if (y) {
         CGRUN(run(nullptr, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ADJOINT));
         CGCK(prof_mark(GLEAM_K_CG_VEC, s));
@@ -361,9 +366,13 @@ static int modl_cg(const void* z, const void* y, const void* sens, const float* 
             CGCK(launch_overlapped(true, cg_dot_kernel, grid, dim3(CG_THREADS), 0, s, a));
         }
         CGCK(prof_mark(GLEAM_K_CG_VEC, s));
-        auto step = !from_rows ? (last ? cg_step_kernel<false, true, true> : cg_step_kernel<false, true, false>)
-                  : a.dot_count <= CG_DEALT ? (last ? cg_step_kernel<true, true, true> : cg_step_kernel<true, true, false>)
-                                            : (last ? cg_step_kernel<true, false, true> : cg_step_kernel<true, false, false>);
+        auto pick = [&](auto n) {
+            constexpr int N = decltype(n)::value;
+            return !from_rows ? (last ? cg_step_kernel<false, true, true, N> : cg_step_kernel<false, true, false, N>)
+                 : a.dot_count <= CG_DEALT ? (last ? cg_step_kernel<true, true, true, N> : cg_step_kernel<true, true, false, N>)
+                                           : (last ? cg_step_kernel<true, false, true, N> : cg_step_kernel<true, false, false, N>);
+        };
+        auto step = batch == 4 ? pick(std::integral_constant<int, 4>{}) : batch == 3 ? pick(std::integral_constant<int, 3>{}) : pick(std::integral_constant<int, 2>{});
         CGCK(launch_overlapped(true, step, grid, dim3(CG_THREADS), 0, s, a));
         CGCK(cudaGetLastError());
     }

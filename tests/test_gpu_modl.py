@@ -203,6 +203,24 @@ def test_sums_of_the_operator_and_examples_of_unlike_scale(oracle, shape, thread
     assert all("cg_step_kernelILb1ELb%d" % dealt in k["name"] for k in steps), steps[0]
 
 
+# vector launches: two, four and three elements a thread at once, four in rounds of two; blocks that are full, nearly empty and part
+# full at the end, several examples
+@pytest.mark.parametrize("shape,blocks", [
+    ((1, 2, 1, 46, 46), 3), ((2, 2, 2, 184, 192), 138), ((1, 2, 3, 320, 160), 75), ((3, 3, 1, 320, 256), 120), ((1, 2, 18, 192, 160), 270),
+    ((1, 2, 20, 192, 160), 400), ((1, 2, 22, 192, 160), 440), ((1, 2, 23, 192, 160), 345), ((1, 2, 24, 320, 192), 592)])
+def test_vector_launches(oracle, shape, blocks):
+    import torch
+    import paper_2207_08393_b200 as g
+    from tests.test_gpu_dispatch import captured
+    B, C, T, n1, n2 = shape
+    d, z, y, sens, mask = problem(2, B, C, T, (1, n1, n2), MASK_READOUT_INVARIANT, seed=sum(shape), density=0.3)
+    close(run_gpu_modl(z, y, sens, mask, 0.5, 3, 2, 0, MASK_READOUT_INVARIANT), oracle.modl_cg_forward(z, y, sens, mask, 0.5, 3, d, nthreads=8), "%s solve" % (shape,))
+    cg = g.ModlCG(B, C, T, 2, (1, n1, n2))
+    tz, ts, tm = (torch.from_numpy(a).to("cuda:0") for a in (z, sens, mask))
+    steps = [k for k in captured(lambda: cg.solve_vjp(tz, ts, tm, 0.5)) if "cg_step_kernel" in k["name"]]
+    assert len(steps) == 10 and all(k["blocks"] == blocks for k in steps), steps[0]
+
+
 def textbook_steps(z, sens, mask, mu, n_iter, dtype):
     """Textbook conjugate gradients on the VJP's system in numpy, vectors in ``dtype``, scalars in double; one coil
     expansion, transforms along the last axis only (a readout-invariant mask).  All iterates."""
