@@ -60,7 +60,13 @@ struct Tile {
     // sum are kept over the coil loop next to a butterfly (a prime radix also holds its sums and differences).
     // A block has a thread per column, so 640-point rows have at most 96 registers and spill up to 180 B whatever the bound.
     static constexpr bool PRIME = RMAX > 4 && RMAX % 2 == 1 && smallest_odd_factor(RMAX) == RMAX;
-    static constexpr int REGS = 2 * RY + (PRIME ? 4 : 2) * RMAX + 16;
+    // The outputs of a prime radix are stored as they are formed on long rows (8 coils of 96 x 240 x 368 807 -> 804 us, 12 of 96 x
+    // 240 x 184 493 -> 488; but 128 x 92 x 92 125 -> 129).  A bound without room for them spills all the same (up to 80 B); more
+    // blocks outweigh that where few image rows are kept and blocks are large: VJP of 8 coils, us, 128 x 92 x 184 283 -> 234,
+    // 128 x 92 x 368 602 -> 485, 256 x 46 x 184 361 -> 325, 4 slices of 92 x 184 23.6 -> 18.9; not with 16 rows (up to 244 B; 128 x
+    // 256 x 92 239 -> 264, 128 x 96 x 184 193 -> 202) nor on short rows (24 x 92 x 92, 4 coils, 17.8 -> 18.8).
+    static constexpr bool EARLY = NZ >= 184, TIGHT = PRIME && RY <= 4 && EARLY;
+    static constexpr int REGS = 2 * RY + (PRIME && !TIGHT ? 4 : 2) * RMAX + (TIGHT ? 24 : 16);
     static constexpr int blocks(size_t bytes) {
         const int n = cmin(16, cmin((int)(LIMIT / (bytes + 1024)), 65536 / (TH * ((REGS + 7) / 8 * 8))));
         return cmax(1, cmin(n, 2048 / TH));
@@ -177,10 +183,8 @@ tile_fwd_kernel(const TileArgs a) {
                 cf u[RL];
 #pragma unroll
                 for (int m = 0; m < RL; ++m) u[m] = e[m];
-                Dft<RL, -1, true>::run(u);
                 cf* o = Vp + row * a.v_k0 + j;
-#pragma unroll
-                for (int k = 0; k < RL; ++k) o[R0 * k] = u[k];
+                dft_emit<RL, -1, true, TL::EARLY>(u, [&](auto k, cf x) { o[R0 * decltype(k)::value] = x; });
             }
         }
     }
@@ -226,9 +230,7 @@ tile_inv_kernel(const TileArgs a) {
                 cf u[RL];
 #pragma unroll
                 for (int k = 0; k < RL; ++k) u[k] = o[R0 * k];
-                Dft<RL, +1, true>::run(u);
-#pragma unroll
-                for (int m = 0; m < RL; ++m) e[m] = u[m];
+                dft_emit<RL, +1, true, TL::EARLY>(u, [&](auto m, cf x) { e[decltype(m)::value] = x; });
             }
             __syncthreads();
             if (TL::ONE_STAGE) stage_rows<NZ, RY>(sS, sp + c * s_stride, row_stride);

@@ -156,12 +156,13 @@ template <int DIR, bool FOLD> struct Dft<4, DIR, FOLD> {
     }
 };
 
-// odd prime P: symmetric direct evaluation
+// odd prime P: symmetric direct evaluation.  emit: every output goes to f(k, X[k]) as soon as it is formed, so that the
+// outputs take no registers next to the sums and differences of the inputs.
 template <int P, int DIR> struct DftPrime {
-    static GLEAM_HD void run(cf (&v)[P]) {
+    template <class F> static GLEAM_HD void emit(const cf (&v)[P], F&& f) {
         constexpr int H = (P - 1) / 2;
         cf a[H], b[H];
-        cf x0 = v[0];
+        const cf x0 = v[0];
         cf sum = x0;
         static_for<0, H>([&](auto mi) {
             constexpr int m = decltype(mi)::value + 1;
@@ -169,7 +170,7 @@ template <int P, int DIR> struct DftPrime {
             b[m - 1] = csub(v[m], v[P - m]);
             sum = cadd(sum, a[m - 1]);
         });
-        v[0] = sum;
+        f(IC<0>{}, sum);
         static_for<0, H>([&](auto ki) {
             constexpr int k = decltype(ki)::value + 1;
             cf C = x0, D = make_float2(0.f, 0.f);
@@ -181,15 +182,12 @@ template <int P, int DIR> struct DftPrime {
                 D = caxpy(s, b[m - 1], D);
             });
             // X[k] = C + DIR * i * D ,  X[P-k] = C - DIR * i * D
-            if (DIR > 0) {
-                v[k] = make_float2(C.x - D.y, C.y + D.x);
-                v[P - k] = make_float2(C.x + D.y, C.y - D.x);
-            } else {
-                v[k] = make_float2(C.x + D.y, C.y - D.x);
-                v[P - k] = make_float2(C.x - D.y, C.y + D.x);
-            }
+            const cf p = make_float2(C.x - D.y, C.y + D.x), q = make_float2(C.x + D.y, C.y - D.x);
+            f(IC<k>{}, DIR > 0 ? p : q);
+            f(IC<P - k>{}, DIR > 0 ? q : p);
         });
     }
+    static GLEAM_HD void run(cf (&v)[P]) { emit(v, [&](auto k, cf x) { v[decltype(k)::value] = x; }); }
 };
 
 // composite R = A * B, decimation in time:  n = A n2 + n1,  k = k2 + B k1
@@ -326,5 +324,14 @@ template <int R, int DIR, bool FOLD> struct Dft {
         else DftComposite<R, DIR>::run(v);
     }
 };
+
+// the transform of v, every output to f(k, X[k]); v is used up.  EARLY: those of a prime radix as they are formed
+template <int R, int DIR, bool FOLD, bool EARLY, class F> GLEAM_HD void dft_emit(cf (&v)[R], F&& f) {
+    if constexpr (EARLY && R > 4 && R % 2 == 1 && smallest_odd_factor(R) == R) DftPrime<R, DIR>::emit(v, f);
+    else {
+        Dft<R, DIR, FOLD>::run(v);
+        static_for<0, R>([&](auto k) { f(k, v[decltype(k)::value]); });
+    }
+}
 
 }  // namespace gleam

@@ -35,6 +35,15 @@ def test_slices_with_an_arbitrary_mask(oracle, n, coils):
     check_all(oracle, d, x, y, sens, mask, 0.9, "slice %s" % (n,))
 
 
+# 23-point rows: outputs stored as they are formed (long rows) or after the butterfly, few and many rows a block
+@pytest.mark.parametrize("n", [(4, 92, 184), (2, 46, 368), (6, 20, 184), (2, 92, 92), (2, 64, 184), (2, 92, 46), (2, 240, 184), (1, 92, 368), (1, 6, 184)])
+def test_rows_of_23_points(oracle, n):
+    rank = 3 if n[0] > 1 else 2
+    for kind in (MASK_READOUT_INVARIANT, MASK_FULL) if rank == 3 else (MASK_FULL,):
+        d, x, y, sens, mask = problem(rank, 1, 3, 1, n, kind, seed=sum(n), density=0.3)
+        check_all(oracle, d, x, y, sens, mask, 0.9, "rows of 23 points %s" % (n,))
+
+
 # middle radix 16 with full blocks: weights and measurements take 48 KB of shared memory, the twiddles come on top
 @pytest.mark.parametrize("n", [(1, 160, 240), (1, 256, 256), (1, 160, 512)])
 def test_slices_whose_middle_pass_takes_48_kb(oracle, n):
