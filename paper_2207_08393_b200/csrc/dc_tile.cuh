@@ -36,18 +36,33 @@ struct Tile {
     static constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, S = PZ::S;
     static constexpr int BF0 = PZ::BF0;                      // butterflies per row of the first kz stage
     static constexpr int LS1 = PZ::LS1;                      // odd run length: the second stage reads without bank conflicts
-    // Slots of a row in the exchange tile.  Congruent to BF0 modulo 16: threads take the butterflies of the first kz stage row
+    static constexpr int TH = ((NZ + 31) / 32) * 32;         // one thread per kz column
+    static constexpr int RMAX = cmax(RY, cmax(R0, RL));
+    static constexpr bool PRIME = RMAX > 4 && RMAX % 2 == 1 && smallest_odd_factor(RMAX) == RMAX;
+    // The outputs of a prime radix are stored as they are formed on long rows (8 coils of 96 x 240 x 368 807 -> 804 us, 12 of 96 x
+    // 240 x 184 493 -> 488; but 128 x 92 x 92 125 -> 129).  A bound without room for them spills all the same (up to 80 B); more
+    // blocks outweigh that where few image rows are kept and blocks are large: VJP of 8 coils, us, 128 x 92 x 184 283 -> 234,
+    // 128 x 92 x 368 602 -> 485, 256 x 46 x 184 361 -> 325, 4 slices of 92 x 184 23.6 -> 18.9; not with 16 rows (up to 244 B; 128 x
+    // 256 x 92 239 -> 264, 128 x 96 x 184 193 -> 202) nor on short rows (24 x 92 x 92, 4 coils, 17.8 -> 18.8).
+    static constexpr bool EARLY = NZ >= 184, TIGHT = PRIME && RY <= 4 && EARLY;
+    // Threads per row in the first kz stage.  Half warps of 23 butterflies a row met on one bank where they cross to the next row, in
+    // every read and write of the stage; with a thread left out per row, and rows congruent to 24 modulo 16, they do not.  VJP of
+    // 12 coils of 96 x 240 x 184 490 -> 476 us, of 8 of 96 x 240 x 368 804 -> 781.
+    static constexpr int BFP = RL == 23 && R0 >= 8 ? 24 : BF0;
+    // A thread whose butterflies all have one place in their rows keeps their twiddles: 476 -> 458 and 781 -> 772 us, 4 slices of
+    // 320 x 384 77 -> 74, 8 coils of 128 x 160 x 64 90 -> 87.  Where registers admit it: not 10- and 12-point stages next to short
+    // ones (64 x 96 rows of 96 46.9 -> 51.1, 128 x 240 of 160 347 -> 357), nor 512 points (320 x 512 94 -> 95).
+    static constexpr bool OWN_TW = S == 2 && TH % BFP == 0 && (R0 <= 8 || (RL >= 23 && NZ <= 384)) && !TIGHT;
+    // Slots of a row in the exchange tile.  Congruent to BFP modulo 16: threads take the butterflies of the first kz stage row
     // after row, and each then has the bank of its thread number.  With rows of R0 runs (odd, packed) two rows of a half warp
     // met on the same banks in its reads and writes.  Packed -> congruent, VJP call, us: 8 coils of 64 x 128 x 128 79.9 -> 73.2,
     // 96 x 96 x 96 76.7 -> 72.0, 64 x 240 x 192 226 -> 217, 48 x 320 x 240 281 -> 272, 48 x 320 x 320 386 -> 375.
     // Not for short rows and first radices below 8, where the second stage crosses rows more often than that
-    // gains: 64 x 92 x 92 62.7 -> 63.9, 80 x 64 x 46 40.8 -> 41.8, 64 x 96 x 40 30.1 -> 30.2.  Nor for 23-point stages: forward of
-    // 15 coils of 128 x 160 x 184 746 -> 793, of 14 of 24 x 24 x 368 76 -> 81.
+    // gains: 64 x 92 x 92 62.7 -> 63.9, 80 x 64 x 46 40.8 -> 41.8, 64 x 96 x 40 30.1 -> 30.2.  (Rows of 23-point
+    // stages congruent to 23 were slower, too: forward of 15 coils of 128 x 160 x 184 746 -> 793.)
     static constexpr int PACKED = R0 * LS1;
-    static constexpr int ROW = S != 2 ? NZ : (R0 < 8 || NZ < 64 || RL == 23) ? PACKED : PACKED + ((BF0 - PACKED) % 16 + 16) % 16;
-    static constexpr int TH = ((NZ + 31) / 32) * 32;         // one thread per kz column
-    static constexpr int T_ELEMS = (RY * ROW + 1) / 2 * 2, STAGE = RY * NZ, TW = (S == 2) ? NZ : 0;
-    static constexpr int RMAX = cmax(RY, cmax(R0, RL));
+    static constexpr int ROW = S != 2 ? NZ : (R0 < 8 || NZ < 64) ? PACKED : PACKED + ((BFP - PACKED) % 16 + 16) % 16;
+    static constexpr int T_ELEMS = (RY * ROW + 1) / 2 * 2, STAGE = RY * NZ, TW = (S == 2 && !OWN_TW) ? NZ : 0;
     static constexpr int slot(int kz) { return (S == 2) ? (kz / BF0) * LS1 + kz % BF0 : kz; }
     static constexpr size_t LIMIT = 227 * 1024;
     static constexpr size_t FWD_BYTES = sizeof(cf) * (T_ELEMS + STAGE + TW);
@@ -59,13 +74,6 @@ struct Tile {
     // The register bound lets the blocks that shared memory admits be resident.  RY values of the image or of the coil
     // sum are kept over the coil loop next to a butterfly (a prime radix also holds its sums and differences).
     // A block has a thread per column, so 640-point rows have at most 96 registers and spill up to 180 B whatever the bound.
-    static constexpr bool PRIME = RMAX > 4 && RMAX % 2 == 1 && smallest_odd_factor(RMAX) == RMAX;
-    // The outputs of a prime radix are stored as they are formed on long rows (8 coils of 96 x 240 x 368 807 -> 804 us, 12 of 96 x
-    // 240 x 184 493 -> 488; but 128 x 92 x 92 125 -> 129).  A bound without room for them spills all the same (up to 80 B); more
-    // blocks outweigh that where few image rows are kept and blocks are large: VJP of 8 coils, us, 128 x 92 x 184 283 -> 234,
-    // 128 x 92 x 368 602 -> 485, 256 x 46 x 184 361 -> 325, 4 slices of 92 x 184 23.6 -> 18.9; not with 16 rows (up to 244 B; 128 x
-    // 256 x 92 239 -> 264, 128 x 96 x 184 193 -> 202) nor on short rows (24 x 92 x 92, 4 coils, 17.8 -> 18.8).
-    static constexpr bool EARLY = NZ >= 184, TIGHT = PRIME && RY <= 4 && EARLY;
     static constexpr int REGS = 2 * RY + (PRIME && !TIGHT ? 4 : 2) * RMAX + (TIGHT ? 24 : 16);
     static constexpr int blocks(size_t bytes) {
         const int n = cmin(16, cmin((int)(LIMIT / (bytes + 1024)), 65536 / (TH * ((REGS + 7) / 8 * 8))));
@@ -121,7 +129,7 @@ __global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY>::blocks(Tile<PZ
 tile_fwd_kernel(const TileArgs a) {
     grid_dependency_wait();
     using TL = Tile<PZ, RY>;
-    constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
+    constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, BFP = TL::BFP, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
     extern __shared__ __align__(16) float2 smem[];
     cf* sT = smem;
     cf* sS = smem + TL::T_ELEMS;
@@ -134,7 +142,13 @@ tile_fwd_kernel(const TileArgs a) {
     const cf* sp = a.sens + ((long long)(id.b * a.C) * a.Ts + (a.Ts > 1 ? id.t : 0)) * V3 + row_elems;
     const long long s_stride = (long long)a.Ts * V3;
     if (id.c0 < id.c1) stage_rows<NZ, RY>(sS, sp + id.c0 * s_stride, row_stride);
-    if (TL::S == 2) for (int i = tid; i < NZ; i += TH) sTw[i] = unit_root_fwd<NZ>(((i / BF0) * (i % BF0)) % NZ);
+    if (TL::S == 2 && !TL::OWN_TW) for (int i = tid; i < NZ; i += TH) sTw[i] = unit_root_fwd<NZ>(((i / BF0) * (i % BF0)) % NZ);
+    cf tw[TL::OWN_TW ? R0 : 1];
+    if (TL::OWN_TW) {
+#pragma unroll
+        for (int k = 1; k < (TL::OWN_TW ? R0 : 1); ++k) tw[k] = unit_root_fwd<NZ>((k * (tid % BFP)) % NZ);
+    }
+    auto twiddle = [&](int k, int j) -> cf { return TL::OWN_TW ? tw[TL::OWN_TW ? k : 0] : sTw[k * BF0 + j]; };
     cf xv[RY];
 #pragma unroll
     for (int m = 0; m < RY; ++m)
@@ -157,8 +171,9 @@ tile_fwd_kernel(const TileArgs a) {
         cf* Vp = a.V + unit * a.v_unit + id.gi * a.v_slab + id.j * a.v_j;
         // first kz stage, in place: butterfly j of a row reads and writes the slots {k * LS1 + j}
 #pragma unroll 1
-        for (int t = tid; t < RY * BF0; t += TH) {
-            const int row = t / BF0, j = t - row * BF0;
+        for (int t = tid; t < RY * BFP; t += TH) {
+            const int row = t / BFP, j = t - row * BFP;
+            if (BFP != BF0 && j >= BF0) continue;
             cf* e = sT + row * ROW + j;
             cf v[R0];
 #pragma unroll
@@ -166,7 +181,7 @@ tile_fwd_kernel(const TileArgs a) {
             Dft<R0, -1, true>::run(v);
             if (TL::S == 2) {
 #pragma unroll
-                for (int k = 0; k < R0; ++k) e[k * LS1] = (k == 0) ? v[0] : cmul(v[k], sTw[k * BF0 + j]);
+                for (int k = 0; k < R0; ++k) e[k * LS1] = (k == 0) ? v[0] : cmul(v[k], twiddle(k, j));
             } else {
                 cf* o = Vp + row * a.v_k0;
 #pragma unroll
@@ -196,7 +211,7 @@ __global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY>::blocks(Tile<PZ
 tile_inv_kernel(const TileArgs a) {
     grid_dependency_wait();
     using TL = Tile<PZ, RY>;
-    constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
+    constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, BFP = TL::BFP, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
     extern __shared__ __align__(16) float2 smem[];
     cf* sT = smem;
     cf* sV = smem + TL::T_ELEMS;
@@ -211,7 +226,13 @@ tile_inv_kernel(const TileArgs a) {
     const long long s_stride = (long long)a.Ts * V3, x_off = id.bt * V3 + row_elems + tid;
     auto v_ptr = [&](int c) { return a.V + (((long long)(id.b * a.C + c)) * a.T + id.t) * a.v_unit + id.gi * a.v_slab + id.j * a.v_j; };
     if (id.c0 < id.c1) stage_rows<NZ, RY>(sV, v_ptr(id.c0), a.v_k0);
-    if (TL::S == 2) for (int i = tid; i < NZ; i += TH) sTw[i] = unit_root_fwd<NZ>(((i / BF0) * (i % BF0)) % NZ);
+    if (TL::S == 2 && !TL::OWN_TW) for (int i = tid; i < NZ; i += TH) sTw[i] = unit_root_fwd<NZ>(((i / BF0) * (i % BF0)) % NZ);
+    cf tw[TL::OWN_TW ? R0 : 1];
+    if (TL::OWN_TW) {
+#pragma unroll
+        for (int k = 1; k < (TL::OWN_TW ? R0 : 1); ++k) tw[k] = unit_root_fwd<NZ>((k * (tid % BFP)) % NZ);
+    }
+    auto twiddle = [&](int k, int j) -> cf { return TL::OWN_TW ? tw[TL::OWN_TW ? k : 0] : sTw[k * BF0 + j]; };
     cf acc[RY];
 #pragma unroll
     for (int m = 0; m < RY; ++m)
@@ -237,12 +258,13 @@ tile_inv_kernel(const TileArgs a) {
             else if (c + 1 < id.c1) stage_rows<NZ, RY>(sV, v_ptr(c + 1), a.v_k0);
             else cp_async_commit();
 #pragma unroll 1
-            for (int t = tid; t < RY * BF0; t += TH) {
-                const int row = t / BF0, j = t - row * BF0;
+            for (int t = tid; t < RY * BFP; t += TH) {
+                const int row = t / BFP, j = t - row * BFP;
+                if (BFP != BF0 && j >= BF0) continue;
                 cf* e = sT + row * ROW + j;
                 cf v[R0];
 #pragma unroll
-                for (int k = 0; k < R0; ++k) { const cf r = e[k * LS1]; v[k] = (k == 0) ? r : cmulc(r, sTw[k * BF0 + j]); }
+                for (int k = 0; k < R0; ++k) { const cf r = e[k * LS1]; v[k] = (k == 0) ? r : cmulc(r, twiddle(k, j)); }
                 Dft<R0, +1, true>::run(v);
 #pragma unroll
                 for (int m = 0; m < R0; ++m) e[m * LS1] = v[m];
