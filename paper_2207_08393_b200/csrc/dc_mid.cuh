@@ -21,8 +21,8 @@ struct MidArgs {
     cf* V; long long v_unit, v_slab, v_k0, v_j;
     const float* mask;                        // MID_SEP*: (B,T,N1,NZ); MID_FULL*, MID_GRADY: (B,T,N1,NZ) or (B,T,NZ)
     int mask_row;                             // MID_GRADY: the mask has one row per (b,t)
-    const cf* zin; const int* zidx;           // compact z table and rank map
-    const float* m2c; const int* zstart;      // squared mask weights by rank; (B,T,33) first rank of each k0 group
+    const cf* zin; const int* zidx;           // compact z table; ranks inside the k0 group, -1 where nothing was sampled
+    const float* m2c; const int* zstart;      // squared mask weights by rank, times scale2; (B,T,33) first rank of each k0 group
     const cf* y; cf* ky_out;
     float scale, scale2;                      // g / sqrt(N1 NZ) (times eta: MID_GRADY), 1 / (N1 NZ)
     int C, T, n0, G, i0_start, NZ, zcap;
@@ -74,11 +74,15 @@ mid_kernel(const MidArgs a) {
     };
 
     // The z values of this block's ky group are contiguous in the compact table (ranks zstart[k0] .. zstart[k0+1]);
-    // they are staged in shared memory while the transform runs, with their scaled squared mask weights.  Slot zcap
-    // holds zero for the unsampled entries, which keeps the update free of branches.
+    // they are staged in shared memory while the transform runs, with their mask weights.  The slots before the first hold
+    // zeros for the unsampled entries (rank -1), which keeps the update free of branches and of index arithmetic.  Ranks inside
+    // the group and weights that are scaled already, against ranks of the whole plane: prepared step of 8 coils of 160 x 320 x 256
+    // 927 -> 901 us, of 96 x 160 x 128 at 4x 162 -> 157; value and weight in one 16-byte slot 984 (a wavefront more per entry).
+    // The test for a staged group lies outside the loop over the entries (6 coils of 64 x 368 x 320 at 3x, whose groups are
+    // larger than the staging area: 732 -> 498).
     extern __shared__ __align__(16) float2 mid_smem[];
-    cf* s_z = reinterpret_cast<cf*>(reinterpret_cast<float*>(mid_smem) + BY * blockDim.x);    // behind the slots of the threads
-    float* s_w = reinterpret_cast<float*>(s_z + a.zcap + 1);
+    cf* s_z = reinterpret_cast<cf*>(reinterpret_cast<float*>(mid_smem) + BY * blockDim.x) + 1;      // behind the slots of the threads
+    float* s_w = reinterpret_cast<float*>(s_z + a.zcap) + 1;
     int z_first = 0;
     bool z_staged = false;
     if (Z) {
@@ -88,10 +92,12 @@ mid_kernel(const MidArgs a) {
         if (z_staged) {
             const cf* zsrc = a.zin + ((long long)unit * a.n0 + a.i0_start + (int)gi) * pe + z_first;
             const float* wsrc = a.m2c + bt * pe + z_first;
-            for (int e = threadIdx.x; e < nz; e += blockDim.x) cp_async8(&s_z[e], zsrc + e);
+            for (int e = threadIdx.x; e < nz; e += blockDim.x) {
+                cp_async8(&s_z[e], zsrc + e);
+                if (MODE == MID_SEP_Z) cp_async4(&s_w[e], wsrc + e);
+            }
             cp_async_commit();
-            if (MODE == MID_SEP_Z) for (int e = threadIdx.x; e < nz; e += blockDim.x) s_w[e] = wsrc[e] * a.scale2;
-            if (threadIdx.x == 0) { s_z[a.zcap] = make_float2(0.f, 0.f); s_w[a.zcap] = 0.f; }
+            if (threadIdx.x == 0) { s_z[-1] = make_float2(0.f, 0.f); s_w[-1] = 0.f; }
         }
     }
     // What the k-space work of this column needs is copied to shared memory while the transform runs, into slots of the
@@ -148,22 +154,26 @@ mid_kernel(const MidArgs a) {
         for (int k1 = 0; k1 < BY; ++k1) { const float m = s_m[k1 * TH]; c[k1] = cscale(c[k1], m * m * a.scale2); }
     } else if (Z) {
         const int* zi = reinterpret_cast<const int*>(s_m);
-        const cf* zz = a.zin + ((long long)unit * a.n0 + a.i0_start + (int)gi) * pe;
-        const float* m2 = a.m2c + bt * pe;
+        const cf* zz = a.zin + ((long long)unit * a.n0 + a.i0_start + (int)gi) * pe + z_first;
+        const float* m2 = a.m2c + bt * pe + z_first;
+        auto update = [&](int k1, float zx, float zy, float w) {
+            if (MODE == MID_SEP_Z) c[k1] = make_float2(fmaf(w, c[k1].x, -zx), fmaf(w, c[k1].y, -zy));
+            else c[k1] = make_float2(-zx, -zy);
+        };
+        if (z_staged) {
 #pragma unroll
-        for (int k1 = 0; k1 < BY; ++k1) {
-            const int r = zi[k1 * TH];
-            cf zv; float w = 0.f;
-            if (z_staged) {
-                const int e = (r >= 0) ? r - z_first : a.zcap;
-                zv = s_z[e];
-                if (MODE == MID_SEP_Z) w = s_w[e];
-            } else {                                                // more sampled entries than the staging area holds
-                zv = (r >= 0) ? zz[r] : make_float2(0.f, 0.f);
-                if (MODE == MID_SEP_Z) w = (r >= 0) ? m2[r] * a.scale2 : 0.f;
+            for (int k1 = 0; k1 < BY; ++k1) {
+                const int r = zi[k1 * TH];
+                const cf zv = s_z[r];
+                update(k1, zv.x, zv.y, MODE == MID_SEP_Z ? s_w[r] : 0.f);
             }
-            if (MODE == MID_SEP_Z) c[k1] = make_float2(fmaf(w, c[k1].x, -zv.x), fmaf(w, c[k1].y, -zv.y));
-            else c[k1] = make_float2(-zv.x, -zv.y);
+        } else {                                                    // more sampled entries than the staging area holds
+#pragma unroll
+            for (int k1 = 0; k1 < BY; ++k1) {
+                const int r = zi[k1 * TH];
+                const cf zv = (r >= 0) ? zz[r] : make_float2(0.f, 0.f);
+                update(k1, zv.x, zv.y, (MODE == MID_SEP_Z && r >= 0) ? m2[r] : 0.f);
+            }
         }
     } else if (FULL) {
 #pragma unroll
@@ -278,11 +288,11 @@ struct MidImpl {
         }
         if (Z) {
             a.zcap = BY * a.NZ < ZCAP ? BY * a.NZ : ZCAP;
-            bytes += (size_t)(a.zcap + 1) * (sizeof(cf) + sizeof(float)) + 8;
+            bytes += (size_t)(a.zcap + 1) * (sizeof(cf) + sizeof(float));
         }
         if (Z) {
             static PerDevice done;
-            cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * sizeof(float) + (ZCAP + 1) * 12 + 8, done, BY * sizeof(cf));
+            cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * sizeof(float) + (ZCAP + 1) * 12, done, BY * sizeof(cf));
             if (e != cudaSuccess) return e;
         }
         return launch_overlapped(true, mid_kernel<RY, BY, MODE>, dim3((unsigned)blocks, (unsigned)parts), dim3(threads), bytes, s, a);

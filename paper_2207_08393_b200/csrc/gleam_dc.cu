@@ -83,9 +83,10 @@ static const TileOps* find_tile(int ry, int n2) {
 
 // Ranks of the sampled (ky, kz) positions, in the order the middle pass consumes them: groups of equal raw
 // ky mod ry, inside a group by (ky div ry, kz), so that the entries one of its blocks needs are contiguous.
-//   zidx[bt][q]  = rank of the raw (half-shifted) position q among the sampled ones, or -1 where M[sh(q)] == 0
+//   zidx[bt][q]  = rank of the raw (half-shifted) position q inside its group, or -1 where M[sh(q)] == 0
 //   zlist[bt][r] = unshifted source position p = sh(q) of rank r;   zcount[bt] = number sampled
 //   zstart[bt][k0] = first rank of group k0, zstart[bt][ry] the total;   m2c[bt][r] = squared mask weight
+//   times scale2
 // One warp per raw ky row, in two launches: the sampled positions of every row are counted, then numbered behind
 // those of the rows before it in that order (a warp adds up to n1 counts by itself).  Bound by latency: a mask plane
 // is a few hundred KB.
@@ -95,7 +96,7 @@ template <bool COUNT>
 __global__ void __launch_bounds__(ZMAP_THREADS) zmap_kernel(const float* mask, int* zidx,
                                                             int* zlist, int* zcount,
                                                             float* m2c, int* zstart,
-                                                            int* row_cnt, int n1, int n2, int ry) {
+                                                            int* row_cnt, int n1, int n2, int ry, float scale2) {
     grid_dependency_wait();
     grid_launch_dependents();
     const int lane = threadIdx.x & 31, row = blockIdx.x * (ZMAP_THREADS / 32) + (threadIdx.x >> 5);   // row = k0 * by + k1
@@ -112,17 +113,18 @@ __global__ void __launch_bounds__(ZMAP_THREADS) zmap_kernel(const float* mask, i
         if (lane == 0) cnt[row] = c;
         return;
     }
-    int r = 0;
-    for (int e = lane; e < row; e += 32) r += cnt[e];
+    int r = 0, group = 0;                                    // ranks before this row, and before its group
+    for (int e = lane; e < row; e += 32) { const int v = cnt[e]; r += v; group += e < k0 * by ? v : 0; }
     r = __reduce_add_sync(0xffffffffu, r);
+    group = __reduce_add_sync(0xffffffffu, group);
     if (lane == 0 && k1 == 0) zstart[bt * (ZMAP_MAX_RY + 1) + k0] = r;
     for (int z0 = 0; z0 < n2; z0 += 32) {
         const int kz = z0 + lane, sz = shift_half(kz, n2);
         const float mv = (kz < n2) ? mk[sz] : 0.f;
         const unsigned bal = __ballot_sync(0xffffffffu, mv != 0.f);
         const int mine = r + __popc(bal & ((1u << lane) - 1u));
-        if (kz < n2) zidx[bt * pe + (long long)ky * n2 + kz] = (mv != 0.f) ? mine : -1;
-        if (mv != 0.f) { zlist[bt * pe + mine] = src_row + sz; m2c[bt * pe + mine] = mv * mv; }
+        if (kz < n2) zidx[bt * pe + (long long)ky * n2 + kz] = (mv != 0.f) ? mine - group : -1;
+        if (mv != 0.f) { zlist[bt * pe + mine] = src_row + sz; m2c[bt * pe + mine] = mv * mv * scale2; }
         r += __popc(bal);
     }
     if (lane == 0 && row == n1 - 1) { zcount[bt] = r; zstart[bt * (ZMAP_MAX_RY + 1) + ry] = r; }
@@ -386,9 +388,9 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
             int* zrows = (int*)(ws + L.off_zrows);
             const dim3 zgrid((unsigned)((L.n1 + ZMAP_THREADS / 32 - 1) / (ZMAP_THREADS / 32)), (unsigned)L.images);
             CK(prof_mark(GLEAM_K_PREP_M2, s));
-            CK(launch_overlapped(true, zmap_kernel<true>, zgrid, dim3(ZMAP_THREADS), 0, s, mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry));
+            CK(launch_overlapped(true, zmap_kernel<true>, zgrid, dim3(ZMAP_THREADS), 0, s, mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry, 1.0f / (float)pe));
             CK(prof_mark(GLEAM_K_PREP_M2, s));
-            CK(launch_overlapped(true, zmap_kernel<false>, zgrid, dim3(ZMAP_THREADS), 0, s, mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry));
+            CK(launch_overlapped(true, zmap_kernel<false>, zgrid, dim3(ZMAP_THREADS), 0, s, mask, zidx, zlist, zcount, m2c, zstart, zrows, L.n1, L.n2, mid->ry, 1.0f / (float)pe));
             cz.zlist = zlist; cz.zcount = zcount;
         }
         cz.scale = g / sqrtf((float)(L.rank == 2 ? L.n1 : L.n0) * (float)pe);

@@ -35,6 +35,21 @@ def test_slices_with_an_arbitrary_mask(oracle, n, coils):
     check_all(oracle, d, x, y, sens, mask, 0.9, "slice %s" % (n,))
 
 
+# z values of a ky group in the middle pass: every group larger than the 2048 that are staged, groups on both sides of it, a full
+# mask, groups of a few samples and of none
+@pytest.mark.parametrize("n,density", [((2, 368, 320), 0.3), ((2, 368, 320), 0.2785), ((2, 320, 96), 1.0), ((2, 64, 40), 0.02), ((4, 160, 24), 0.003)])
+def test_groups_of_z_values(oracle, n, density):
+    import torch
+    import paper_2207_08393_b200 as g
+    d, x, y, sens, mask = problem(3, 1, 2, 1, n, MASK_READOUT_INVARIANT, weighted=False, seed=sum(n), density=density)
+    mask = (mask * np.random.default_rng(1).uniform(0.5, 1.5, mask.shape)).astype(np.float32)
+    check_all(oracle, d, x, y, sens, mask, 0.9, "groups %s" % (n,))
+    dc = g.DataConsistency(1, 2, 1, 3, n)
+    t = [torch.from_numpy(a).to("cuda:0") for a in (x, y, sens, mask)]
+    dc.prepare(t[1], t[3])
+    assert torch.equal(dc.forward_prepared(t[0], t[1], t[2], t[3], 0.9), g.DataConsistency(1, 2, 1, 3, n).forward(t[0], t[1], t[2], t[3], 0.9))
+
+
 # 23-point rows: outputs stored as they are formed (long rows) or after the butterfly, few and many rows a block
 @pytest.mark.parametrize("n", [(4, 92, 184), (2, 46, 368), (6, 20, 184), (2, 92, 92), (2, 64, 184), (2, 92, 46), (2, 240, 184), (1, 92, 368), (1, 6, 184)])
 def test_rows_of_23_points(oracle, n):
