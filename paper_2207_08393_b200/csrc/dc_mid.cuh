@@ -7,10 +7,10 @@
 namespace gleam {
 
 enum MidMode {
-    MID_SEP = 0,     // readout-invariant mask, no measurements (VJP, normal-equations form)
+    MID_SEP = 0,     // no measurements (VJP, normal-equations form): readout-invariant mask, or 2-D problem with an arbitrary one
     MID_SEP_Z = 1,   // readout-invariant mask and the table z of the measurements
     MID_ADJ_Z = 2,   // A^H y: minus the table z alone, nothing is read from the workspace
-    MID_FULL = 3,    // 2-D problem with an arbitrary mask; measurements may be null
+    MID_FULL = 3,    // 2-D problem with an arbitrary mask and measurements
     MID_ADJ_FULL = 4,
     MID_FWD = 5,     // forward half alone (arbitrary 3-D masks: the readout axis follows)
     MID_INV = 6,     // inverse half alone
@@ -135,7 +135,7 @@ mid_kernel(const MidArgs a) {
             const int off = centred(k1) * NZ;
             const float m = mk[off];
             s_m[k1 * TH] = m;
-            if (a.y && m != 0.f) cp_async8(s_y + k1 * TH, yy + off);
+            if (m != 0.f) cp_async8(s_y + k1 * TH, yy + off);
         }
         cp_async_commit();
     }
@@ -179,14 +179,10 @@ mid_kernel(const MidArgs a) {
 #pragma unroll
         for (int k1 = 0; k1 < BY; ++k1) {
             const float m = s_m[k1 * TH], w = m * m * a.scale2;
-            if (a.y) {
-                const cf yv = (m != 0.f) ? s_y[k1 * TH] : make_float2(0.f, 0.f);
-                const float f = (((centred(k1) + s2) & 1) ? -a.scale : a.scale) * m;
-                if (MODE == MID_FULL) c[k1] = make_float2(fmaf(w, c[k1].x, -f * yv.x), fmaf(w, c[k1].y, -f * yv.y));
-                else c[k1] = make_float2(-f * yv.x, -f * yv.y);
-            } else {
-                c[k1] = cscale(c[k1], w);
-            }
+            const cf yv = (m != 0.f) ? s_y[k1 * TH] : make_float2(0.f, 0.f);
+            const float f = (((centred(k1) + s2) & 1) ? -a.scale : a.scale) * m;
+            if (MODE == MID_FULL) c[k1] = make_float2(fmaf(w, c[k1].x, -f * yv.x), fmaf(w, c[k1].y, -f * yv.y));
+            else c[k1] = make_float2(-f * yv.x, -f * yv.y);
         }
     } else if (MODE == MID_GRADY) {
         const float* mk = a.mask + bt * (a.mask_row ? NZ : pe) + s2;
@@ -284,7 +280,7 @@ struct MidImpl {
             static PerDevice done;
             cudaError_t e = ensure_smem(mid_kernel<RY, BY, MODE>, BY * 256 * (sizeof(cf) + sizeof(float)), done, BY * sizeof(cf));
             if (e != cudaSuccess) return e;
-            if (a.y) bytes += (size_t)BY * threads * sizeof(cf);
+            bytes += (size_t)BY * threads * sizeof(cf);
         }
         if (Z) {
             a.zcap = BY * a.NZ < ZCAP ? BY * a.NZ : ZCAP;

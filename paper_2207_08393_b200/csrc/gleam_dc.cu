@@ -446,7 +446,7 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
         if (L.separable) {
             LAUNCH(GLEAM_K_COL_MID_SEP, mid->launch(!z ? MID_SEP : adjoint ? MID_ADJ_Z : MID_SEP_Z, ma, s));
         } else if (L.rank == 2) {
-            LAUNCH(GLEAM_K_COL_MID_FULL, mid->launch(adjoint ? MID_ADJ_FULL : MID_FULL, ma, s));
+            LAUNCH(GLEAM_K_COL_MID_FULL, mid->launch(adjoint ? MID_ADJ_FULL : y ? MID_FULL : MID_SEP, ma, s));
         } else {
             BrickArgs br{};
             br.V = ta.V; br.y = (const cf*)y; br.mask = mask; br.adjoint = adjoint ? 1 : 0;
