@@ -199,7 +199,7 @@ tile_fwd_kernel(const TileArgs a) {
 #pragma unroll
                 for (int m = 0; m < RL; ++m) u[m] = e[m];
                 cf* o = Vp + row * a.v_k0 + j;
-                dft_emit<RL, -1, true, TL::EARLY>(u, [&](auto k, cf x) { o[R0 * decltype(k)::value] = x; });
+                dft_emit<RL, -1, true, TL::EARLY>(u, [&](int k, cf x) { o[R0 * k] = x; });
             }
         }
     }
@@ -251,7 +251,7 @@ tile_inv_kernel(const TileArgs a) {
                 cf u[RL];
 #pragma unroll
                 for (int k = 0; k < RL; ++k) u[k] = o[R0 * k];
-                dft_emit<RL, +1, true, TL::EARLY>(u, [&](auto m, cf x) { e[decltype(m)::value] = x; });
+                dft_emit<RL, +1, true, TL::EARLY>(u, [&](int m, cf x) { e[m] = x; });
             }
             __syncthreads();
             if (TL::ONE_STAGE) stage_rows<NZ, RY>(sS, sp + c * s_stride, row_stride);

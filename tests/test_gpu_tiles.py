@@ -59,6 +59,23 @@ def test_rows_of_23_points(oracle, n):
         check_all(oracle, d, x, y, sens, mask, 0.9, "rows of 23 points %s" % (n,))
 
 
+# blocks of passes 1 and 3 that are resident on an SM (their registers decide), per pass
+@pytest.mark.parametrize("n,fwd,inv", [((24, 80, 46), 10, 8)])
+def test_resident_blocks_of_the_row_tile_passes(n, fwd, inv):
+    import torch
+    import paper_2207_08393_b200 as g
+    from tests.test_gpu_dispatch import captured
+    dev = torch.device("cuda:0")
+    x = torch.zeros((1, 1) + n, dtype=torch.complex64, device=dev)
+    s = torch.zeros((1, 3) + n, dtype=torch.complex64, device=dev)
+    dc, m = g.DataConsistency(1, 3, 1, 3, n), torch.ones((1, 1) + n[1:], device=dev)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    launches = captured(lambda: dc.vjp(x, s, m, 1.0))
+    for name, least in (("tile_fwd_kernel", fwd), ("tile_inv_kernel", inv)):
+        k, = [k for k in launches if name in k["name"]]
+        assert k["resident"] >= least * sms, k
+
+
 # middle radix 16 with full blocks: weights and measurements take 48 KB of shared memory, the twiddles come on top
 @pytest.mark.parametrize("n", [(1, 160, 240), (1, 256, 256), (1, 160, 512)])
 def test_slices_whose_middle_pass_takes_48_kb(oracle, n):
