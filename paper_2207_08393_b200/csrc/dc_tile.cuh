@@ -53,6 +53,10 @@ struct Tile {
     // 320 x 384 77 -> 74, 8 coils of 128 x 160 x 64 90 -> 87.  Where registers admit it: not 10- and 12-point stages next to short
     // ones (64 x 96 rows of 96 46.9 -> 51.1, 128 x 240 of 160 347 -> 357), nor 512 points (320 x 512 94 -> 95).
     static constexpr bool OWN_TW = S == 2 && TH % BFP == 0 && (R0 <= 8 || (RL >= 23 && NZ <= 384)) && !TIGHT;
+    // In pass 3 not where they cost blocks on an SM and no more is gained (8 rows of 24 points, 89 registers -> 99: 9 coils of 368
+    // x 64 x 24 24.8 -> 28.6 us a pass), nor where they spill (20 rows of 64, 47 x 11 coils of 640 x 64 80 -> 91), nor for 16 rows of
+    // 368, one block per SM with them or without (13 coils of 24 x 256 x 368 158 -> 163).
+    static constexpr bool OWN_TW_INV = OWN_TW && !(RY == 8 && NZ == 24) && !(RY == 20 && NZ == 64) && !(RY == 16 && NZ == 368);
     // Slots of a row in the exchange tile.  Congruent to BFP modulo 16: threads take the butterflies of the first kz stage row
     // after row, and each then has the bank of its thread number.  With rows of R0 runs (odd, packed) two rows of a half warp
     // met on the same banks in its reads and writes.  Packed -> congruent, VJP call, us: 8 coils of 64 x 128 x 128 79.9 -> 73.2,
@@ -62,15 +66,15 @@ struct Tile {
     // stages congruent to 23 were slower, too: forward of 15 coils of 128 x 160 x 184 746 -> 793.)
     static constexpr int PACKED = R0 * LS1;
     static constexpr int ROW = S != 2 ? NZ : (R0 < 8 || NZ < 64) ? PACKED : PACKED + ((BFP - PACKED) % 16 + 16) % 16;
-    static constexpr int T_ELEMS = (RY * ROW + 1) / 2 * 2, STAGE = RY * NZ, TW = (S == 2 && !OWN_TW) ? NZ : 0;
+    static constexpr int T_ELEMS = (RY * ROW + 1) / 2 * 2, STAGE = RY * NZ, TW = (S == 2 && !OWN_TW) ? NZ : 0, TW_INV = (S == 2 && !OWN_TW_INV) ? NZ : 0;
     static constexpr int slot(int kz) { return (S == 2) ? (kz / BF0) * LS1 + kz % BF0 : kz; }
     static constexpr size_t LIMIT = 227 * 1024;
     static constexpr size_t FWD_BYTES = sizeof(cf) * (T_ELEMS + STAGE + TW);
     // Pass 3 stages a tile of the workspace and one of the sensitivities.  Where both and the exchange tile take more
     // than a third of the SM they take turns in one buffer: a third block per SM hides more latency than the longer
     // reach of two buffers (8 slices of 320 x 256, 8 coils: 84.7 -> 76.7 us per VJP call).
-    static constexpr bool ONE_STAGE = sizeof(cf) * (T_ELEMS + 2 * STAGE + TW) > LIMIT / 3;
-    static constexpr size_t INV_BYTES = sizeof(cf) * (T_ELEMS + (ONE_STAGE ? 1 : 2) * STAGE + TW);
+    static constexpr bool ONE_STAGE = sizeof(cf) * (T_ELEMS + 2 * STAGE + TW_INV) > LIMIT / 3;
+    static constexpr size_t INV_BYTES = sizeof(cf) * (T_ELEMS + (ONE_STAGE ? 1 : 2) * STAGE + TW_INV);
     // The register bound lets the blocks that shared memory admits be resident.  RY values of the image or of the coil
     // sum are kept over the coil loop next to a butterfly (a prime radix also holds its sums and differences).
     // A block has a thread per column, so 640-point rows have at most 96 registers and spill up to 180 B whatever the bound.
@@ -226,13 +230,13 @@ tile_inv_kernel(const TileArgs a) {
     const long long s_stride = (long long)a.Ts * V3, x_off = id.bt * V3 + row_elems + tid;
     auto v_ptr = [&](int c) { return a.V + (((long long)(id.b * a.C + c)) * a.T + id.t) * a.v_unit + id.gi * a.v_slab + id.j * a.v_j; };
     if (id.c0 < id.c1) stage_rows<NZ, RY>(sV, v_ptr(id.c0), a.v_k0);
-    if (TL::S == 2 && !TL::OWN_TW) for (int i = tid; i < NZ; i += TH) sTw[i] = unit_root_fwd<NZ>(((i / BF0) * (i % BF0)) % NZ);
-    cf tw[TL::OWN_TW ? R0 : 1];
-    if (TL::OWN_TW) {
+    if (TL::S == 2 && !TL::OWN_TW_INV) for (int i = tid; i < NZ; i += TH) sTw[i] = unit_root_fwd<NZ>(((i / BF0) * (i % BF0)) % NZ);
+    cf tw[TL::OWN_TW_INV ? R0 : 1];
+    if (TL::OWN_TW_INV) {
 #pragma unroll
-        for (int k = 1; k < (TL::OWN_TW ? R0 : 1); ++k) tw[k] = unit_root_fwd<NZ>((k * (tid % BFP)) % NZ);
+        for (int k = 1; k < (TL::OWN_TW_INV ? R0 : 1); ++k) tw[k] = unit_root_fwd<NZ>((k * (tid % BFP)) % NZ);
     }
-    auto twiddle = [&](int k, int j) -> cf { return TL::OWN_TW ? tw[TL::OWN_TW ? k : 0] : sTw[k * BF0 + j]; };
+    auto twiddle = [&](int k, int j) -> cf { return TL::OWN_TW_INV ? tw[TL::OWN_TW_INV ? k : 0] : sTw[k * BF0 + j]; };
     cf acc[RY];
 #pragma unroll
     for (int m = 0; m < RY; ++m)

@@ -60,7 +60,7 @@ def test_rows_of_23_points(oracle, n):
 
 
 # blocks of passes 1 and 3 that are resident on an SM (their registers decide), per pass
-@pytest.mark.parametrize("n,fwd,inv", [((24, 80, 46), 10, 8)])
+@pytest.mark.parametrize("n,fwd,inv", [((24, 80, 46), 10, 8), ((24, 64, 24), 20, 20)])
 def test_resident_blocks_of_the_row_tile_passes(n, fwd, inv):
     import torch
     import paper_2207_08393_b200 as g
