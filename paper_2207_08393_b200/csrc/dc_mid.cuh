@@ -235,31 +235,55 @@ inline int coil_split(long long tiles, int threads, int sms, int C) {
 template <class PZ, int RY>
 struct TileImpl {
     using TL = Tile<PZ, RY>;
-    static cudaError_t fwd(const TileArgs& a0, long long images, long long tiles, cudaStream_t s) {
-        static PerDevice done;
-        cudaError_t e = ensure_smem(tile_fwd_kernel<PZ, RY>, TL::FWD_BYTES, done);
-        if (e != cudaSuccess) return e;
-        int sms = 0;
-        if ((e = device_sms(&sms)) != cudaSuccess) return e;
-        TileArgs a = a0;
-        a.csplit = coil_split(tiles, TL::TH, sms, a.C);
-        const long long blocks = images * a.G * a.BY * a.csplit;
-        if (blocks <= 0) return cudaSuccess;
-        if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-        return launch_overlapped(true, tile_fwd_kernel<PZ, RY>, dim3((unsigned)blocks), dim3(TL::TH), TL::FWD_BYTES, s, a);
+    using LL = Tile<PZ, RY, true>;
+    static cudaError_t fwd(const TileArgs& a, long long images, long long tiles, cudaStream_t s) {
+        if constexpr (TL::TIGHT) return launch_either<tile_fwd_kernel<PZ, RY>, tile_fwd_kernel<PZ, RY, true>>(TL::FWD_BYTES, LL::FWD_BYTES, false, a, images, tiles, s);
+        else return launch<tile_fwd_kernel<PZ, RY>>(TL::FWD_BYTES, false, a, images, tiles, s);
     }
-    static cudaError_t inv(const TileArgs& a0, long long images, long long tiles, cudaStream_t s) {
-        static PerDevice done;
-        cudaError_t e = ensure_smem(tile_inv_kernel<PZ, RY>, TL::INV_BYTES, done);
-        if (e != cudaSuccess) return e;
+    static cudaError_t inv(const TileArgs& a, long long images, long long tiles, cudaStream_t s) {
+        if constexpr (TL::TIGHT) return launch_either<tile_inv_kernel<PZ, RY>, tile_inv_kernel<PZ, RY, true>>(TL::INV_BYTES, LL::INV_BYTES, true, a, images, tiles, s);
+        else return launch<tile_inv_kernel<PZ, RY>>(TL::INV_BYTES, true, a, images, tiles, s);
+    }
+
+private:
+    static cudaError_t count_blocks(const TileArgs& a, long long images, long long tiles, int* csplit, long long* blocks) {
         int sms = 0;
-        if ((e = device_sms(&sms)) != cudaSuccess) return e;
+        const cudaError_t e = device_sms(&sms);
+        if (e != cudaSuccess) return e;
+        *csplit = coil_split(tiles, TL::TH, sms, a.C);
+        *blocks = images * a.G * a.BY * *csplit;
+        return cudaSuccess;
+    }
+    template <auto KERNEL> static cudaError_t resident(size_t bytes, int* slots) {
+        static PerDevice done, cache;
+        const cudaError_t e = ensure_smem(KERNEL, bytes, done);
+        return e != cudaSuccess ? e : resident_slots(KERNEL, TL::TH, bytes, cache, slots);
+    }
+    // The spills of the tight bound pay where its further blocks save a round.  VJP, us, loose / tight: 5 coils of 32 x 46 x 184 (736 blocks,
+    // two rounds of either) 32.6 / 36.0, 12 of 12 slices of 92 x 184 (276 blocks, one round) 37.0 / 41.4; 8 coils of 128 x 92 x 184 283 / 234.
+    template <auto TIGHT, auto LOOSE>
+    static cudaError_t launch_either(size_t tight_bytes, size_t loose_bytes, bool cluster, const TileArgs& a, long long images, long long tiles, cudaStream_t s) {
+        int csplit = 1, tight = 1, loose = 1;
+        long long blocks = 0;
+        cudaError_t e;
+        if ((e = count_blocks(a, images, tiles, &csplit, &blocks)) != cudaSuccess) return e;
+        if ((e = resident<TIGHT>(tight_bytes, &tight)) != cudaSuccess || (e = resident<LOOSE>(loose_bytes, &loose)) != cudaSuccess) return e;
+        if ((blocks + tight - 1) / tight < (blocks + loose - 1) / loose) return launch<TIGHT>(tight_bytes, cluster, a, images, tiles, s);
+        return launch<LOOSE>(loose_bytes, cluster, a, images, tiles, s);
+    }
+    // cluster: the blocks that share a tile form one
+    template <auto KERNEL>
+    static cudaError_t launch(size_t bytes, bool cluster, const TileArgs& a0, long long images, long long tiles, cudaStream_t s) {
+        static PerDevice done;
+        cudaError_t e = ensure_smem(KERNEL, bytes, done);
+        if (e != cudaSuccess) return e;
         TileArgs a = a0;
-        a.csplit = coil_split(tiles, TL::TH, sms, a.C);
-        const long long blocks = images * a.G * a.BY * a.csplit;
+        long long blocks = 0;
+        if ((e = count_blocks(a, images, tiles, &a.csplit, &blocks)) != cudaSuccess) return e;
         if (blocks <= 0) return cudaSuccess;
         if (blocks > 2147483647LL) return cudaErrorInvalidConfiguration;
-        return launch_overlapped_cluster((unsigned)a.csplit, tile_inv_kernel<PZ, RY>, dim3((unsigned)blocks), dim3(TL::TH), TL::INV_BYTES, s, a);
+        if (cluster) return launch_overlapped_cluster((unsigned)a.csplit, KERNEL, dim3((unsigned)blocks), dim3(TL::TH), bytes, s, a);
+        return launch_overlapped(true, KERNEL, dim3((unsigned)blocks), dim3(TL::TH), bytes, s, a);
     }
 };
 

@@ -31,7 +31,8 @@ struct TileArgs {
     const cf* aty;                            // A^H y image of the normal-equations form, or null (see RowArgs)
 };
 
-template <class PZ, int RY>
+// LOOSE: the form of short tiles with 23-point rows without the tight register bound (TIGHT, below).
+template <class PZ, int RY, bool LOOSE = false>
 struct Tile {
     static constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, S = PZ::S;
     static constexpr int BF0 = PZ::BF0;                      // butterflies per row of the first kz stage
@@ -43,16 +44,17 @@ struct Tile {
     // 240 x 184 493 -> 488; but 128 x 92 x 92 125 -> 129).  A bound without room for them spills all the same (up to 80 B); more
     // blocks outweigh that where few image rows are kept and blocks are large: VJP of 8 coils, us, 128 x 92 x 184 283 -> 234,
     // 128 x 92 x 368 602 -> 485, 256 x 46 x 184 361 -> 325, 4 slices of 92 x 184 23.6 -> 18.9; not with 16 rows (up to 244 B; 128 x
-    // 256 x 92 239 -> 264, 128 x 96 x 184 193 -> 202) nor on short rows (24 x 92 x 92, 4 coils, 17.8 -> 18.8).
-    static constexpr bool EARLY = NZ >= 184, TIGHT = PRIME && RY <= 4 && EARLY;
+    // 256 x 92 239 -> 264, 128 x 96 x 184 193 -> 202) nor on short rows (24 x 92 x 92, 4 coils, 17.8 -> 18.8).  Only where they save a
+    // round of blocks (LOOSE otherwise, TileImpl).
+    static constexpr bool EARLY = NZ >= 184, SHORT = PRIME && RY <= 4 && EARLY, TIGHT = SHORT && !LOOSE;
     // Threads per row in the first kz stage.  Half warps of 23 butterflies a row met on one bank where they cross to the next row, in
     // every read and write of the stage; with a thread left out per row, and rows congruent to 24 modulo 16, they do not.  VJP of
     // 12 coils of 96 x 240 x 184 490 -> 476 us, of 8 of 96 x 240 x 368 804 -> 781.
     static constexpr int BFP = RL == 23 && R0 >= 8 ? 24 : BF0;
     // A thread whose butterflies all have one place in their rows keeps their twiddles: 476 -> 458 and 781 -> 772 us, 4 slices of
     // 320 x 384 77 -> 74, 8 coils of 128 x 160 x 64 90 -> 87.  Where registers admit it: not 10- and 12-point stages next to short
-    // ones (64 x 96 rows of 96 46.9 -> 51.1, 128 x 240 of 160 347 -> 357), nor 512 points (320 x 512 94 -> 95).
-    static constexpr bool OWN_TW = S == 2 && TH % BFP == 0 && (R0 <= 8 || (RL >= 23 && NZ <= 384)) && !TIGHT;
+    // ones (64 x 96 rows of 96 46.9 -> 51.1, 128 x 240 of 160 347 -> 357), nor 512 points (320 x 512 94 -> 95), nor SHORT tiles.
+    static constexpr bool OWN_TW = S == 2 && TH % BFP == 0 && (R0 <= 8 || (RL >= 23 && NZ <= 384)) && !SHORT;
     // In pass 3 not where they cost blocks on an SM and no more is gained (8 rows of 24 points, 89 registers -> 99: 9 coils of 368
     // x 64 x 24 24.8 -> 28.6 us a pass), nor where they spill (20 rows of 64, 47 x 11 coils of 640 x 64 80 -> 91), nor for 16 rows of
     // 368, one block per SM with them or without (13 coils of 24 x 256 x 368 158 -> 163).
@@ -128,11 +130,11 @@ __device__ __forceinline__ void stage_rows(cf* dst, const cf* src, long long row
     cp_async_commit();
 }
 
-template <class PZ, int RY>
-__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY>::blocks(Tile<PZ, RY>::FWD_BYTES))
+template <class PZ, int RY, bool LOOSE = false>
+__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY, LOOSE>::blocks(Tile<PZ, RY, LOOSE>::FWD_BYTES))
 tile_fwd_kernel(const TileArgs a) {
     grid_dependency_wait();
-    using TL = Tile<PZ, RY>;
+    using TL = Tile<PZ, RY, LOOSE>;
     constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, BFP = TL::BFP, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
     extern __shared__ __align__(16) float2 smem[];
     cf* sT = smem;
@@ -210,11 +212,11 @@ tile_fwd_kernel(const TileArgs a) {
     cp_async_wait<0>();
 }
 
-template <class PZ, int RY>
-__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY>::blocks(Tile<PZ, RY>::INV_BYTES))
+template <class PZ, int RY, bool LOOSE = false>
+__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY, LOOSE>::blocks(Tile<PZ, RY, LOOSE>::INV_BYTES))
 tile_inv_kernel(const TileArgs a) {
     grid_dependency_wait();
-    using TL = Tile<PZ, RY>;
+    using TL = Tile<PZ, RY, LOOSE>;
     constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, BF0 = TL::BF0, BFP = TL::BFP, LS1 = TL::LS1, ROW = TL::ROW, TH = TL::TH;
     extern __shared__ __align__(16) float2 smem[];
     cf* sT = smem;

@@ -76,6 +76,30 @@ def test_resident_blocks_of_the_row_tile_passes(n, fwd, inv):
         assert k["resident"] >= least * sms, k
 
 
+# short tiles with 23-point rows: the form with more blocks on an SM only where that saves a round of them
+@pytest.mark.parametrize("n,coils,batch", [((32, 46, 184), 3, 1), ((24, 46, 184), 3, 1), ((1, 92, 184), 5, 12), ((1, 46, 368), 3, 6), ((1, 46, 368), 3, 8),
+                                           ((48, 92, 184), 2, 1), ((1, 20, 368), 3, 3), ((1, 92, 184), 6, 3)])
+def test_form_of_short_tiles(oracle, n, coils, batch):
+    import torch
+    import paper_2207_08393_b200 as g
+    from tests.test_gpu_dispatch import captured
+    rank, kind = (3, MASK_READOUT_INVARIANT) if n[0] > 1 else (2, MASK_FULL)
+    d, x, y, sens, mask = problem(rank, batch, coils, 1, n, kind, seed=sum(n), density=0.3)
+    check_all(oracle, d, x, y, sens, mask, 0.9, "short tiles %s" % (n,))
+    dc = g.DataConsistency(batch, coils, 1, rank, n, 0, kind)
+    t = [torch.from_numpy(a).to("cuda:0") for a in (x, sens, mask)]
+    launches = captured(lambda: dc.vjp(t[0], t[1], t[2], 1.0))
+    for name in ("tile_fwd_kernel", "tile_inv_kernel"):
+        k, = [k for k in launches if name in k["name"]]
+        rounds = lambda per_sm: -(-k["blocks"] // (per_sm * torch.cuda.get_device_properties(0).multi_processor_count))
+        taken = -(-k["blocks"] // k["resident"])
+        # blocks on an SM of the tight form (80 registers), and of the other one at most (92 and more)
+        if "Lb1E" in k["name"]:
+            assert taken <= rounds(4 if n[2] == 184 else 2), k
+        else:
+            assert taken < rounds(3 if n[2] == 184 else 1), k
+
+
 # middle radix 16 with full blocks: weights and measurements take 48 KB of shared memory, the twiddles come on top
 @pytest.mark.parametrize("n", [(1, 160, 240), (1, 256, 256), (1, 160, 512)])
 def test_slices_whose_middle_pass_takes_48_kb(oracle, n):
