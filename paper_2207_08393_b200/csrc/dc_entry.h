@@ -10,6 +10,13 @@ namespace gleam {
 // (x and eta are ignored; the transforms of a zero image are left out).
 enum { RUN_ALL = 0, RUN_PREPARE = 1, RUN_APPLY = 2, RUN_ADJOINT = 3 };
 
+// How the one-pass 2-D kernel of a call leaves its inner products (dot_rows), and the shape of its launch.
+struct DotForm {
+    int sums;            // sums per example in each half of dot_rows
+    int warps;           // warps of its blocks where it is one block per SM, 0 in its other forms
+    bool shared;         // such a block: four warps share a line group
+};
+
 // out = x - eta A^H (A x - y)   (y == nullptr: out = x - eta A^H A x).  Validates its arguments,
 // enqueues on d->stream, returns GLEAM_OK or a GLEAM_ERR_* code.  check_only: the argument checks
 // alone (callers that must enqueue something of their own before the step run them first).
@@ -17,7 +24,7 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
         const gleam_dims* d, int mode = RUN_ALL, double* dot_rows = nullptr, bool check_only = false,
         int layout = 0,      // layout: GLEAM_X_CHANNELS | GLEAM_OUT_CHANNELS (two-real-channel image arrays)
         const void* aty = nullptr,    // with y == nullptr: out = x - eta (A^H A x - aty), aty = A^H y as an image
-        int* dot_count = nullptr);    // set (also by check_only) to the number of sums per example in each half of dot_rows
+        DotForm* dot_form = nullptr);    // set (also by check_only) to the form of the call's one-pass launch
 
 // dot_rows (device, two arrays of one double per image row, B*T*n1): the one-pass 2-D kernel also stores
 // Re<x_row, out_row> and <out_row, out_row> of every row it writes, so that a caller's inner products need no

@@ -12,6 +12,7 @@
 // way out.  The column kernel here turns y into the table z.
 #pragma once
 #include "fft_line.cuh"
+#include "dc_entry.h"
 #include "launch_overlap.cuh"
 #include <stdint.h>
 
@@ -48,7 +49,7 @@ struct RowArgs {
     int RPB;            // rows of an image (n1)
     long long nrows;    // B*T*n1
     double* dot_rows;   // if not null, Re<x, out> of every image row, (B*T*n1), followed by <out, out> of every row
-    int* dot_count;     // host: if not null, set by the launch to the number of such sums per example
+    DotForm* dot_form;  // host: if not null, the launch says how it leaves them
     int dot_blocks;     // set by the launch, if not 0 the number of examples: the sums of a whole block instead of a row, by block
     // Two-real-channel layout (B, 2, T, n0, n1, n2) float32 of the image-side arrays (the form the learned
     // prior takes and returns): real index of complex element e of example b = e + b * plane, the imaginary

@@ -300,7 +300,7 @@ bool dot_rows_supported(const gleam_dims* d) {
 }
 
 int run(const void* x, const void* y, const void* sens, const float* mask, float eta, void* out,
-        const gleam_dims* d, int mode, double* dot_rows, bool check_only, int layout, const void* aty, int* dot_count) {
+        const gleam_dims* d, int mode, double* dot_rows, bool check_only, int layout, const void* aty, DotForm* dot_form) {
     if (!d || !mask) return GLEAM_ERR_NULL_POINTER;
     if (aty && (y || mode != RUN_ALL)) return GLEAM_ERR_BAD_DIMS;      // the given A^H y stands in for y
     if (mode == RUN_PREPARE) {
@@ -350,7 +350,7 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
             (aty && overlaps(w, L.total, aty, img_b)))
             return GLEAM_ERR_ALIAS;
     }
-    if (check_only && !dot_count) return GLEAM_OK;          // every argument check has passed; nothing is enqueued
+    if (check_only && !dot_form) return GLEAM_OK;          // every argument check has passed; nothing is enqueued
 
     cudaStream_t s = (cudaStream_t)d->stream;
     char* ws = (char*)d->workspace;
@@ -368,8 +368,8 @@ int run(const void* x, const void* y, const void* sens, const float* mask, float
     ra.x = (const cf*)x; ra.sens = (const cf*)sens; ra.out = (cf*)out; ra.eta = eta; ra.mask = mask; ra.z = z;
     ra.C = L.C; ra.T = L.T; ra.Ts = L.Ts; ra.RPB = L.n1; ra.nrows = L.images * L.n1;
     ra.x_planar = x_planar; ra.out_planar = out_planar; ra.plane = plane;
-    ra.aty = (const cf*)aty; ra.dot_rows = dot_rows; ra.dot_count = dot_count;
-    if (dot_count) *dot_count = L.T * L.n1;          // one per row unless the launch says otherwise
+    ra.aty = (const cf*)aty; ra.dot_rows = dot_rows; ra.dot_form = dot_form;
+    if (dot_form) *dot_form = DotForm{L.T * L.n1, 0, false};      // a sum per row unless the launch says otherwise
     if (check_only) {
         bool lets_in = false;                        // not asked for, but nothing is launched
         if (dot_rows) { ra.z = nullptr; CK(find_size(L.n2)->row(ra, s, &lets_in)); }

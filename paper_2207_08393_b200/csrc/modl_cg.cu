@@ -175,6 +175,8 @@ __global__ void __launch_bounds__(CG_THREADS) cg_dot_kernel(const CgArgs a) {
 }
 
 // BATCH elements of every vector are requested before the sums are formed, so that their latency covers that of the sums.
+// The bounds (four, three and two blocks on an SM) make the forms that are not the last step and request two or three elements spill 32 to
+// 96 B, two with sums per row also in the last step (8 B); four elements fit their 128 registers.
 template <bool FROM_ROWS, bool DEALT, bool LAST, int BATCH>
 __global__ void __launch_bounds__(CG_THREADS, BATCH == 2 ? 4 : BATCH == 3 ? 3 : 2) cg_step_kernel(const CgArgs a) {
     grid_dependency_wait();
@@ -332,21 +334,30 @@ static int modl_cg(const void* z, const void* y, const void* sens, const float* 
     a.dot_rows = dot_rows; a.rows_per_example = d->frames * d->n[1];
 
     // the operator's own argument checks (y, sens, mask) before anything is enqueued
-    CGRUN(run(ws + L.off_r, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ALL, dot_rows, true, 0, nullptr, &a.dot_count));
+    DotForm op{};
+    CGRUN(run(ws + L.off_r, y, sens, mask, 1.0f, ws + L.off_q, &dd, RUN_ALL, dot_rows, true, 0, nullptr, &op));
+    a.dot_count = op.sums;
     // Elements a thread of the vector launches, and how many of them a step requests at once.  All of them where that is one
     // round of resident blocks: a thread that comes back for a few more waits for memory once more after the sums (20 frames of
     // 192 x 160: 4096 of 307,200 elements were left over by 592 blocks of two a thread; 10 steps 240 -> 227 us with three).  Two
     // while the blocks are one per SM, then four (two blocks per SM), three (three) and, beyond that, four in two rounds.
     // Measured against two and four elements in rounds of two, 10 steps: 5 coils of 384 x 640 251 -> 219, of 640 x 320 129 -> 119,
-    // 6 x 18 of 384 x 80 220 -> 203, 3 x 5 of 320 x 256 135 -> 125, 8 x 24 x 3 of 64 x 128 203 -> 199; 4 x 4 of 92 x 640 209 -> 213.
-    // Where the operator sums per block (one block of many warps per SM) and the step is no more than a block per SM, those
-    // of fewer registers come in while the operator drains: two at once (3 x 5 x 8 of 128 x 96 119 against 125).
+    // 6 x 18 of 384 x 80 220 -> 203, 3 x 5 of 320 x 256 135 -> 125, 8 x 24 x 3 of 64 x 128 203 -> 199; 4 x 4 of 92 x 640 equal (210).
+    // Some problems of short vectors lose: 10 x 2 x 7 of 46 x 120 111 -> 114, 32 x 2 x 6 of 32 x 46 174 -> 179.
+    // No more than a block per SM: what counts is how the blocks spread over the SMs that an operator of one block per SM gives free (us
+    // of 10 steps, two at once / four).  Behind 13 to 16 warps of it nothing fits before they end, and then blocks of 64 registers a
+    // thread crowd by fours on the first SMs, of 128 by twos: 36 x 5 coils of 128 x 64 154 / 122, 10 coils x 7 of 512 x 80 195 / 165.
+    // Next to 11 or 12 warps one block of 64 registers fits, none of 128, and comes in while the operator drains: 24 x 4 x 8 of 32 x 48
+    // 116 / 122, 48 x 6 of 64 x 64 107 / 115, 3 x 5 x 8 of 128 x 96 119 / 128; next to 8 warps two would: 6 coils x 28 of 80 x 128
+    // 125 / 119.  Where 12 warps share groups by fours the sums tell: per block two at once (4 coils x 10 of 256 x 80 102 / 111), per
+    // row four (38 x 6 of 64 x 96 120 / 115).  12 warps of 32 points take four as well (3 x 4 x 24 of 96 x 32 139 / 112).
     auto blocks_of = [&](int each) { const long long n = (L.ne2 + (long long)CG_THREADS * each - 1) / ((long long)CG_THREADS * each); return n < 1 ? 1 : n; };
     const long long one = CG_MAX_BLOCKS / 4;                 // a block per SM
-    const bool sums_per_block = from_rows && a.dot_count != a.rows_per_example;
+    const bool sums_per_block = op.sums != a.rows_per_example;
+    const bool beside = op.warps == 11 || (op.warps == 12 && d->n[2] >= 48 && (!op.shared || sums_per_block));
     int each = 4, batch = 2;
     if (blocks_of(2) * L.B <= one) each = batch = 2;
-    else if (blocks_of(4) * L.B <= 2 * one) batch = (sums_per_block && blocks_of(4) * L.B <= one) ? 2 : 4;
+    else if (blocks_of(4) * L.B <= 2 * one) batch = (beside && blocks_of(4) * L.B <= one) ? 2 : 4;
     else if (blocks_of(3) * L.B <= 3 * one) each = batch = 3;
     const dim3 grid((unsigned)(blocks_of(each) < CG_MAX_BLOCKS ? blocks_of(each) : CG_MAX_BLOCKS), (unsigned)L.B);
     if (y) {

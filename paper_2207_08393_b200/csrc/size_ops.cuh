@@ -138,7 +138,7 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* le
                 // 224, but 5 of 640 214 -> 223, 6 of 640 249 -> 259, 8 of 480 251 -> 265.
                 const long long rows = (long long)a.T * a.RPB;
                 const bool whole = DOT && rows >= sms && rows % WF::LW == 0 && a.nrows <= 3 * rows;
-                if (whole && a.dot_count) *a.dot_count = sms;
+                if (DOT && a.dot_form) *a.dot_form = DotForm{whole ? sms : (int)rows, warps, nsplit > 0};
                 if (lets_in) { *lets_in = true; return cudaSuccess; }
                 RowArgs b = a;
                 b.dot_blocks = whole ? (int)(a.nrows / rows) : 0;

@@ -203,12 +203,21 @@ def test_sums_of_the_operator_and_examples_of_unlike_scale(oracle, shape, thread
     assert all("cg_step_kernelILb1ELb%d" % dealt in k["name"] for k in steps), steps[0]
 
 
-# vector launches: two, four and three elements a thread at once, four in rounds of two; blocks that are full, nearly empty and part
-# full at the end, several examples
-@pytest.mark.parametrize("shape,blocks", [
-    ((1, 2, 1, 46, 46), 3), ((2, 2, 2, 184, 192), 138), ((1, 2, 3, 320, 160), 75), ((3, 3, 1, 320, 256), 120), ((1, 2, 18, 192, 160), 270),
-    ((1, 2, 20, 192, 160), 400), ((1, 2, 22, 192, 160), 440), ((1, 2, 23, 192, 160), 345), ((1, 2, 24, 320, 192), 592)])
-def test_vector_launches(oracle, shape, blocks):
+# vector launches: blocks, and elements that a thread requests at once; two, four and three a thread at once, four in rounds of two; blocks
+# that are full, nearly empty and part full at the end, several examples.  Behind an operator of one block per SM (11, 12 and 16
+# warps, with and without shared groups, sums per block and per row) four at once unless a block of two fits next to it
+@pytest.mark.parametrize("shape,blocks,batch", [
+    ((1, 2, 1, 46, 46), 3, 2), ((2, 2, 2, 184, 192), 138, 2), ((1, 2, 3, 320, 160), 75, 4), ((3, 3, 1, 320, 256), 120, 4), ((1, 2, 18, 192, 160), 270, 4),
+    ((1, 2, 20, 192, 160), 400, 3), ((1, 2, 22, 192, 160), 440, 3), ((1, 2, 23, 192, 160), 345, 2), ((1, 2, 24, 320, 192), 592, 2),
+    ((3, 5, 8, 128, 96), 144, 2),             # 11 warps, sums per block
+    ((48, 6, 1, 64, 64), 96, 2),              # 11 warps, sums per row
+    ((11, 12, 1, 240, 64), 88, 4),            # 12 warps, a group shared, sums per row
+    ((11, 12, 1, 320, 64), 110, 2),           # 12 warps, none shared
+    ((1, 4, 10, 256, 80), 100, 2),            # 12 warps, a group shared, sums per block
+    ((3, 4, 24, 96, 32), 108, 4),             # 12 warps of 32 points
+    ((1, 6, 28, 80, 128), 140, 4),            # 8 warps
+    ((1, 10, 7, 512, 80), 140, 4)])           # 16 warps
+def test_vector_launches(oracle, shape, blocks, batch):
     import torch
     import paper_2207_08393_b200 as g
     from tests.test_gpu_dispatch import captured
@@ -218,7 +227,7 @@ def test_vector_launches(oracle, shape, blocks):
     cg = g.ModlCG(B, C, T, 2, (1, n1, n2))
     tz, ts, tm = (torch.from_numpy(a).to("cuda:0") for a in (z, sens, mask))
     steps = [k for k in captured(lambda: cg.solve_vjp(tz, ts, tm, 0.5)) if "cg_step_kernel" in k["name"]]
-    assert len(steps) == 10 and all(k["blocks"] == blocks for k in steps), steps[0]
+    assert len(steps) == 10 and all(k["blocks"] == blocks and "ELi%dE" % batch in k["name"] for k in steps), steps[0]
 
 
 def textbook_steps(z, sens, mask, mu, n_iter, dtype):
