@@ -150,15 +150,21 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* le
         }
     }
     if (lets_in) return cudaSuccess;
-    // A last round that fills no more than a quarter of the warps: blocks of four warps that share each group of it, a quarter
-    // of the coils each (FLAT_TAIL).  Such a round costs a warp's whole run time however few groups it has: 4 x 15 coils of 640 x
-    // 368 are 1280 groups on 1184 warps, VJP 77.6 -> 63.6 us, and 2560 with z, prepared step 92 -> 84.  Where no more than 8
-    // warps are on an SM (368, 512, 640 points; 6 to 16 coils) it makes a VJP behind one full round 1.05-1.30 times as fast and a
-    // prepared step behind one to three 1.04-1.33.  With more warps an SM the single-warp blocks, which finish one by one, fill
-    // the last round themselves (VJP, 7 to 12 coils of 320 and 384 points, 0.82-0.93 times as fast in fours); only prepared steps
-    // gain there, 1.04-1.29 with 12 to 16 coils and a last round that is not too full (0.95-0.98 with fewer or more groups).
+    // A nearly empty last round: blocks of four warps that share each group of it, a quarter of the coils each (FLAT_TAIL).  Such a
+    // round costs a warp's whole run time however few groups it has: 4 x 15 coils of 640 x 368 are 1280 groups on 1184 warps, VJP
+    // 77.6 -> 63.6 us, and 2560 with z, prepared step 92 -> 84.  Two lines, by the warps an SM holds:
+    // 8 or fewer (368, 512, 640 points): a last round of at most a quarter of the warps.  6 to 32 coils: VJP behind one full round 1.05-
+    // 1.30 times as fast; prepared step behind one to fourteen 1.00-1.33, 368 points 1.02 in the mean at 14 rounds, 640 points 1.05 (with
+    // every second line sampled and 6 rounds or more 0.96-1.02).  The warps of a block drift apart over the rounds and wait for
+    // one another before the last: with 512 points 1.03 at 5 rounds, 1.01 at 6, 0.99 from 8 on (0.96 at worst), so at most 6.
+    // More: the single-warp blocks, which finish one by one, fill the last round themselves (VJP, 7 to 12 coils of 320 and 384 points,
+    // 0.82-0.93 times as fast in fours); only prepared steps behind one full round gain, 1.04-1.29 with 12 to 16 coils and at most 15
+    // % of the warps in the last round (0.95-0.98 with fewer coils or more groups).
     // Two groups a block: 368 points 1.09, most others slower.  A group of few units is one round whoever shares it.
+    // Spilled for it (128 threads, the bound of the single warps): VJP of 368 points 56 B, with A^H y 52; prepared step of 384 points 92
+    // (single warps 32), 160 points 48, 320 points 12, 256 points 4 (none).
     constexpr bool FEW_WARPS = WF::SINGLE_BLOCKS <= 8;
+    constexpr long long MOST_ROUNDS = P::N == 512 ? 6 : 1LL << 40;
     if constexpr ((FEW_WARPS || HAS_Z) && 4 * WF::WARP_BYTES <= 227 * 1024) {
         if (groups > slots && a.C >= (FEW_WARPS ? 6 : 12) && WF::UPC * a.C > 64) {
             static PerDevice tail_attr_done, tail_cache;
@@ -167,7 +173,7 @@ inline cudaError_t launch_warpflat_zy(const RowArgs& a, cudaStream_t s, bool* le
             if ((e = ensure_smem(warpflat_kernel<P, HAS_Z, FLAT_TAIL, HAS_ATY, ADJ, DOT>, BYTES, tail_attr_done)) != cudaSuccess) return e;
             if ((e = resident_slots(warpflat_kernel<P, HAS_Z, FLAT_TAIL, HAS_ATY, ADJ, DOT>, 128, BYTES, tail_cache, &resident)) != cudaSuccess) return e;
             const long long full = groups / (4LL * resident), tail = groups % (4LL * resident);
-            if (4 * resident >= slots && tail > 0 && (FEW_WARPS ? tail <= resident : 5 * tail <= 3 * resident) && (full == 1 || (FEW_WARPS && HAS_Z)))
+            if (4 * resident >= slots && tail > 0 && (FEW_WARPS ? tail <= resident : 5 * tail <= 3 * resident) && (full == 1 || (FEW_WARPS && HAS_Z && full <= MOST_ROUNDS)))
                 return launch_overlapped(true, warpflat_kernel<P, HAS_Z, FLAT_TAIL, HAS_ATY, ADJ, DOT>, dim3((unsigned)resident), dim3(128), BYTES, s, a, 4);
         }
     }

@@ -140,6 +140,14 @@ def test_last_round_of_the_row_kernel(oracle, shape, shared):
     assert_close(got, oracle.dc_forward(x, y, sens, mask, 0.9, d, nthreads=8), x, "%s normal equations" % (shape,))
 
 
+# prepared steps of 512 points share the groups of the last round behind at most six full ones, of 368 and 640 points behind any number
+@pytest.mark.parametrize("shape,shared", [((23, 6, 1, 320, 512), True), ((26, 6, 1, 320, 512), False), ((23, 6, 1, 320, 640), True), ((23, 6, 1, 320, 368), True)])
+def test_rounds_before_a_shared_one(shape, shared):
+    dc, x, y, s, m = holder(shape)
+    row = [k for k in captured(lambda: dc.forward_prepared(x, y, s, m, 1.0)) if "warpflat_kernel" in k["name"]][-1]
+    assert (row["threads"] == 128) == shared, row
+
+
 # z table: more sampled tiles than blocks (a block walks over several, also with the last tile part full) and fewer, one-, two-
 # and three-stage readouts, staged and direct tiles
 @pytest.mark.parametrize("rank,coils,n,density", [
