@@ -140,6 +140,31 @@ def test_last_round_of_the_row_kernel(oracle, shape, shared):
     assert_close(got, oracle.dc_forward(x, y, sens, mask, 0.9, d, nthreads=8), x, "%s normal equations" % (shape,))
 
 
+# the shared last round with sensitivities that move with the frames, in place (four warps read the rows that one of them writes) and in
+# the two-channel layout, bit for bit as the complex calls
+@pytest.mark.parametrize("shape", [(4, 7, 2, 320, 368), (1, 6, 4, 320, 640), (4, 9, 2, 160, 512)])
+def test_shared_last_round_in_place_and_in_channels(oracle, shape):
+    import torch
+    import paper_2207_08393_b200 as g
+    from tests.test_gpu_bridge import _run
+    B, C, T, n1, n2 = shape
+    d, x, y, sens, mask = problem(2, B, C, T, (1, n1, n2), MASK_READOUT_INVARIANT, sens_has_frames=1, seed=sum(shape), density=0.3)
+    dc = g.DataConsistency(B, C, T, 2, (1, n1, n2), 1)
+    t = [torch.from_numpy(a).to("cuda:0") for a in (x, y, sens, mask)]
+    dc.prepare(t[1], t[3])
+    for fn in (lambda: dc.vjp(t[0], t[2], t[3], 1.0), lambda: dc.forward_prepared(t[0], t[1], t[2], t[3], 1.0)):
+        assert captured(fn)[-1]["threads"] == 128
+    both, x_ch = g.GLEAM_X_CHANNELS | g.GLEAM_OUT_CHANNELS, oracle.complex_to_channels(x)
+    for yy in (y, None):
+        plain = _run(d, x, yy, sens, mask, 0.9, 0)
+        ref = oracle.dc_forward(x, yy, sens, mask, 0.9, d, nthreads=8) if yy is not None else oracle.dc_vjp(x, sens, mask, 0.9, d, nthreads=8)
+        assert_close(plain, ref, x, "moving coils %s" % (shape,))
+        assert _run(d, x, yy, sens, mask, 0.9, 0, in_place=True).tobytes() == plain.tobytes()
+        plain_ch = oracle.complex_to_channels(plain).tobytes()
+        assert _run(d, x_ch, yy, sens, mask, 0.9, both).tobytes() == plain_ch
+        assert _run(d, x_ch, yy, sens, mask, 0.9, both, in_place=True).tobytes() == plain_ch
+
+
 # prepared steps of 512 points share the groups of the last round behind at most six full ones, of 368 and 640 points behind any number
 @pytest.mark.parametrize("shape,shared", [((23, 6, 1, 320, 512), True), ((26, 6, 1, 320, 512), False), ((23, 6, 1, 320, 640), True), ((23, 6, 1, 320, 368), True)])
 def test_rounds_before_a_shared_one(shape, shared):
