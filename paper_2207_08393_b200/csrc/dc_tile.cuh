@@ -79,6 +79,8 @@ struct Tile {
     static constexpr size_t INV_BYTES = sizeof(cf) * (T_ELEMS + (ONE_STAGE ? 1 : 2) * STAGE + TW_INV);
     // The register bound lets the blocks that shared memory admits be resident.  RY values of the image or of the coil
     // sum are kept over the coil loop next to a butterfly (a prime radix also holds its sums and differences).
+    // The twiddles of OWN_TW are not counted: under bounds that leave room for them pass 1 of 64-point rows would not spill (up to 68 B),
+    // but with fewer blocks; with the spills it is 1.00-1.07 times as fast as with twiddles in shared memory.
     // A block has a thread per column, so 640-point rows have at most 96 registers and spill up to 180 B whatever the bound.
     static constexpr int REGS = 2 * RY + (PRIME && !TIGHT ? 4 : 2) * RMAX + (TIGHT ? 24 : 16);
     static constexpr int blocks(size_t bytes) {
