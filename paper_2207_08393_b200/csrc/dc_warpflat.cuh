@@ -351,36 +351,24 @@ warpflat_kernel(const RowArgs a, const int nwhole) {
         }
         cp_async_wait<0>();
         __syncwarp();
-        if (SMW && split) {
-            // partial coil sums of the other three warps are added by the first in warp order (the ring is free by now)
+        if ((SMW || TAIL) && split) {
+            // partial coil sums of the other three warps are added by the first in warp order (the ring is free by now); all four
+            // warps of the group get here
             if (q > 0) {
 #pragma unroll
                 for (int m = 0; m < R0; ++m) sE[m * 32 + lane] = acc[m];
             }
-            // the four warps of this group (every one gets here: same g)
-            if (set == 0) asm volatile("bar.sync 1, 128;" ::: "memory"); else asm volatile("bar.sync 2, 128;" ::: "memory");
-            if (q > 0) continue;
-            for (int w = 1; w < 4; ++w) {
-                const cf* o = smem + (nwhole + 4 * set + w) * WF::ELEMS + WF::OFF_E;
-#pragma unroll
-                for (int m = 0; m < R0; ++m) acc[m] = cadd(acc[m], o[m * 32 + lane]);
-            }
-        }
-        if (TAIL && split) {
-            // as above; the second barrier: a warp's ring is free again once its sums have been read
-            if (q > 0) {
-#pragma unroll
-                for (int m = 0; m < R0; ++m) sE[m * 32 + lane] = acc[m];
-            }
-            __syncthreads();
+            if (TAIL) __syncthreads();
+            else if (set == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
+            else asm volatile("bar.sync 2, 128;" ::: "memory");
             if (q == 0) {
                 for (int w = 1; w < 4; ++w) {
-                    const cf* o = smem + w * WF::ELEMS + WF::OFF_E;
+                    const cf* o = smem + ((TAIL ? 0 : nwhole + 4 * set) + w) * WF::ELEMS + WF::OFF_E;
 #pragma unroll
                     for (int m = 0; m < R0; ++m) acc[m] = cadd(acc[m], o[m * 32 + lane]);
                 }
             }
-            __syncthreads();
+            if (TAIL) __syncthreads();          // a warp's ring is free again once its sums have been read
             if (q > 0) continue;
         }
         // ---- out = x - eta * sum, and Re<x, out>, <out, out> per row for the caller's inner products ----
