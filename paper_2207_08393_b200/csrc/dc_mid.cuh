@@ -237,11 +237,11 @@ struct TileImpl {
     using TL = Tile<PZ, RY>;
     using LL = Tile<PZ, RY, true>;
     static cudaError_t fwd(const TileArgs& a, long long images, long long tiles, cudaStream_t s) {
-        if constexpr (TL::TIGHT) return launch_either<tile_fwd_kernel<PZ, RY>, tile_fwd_kernel<PZ, RY, true>>(TL::FWD_BYTES, LL::FWD_BYTES, false, a, images, tiles, s);
+        if constexpr (TL::TWO_FWD) return launch_either<tile_fwd_kernel<PZ, RY>, tile_fwd_kernel<PZ, RY, true>>(TL::FWD_BYTES, LL::FWD_BYTES, false, a, images, tiles, s);
         else return launch<tile_fwd_kernel<PZ, RY>>(TL::FWD_BYTES, false, a, images, tiles, s);
     }
     static cudaError_t inv(const TileArgs& a, long long images, long long tiles, cudaStream_t s) {
-        if constexpr (TL::TIGHT) return launch_either<tile_inv_kernel<PZ, RY>, tile_inv_kernel<PZ, RY, true>>(TL::INV_BYTES, LL::INV_BYTES, true, a, images, tiles, s);
+        if constexpr (TL::TWO_INV) return launch_either<tile_inv_kernel<PZ, RY>, tile_inv_kernel<PZ, RY, true>>(TL::INV_BYTES, LL::INV_BYTES, true, a, images, tiles, s);
         else return launch<tile_inv_kernel<PZ, RY>>(TL::INV_BYTES, true, a, images, tiles, s);
     }
 
@@ -259,16 +259,17 @@ private:
         const cudaError_t e = ensure_smem(KERNEL, bytes, done);
         return e != cudaSuccess ? e : resident_slots(KERNEL, TL::TH, bytes, cache, slots);
     }
-    // The spills of the tight bound pay where its further blocks save a round.  VJP, us, loose / tight: 5 coils of 32 x 46 x 184 (736 blocks,
-    // two rounds of either) 32.6 / 36.0, 12 of 12 slices of 92 x 184 (276 blocks, one round) 37.0 / 41.4; 8 coils of 128 x 92 x 184 283 / 234.
-    template <auto TIGHT, auto LOOSE>
-    static cudaError_t launch_either(size_t tight_bytes, size_t loose_bytes, bool cluster, const TileArgs& a, long long images, long long tiles, cudaStream_t s) {
-        int csplit = 1, tight = 1, loose = 1;
+    // The form with more blocks on an SM pays for its spills, or its twiddles in shared memory, where it saves a round of blocks.  VJP, us,
+    // loose / dense: 5 coils of 32 x 46 x 184 (736 blocks, two rounds of either) 32.6 / 36.0, 12 of 12 slices of 92 x 184 (276 blocks,
+    // one round) 37.0 / 41.4; 8 coils of 128 x 92 x 184 283 / 234.
+    template <auto DENSE, auto LOOSE>
+    static cudaError_t launch_either(size_t dense_bytes, size_t loose_bytes, bool cluster, const TileArgs& a, long long images, long long tiles, cudaStream_t s) {
+        int csplit = 1, dense = 1, loose = 1;
         long long blocks = 0;
         cudaError_t e;
         if ((e = count_blocks(a, images, tiles, &csplit, &blocks)) != cudaSuccess) return e;
-        if ((e = resident<TIGHT>(tight_bytes, &tight)) != cudaSuccess || (e = resident<LOOSE>(loose_bytes, &loose)) != cudaSuccess) return e;
-        if ((blocks + tight - 1) / tight < (blocks + loose - 1) / loose) return launch<TIGHT>(tight_bytes, cluster, a, images, tiles, s);
+        if ((e = resident<DENSE>(dense_bytes, &dense)) != cudaSuccess || (e = resident<LOOSE>(loose_bytes, &loose)) != cudaSuccess) return e;
+        if ((blocks + dense - 1) / dense < (blocks + loose - 1) / loose) return launch<DENSE>(dense_bytes, cluster, a, images, tiles, s);
         return launch<LOOSE>(loose_bytes, cluster, a, images, tiles, s);
     }
     // cluster: the blocks that share a tile form one

@@ -31,7 +31,7 @@ struct TileArgs {
     const cf* aty;                            // A^H y image of the normal-equations form, or null (see RowArgs)
 };
 
-// LOOSE: the form of short tiles with 23-point rows without the tight register bound (TIGHT, below).
+// LOOSE: of kernels that are built in two forms, the one with more registers and fewer blocks on an SM (TWO_FWD, TWO_INV).
 template <class PZ, int RY, bool LOOSE = false>
 struct Tile {
     static constexpr int NZ = PZ::N, R0 = PZ::R0, RL = PZ::RL, S = PZ::S;
@@ -55,10 +55,12 @@ struct Tile {
     // 320 x 384 77 -> 74, 8 coils of 128 x 160 x 64 90 -> 87.  Where registers admit it: not 10- and 12-point stages next to short
     // ones (64 x 96 rows of 96 46.9 -> 51.1, 128 x 240 of 160 347 -> 357), nor 512 points (320 x 512 94 -> 95), nor SHORT tiles.
     static constexpr bool OWN_TW = S == 2 && TH % BFP == 0 && (R0 <= 8 || (RL >= 23 && NZ <= 384)) && !SHORT;
-    // In pass 3 not where they cost blocks on an SM and no more is gained (8 rows of 24 points, 89 registers -> 99: 9 coils of 368
-    // x 64 x 24 24.8 -> 28.6 us a pass), nor where they spill (20 rows of 64, 47 x 11 coils of 640 x 64 80 -> 91), nor for 16 rows of
-    // 368, one block per SM with them or without (13 coils of 24 x 256 x 368 158 -> 163).
-    static constexpr bool OWN_TW_INV = OWN_TW && !(RY == 8 && NZ == 24) && !(RY == 20 && NZ == 64) && !(RY == 16 && NZ == 368);
+    // In pass 3 not where they spill (20 rows of 64, 47 x 11 coils of 640 x 64 80 -> 91 us a pass), nor for 16 rows of 368, one block per
+    // SM with them or without (13 coils of 24 x 256 x 368 158 -> 163).  With 8 rows of 24 points they cost blocks on an SM (89
+    // registers -> 99, 20 blocks -> 16: 9 coils of 368 x 64 x 24 24.8 -> 28.6), so only where that takes no further round (LOOSE).
+    static constexpr bool FEWER_BLOCKS = RY == 8 && NZ == 24;
+    static constexpr bool OWN_TW_INV = OWN_TW && (LOOSE || !FEWER_BLOCKS) && !(RY == 20 && NZ == 64) && !(RY == 16 && NZ == 368);
+    static constexpr bool TWO_FWD = SHORT, TWO_INV = SHORT || FEWER_BLOCKS;      // kernels in two forms, chosen by rounds (TileImpl)
     // Slots of a row in the exchange tile.  Congruent to BFP modulo 16: threads take the butterflies of the first kz stage row
     // after row, and each then has the bank of its thread number.  With rows of R0 runs (odd, packed) two rows of a half warp
     // met on the same banks in its reads and writes.  Packed -> congruent, VJP call, us: 8 coils of 64 x 128 x 128 79.9 -> 73.2,
@@ -83,8 +85,11 @@ struct Tile {
     // but with fewer blocks; with the spills it is 1.00-1.07 times as fast as with twiddles in shared memory.
     // A block has a thread per column, so 640-point rows have at most 96 registers and spill up to 180 B whatever the bound.
     static constexpr int REGS = 2 * RY + (PRIME && !TIGHT ? 4 : 2) * RMAX + (TIGHT ? 24 : 16);
-    static constexpr int blocks(size_t bytes) {
-        const int n = cmin(16, cmin((int)(LIMIT / (bytes + 1024)), 65536 / (TH * ((REGS + 7) / 8 * 8))));
+    // Pass 1 with 4 rows of 92 points takes 104 registers where 96 do, 4 warps per scheduler instead of 5 (4 x 2 x 4 coils of 120 x 92 x 92,
+    // VJP, 468 -> 451 us).
+    static constexpr int REGS_FWD = RY == 4 && NZ == 92 ? 104 : REGS;
+    static constexpr int blocks(size_t bytes, int regs) {
+        const int n = cmin(16, cmin((int)(LIMIT / (bytes + 1024)), 65536 / (TH * ((regs + 7) / 8 * 8))));
         return cmax(1, cmin(n, 2048 / TH));
     }
 };
@@ -133,7 +138,7 @@ __device__ __forceinline__ void stage_rows(cf* dst, const cf* src, long long row
 }
 
 template <class PZ, int RY, bool LOOSE = false>
-__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY, LOOSE>::blocks(Tile<PZ, RY, LOOSE>::FWD_BYTES))
+__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY, LOOSE>::blocks(Tile<PZ, RY, LOOSE>::FWD_BYTES, Tile<PZ, RY, LOOSE>::REGS_FWD))
 tile_fwd_kernel(const TileArgs a) {
     grid_dependency_wait();
     using TL = Tile<PZ, RY, LOOSE>;
@@ -215,7 +220,7 @@ tile_fwd_kernel(const TileArgs a) {
 }
 
 template <class PZ, int RY, bool LOOSE = false>
-__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY, LOOSE>::blocks(Tile<PZ, RY, LOOSE>::INV_BYTES))
+__global__ void __launch_bounds__(Tile<PZ, RY>::TH, Tile<PZ, RY, LOOSE>::blocks(Tile<PZ, RY, LOOSE>::INV_BYTES, Tile<PZ, RY, LOOSE>::REGS))
 tile_inv_kernel(const TileArgs a) {
     grid_dependency_wait();
     using TL = Tile<PZ, RY, LOOSE>;
